@@ -78,14 +78,10 @@ extern "C" size_t lrq_act_workspace_bytes(int M, int K, const lrq_act_params* p)
     return 0;
 }
 
-extern "C" lrq_status lrq_rotate_quantize_act(const void* X, int M, int K, long ldx, const lrq_act_params* p,
-                                              uint8_t* a_codes, float* a_scale, int32_t* a_zp,
-                                              void* workspace, size_t workspace_bytes, void* cuda_stream) {
-    if (!X || !a_codes || !a_scale || !a_zp || M <= 0) return LRQ_ERR_INVALID_ARG;
-    lrq_status st = check_act(p, K);
-    if (st != LRQ_OK) return st;
-    if (ldx < K || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(a_codes, 16)) return LRQ_ERR_INVALID_ARG;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
+// Rotation + quantization of checked arguments; out16: the contraction's bf16 operand instead of packed codes.
+static lrq_status run_act(const void* X, int M, int K, long ldx, const lrq_act_params* p, int out16, uint8_t* a_codes,
+                          float* a_scale, int32_t* a_zp, void* workspace, size_t workspace_bytes, cudaStream_t stream) {
+    lrq_status st;
     if (p->kind == LRQ_ROT_DENSE) {
         const size_t need = lrq_act_workspace_bytes(M, K, p);
         if (!workspace || workspace_bytes < need || !lrq_aligned(workspace, 256)) return LRQ_ERR_WORKSPACE;
@@ -94,7 +90,7 @@ extern "C" lrq_status lrq_rotate_quantize_act(const void* X, int M, int K, long 
         // quantizer reads them and then writes the real values there
         st = lrq_launch_rotgemm(X, M, K, ldx, p->R_bf16, Yr, reinterpret_cast<int*>(a_scale), reinterpret_cast<int*>(a_zp), stream);
         if (st != LRQ_OK) return st;
-        return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, a_codes, a_scale, a_zp, stream);
+        return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, stream);
     }
     if (p->kind == LRQ_ROT_DUAL) {
         const size_t need = lrq_act_workspace_bytes(M, K, p);
@@ -108,10 +104,20 @@ extern "C" lrq_status lrq_rotate_quantize_act(const void* X, int M, int K, long 
         st = lrq_launch_bdiag_gemm(V3, M, K, 3L * K, 3, p->R2_bf16, Yr, reinterpret_cast<int*>(a_scale),
                                    reinterpret_cast<int*>(a_zp), stream);
         if (st != LRQ_OK) return st;
-        return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, a_codes, a_scale, a_zp, stream);
+        return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, stream);
     }
     const int B = p->kind == LRQ_ROT_HADAMARD ? p->had_block : 1;
-    return lrq_launch_rotq_hadamard(X, M, K, ldx, B, p->a_bits, p->mode, p->prescale, a_codes, a_scale, a_zp, stream);
+    return lrq_launch_rotq_hadamard(X, M, K, ldx, B, p->a_bits, p->mode, out16, p->prescale, a_codes, a_scale, a_zp, stream);
+}
+
+extern "C" lrq_status lrq_rotate_quantize_act(const void* X, int M, int K, long ldx, const lrq_act_params* p,
+                                              uint8_t* a_codes, float* a_scale, int32_t* a_zp,
+                                              void* workspace, size_t workspace_bytes, void* cuda_stream) {
+    if (!X || !a_codes || !a_scale || !a_zp || M <= 0) return LRQ_ERR_INVALID_ARG;
+    lrq_status st = check_act(p, K);
+    if (st != LRQ_OK) return st;
+    if (ldx < K || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(a_codes, 16)) return LRQ_ERR_INVALID_ARG;
+    return run_act(X, M, K, ldx, p, 0, a_codes, a_scale, a_zp, workspace, workspace_bytes, (cudaStream_t)cuda_stream);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -207,13 +213,41 @@ extern "C" lrq_status lrq_layer_create(lrq_layer** out, int N, int K, int w_bits
 extern "C" void lrq_layer_destroy(lrq_layer* L) { delete L; }
 
 namespace {
-struct WsLayout { size_t codes, scale, zp, rot, total; };
+// How lrq_qlinear runs a layer on M tokens.
+//   expanded  the quantizer writes the contraction's bf16 operand, the weight codes are decoded to bf16 once, and the
+//             contraction streams both (qgemm_bf16.cu)
+//   packed    both operands stay packed, 256 x 256 tiles that decode them (qgemm_tc.cu)
+//   small     both operands stay packed, 128 x 32 tiles (qgemm_small.cu)
+// The choice depends on the layer and M alone, since the workspace is laid out by it.  Expanded is the rule: a k-block of
+// a tile takes 0.34 us there and 0.1 (3-bit weights, 4-bit activations) to 0.2 us more where it is decoded on the
+// way.  It costs a pass over 2.5 bytes per weight, 0.46 us per million, less a microsecond by which the decoding kernel
+// starts later; few tokens on a large matrix do not earn that back (us per call, expanded / packed, 11360 x 3456, W4A8:
+// M = 256 45.0 / 37.1, M = 333 53.6 / 60.9, M = 1024 75 / 85; W3A4: 256 45.8 / 31.9, 2048 124 / 128; 1152 x 4608, W4A8:
+// 256 26.2 / 36.7).  Batches with fewer than 37 tiles of 256 x 128 keep the small tiles: two launches instead of three, which is
+// what the host can issue in the time such a layer takes.
+enum Form { FORM_SMALL, FORM_PACKED, FORM_EXPANDED };
+Form pick_form(const lrq_layer* L, int M) {
+    const long narrow_tiles = (long)((M + 255) / 256) * ((L->N + 127) / 128);
+    if (narrow_tiles * 4 < 148 && lrq_qgemm_small_takes(L)) return FORM_SMALL;
+    if (lrq_qgemm_tc_takes(L)) {
+        const long tiles = (long)((M + 255) / 256) * ((L->N + 255) / 256);
+        const double rounds = (double)((tiles + 73) / 74);           // of tiles over the CTA pairs
+        const double decode_us = rounds * (L->K / 64) * (L->w_bits == 3 && L->act.a_bits == 4 ? 0.1 : 0.2);
+        if (decode_us < 0.46e-6 * L->N * (double)L->K - 1.0) return FORM_PACKED;
+    }
+    return FORM_EXPANDED;
+}
+
+struct WsLayout { size_t codes, scale, zp, wexp, rot, total; Form form; };
 WsLayout ws_layout(const lrq_layer* L, int M) {
     WsLayout w;
     size_t off = 0;
-    w.codes = off; off += lrq_round_up((size_t)M * L->K * L->act.a_bits / 8, 256);
+    w.form = pick_form(L, M);
+    const bool ex = w.form == FORM_EXPANDED;
+    w.codes = off; off += lrq_round_up(ex ? (size_t)M * L->K * 2 : (size_t)M * L->K * L->act.a_bits / 8, 256);
     w.scale = off; off += lrq_round_up((size_t)M * sizeof(float), 256);
     w.zp = off;    off += lrq_round_up((size_t)M * sizeof(int32_t), 256);
+    w.wexp = off;  off += ex ? lrq_round_up((size_t)L->N * L->K * 2, 256) : 0;
     w.rot = off;   off += lrq_act_workspace_bytes(M, L->K, &L->act);
     w.total = off;
     return w;
@@ -233,30 +267,6 @@ static lrq_status check_out(const void* Y, lrq_dtype dt, long ldy, int N) {
     return LRQ_OK;
 }
 
-// Which contraction kernel a call takes.  impl: 0 large-tile tcgen05, 1 CUDA cores, 2 small-tile tcgen05, 3 CUDA cores
-// in the integer shift form, -1 automatic:
-// the small-tile kernel for packed 3-bit codes and for batches that give the large-tile kernel fewer tiles than half
-// the CTA pairs of the device (a few hundred tokens), the large-tile kernel otherwise, the CUDA cores for shapes
-// neither takes.
-static lrq_status qgemm_dispatch(const lrq_layer* L, const uint8_t* a_codes, const float* a_scale,
-                                 const int32_t* a_zp, int M, void* Y, lrq_dtype dt, long ldy, int impl,
-                                 cudaStream_t st) {
-    if (impl == 1) return lrq_launch_qgemm_simple(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, st);
-    if (impl == 2) return lrq_launch_qgemm_small(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, st);
-    if (impl == 3) return lrq_launch_qgemm_shift(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, st);
-    if (impl == 0) return lrq_launch_qgemm_tc(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, st);
-    lrq_status s = LRQ_ERR_UNSUPPORTED;
-    if (lrq_qgemm_small_takes(L)) {
-        int sms = 0;
-        if (lrq_current_device(nullptr, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
-        const long narrow_tiles = (long)((M + 255) / 256) * ((L->N + 127) / 128);
-        if (L->packed3 || narrow_tiles * 4 < sms) s = lrq_launch_qgemm_small(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, st);
-    }
-    if (s == LRQ_ERR_UNSUPPORTED) s = lrq_launch_qgemm_tc(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, st);
-    if (s == LRQ_ERR_UNSUPPORTED) s = lrq_launch_qgemm_simple(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, st);
-    return s;
-}
-
 extern "C" lrq_status lrq_qgemm_codes(const lrq_layer* L, const uint8_t* a_codes, const float* a_scale,
                                       const int32_t* a_zp, int M, void* Y, lrq_dtype dt, long ldy, int impl,
                                       void* cuda_stream) {
@@ -265,7 +275,13 @@ extern "C" lrq_status lrq_qgemm_codes(const lrq_layer* L, const uint8_t* a_codes
     lrq_status st = check_out(Y, dt, ldy, L->N);
     if (st != LRQ_OK) return st;
     if (!lrq_aligned(a_codes, 16)) return LRQ_ERR_INVALID_ARG;
-    return qgemm_dispatch(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, impl, (cudaStream_t)cuda_stream);
+    cudaStream_t stream = (cudaStream_t)cuda_stream;
+    switch (impl) {
+        case 0: return lrq_launch_qgemm_tc(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
+        case 1: return lrq_launch_qgemm_simple(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
+        case 2: return lrq_launch_qgemm_small(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
+        default: return lrq_launch_qgemm_shift(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
+    }
 }
 
 // Every check lrq_qlinear makes on one layer's arguments; nothing is launched here.
@@ -288,10 +304,17 @@ extern "C" lrq_status lrq_qlinear(const lrq_layer* L, const void* X, int M, long
     uint8_t* a_codes = reinterpret_cast<uint8_t*>(base + w.codes);
     float* a_scale = reinterpret_cast<float*>(base + w.scale);
     int32_t* a_zp = reinterpret_cast<int32_t*>(base + w.zp);
-    st = lrq_rotate_quantize_act(X, M, L->K, ldx, &L->act, a_codes, a_scale, a_zp, base + w.rot,
-                                 w.total - w.rot, cuda_stream);
+    cudaStream_t stream = (cudaStream_t)cuda_stream;
+    const bool ex = w.form == FORM_EXPANDED;
+    if (ex) {
+        st = lrq_launch_expand_w(L, base + w.wexp, stream);
+        if (st != LRQ_OK) return st;
+    }
+    st = run_act(X, M, L->K, ldx, &L->act, ex ? 1 : 0, a_codes, a_scale, a_zp, base + w.rot, w.total - w.rot, stream);
     if (st != LRQ_OK) return st;
-    return qgemm_dispatch(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, -1, (cudaStream_t)cuda_stream);
+    if (ex) return lrq_launch_qgemm_bf16(L, a_codes, base + w.wexp, a_scale, a_zp, M, Y, dt, ldy, stream);
+    if (w.form == FORM_PACKED) return lrq_launch_qgemm_tc(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
+    return lrq_launch_qgemm_small(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
 }
 
 extern "C" lrq_status lrq_qlinear_stack(const lrq_layer* const* layers, int n_layers, const void* const* X,

@@ -58,11 +58,13 @@ inline cudaError_t lrq_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block,
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// Quantizers: out16 == 0 writes packed 8- or 4-bit codes, out16 == 1 the contraction's operand instead, bf16 [M,K] of
+// q - 2^(a_bits-1) (16-byte aligned rows), from the same arithmetic.
 // rotq.cu
-lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, const float* prescale,
+lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                                     uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st);
 // rotq_blk.cu : the same for blocks of 8..128 channels with K a multiple of 128; LRQ_ERR_UNSUPPORTED otherwise
-lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, const float* prescale,
+lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                                uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st);
 // rotgemm.cu : Y[M,K] (fp32) = X[M,K] (bf16) . R[K,K] (bf16) on the tensor cores; also leaves every row's minimum and
 // maximum in ext_min[M] / ext_max[M] as order-preserving integers.
@@ -76,7 +78,7 @@ lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int part
 lrq_status lrq_launch_dual_gather_split(const float* U, int M, int K, const int32_t* perm, void* V3, cudaStream_t st);
 // rotq.cu : per-token quantization of fp32 rows whose extremes are already known (ext_min / ext_max alias the
 // scale / zero-point outputs: each row's extremes are read before its results are written).
-lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int a_bits, int mode, uint8_t* codes,
+lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int a_bits, int mode, int out16, uint8_t* codes,
                                        float* scale, int32_t* zp, cudaStream_t st);
 
 // rotq.cu : fluctuation metric J (Eq. 11) and the kind Eq. 12 picks; acc is one double of device scratch
@@ -107,12 +109,18 @@ lrq_status lrq_launch_qgemm_simple(const lrq_layer* L, const uint8_t* a_codes, c
 // qgemm_simple.cu : the integer form of Eq. 10 (mantissa products, shifts, exact integer accumulation) on the CUDA cores
 lrq_status lrq_launch_qgemm_shift(const lrq_layer* L, const uint8_t* a_codes, const float* a_scale,
                                   const int32_t* a_zp, int M, void* Y, lrq_dtype dt, long ldy, cudaStream_t st);
+bool lrq_qgemm_tc_takes(const lrq_layer* L);
 lrq_status lrq_launch_qgemm_tc(const lrq_layer* L, const uint8_t* a_codes, const float* a_scale,
                                const int32_t* a_zp, int M, void* Y, lrq_dtype dt, long ldy, cudaStream_t st);
 // qgemm_small.cu : 128 x 32 tiles, one CTA each, for small token counts and for packed 3-bit codes
 bool lrq_qgemm_small_takes(const lrq_layer* L);
 lrq_status lrq_launch_qgemm_small(const lrq_layer* L, const uint8_t* a_codes, const float* a_scale,
                                   const int32_t* a_zp, int M, void* Y, lrq_dtype dt, long ldy, cudaStream_t st);
+// expand_w.cu : the layer's weight codes decoded to bf16 [N,K]
+lrq_status lrq_launch_expand_w(const lrq_layer* L, void* out, cudaStream_t st);
+// qgemm_bf16.cu : contraction of bf16 operands, A [M,K] of q - 2^(a_bits-1), W [N,K] of decoded levels (both 16-byte aligned)
+lrq_status lrq_launch_qgemm_bf16(const lrq_layer* L, const void* A, const void* W, const float* a_scale, const int32_t* a_zp, int M,
+                                 void* Y, lrq_dtype dt, long ldy, cudaStream_t st);
 // fills the layer's cached TMA descriptors (called once by lrq_layer_create; never fails: without a driver, or for
 // shapes the tensor-core kernel does not take, the layer is simply left without them)
 void lrq_qgemm_tc_prepare(lrq_layer* L);

@@ -1,0 +1,422 @@
+// Contraction + epilogue on operands that are already bf16 (Sec. 4.1, Eq. 10): the kernel lrq_qlinear takes for
+// almost every layer (the rule is in api.cu).
+//
+//   acc[m,n] = sum_k a[m,k] * w[n,k]                     exact bf16 products, fp32 accumulation in TMEM
+//   Y[m,n]   = s_m * (acc + (z_m + C) * wsum_n) * wscale_n + bias_n
+//
+// a = q - C are the centred activation codes (C = 128 or 8) as the quantizer wrote them, w the decoded levels
+// (expand_w.cu).  Nothing is left to do between the copy and the tensor core, so both operands go from global memory
+// to their stages by TMA alone, and the kernel is bound by the tensor pipe and, over more than a tenth of a second, by
+// the power cap: what counts then is the energy of a tile, of which DRAM and cross-die L2 traffic are a good part.
+//
+// A pair of CTAs (cluster of two, cta_group::2) owns 256 tokens x up to 256 channels; each CTA holds its 128 rows of A
+// and half of the B rows (32 KB per 64-deep k-block, STAGES deep).  Both CTAs' copies complete on the even CTA's
+// barrier, whose MMA warp issues the MMAs; stage release and accumulator completion come back by multicast commit.
+//   warp 0  TMA producer   warp 1  TMEM, MMA issue   warps 2-5  epilogue (tcgen05.ld, scale, TMA store)
+// The accumulator is double-buffered (2 x 256 columns): one tile's epilogue overlaps the next one's main loop.
+// Tiles are dealt in the order of struct Plan; with neighbouring tiles at different columns instead, DRAM reads of the
+// 4608 x 12288 x 3072 contraction were 940 MB instead of 190 and it took 265 us instead of 211 (1650 TFLOP/s, at the
+// matmul peak; the kernel that decodes on the way: 300).  Issued by whole warps (see elect_one): 4096 x 1152 x 4608
+// takes 35 us, with a loop inside `lane == 0` 47.
+// Every wait is bounded, as in the other kernels; on expiry the CTA records a code, its copies in flight land, and both
+// CTAs meet at the final cluster barrier.
+#include "lrq_internal.cuh"
+#include "tc_ptx.cuh"
+#include "f32x2.cuh"
+#include "tma_host.cuh"
+#include <mutex>
+
+namespace {
+using namespace lrq_tc;
+using namespace lrq_f2;
+
+constexpr int BM_CTA = 128, BM = 2 * BM_CTA, BN = 256, BK = 64;
+constexpr int UNIT = 64;                                    // granularity of tile widths
+constexpr int STAGES = 6;
+constexpr int A_STAGE_BYTES = BM_CTA * BK * 2;              // 16 KB
+constexpr int B_STAGE_BYTES = (BN / 2) * BK * 2;            // 16 KB
+constexpr int TMA_WARP = 0, MMA_WARP = 1, EPI_WARP0 = 2, NUM_EPI_WARPS = 4;
+constexpr int NUM_THREADS = (EPI_WARP0 + NUM_EPI_WARPS) * 32;
+constexpr int TMEM_COLS = 512;
+constexpr int EPI_TILE_BYTES = 32 * 128;                    // 32 rows of 128 bytes per epilogue warp, staged for a TMA store
+
+struct __align__(16) Ctl {
+    uint64_t full[STAGES];        // stage filled in both CTAs            (even CTA; both CTAs' copies complete on it)
+    uint64_t empty[STAGES];       // stage consumed by the MMAs           (each CTA, multicast commit)
+    uint64_t tmem_full[2];        // accumulator complete                 (each CTA, multicast commit)
+    uint64_t tmem_empty[2];       // accumulator drained by both CTAs     (even CTA)
+    uint32_t tmem_base;
+    volatile int abort_flag;
+    alignas(16) float col[2][3][BN];    // per TMEM buffer: wsum, wscale, bias of the tile's columns
+};
+constexpr size_t SMEM_BYTES = 1024 + (size_t)STAGES * (A_STAGE_BYTES + B_STAGE_BYTES) + (size_t)NUM_EPI_WARPS * EPI_TILE_BYTES + sizeof(Ctl);
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
+
+// Order of the tiles.  Whole tiles (256 x 256) come first, panel by panel (gm token rows each), a panel's columns one
+// after the other, its rows fastest, so that the tiles which run at the same time form a compact rectangle of the output
+// and share both operands in L2.  The last `split` whole tiles are cut into `pieces` parts each when that lets the
+// last round spread over pairs that would idle.  The ragged last column (width < 256) comes at the end.
+// Pair p takes positions p, 2P-1-p, 2P+p, 4P-1-p, ...: rounds run forwards and backwards in turn, so that the pairs
+// whose last tile was a narrow one get the next.
+struct Plan {
+    int rows, cols, gm;           // 256-token rows, whole columns, rows per panel
+    int whole, split, pieces;     // whole tiles in all, of which cut at the end, parts per cut tile
+    int ragged, total;            // width of the ragged column (0: none), positions in all
+};
+struct Tile { int row, col, width; };            // 256-token row, first channel, channels (a multiple of UNIT)
+
+__device__ inline Tile tile_at(const Plan& p, int i) {
+    Tile t;
+    const int uncut = p.whole - p.split, cut = uncut + p.split * p.pieces;
+    if (i >= cut) { t.row = i - cut; t.col = p.cols * BN; t.width = p.ragged; return t; }
+    int q = i, part = 0;
+    t.width = BN;
+    if (i >= uncut) { q = uncut + (i - uncut) / p.pieces; part = (i - uncut) % p.pieces; t.width = BN / p.pieces; }
+    const int panel = q / (p.gm * p.cols), r0 = panel * p.gm, in = q - r0 * p.cols;
+    const int h = p.rows - r0 < p.gm ? p.rows - r0 : p.gm;
+    t.col = (in / h) * BN + part * t.width;
+    t.row = r0 + in % h;
+    return t;
+}
+
+struct Params {
+    const float* a_scale; const int32_t* a_zp; const float* wsum; const float* wscale; const float* bias;
+    int M, N, K, bf16_out; float zoff; int* status;
+    Plan plan;
+};
+
+__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+// Named barrier 1 over the epilogue warps, returning the OR of `pred` over all of them.
+__device__ __forceinline__ bool bar_or_epilogue(bool pred) {
+    uint32_t r;
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.u32 q, %1, 0;\n"
+        "bar.red.or.pred p, 1, %2, q;\n"
+        "selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(r) : "r"((uint32_t)pred), "n"(NUM_EPI_WARPS * 32) : "memory");
+    return r != 0;
+}
+
+// A pair's walk over its positions.
+struct Walk {
+    const Plan& p;
+    int pair, pairs, round;
+    Tile t;
+    __device__ Walk(const Plan& plan, int pair_, int pairs_) : p(plan), pair(pair_), pairs(pairs_), round(0) {}
+    __device__ __forceinline__ bool next() {
+        const int i = round * pairs + ((round & 1) ? pairs - 1 - pair : pair);
+        ++round;
+        if (i >= p.total) return false;
+        t = tile_at(p, i);
+        return true;
+    }
+};
+
+// Copies of a CTA pair: the transaction is counted on the barrier at `bar` of the even CTA (a shared::cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void* tmap, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
+template <bool OUT16>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
+                  const __grid_constant__ CUtensorMap tmWs, const __grid_constant__ CUtensorMap tmWr, const __grid_constant__ CUtensorMap tmY) {
+    extern __shared__ unsigned char smem_dyn[];
+    unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+    const uint32_t sA = smem_u32(base), sB = sA + STAGES * A_STAGE_BYTES, sEpi = sB + STAGES * B_STAGE_BYTES;
+    Ctl* ctl = reinterpret_cast<Ctl*>(base + STAGES * (A_STAGE_BYTES + B_STAGE_BYTES) + NUM_EPI_WARPS * EPI_TILE_BYTES);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();
+    const int kblocks = (p.K + BK - 1) / BK;                 // a ragged last block is zero-filled in both operands
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) { mbar_init(smem_u32(&ctl->full[s]), 1); mbar_init(smem_u32(&ctl->empty[s]), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&ctl->tmem_full[b]), 1); mbar_init(smem_u32(&ctl->tmem_empty[b]), 2 * NUM_EPI_WARPS); }
+        ctl->abort_flag = 0;
+        mbar_init_fence();
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmW);
+        if (p.plan.split) tma_prefetch_desc(&tmWs);
+        if (p.plan.ragged) tma_prefetch_desc(&tmWr);
+        tma_prefetch_desc(&tmY);
+    }
+    if (warp == MMA_WARP) tmem_alloc_pair(smem_u32(&ctl->tmem_base), TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                       // the peer's barriers exist before anyone arrives on them
+    tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    lrq_pdl_trigger();
+    lrq_pdl_wait();                           // everything above overlaps the previous kernel's tail
+    Walk walk(p.plan, blockIdx.x >> 1, gridDim.x >> 1);
+
+    if (warp == TMA_WARP) {
+        const bool lead = elect_one();
+        int s = 0;
+        uint32_t ph = 1, issued = 0;
+        bool ok = true;
+        const uint32_t full0 = map_to_cta(smem_u32(&ctl->full[0]), 0);
+        while (ok && walk.next()) {
+            const int m0 = walk.t.row * BM + (int)rank * BM_CTA;
+            const int half = walk.t.width / 2;               // B rows of this CTA
+            const int n0 = walk.t.col + (int)rank * half;
+            const uint32_t tx = 2u * (A_STAGE_BYTES + (uint32_t)half * (BK * 2));
+            const CUtensorMap* map_w = walk.t.width == BN ? &tmW : walk.t.col == p.plan.cols * BN ? &tmWr : &tmWs;
+            for (int kb = 0; kb < kblocks; ++kb) {
+                ok = mbar_wait_warp(smem_u32(&ctl->empty[s]), ph, &ctl->abort_flag, p.status, 41);
+                if (!ok) break;
+                if (lead) {
+                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[s]), tx);
+                    tma_load_2d_pair(sA + s * A_STAGE_BYTES, &tmA, kb * BK, m0, full0 + 8 * s);
+                    tma_load_2d_pair(sB + s * B_STAGE_BYTES, map_w, kb * BK, n0, full0 + 8 * s);
+                }
+                __syncwarp();
+                ++issued;
+                if (++s == STAGES) { s = 0; ph ^= 1; }
+            }
+        }
+        if (!ok && issued) {
+            // Copies in flight still write this CTA's shared memory, and the peer's barrier counts them: they have
+            // a millisecond to land, three orders above their latency, before the CTAs meet and end.
+            const long long t0 = clock64();
+            while (clock64() - t0 < 2000000) __nanosleep(1000);
+        }
+        __syncwarp();
+    } else if (warp == MMA_WARP) {
+        if (rank == 0) {
+            const bool lead = elect_one();
+            const uint64_t a0 = umma_desc_sw128(sA, 16, 1024), b0 = umma_desc_sw128(sB, 16, 1024);
+            int s = 0;
+            uint32_t ph = 0, t = 0;
+            bool ok = true;
+            while (ok && walk.next()) {
+                const uint32_t buf = t & 1;
+                ok = mbar_wait_warp(smem_u32(&ctl->tmem_empty[buf]), ((t >> 1) & 1) ^ 1, &ctl->abort_flag, p.status, 42);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + buf * BN;
+                const uint32_t idesc = umma_idesc_bf16(BM, walk.t.width, false, false);
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    ok = mbar_wait_warp(smem_u32(&ctl->full[s]), ph, &ctl->abort_flag, p.status, 43);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (lead) {
+                        const uint64_t a = a0 + (uint64_t)(s * (A_STAGE_BYTES >> 4)), b = b0 + (uint64_t)(s * (B_STAGE_BYTES >> 4));
+#pragma unroll
+                        for (int k = 0; k < BK / 16; ++k)    // 16 k = 32 bytes along the row: 2 in descriptor units
+                            tc_mma_f16_pair(d_tmem, a + 2 * k, b + 2 * k, idesc, (kb | k) ? 1u : 0u);
+                        tc_commit_pair(smem_u32(&ctl->empty[s]), 3);
+                    }
+                    __syncwarp();
+                    if (++s == STAGES) { s = 0; ph ^= 1; }
+                }
+                if (ok && lead) tc_commit_pair(smem_u32(&ctl->tmem_full[buf]), 3);
+                __syncwarp();
+                ++t;
+            }
+        }
+        __syncwarp();
+    } else {
+        const int ew = warp & 3;                             // TMEM lane quadrant this warp may read
+        const int et = threadIdx.x - EPI_WARP0 * 32;
+        const bool has_ws = p.wscale != nullptr, has_bias = p.bias != nullptr;
+        const uint32_t tile = sEpi + (uint32_t)(warp - EPI_WARP0) * EPI_TILE_BYTES;
+        uint32_t t = 0;
+        while (walk.next()) {
+            const int mw = walk.t.row * BM + (int)rank * BM_CTA + ew * 32, m = mw + lane, n0 = walk.t.col;
+            const int width = min(walk.t.width, p.N - n0);
+            const uint32_t buf = t & 1;
+            float (*col)[BN] = ctl->col[buf];
+            for (int c = et; c < walk.t.width; c += NUM_EPI_WARPS * 32) {
+                const int n = n0 + c;
+                const bool okc = c < width;
+                col[0][c] = okc ? __ldg(p.wsum + n) : 0.f;
+                if (has_ws) col[1][c] = okc ? __ldg(p.wscale + n) : 1.f;
+                if (has_bias) col[2][c] = okc ? __ldg(p.bias + n) : 0.f;
+            }
+            if (bar_or_epilogue(ctl->abort_flag != 0)) break;     // the epilogue warps leave together
+            const bool row_ok = m < p.M;
+            const float sm = row_ok ? __ldg(p.a_scale + m) : 0.f;
+            const float zm = row_ok ? (float)__ldg(p.a_zp + m) + p.zoff : 0.f;
+            const f32x2 SM = pack2(sm, sm), ZM = pack2(zm, zm);
+            const bool ok = mbar_wait_warp<100>(smem_u32(&ctl->tmem_full[buf]), (t >> 1) & 1, &ctl->abort_flag, p.status, 44);
+            tc_fence_after();
+            if (ok && mw < p.M) {
+                const uint32_t acc0 = tmem_base + ((uint32_t)(ew * 32) << 16) + buf * BN;
+#pragma unroll 1
+                for (int c0 = 0; c0 < width; c0 += 32) {
+                    uint32_t acc[32];
+                    tc_ld32(acc0 + (uint32_t)c0, acc);
+                    tc_wait_ld();
+                    // y = s_m * (acc + z_m * wsum_n) [* wscale_n] [+ bias_n], two columns per instruction
+                    f32x2 y[16];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 ws = *reinterpret_cast<const float4*>(&col[0][c0 + 4 * j]);
+                        f32x2 a0 = fma2(ZM, pack2(ws.x, ws.y), pack2(__uint_as_float(acc[4 * j]), __uint_as_float(acc[4 * j + 1])));
+                        f32x2 a1 = fma2(ZM, pack2(ws.z, ws.w), pack2(__uint_as_float(acc[4 * j + 2]), __uint_as_float(acc[4 * j + 3])));
+                        a0 = mul2(a0, SM); a1 = mul2(a1, SM);
+                        if (has_ws) {
+                            const float4 sc = *reinterpret_cast<const float4*>(&col[1][c0 + 4 * j]);
+                            a0 = mul2(a0, pack2(sc.x, sc.y)); a1 = mul2(a1, pack2(sc.z, sc.w));
+                        }
+                        if (has_bias) {
+                            const float4 bi = *reinterpret_cast<const float4*>(&col[2][c0 + 4 * j]);
+                            a0 = add2(a0, pack2(bi.x, bi.y)); a1 = add2(a1, pack2(bi.z, bi.w));
+                        }
+                        y[2 * j] = a0; y[2 * j + 1] = a1;
+                    }
+                    // The warp lays its 32 x 128-byte chunk out in shared memory (128-byte swizzle: conflict-free) and
+                    // one lane hands it to the TMA, which writes whole lines and clips rows past M and columns past N.
+                    const int half = OUT16 ? (c0 >> 5) & 1 : 0;
+                    if (half == 0) {
+                        if (lane == 0) tma_store_wait_read<0>();         // the store that last read this tile is done with it
+                        __syncwarp();
+                    }
+                    if (OUT16) {
+                        uint32_t h[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            float a, b;
+                            unpack2(y[j], a, b);
+                            if (p.bf16_out) { __nv_bfloat162 v = __floats2bfloat162_rn(a, b); h[j] = *reinterpret_cast<uint32_t*>(&v); }
+                            else { __half2 v = __floats2half2_rn(a, b); h[j] = *reinterpret_cast<uint32_t*>(&v); }
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            sts128(tile + (uint32_t)(lane * 128 + (((half * 4 + j) ^ (lane & 7)) << 4)), h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            float a, b, c, d;
+                            unpack2(y[2 * j], a, b); unpack2(y[2 * j + 1], c, d);
+                            sts128(tile + (uint32_t)(lane * 128 + ((j ^ (lane & 7)) << 4)), __float_as_uint(a), __float_as_uint(b),
+                                   __float_as_uint(c), __float_as_uint(d));
+                        }
+                    }
+                    if (!OUT16 || half == 1 || c0 + 32 >= width) {
+                        fence_async_smem();
+                        __syncwarp();
+                        if (lane == 0) tma_store_2d(&tmY, n0 + (OUT16 ? (c0 & ~63) : c0), mw, tile);
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            // CTA-scope release is enough: the accumulator reads above have completed (tcgen05.wait::ld)
+            if (lane == 0) mbar_arrive_cluster_light(smem_u32(&ctl->tmem_empty[buf]), 0);
+            ++t;
+        }
+        if (lane == 0) tma_store_wait_all();                 // output tiles still in flight read this CTA's shared memory
+    }
+
+    // teardown: neither CTA may exit (or release TMEM) while its peer can still arrive on its barriers or have MMAs
+    // reading its shared memory
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    if (warp == MMA_WARP) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, TMEM_COLS);
+    }
+}
+
+template <bool OUT16>
+lrq_status max_pairs(int dev, int sms, int* out) {
+    // per device and kernel variant: the shared-memory opt-in and the number of CTA pairs that can be resident
+    static std::mutex mu;
+    static int max_pairs_of[LRQ_MAX_DEVICES] = {};
+    std::lock_guard<std::mutex> lock(mu);
+    if (!max_pairs_of[dev]) {
+        LRQ_CUDA_TRY(cudaFuncSetAttribute(qgemm_bf16_kernel<OUT16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(sms & ~1); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = SMEM_BYTES;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int clusters = 0;
+        LRQ_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, qgemm_bf16_kernel<OUT16>, &cfg));
+        if (clusters < 1) return LRQ_ERR_CUDA;
+        max_pairs_of[dev] = clusters < sms / 2 ? clusters : sms / 2;
+    }
+    *out = max_pairs_of[dev];
+    return LRQ_OK;
+}
+
+Plan make_plan(int M, int N, int K, int pairs) {
+    Plan p;
+    p.rows = (M + BM - 1) / BM;
+    p.cols = N / BN;
+    p.ragged = (N % BN + UNIT - 1) / UNIT * UNIT;
+    if (p.ragged == BN) { ++p.cols; p.ragged = 0; }          // the last whole column is clipped by the copies
+    p.whole = p.rows * p.cols;
+    const int narrow = p.ragged ? p.rows : 0, left = p.whole % pairs;
+    p.pieces = left * 4 + narrow <= pairs ? 4 : left * 2 + narrow <= pairs ? 2 : 1;
+    p.split = p.pieces > 1 ? left : 0;
+    p.total = p.whole - p.split + p.split * p.pieces + narrow;
+    // Rows per panel: the fewest bytes from DRAM.  A panel's A is read once while it fits into half of the L2 (the other half
+    // holds B's moving window and the outputs), else once per round of its columns; B once per panel unless it fits itself.
+    const double a_row = 2.0 * BM * K, b_all = 2.0 * N * K, l2 = 60e6;
+    double best = 1e300;
+    p.gm = 1;
+    for (int panels = 1; panels <= 16 && panels <= p.rows; ++panels) {
+        const int gm = (p.rows + panels - 1) / panels;
+        const double rounds = gm * a_row <= l2 ? 1.0 : (double)p.cols * gm / pairs;
+        const double cost = p.rows * a_row * (rounds < 1.0 ? 1.0 : rounds) + (b_all <= l2 / 2 ? 1.0 : (double)panels) * b_all +
+                            1e-3 * gm * a_row;               // among equals the smaller panel
+        if (cost < best) { best = cost; p.gm = gm; }
+    }
+    return p;
+}
+
+}  // namespace
+
+lrq_status lrq_launch_qgemm_bf16(const lrq_layer* L, const void* A, const void* W, const float* a_scale, const int32_t* a_zp, int M,
+                                 void* Y, lrq_dtype dt, long ldy, cudaStream_t st) {
+    const size_t es = dt == LRQ_F32 ? 4 : 2;
+    int dev = 0, sms = 0, pairs = 0;
+    if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
+    const lrq_status rs = dt == LRQ_F32 ? max_pairs<false>(dev, sms, &pairs) : max_pairs<true>(dev, sms, &pairs);
+    if (rs != LRQ_OK) return rs;
+    Params p;
+    p.a_scale = a_scale; p.a_zp = a_zp; p.wsum = L->wsum; p.wscale = L->wscale; p.bias = L->bias;
+    p.M = M; p.N = L->N; p.K = L->K; p.bf16_out = dt == LRQ_BF16; p.zoff = L->act.a_bits == 8 ? 128.f : 8.f;
+    p.status = lrq_status_word();
+    if ((long)((M + BM - 1) / BM) * ((L->N + BN - 1) / BN) > (1l << 28)) return LRQ_ERR_UNSUPPORTED;
+    p.plan = make_plan(M, L->N, L->K, pairs);
+    // weight boxes are half a tile's width: whole tiles, the parts of cut ones, the ragged column
+    CUtensorMap tmA, tmW, tmWs, tmWr, tmY;
+    auto map_w = [&](CUtensorMap* tm, int width) {
+        return lrq_tma::make_map_2d(tm, W, 2, (uint64_t)L->N, (uint64_t)L->K, (uint64_t)L->K, BK, (uint32_t)width / 2, true);
+    };
+    if (!lrq_tma::make_map_2d(&tmA, A, 2, (uint64_t)M, (uint64_t)L->K, (uint64_t)L->K, BK, BM_CTA, true) || !map_w(&tmW, BN) ||
+        !lrq_tma::make_map_2d(&tmY, Y, (int)es, (uint64_t)M, (uint64_t)L->N, (uint64_t)ldy, dt == LRQ_F32 ? 32 : 64, 32, true))
+        return LRQ_ERR_CUDA;
+    tmWs = tmWr = tmW;
+    if (p.plan.split && !map_w(&tmWs, BN / p.plan.pieces)) return LRQ_ERR_CUDA;
+    if (p.plan.ragged && !map_w(&tmWr, p.plan.ragged)) return LRQ_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(2 * (p.plan.total < pairs ? p.plan.total : pairs));
+    cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = st;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    LRQ_CUDA_TRY(dt == LRQ_F32 ? cudaLaunchKernelEx(&cfg, qgemm_bf16_kernel<false>, p, tmA, tmW, tmWs, tmWr, tmY)
+                               : cudaLaunchKernelEx(&cfg, qgemm_bf16_kernel<true>, p, tmA, tmW, tmWs, tmWr, tmY));
+    return LRQ_OK;
+}

@@ -689,6 +689,8 @@ bool make_w_map(const lrq_layer* L, bool narrow, CUtensorMap* tm) {
 
 }  // namespace
 
+bool lrq_qgemm_tc_takes(const lrq_layer* L) { return tc_shape_ok(L); }
+
 void lrq_qgemm_tc_prepare(lrq_layer* L) {
     L->have_tm_w = tc_shape_ok(L) && make_w_map(L, false, &L->tm_w_wide) && make_w_map(L, true, &L->tm_w_narrow);
 }

@@ -68,7 +68,7 @@ __device__ __forceinline__ int quant1(float u, const TokenQ& t, int qmax) {
 // Any B = 2^n (8..4096) dividing K, any K that is a multiple of 8.
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log2B, int a_bits, int mode,
+rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log2B, int a_bits, int mode, int out16,
                     const float* __restrict__ prescale,
                     uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp) {
     extern __shared__ float row[];
@@ -136,7 +136,11 @@ rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log
     __syncthreads();
     const TokenQ t = tq;
     const int qmax = (1 << a_bits) - 1;
-    if (a_bits == 8) {
+    if (out16) {                                              // the contraction's centred bf16 operand
+        const int C = 1 << (a_bits - 1);
+        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(codes) + (size_t)m * K;
+        for (int k = tid; k < K; k += nthr) dst[k] = __float2bfloat16_rn((float)(quant1(row[k], t, qmax) - C));
+    } else if (a_bits == 8) {
         uint2* dst = reinterpret_cast<uint2*>(codes + (size_t)m * K);
         for (int c = tid; c < nchunk; c += nthr) {
             uint32_t w[2] = {0, 0};
@@ -197,7 +201,7 @@ __device__ __forceinline__ void load_raw(const __nv_bfloat16* p, uint4* raw) {
 
 template <int LOG2B, int A_BITS, int MAX_THREADS, int MIN_CTAS, bool WIDE>
 __global__ void __launch_bounds__(MAX_THREADS, MIN_CTAS)
-rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int mode, int tok_per_cta, int num_groups,
+rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int mode, int out16, int tok_per_cta, int num_groups,
                  const float* __restrict__ prescale,
                  uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -310,6 +314,14 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
         if (tid < 2 * tok_per_cta) ext[((it + 2) % 3) * 2 * tok_per_cta + tid] = (tid & 1) ? INT_MIN : INT_MAX;
         if (live) {
             const f32x2 INV = pack2(t.inv, t.inv), NEGZ = pack2(t.negz, t.negz);
+            if (out16) {                                      // the contraction's centred bf16 operand
+                uint4* dst = reinterpret_cast<uint4*>(codes + 2 * ((size_t)m * K + (size_t)j * EPT));
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    dst[i] = make_uint4(centred_bf16x2<A_BITS>(fma2(P[4 * i], INV, NEGZ)), centred_bf16x2<A_BITS>(fma2(P[4 * i + 1], INV, NEGZ)),
+                                        centred_bf16x2<A_BITS>(fma2(P[4 * i + 2], INV, NEGZ)), centred_bf16x2<A_BITS>(fma2(P[4 * i + 3], INV, NEGZ)));
+                continue;
+            }
             int q[EPT];
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
@@ -360,7 +372,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
 // ------------------------------------------------------------------------------------------------
 template <int LOG2B, int A_BITS, int MAX_THREADS, int MIN_CTAS, bool WIDE>
 __global__ void __launch_bounds__(MAX_THREADS, MIN_CTAS)
-rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int mode, int tok_per_cta, int num_groups,
+rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int mode, int out16, int tok_per_cta, int num_groups,
                 const float* __restrict__ prescale,
                 uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp) {
     static_assert(LOG2B >= 10 && LOG2B <= 12, "block sizes 1024..4096");
@@ -516,6 +528,13 @@ rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int
             const size_t e0 = (size_t)m * K + (size_t)unit_in_token * (U * 1024) + (size_t)tau * 8;
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
+                const size_t e = e0 + (size_t)r * (U * 256);
+                if (out16) {                                  // the contraction's centred bf16 operand
+                    *reinterpret_cast<uint4*>(codes + 2 * e) =
+                        make_uint4(centred_bf16x2<A_BITS>(fma2(P[4 * r], INV, NEGZ)), centred_bf16x2<A_BITS>(fma2(P[4 * r + 1], INV, NEGZ)),
+                                   centred_bf16x2<A_BITS>(fma2(P[4 * r + 2], INV, NEGZ)), centred_bf16x2<A_BITS>(fma2(P[4 * r + 3], INV, NEGZ)));
+                    continue;
+                }
                 int q[8];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -523,7 +542,6 @@ rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int
                     unpack2(fma2(P[4 * r + i], INV, NEGZ), x, y);
                     q[2 * i] = __float2int_rn(x); q[2 * i + 1] = __float2int_rn(y);
                 }
-                const size_t e = e0 + (size_t)r * (U * 256);
                 if (A_BITS == 8) {
                     *reinterpret_cast<uint2*>(codes + e) = make_uint2(pack_u8x4(q[0], q[1], q[2], q[3]), pack_u8x4(q[4], q[5], q[6], q[7]));
                 } else {
@@ -540,7 +558,7 @@ rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int
 // streams the row: 32 bytes in (one 256-bit load), 8 or 4 code bytes out per lane and step.
 // ext_min / ext_max alias scale / zp: the warp reads its row's extremes before it writes the results.
 // ------------------------------------------------------------------------------------------------
-template <int A_BITS>
+template <int A_BITS, bool OUT16>
 __global__ void __launch_bounds__(256)
 quant_rows_f32_kernel(const float* __restrict__ Y, int M, int K, int mode, uint8_t* __restrict__ codes,
                       float* scale, int32_t* zp) {
@@ -567,6 +585,13 @@ quant_rows_f32_kernel(const float* __restrict__ Y, int M, int K, int mode, uint8
             asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                          : "l"(row + 8 * c));
+            if constexpr (OUT16) {                            // the contraction's centred bf16 operand
+                uint32_t h[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    h[i] = centred_bf16x2<A_BITS>(fma2(pack2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), INV, NEGZ));
+                *reinterpret_cast<uint4*>(codes + 2 * ((size_t)m * K + 8 * c)) = make_uint4(h[0], h[1], h[2], h[3]);
+            } else {
             int q[8];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -578,21 +603,23 @@ quant_rows_f32_kernel(const float* __restrict__ Y, int M, int K, int mode, uint8
                 *reinterpret_cast<uint2*>(codes + (size_t)m * K + 8 * c) = make_uint2(pack_u8x4(q[0], q[1], q[2], q[3]), pack_u8x4(q[4], q[5], q[6], q[7]));
             else
                 *reinterpret_cast<uint32_t*>(codes + (((size_t)m * K) >> 1) + 4 * c) = pack_u4x8(q);
+            }
         }
     }
 }
 
 }  // namespace
 
-lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int a_bits, int mode, uint8_t* codes,
+lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int a_bits, int mode, int out16, uint8_t* codes,
                                        float* scale, int32_t* zp, cudaStream_t st) {
     if (!lrq_aligned(Y, 32)) return LRQ_ERR_INVALID_ARG;          // rows are K*4 bytes with K % 8 == 0: 32-byte aligned chunks
     int sms = 0;
     if (lrq_current_device(nullptr, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
     const int blocks_needed = (M + 7) / 8;                        // 8 warps per CTA, one token per warp and step
     const int grid = blocks_needed < sms * 8 ? blocks_needed : sms * 8;
-    if (a_bits == 8) LRQ_CUDA_TRY(lrq_launch_pdl(quant_rows_f32_kernel<8>, dim3(grid), dim3(256), 0, st, Y, M, K, mode, codes, scale, zp));
-    else LRQ_CUDA_TRY(lrq_launch_pdl(quant_rows_f32_kernel<4>, dim3(grid), dim3(256), 0, st, Y, M, K, mode, codes, scale, zp));
+    auto kern = a_bits == 8 ? (out16 ? quant_rows_f32_kernel<8, true> : quant_rows_f32_kernel<8, false>)
+                            : (out16 ? quant_rows_f32_kernel<4, true> : quant_rows_f32_kernel<4, false>);
+    LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(256), 0, st, Y, M, K, mode, codes, scale, zp));
     return LRQ_OK;
 }
 
@@ -690,7 +717,7 @@ static lrq_status resident_ctas(const void* kern, int dev, int threads, size_t s
     return LRQ_OK;
 }
 
-static lrq_status launch_generic(const void* X, int M, int K, long ldx, int log2B, int a_bits, int mode, const float* prescale,
+static lrq_status launch_generic(const void* X, int M, int K, long ldx, int log2B, int a_bits, int mode, int out16, const float* prescale,
                                  uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st) {
     const size_t smem = (size_t)K * sizeof(float);
     if (smem > 200 * 1024) return LRQ_ERR_UNSUPPORTED;
@@ -699,7 +726,7 @@ static lrq_status launch_generic(const void* X, int M, int K, long ldx, int log2
     const int threads = (K >= 2048) ? 256 : (K >= 1024 ? 128 : 64);
     lrq_status rs = resident_ctas(reinterpret_cast<const void*>(rotq_generic_kernel), dev, threads, smem, &per_sm);   // sets the shared-memory opt-in
     if (rs != LRQ_OK) return rs;
-    LRQ_CUDA_TRY(lrq_launch_pdl(rotq_generic_kernel, dim3(M), dim3(threads), smem, st, X, M, K, ldx, log2B, a_bits, mode, prescale, codes,
+    LRQ_CUDA_TRY(lrq_launch_pdl(rotq_generic_kernel, dim3(M), dim3(threads), smem, st, X, M, K, ldx, log2B, a_bits, mode, out16, prescale, codes,
                                 scale, zp));
     return LRQ_OK;
 }
@@ -714,7 +741,7 @@ struct RotqPick<LOG2B, true, A_BITS, NT, NB, WIDE> {
 };
 
 template <int LOG2B, bool BIG = false>
-static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits, int mode, const float* prescale, uint8_t* codes,
+static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits, int mode, int out16, const float* prescale, uint8_t* codes,
                               float* scale, int32_t* zp, cudaStream_t st) {
     const int tpt = K / EPT;
     // whole tokens per CTA: thread count a multiple of 32, at least 256 when the token is small
@@ -730,7 +757,7 @@ static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits,
         smem += (size_t)(threads * EPT / B) * (size_t)(B + 32) * sizeof(float);
     }
     // register budget by CTA size: three CTAs of up to 288 threads, two of up to 384, else one
-    typedef void (*Kern)(const __nv_bfloat16*, int, int, long, int, int, int, const float*, uint8_t*, float*, int32_t*);
+    typedef void (*Kern)(const __nv_bfloat16*, int, int, long, int, int, int, int, const float*, uint8_t*, float*, int32_t*);
     // 256-bit accesses when every thread's 64 input bytes and 32 code bytes start on 32-byte boundaries
     const bool wide = lrq_aligned(X, 32) && (ldx % 16) == 0 && lrq_aligned(codes, 32);
     Kern kern;
@@ -747,16 +774,16 @@ static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits,
     if (rs != LRQ_OK) return rs;
     const int groups = (M + T - 1) / T;
     const int grid = groups < sms * per_sm ? groups : sms * per_sm;
-    LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, static_cast<const __nv_bfloat16*>(X), M, K, ldx, mode, T,
+    LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, static_cast<const __nv_bfloat16*>(X), M, K, ldx, mode, out16, T,
                                 groups, prescale, codes, scale, zp));
     return LRQ_OK;
 }
 
-lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, const float* prescale,
+lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                                     uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st) {
     // blocks of up to 128 channels: whole blocks per thread, TMA-fed (rotq_blk.cu), when the shape allows
     {
-        const lrq_status r = lrq_launch_rotq_blk(X, M, K, ldx, B, a_bits, mode, prescale, codes, scale, zp, st);
+        const lrq_status r = lrq_launch_rotq_blk(X, M, K, ldx, B, a_bits, mode, out16, prescale, codes, scale, zp, st);
         if (r != LRQ_ERR_UNSUPPORTED) return r;
     }
     int log2B = 0;
@@ -766,15 +793,15 @@ lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B
     if (fast_ok) {
         lrq_status r = LRQ_ERR_UNSUPPORTED;
         switch (log2B) {
-#define LRQ_CASE(L) case L: r = launch_fast<L>(X, M, K, ldx, a_bits, mode, prescale, codes, scale, zp, st); break;
+#define LRQ_CASE(L) case L: r = launch_fast<L>(X, M, K, ldx, a_bits, mode, out16, prescale, codes, scale, zp, st); break;
             LRQ_CASE(3) LRQ_CASE(4) LRQ_CASE(5) LRQ_CASE(6) LRQ_CASE(7) LRQ_CASE(8) LRQ_CASE(9)
 #undef LRQ_CASE
-#define LRQ_CASE(L) case L: r = launch_fast<L, true>(X, M, K, ldx, a_bits, mode, prescale, codes, scale, zp, st); break;
+#define LRQ_CASE(L) case L: r = launch_fast<L, true>(X, M, K, ldx, a_bits, mode, out16, prescale, codes, scale, zp, st); break;
             LRQ_CASE(10) LRQ_CASE(11) LRQ_CASE(12)
 #undef LRQ_CASE
             default: break;
         }
         if (r != LRQ_ERR_UNSUPPORTED) return r;
     }
-    return launch_generic(X, M, K, ldx, log2B, a_bits, mode, prescale, codes, scale, zp, st);
+    return launch_generic(X, M, K, ldx, log2B, a_bits, mode, out16, prescale, codes, scale, zp, st);
 }

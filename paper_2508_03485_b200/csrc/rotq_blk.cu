@@ -111,9 +111,22 @@ __device__ __forceinline__ TokenQ token_params_f32(float mn, float mx, int mode,
     return token_params_fast(mn, mx, A_BITS, mode, nrm, scale_out, zp_out);
 }
 
-// 32 consecutive values (16 pairs) -> codes; A8: 32 bytes (two 128-bit stores), A4: 16 bytes (one)
-template <int A_BITS>
-__device__ __forceinline__ void quantize_store_32(const f32x2* P, f32x2 INV, f32x2 NEGZ, uint8_t* dst) {
+// 32 consecutive values (16 pairs) from channel e of the code matrix on -> codes; A8: 32 bytes (two 128-bit stores),
+// A4: 16 bytes (one), OUT16 (the contraction's centred bf16 operand): 64 bytes (two 256-bit stores, whole sectors)
+template <int A_BITS, bool OUT16>
+__device__ __forceinline__ void quantize_store_32(const f32x2* P, f32x2 INV, f32x2 NEGZ, uint8_t* codes, size_t e) {
+    if (OUT16) {
+        uint32_t h[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) h[i] = centred_bf16x2<A_BITS>(fma2(P[i], INV, NEGZ));
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            asm volatile("st.global.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                         :: "l"(codes + 2 * e + 32 * i), "r"(h[8 * i]), "r"(h[8 * i + 1]), "r"(h[8 * i + 2]), "r"(h[8 * i + 3]),
+                            "r"(h[8 * i + 4]), "r"(h[8 * i + 5]), "r"(h[8 * i + 6]), "r"(h[8 * i + 7]) : "memory");
+        return;
+    }
+    uint8_t* dst = codes + (A_BITS == 8 ? e : e >> 1);
     int q[32];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -135,7 +148,7 @@ __device__ __forceinline__ void quantize_store_32(const f32x2* P, f32x2 INV, f32
     }
 }
 
-template <int LOG2B, int A_BITS>
+template <int LOG2B, int A_BITS, bool OUT16>
 __global__ void __launch_bounds__(MAX_WARPS * 32, 1)
 rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode, int tok_per_step, int num_steps,
                 int sub_warps, uint32_t stage_bytes, float scale_mul, const float* __restrict__ prescale,
@@ -337,8 +350,8 @@ rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode,
             // PAIRED: registers 0-15 are channels 32 odd .. + 31 of the block, registers 16-31 the same 64 further up
             const size_t e0 = (size_t)m * K + (PAIRED ? (size_t)(jh >> 1) * 128 + (size_t)odd * 32 : (size_t)jh * EPT);
             const size_t e1 = e0 + (PAIRED ? 64 : 32);
-            quantize_store_32<A_BITS>(P, INV, NEGZ, codes + (A_BITS == 8 ? e0 : e0 >> 1));
-            quantize_store_32<A_BITS>(P + 16, INVD, NEGZ, codes + (A_BITS == 8 ? e1 : e1 >> 1));
+            quantize_store_32<A_BITS, OUT16>(P, INV, NEGZ, codes, e0);
+            quantize_store_32<A_BITS, OUT16>(P + 16, INVD, NEGZ, codes, e1);
         }
     }
     if (aborted && ts == 0) {
@@ -356,11 +369,11 @@ rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode,
 typedef lrq_status (*BlkLaunch)(const CUtensorMap&, int, int, int, int, int, int, int, uint32_t, float, const float*, uint8_t*, float*,
                                 int32_t*, int, size_t, cudaStream_t);
 
-template <int LOG2B, int A_BITS>
+template <int LOG2B, int A_BITS, bool OUT16>
 lrq_status launch_blk(const CUtensorMap& tm, int M, int K, int mode, int T, int steps, int sub_warps, int nsub, uint32_t stage_bytes,
                       float scale_mul, const float* prescale, uint8_t* codes, float* scale, int32_t* zp, int sms, size_t smem,
                       cudaStream_t st) {
-    auto kern = rotq_blk_kernel<LOG2B, A_BITS>;
+    auto kern = rotq_blk_kernel<LOG2B, A_BITS, OUT16>;
     // the shared-memory opt-in is a per-device function attribute: set once per device and kernel variant
     static std::mutex mu;
     static bool configured[LRQ_MAX_DEVICES] = {};
@@ -384,9 +397,9 @@ lrq_status launch_blk(const CUtensorMap& tm, int M, int K, int mode, int T, int 
 }  // namespace
 
 // Returns LRQ_ERR_UNSUPPORTED for shapes this kernel does not take (the caller then uses the other kernels).
-lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, const float* prescale,
+lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                                uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st) {
-    if (K % 128 || B < 8 || B > 128 || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(codes, 16)) return LRQ_ERR_UNSUPPORTED;
+    if (K % 128 || B < 8 || B > 128 || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(codes, out16 ? 32 : 16)) return LRQ_ERR_UNSUPPORTED;
     const int tpt = K / EPT;
     if (K / 64 > 256) return LRQ_ERR_UNSUPPORTED;
     int log2B = 0;
@@ -420,8 +433,9 @@ lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int
     const double qsteps = mode == LRQ_ACT_ASYM ? (double)((1 << a_bits) - 1) : (double)((1 << (a_bits - 1)) - 1);
     const float scale_mul = (float)(1.0 / (sqrt((double)B) * qsteps));
     BlkLaunch fn = nullptr;
-    switch (log2B * 2 + (a_bits == 8)) {
-#define LRQ_CASE(L) case L * 2: fn = launch_blk<L, 4>; break; case L * 2 + 1: fn = launch_blk<L, 8>; break;
+    switch (log2B * 4 + (a_bits == 8) * 2 + out16) {
+#define LRQ_CASE(L) case L * 4: fn = launch_blk<L, 4, false>; break; case L * 4 + 1: fn = launch_blk<L, 4, true>; break; \
+                    case L * 4 + 2: fn = launch_blk<L, 8, false>; break; case L * 4 + 3: fn = launch_blk<L, 8, true>; break;
         LRQ_CASE(3) LRQ_CASE(4) LRQ_CASE(5) LRQ_CASE(6) LRQ_CASE(7)
 #undef LRQ_CASE
         default: return LRQ_ERR_UNSUPPORTED;

@@ -1,6 +1,7 @@
 // Pieces shared by the rotate + quantize kernels: the per-token parameters of Eq. 1 and the saturating packers.
 #pragma once
 #include "lrq_internal.cuh"
+#include "f32x2.cuh"
 
 namespace lrq_rq {
 
@@ -21,6 +22,22 @@ __device__ __forceinline__ uint32_t pack_u4x8(const int* q) {
     for (int i = 3; i >= 0; --i)
         asm("cvt.pack.sat.u4.s32.b32 %0, %1, %2, %3;" : "=r"(t) : "r"(q[2 * i + 1]), "r"(q[2 * i]), "r"(t));
     return t;
+}
+
+// Two codes as the contraction's bf16 operand: clamp(rint(x), 0, 2^b - 1) - C with C = 2^(b-1) (Eq. 1 before centring;
+// x = y / s - z).  Adding 1.5 * 2^23 rounds to an integer, ties to even, as cvt.rni does; every integer up to 256 is
+// exactly a bf16 number, so the clamp can run on the packed result.
+template <int A_BITS>
+__device__ __forceinline__ uint32_t centred_bf16x2(lrq_f2::f32x2 x) {
+    constexpr float C = A_BITS == 8 ? 128.f : 8.f;
+    const lrq_f2::f32x2 MAGIC = lrq_f2::pack2(12582912.f, 12582912.f), BACK = lrq_f2::pack2(-12582912.f - C, -12582912.f - C);
+    float a, b;
+    lrq_f2::unpack2(lrq_f2::add2(lrq_f2::add2(x, MAGIC), BACK), a, b);
+    uint32_t d;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
+    asm("max.bf16x2 %0, %0, %1;" : "+r"(d) : "r"(A_BITS == 8 ? 0xC300C300u : 0xC100C100u));      // -128 / -8
+    asm("min.bf16x2 %0, %0, %1;" : "+r"(d) : "r"(A_BITS == 8 ? 0x42FE42FEu : 0x40E040E0u));      // 127 / 7
+    return d;
 }
 
 // The same parameters for the fast kernel, where every warp works them out: one fp64 reciprocal refined

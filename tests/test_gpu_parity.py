@@ -532,3 +532,36 @@ def test_small_batches_take_the_small_tile_kernel(P, orc, M, w_bits, a_bits):
     Y2 = P.lrq_qgemm_codes(layer, q, s, z, P.F32, 2)
     assert torch.equal(Y, Y2)                                # lrq_qlinear took the small-tile kernel
     assert P.lrq_device_status() == 0
+
+
+# ------------------------------------------------------------ expanded form: decoded weights, bf16 operands
+@pytest.mark.parametrize("M,K,N,w_bits,a_bits,G,packed3,dt", [
+    (1024, 64, 8, 2, 8, 0, False, "F32"),            # one k-block, one narrow column, a table the packed kernels refuse
+    (1025, 72, 264, 2, 4, 24, False, "F16"),         # ragged k-block, groups of 24, ragged columns
+    (1281, 1152, 1096, 4, 8, 0, False, "BF16"),      # six 256-token rows, the last almost empty; ragged column of 72
+    (2300, 256, 3328, 3, 4, 128, False, "F32"),      # 117 whole tiles: a second round
+    (2500, 200, 2048, 4, 4, 0, False, "F16"),        # 80 whole tiles: a second round whose tiles are cut in quarters
+    (5000, 128, 256, 3, 8, 64, False, "BF16"),       # 20 tiles, one column, several panels' worth of rows
+    (700, 512, 2120, 3, 4, 128, True, "F32"),        # packed 3-bit codes decoded ahead of the contraction
+    (1100, 1152, 1096, 3, 8, 0, True, "BF16"),
+])
+def test_expanded_form_matches_cuda_core(P, M, K, N, w_bits, a_bits, G, packed3, dt):
+    # lrq_qlinear with the operands laid out in bf16 ahead of the contraction, against the CUDA-core kernel on the same
+    # codes: products are exact in both, so fp32 outputs differ by the order of K fp32 additions alone (each within
+    # 2^-24 of a partial sum; sqrt(K) 2^-24 of the rms is 3e-6 here, 1e-4 allows for cancellation with the
+    # zero-point term); 16-bit outputs by one more rounding (an ulp: 2^-7 / 2^-10 of the value).
+    B = min(K & -K, 128)
+    spec = LayerSpec("x", 700 + M, M, K, N, w_bits, a_bits, G, "hadamard", B)
+    layer, _ = PU.gpu_layer(spec, spec.weights(), P, code_layout=P.CODES_PACKED3 if packed3 else P.CODES_NIBBLE)
+    X = PU.bf16_to_device(spec.activations())
+    q, s, z = P.lrq_rotate_quantize_act(X, P.ROT_HADAMARD, a_bits, B)
+    code = getattr(P, dt)
+    ref = P.lrq_qgemm_codes(layer, q, s, z, P.F32, 1)
+    Y = P.lrq_qlinear(layer, X, code).float()
+    again = P.lrq_qlinear(layer, X, code).float()
+    torch.cuda.synchronize()
+    assert P.lrq_device_status() == 0
+    assert torch.equal(Y, again)
+    tol = 1e-4 * ref.pow(2).mean().sqrt() + ref.abs() * {"F32": 0.0, "BF16": 2.0 ** -7, "F16": 2.0 ** -10}[dt]
+    assert ((Y - ref).abs() <= tol).all()
+    layer.close()

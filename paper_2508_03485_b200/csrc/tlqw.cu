@@ -6,9 +6,17 @@
 // was rounded.  The sum is therefore taken exactly as its definition reads - over the side's elements in
 // increasing k, one add after another, products and sums rounded separately - and the parallelism is across
 // candidates instead of across elements: warp 0 scores the positive side, warp 1 the negative side, each lane
-// one clipping factor of the caller's grid, all lanes walking over the same elements (a lane computes log2|w|
-// for one element of a 32-element chunk; the chunk is then handed round by shuffles).  Every decision (codes,
-// chosen factor) is taken in fp64 with explicitly rounded operations, so no multiply-add is ever fused.
+// one clipping factor of the caller's grid, all lanes walking over the same elements.  Every decision (codes,
+// chosen factor) is the one fp64 arithmetic with explicitly rounded operations gives.
+//
+// What bounds it is the number of instructions per element and factor, so nothing but the three operations of the sum
+// itself is left in fp64 there:
+//   * the code is rint(l/s) - z in fp32, from log2f; an element within the fp32 error of a rounding boundary
+//     (|x - rint x| > 1/2 - E, E worked out from the candidate's range) takes the fp64 expression, a division, instead;
+//   * levels have 8-bit significands, so the upper word of the double is the level: 32-bit look-ups;
+//   * a side's elements are compacted into shared memory CHUNK source elements at a time and read as broadcasts.
+// 4608 x 1152, 4 bits, 31 factors a side: 545 us with fp64 codes and elements handed round by shuffles, 211 now;
+// 4608 x 1536, 3 bits, groups of 128: 1086 and 550.
 #include "lrq_internal.cuh"
 #include <climits>
 
@@ -16,6 +24,7 @@ namespace {
 
 constexpr int kMaxGrid = 64;
 constexpr int kThreads = 64;
+constexpr int kChunk = 128;                        // source elements compacted at a time
 struct ClipGrid { double a[kMaxGrid]; double b[kMaxGrid]; int na, nb; };
 
 __device__ __forceinline__ double level_value(double e, int I) {
@@ -25,7 +34,7 @@ __device__ __forceinline__ double level_value(double e, int I) {
     return ldexp(II, (int)f - I);
 }
 
-// code of Eq. 5 on one side: clamp(rint(l / s) - z, 0, nq)
+// code of Eq. 5 on one side: clamp(rint(l / s) - z, 0, nq), l = log2 of the magnitude
 __device__ __forceinline__ int side_code(double l, double s, double z, int nq) {
     return (int)fmin(fmax(__dsub_rn(rint(__ddiv_rn(l, s)), z), 0.0), (double)nq);
 }
@@ -34,14 +43,37 @@ __device__ __forceinline__ double shfl_double(double v, int src) {
     return __hiloint2double(__shfl_sync(0xffffffffu, __double2hiint(v), src), __shfl_sync(0xffffffffu, __double2loint(v), src));
 }
 
+// The same from fp32: x = l32 * inv + negz is within E of the exact l/s - z, with E = 2^-21 (max|l| / s + nq + 2): log2f is
+// within an ulp of l, the reciprocal and the fused multiply-add round once each (2^-23 + 2^-24 + 2^-24 of |l/s|, taken
+// twice over).  `thr` = 1/2 - E; a candidate whose E is too large (E >= 1/2) always takes the fp64 expression, and so
+// does one whose z is not an fp32 integer, since then |l/s| is above 2^23.  Returned in the low bits of a float.
+constexpr float kMagic = 12582912.f;                // 1.5 * 2^23: adding it rounds to an integer, ties to even
+struct FastCode { float inv, negz, thr, top; };
+__device__ __forceinline__ FastCode fast_code(double s, double z, double lmin, double lmax, int nq) {
+    FastCode f;
+    const double e = 4.76837158203125e-7 * (fmax(fabs(lmin), fabs(lmax)) / s + (double)nq + 2.0);
+    f.inv = (float)(1.0 / s);
+    f.negz = (float)-z;
+    f.thr = e < 0.5 ? (float)(0.5 - e) * 0.999999f : -1.f;
+    f.top = kMagic + (float)nq;
+    return f;
+}
+__device__ __forceinline__ float fast_round(float l32, const FastCode& f, bool& exact) {
+    const float x = fmaf(l32, f.inv, f.negz), r = x + kMagic;
+    exact = fabsf(x - (r - kMagic)) <= f.thr;       // false for a NaN or an out-of-range x as well
+    return fminf(fmaxf(r, kMagic), f.top);
+}
+
 struct Side { double s, z, factor; };
+struct __align__(16) Elem { double a; float l32; };  // magnitude and its log2
 
 __global__ void __launch_bounds__(kThreads)
 tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, int I, ClipGrid grid, int pack3,
                     uint8_t* __restrict__ codes, float* __restrict__ levels, double* __restrict__ meta,
                     float* __restrict__ wsum) {
-    __shared__ double cand_lev[2][9][32];          // level table of each lane's candidate, per side
-    __shared__ double ext[2][2][2];                // [warp][side][max, min] of log2|w|
+    __shared__ int cand_lev[2][9][32];             // level table of each lane's candidate, per side (upper word of the double)
+    __shared__ Elem list[2][kChunk + 4];           // a side's elements of one chunk, in increasing k
+    __shared__ float ext[2][2][2];                 // [warp][side][max, min] of |w|
     __shared__ int ext_cnt[2][2];
     __shared__ Side best[2];
     __shared__ double T[16];
@@ -50,36 +82,37 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
     const int n = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = 1 << (bits - 1), nlev = 1 << bits, ngrp = K / G;
     double row_sum = 0.0;                          // meaningful in thread 0
+    lrq_pdl_trigger();
+    lrq_pdl_wait();                                // the weights may be the previous kernel's output
 
     for (int g = 0; g < ngrp; ++g) {
         const float* w = W + (size_t)n * K + (size_t)g * G;
-        // ---- extremes of log2|w| per side (order does not matter for max / min)
-        double lmax[2] = {-INFINITY, -INFINITY}, lmin[2] = {INFINITY, INFINITY};
+        // ---- extremes of |w| per side (order does not matter for max / min, and log2 is monotone on fp32 numbers)
+        float amax[2] = {0.f, 0.f}, amin[2] = {INFINITY, INFINITY};
         int cnt[2] = {0, 0};
         for (int k = tid; k < G; k += kThreads) {
             const float v = w[k];
             if (v != 0.f) {
-                const double l = log2((double)fabsf(v));
                 const int sd = v < 0.f;
-                lmax[sd] = fmax(lmax[sd], l); lmin[sd] = fmin(lmin[sd], l); cnt[sd]++;
+                const float av = fabsf(v);
+                if (sd) { amax[1] = fmaxf(amax[1], av); amin[1] = fminf(amin[1], av); cnt[1]++; }
+                else { amax[0] = fmaxf(amax[0], av); amin[0] = fminf(amin[0], av); cnt[0]++; }
             }
         }
 #pragma unroll
         for (int sd = 0; sd < 2; ++sd) {
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                lmax[sd] = fmax(lmax[sd], shfl_double(lmax[sd], lane ^ o));
-                lmin[sd] = fmin(lmin[sd], shfl_double(lmin[sd], lane ^ o));
-                cnt[sd] += __shfl_xor_sync(0xffffffffu, cnt[sd], o);
-            }
-            if (lane == 0) { ext[warp][sd][0] = lmax[sd]; ext[warp][sd][1] = lmin[sd]; ext_cnt[warp][sd] = cnt[sd]; }
+            // magnitudes: the bit patterns are ordered as the numbers
+            const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(amax[sd])), mn = __reduce_min_sync(0xffffffffu, __float_as_uint(amin[sd]));
+            const int c = __reduce_add_sync(0xffffffffu, cnt[sd]);
+            if (lane == 0) { ext[warp][sd][0] = __uint_as_float(mx); ext[warp][sd][1] = __uint_as_float(mn); ext_cnt[warp][sd] = c; }
         }
         __syncthreads();
         // ---- search of the clipping factor: warp `sd` owns side sd, lane c the c-th factor of that side's grid
         const int sd = warp;
         const int nq = sd ? half : half - 1;       // highest code of the side = denominator of Eq. 6
-        const double smax = fmax(ext[0][sd][0], ext[1][sd][0]), smin = fmin(ext[0][sd][1], ext[1][sd][1]);
+        const float vmax = fmaxf(ext[0][sd][0], ext[1][sd][0]), vmin = fminf(ext[0][sd][1], ext[1][sd][1]);
         const int scnt = ext_cnt[0][sd] + ext_cnt[1][sd];
+        const double smax = scnt ? log2((double)vmax) : -INFINITY, smin = scnt ? log2((double)vmin) : INFINITY;
         const int ng = sd ? grid.nb : grid.na;
         double best_err = INFINITY, best_s = 1.0, best_z = 0.0, best_f = 1.0;
         bool found = false;
@@ -98,26 +131,47 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
             }
             __syncwarp();
             for (int q = 0; q <= nq; ++q)
-                cand_lev[sd][q][lane] = ok ? level_value(__dmul_rn(s, __dadd_rn((double)q, z)), I) : 0.0;
+                cand_lev[sd][q][lane] = ok ? __double2hiint(level_value(__dmul_rn(s, __dadd_rn((double)q, z)), I)) : 0;
+            FastCode fc = fast_code(s, z, smin, smax, nq);
+            if (!ok) { fc.inv = 0.f; fc.negz = 0.f; fc.thr = 1.f; }                 // scored, but never looked at
+            const uint32_t lev0 = (uint32_t)__cvta_generic_to_shared(&cand_lev[sd][0][lane]) - (__float_as_uint(kMagic) << 7);
             __syncwarp();
-            // the side's elements in increasing k, one chunk of 32 at a time
+            // the side's elements in increasing k, one chunk at a time
             double err = 0.0;
-            for (int k0 = 0; k0 < G; k0 += 32) {
-                const int k = k0 + lane;
-                const float v = k < G ? w[k] : 0.f;
-                const bool mine = sd ? (v < 0.f) : (v > 0.f);
-                const double a = (double)fabsf(v);
-                const double l = mine ? log2(a) : 0.0;
-                unsigned m = __ballot_sync(0xffffffffu, mine);
-                while (m) {
-                    const int j = __ffs(m) - 1;
-                    m &= m - 1;
-                    const double lj = shfl_double(l, j), aj = shfl_double(a, j);
-                    if (ok) {
-                        const double d = __dsub_rn(aj, cand_lev[sd][side_code(lj, s, z, nq)][lane]);
-                        err = __dadd_rn(err, __dmul_rn(d, d));
+            for (int k0 = 0; k0 < G; k0 += kChunk) {
+                int n_el = 0;
+#pragma unroll
+                for (int u = 0; u < kChunk / 32; ++u) {
+                    const int k = k0 + 32 * u + lane;
+                    const float v = k < G ? w[k] : 0.f;
+                    const bool mine = sd ? (v < 0.f) : (v > 0.f);
+                    const unsigned m = __ballot_sync(0xffffffffu, mine);
+                    if (mine) {
+                        Elem e;
+                        e.a = (double)fabsf(v); e.l32 = log2f(fabsf(v));
+                        list[sd][n_el + __popc(m & ((1u << lane) - 1u))] = e;
                     }
+                    n_el += __popc(m);
                 }
+                __syncwarp();
+                auto score = [&](const Elem& e) {
+                    bool exact;
+                    float r = fast_round(e.l32, fc, exact);
+                    if (!exact) r = kMagic + (float)side_code(log2(e.a), s, z, nq);
+                    int hi;
+                    asm("ld.shared.b32 %0, [%1];" : "=r"(hi) : "r"(lev0 + (__float_as_uint(r) << 7)));
+                    return __dsub_rn(e.a, __hiloint2double(hi, 0));
+                };
+                int j = 0;
+                for (; j + 4 <= n_el; j += 4) {
+                    double d[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) d[u] = score(list[sd][j + u]);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) err = __dadd_rn(err, __dmul_rn(d[u], d[u]));
+                }
+                for (; j < n_el; ++j) { const double d = score(list[sd][j]); err = __dadd_rn(err, __dmul_rn(d, d)); }
+                __syncwarp();
             }
             // first minimum in grid order: the smallest error, the lowest index among equals
             double e = ok ? err : INFINITY;
@@ -159,14 +213,30 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
         __syncthreads();
         // ---- codes, eight at a time (one 32-bit word of nibbles, or three bytes of packed 3-bit codes)
         double part = 0.0;
+        FastCode fcs[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const float mx = fmaxf(ext[0][q][0], ext[1][q][0]), mn = fminf(ext[0][q][1], ext[1][q][1]);
+            fcs[q] = fast_code(best[q].s, best[q].z, (q ? ncnt : pcnt) ? log2((double)mn) : 0.0, (q ? ncnt : pcnt) ? log2((double)mx) : 0.0,
+                               q ? half : half - 1);
+        }
         for (int j = tid; j < G / 8; j += kThreads) {
             uint32_t word = 0;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const float v = w[8 * j + e];
                 int cc = 0;
-                if (v > 0.f) cc = side_code(log2((double)v), best[0].s, best[0].z, half - 1);
-                else if (v < 0.f) cc = -side_code(log2((double)-v), best[1].s, best[1].z, half);
+                if (v != 0.f) {
+                    const bool neg = v < 0.f;
+                    FastCode f;
+                    f.inv = neg ? fcs[1].inv : fcs[0].inv; f.negz = neg ? fcs[1].negz : fcs[0].negz;
+                    f.thr = neg ? fcs[1].thr : fcs[0].thr; f.top = neg ? fcs[1].top : fcs[0].top;
+                    bool exact;
+                    const float r = fast_round(log2f(fabsf(v)), f, exact);
+                    const int q = exact ? (int)(__float_as_uint(r) - __float_as_uint(kMagic))
+                                        : side_code(log2((double)fabsf(v)), best[neg].s, best[neg].z, neg ? half : half - 1);
+                    cc = neg ? -q : q;
+                }
                 const int u = cc + half;
                 part += T[u];
                 word |= (uint32_t)u << ((pack3 ? 3 : 4) * e);
@@ -210,9 +280,7 @@ extern "C" lrq_status lrq_tlq_quantize_weights(const float* W_rot, int N, int K,
         grid.a[i] = i < grid.na ? p->alpha[i] : 0.0;
         grid.b[i] = i < grid.nb ? p->beta[i] : 0.0;
     }
-    tlq_quantize_kernel<<<N, kThreads, 0, (cudaStream_t)cuda_stream>>>(W_rot, N, K, G, p->w_bits, p->integerize_I, grid,
-                                                                      p->code_layout == LRQ_CODES_PACKED3 ? 1 : 0, codes,
-                                                                      levels, meta, wsum);
-    LRQ_CUDA_TRY(cudaGetLastError());
+    LRQ_CUDA_TRY(lrq_launch_pdl(tlq_quantize_kernel, dim3(N), dim3(kThreads), 0, (cudaStream_t)cuda_stream, W_rot, N, K, G, p->w_bits,
+                                p->integerize_I, grid, p->code_layout == LRQ_CODES_PACKED3 ? 1 : 0, codes, levels, meta, wsum));
     return LRQ_OK;
 }

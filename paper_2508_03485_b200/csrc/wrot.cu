@@ -2,10 +2,9 @@
 // Sec. 5.1 folded in: W_rot = W diag(colmul) R, evaluated in fp64 and rounded once to fp32, which is what
 // the TLQ quantizer reads.
 //
-// Offline step.  Hadamard: one CTA per weight row, the row in shared memory as fp64, log2(B) butterfly
-// stages with a CTA barrier between them.  Dense: an fp64 matrix product on the CUDA cores, 64 x 64
-// output tiles, 4 x 4 accumulators per thread; R is the layer's stored bf16 matrix (exact in fp64), so
-// both sides of Eq. 2 use the same R.  Dual transformation (R = R1hat P R2hat, Sec. 4.2): one CTA per row, the
+// Offline step.  Hadamard: one CTA per weight row, butterflies in registers, up to four stages between two trips
+// through shared memory.  Dense: an fp64 matrix product on the fp64 tensor cores, 64 x 64 output tiles; R is the
+// layer's stored bf16 matrix (exact in fp64), so both sides of Eq. 2 use the same R.  Dual transformation (R = R1hat P R2hat, Sec. 4.2): one CTA per row, the
 // row in shared memory as fp64, block-diagonal product, gather through the index map, second product.
 #include "lrq_internal.cuh"
 
@@ -13,79 +12,162 @@
 
 namespace {
 
-__global__ void __launch_bounds__(256)
+// NB butterfly stages (index bits bit .. bit + NB - 1) of the row: a thread takes the 2^NB elements that differ in these
+// bits, from global memory in the first pass, to global memory in the last.  Elements lie in shared memory with one
+// pad after every 16, which makes both the first pass (runs of 16 per thread) and the later ones (neighbouring
+// threads, neighbouring elements) conflict-free.  Stages run in the order of increasing bits whatever NB is, so the
+// result does not depend on how they are grouped.
+template <int NB>
+__device__ __forceinline__ void hadamard_pass(double* row, int K, int bit, const float* w, const float* colmul, float* o, double norm) {
+    constexpr int E = 1 << NB;
+    for (int g = threadIdx.x; g < (K >> NB); g += blockDim.x) {
+        const int low = g & ((1 << bit) - 1), base = ((g - low) << NB) | low;
+        double v[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int k = base + (e << bit);
+            v[e] = w ? (double)w[k] * (colmul ? (double)colmul[k] : 1.0) : row[k + (k >> 4)];
+        }
+#pragma unroll
+        for (int h = 1; h < E; h <<= 1)
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (!(e & h)) { const double a = v[e], b = v[e | h]; v[e] = a + b; v[e | h] = a - b; }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int k = base + (e << bit);
+            if (o) o[k] = (float)(v[e] * norm); else row[k + (k >> 4)] = v[e];
+        }
+    }
+    __syncthreads();
+}
+
+// 4608 x 1152, B = 128: 34 us with a barrier and a trip through shared memory per stage, 17 now.
+__global__ void __launch_bounds__(128)
 wrot_hadamard_kernel(const float* __restrict__ W, int N, int K, long ldw, const float* __restrict__ colmul, int log2B,
                      float* __restrict__ out, long ldo) {
-    extern __shared__ double row[];                // [K]
-    const int n = blockIdx.x, tid = threadIdx.x, nthr = blockDim.x;
+    extern __shared__ double row[];                // [K + K / 16]
+    const int n = blockIdx.x;
     const float* w = W + (size_t)n * ldw;
-    for (int k = tid; k < K; k += nthr) row[k] = (double)w[k] * (colmul ? (double)colmul[k] : 1.0);
-    __syncthreads();
-    const int pairs = K >> 1;
-    for (int s = 0; s < log2B; ++s) {
-        const int h = 1 << s;
-        for (int i = tid; i < pairs; i += nthr) {
-            const int lo = ((i >> s) << (s + 1)) | (i & (h - 1));
-            const double a = row[lo], b = row[lo + h];
-            row[lo] = a + b;
-            row[lo + h] = a - b;
-        }
-        __syncthreads();
-    }
     // 1/sqrt(B): a power of two for even log2(B), else a power of two times 1/sqrt(2)
     const double norm = ldexp((log2B & 1) ? 0.70710678118654752440 : 1.0, -(log2B >> 1));
     float* o = out + (size_t)n * ldo;
-    for (int k = tid; k < K; k += nthr) o[k] = (float)(row[k] * norm);
+    lrq_pdl_trigger();
+    lrq_pdl_wait();
+    int bit = 0;
+    do {
+        const int left = log2B - bit, nb = left < 4 ? left : 4;
+        const float* src = bit == 0 ? w : nullptr;
+        float* dst = nb == left ? o : nullptr;
+        if (nb == 4) hadamard_pass<4>(row, K, bit, src, colmul, dst, norm);
+        else if (nb == 3) hadamard_pass<3>(row, K, bit, src, colmul, dst, norm);
+        else if (nb == 2) hadamard_pass<2>(row, K, bit, src, colmul, dst, norm);
+        else if (nb == 1) hadamard_pass<1>(row, K, bit, src, colmul, dst, norm);
+        else hadamard_pass<0>(row, K, bit, src, colmul, dst, norm);
+        bit += nb;
+    } while (bit < log2B);
 }
 
+// Dense rotation: out[N,K] = (W diag(colmul)) . R in fp64 on the tensor cores (mma m8n8k4).  A CTA of four warps owns a
+// 64 x 64 tile, a warp 32 x 32 of it (4 x 4 fragments, 64 accumulator registers): per 4-deep step 8 fragment loads feed
+// 16 MMAs, a quarter of the shared-memory traffic that 4 x 4 accumulators per thread needed.  Both operands are
+// widened to fp64 on their way into shared memory, double-buffered, the next 16-deep block in flight in registers.
+// Bound by the fp64 pipe.  4608 x 1536 x 1536: 1924 us on the CUDA cores (11 TFLOP/s), 480 now (45 TFLOP/s).
 constexpr int TM = 64, TN = 64, TK = 16;
+constexpr int A_PITCH = TK + 4, B_PITCH = TN + 4;   // doubles; 4 mod 16: a fragment's 4 x 4 half-warp hits 16 bank pairs
 
-__global__ void __launch_bounds__(256)
+__device__ __forceinline__ void dmma(double* d, double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+
+__global__ void __launch_bounds__(128)
 wrot_dense_kernel(const float* __restrict__ W, int N, int K, long ldw, const float* __restrict__ colmul,
-                  const __nv_bfloat16* __restrict__ R, float* __restrict__ out, long ldo) {
-    __shared__ double sW[TK][TM + 1];              // [k][row]
-    __shared__ double sR[TK][TN];                  // [k][col]
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+                  const __nv_bfloat16* __restrict__ R, float* __restrict__ out, long ldo, int vec_w, int vec_r) {
+    __shared__ __align__(16) double sA[2][TM * A_PITCH];
+    __shared__ __align__(16) double sB[2][TK * B_PITCH];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n0 = blockIdx.y * TM, j0 = blockIdx.x * TN;
-    double acc[4][4];
+    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+    const int ar = tid >> 1, ak = (tid & 1) * 8;               // W: row of the tile, first of eight k
+    const int bk = tid >> 3, bn = (tid & 7) * 8;               // R: k of the block, first of eight columns
+    lrq_pdl_trigger();
+    lrq_pdl_wait();
+    const float* wrow = W + (size_t)(n0 + ar) * ldw;
+    const bool row_ok = n0 + ar < N;
+    float fa[8], fc[8];
+    uint32_t fb[4];
+    auto fetch = [&](int k0) {
+        const int k = k0 + ak;
+        if (vec_w && row_ok && k + 8 <= K) {
+            const float4 x = *reinterpret_cast<const float4*>(wrow + k), y = *reinterpret_cast<const float4*>(wrow + k + 4);
+            fa[0] = x.x; fa[1] = x.y; fa[2] = x.z; fa[3] = x.w; fa[4] = y.x; fa[5] = y.y; fa[6] = y.z; fa[7] = y.w;
+        } else {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-    for (int k0 = 0; k0 < K; k0 += TK) {
-        for (int i = tid; i < TM * TK; i += 256) {
-            const int r = i / TK, k = i % TK;
-            const int n = n0 + r, kk = k0 + k;
-            double v = 0.0;
-            if (n < N && kk < K) v = (double)W[(size_t)n * ldw + kk] * (colmul ? (double)colmul[kk] : 1.0);
-            sW[k][r] = v;
+            for (int i = 0; i < 8; ++i) fa[i] = row_ok && k + i < K ? wrow[k + i] : 0.f;
         }
-        for (int i = tid; i < TK * TN; i += 256) {
-            const int k = i / TN, c = i % TN;
-            const int kk = k0 + k, j = j0 + c;
-            sR[k][c] = (kk < K && j < K) ? (double)__bfloat162float(R[(size_t)kk * K + j]) : 0.0;
+        if (colmul) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) fc[i] = k + i < K ? colmul[k + i] : 0.f;
         }
-        __syncthreads();
+        const int kr = k0 + bk, c = j0 + bn;
+        if (vec_r && kr < K && c + 8 <= K) {
+            const uint4 x = *reinterpret_cast<const uint4*>(R + (size_t)kr * K + c);
+            fb[0] = x.x; fb[1] = x.y; fb[2] = x.z; fb[3] = x.w;
+        } else {
+            const unsigned short* r = reinterpret_cast<const unsigned short*>(R) + (size_t)kr * K + c;
 #pragma unroll
-        for (int k = 0; k < TK; ++k) {
-            double a[4], b[4];
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t lo = kr < K && c + 2 * i < K ? r[2 * i] : 0u, hi = kr < K && c + 2 * i + 1 < K ? r[2 * i + 1] : 0u;
+                fb[i] = lo | (hi << 16);
+            }
+        }
+    };
+    auto stage = [&](int s) {
+        double2* a = reinterpret_cast<double2*>(&sA[s][ar * A_PITCH + ak]);
+        double2* b = reinterpret_cast<double2*>(&sB[s][bk * B_PITCH + bn]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = sW[k][ty * 4 + i]; b[i] = sR[k][tx * 4 + i]; }
+        for (int i = 0; i < 4; ++i) {
+            double x = (double)fa[2 * i], y = (double)fa[2 * i + 1];
+            if (colmul) { x *= (double)fc[2 * i]; y *= (double)fc[2 * i + 1]; }
+            a[i] = make_double2(x, y);
+            b[i] = make_double2((double)__uint_as_float(fb[i] << 16), (double)__uint_as_float(fb[i] & 0xffff0000u));
+        }
+    };
+    double acc[4][4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+    fetch(0);
+    stage(0);
+    __syncthreads();
+    for (int k0 = 0, s = 0; k0 < K; k0 += TK, s ^= 1) {
+        const bool more = k0 + TK < K;
+        if (more) fetch(k0 + TK);
+        const double* a = &sA[s][(wm + (lane >> 2)) * A_PITCH + (lane & 3)];
+        const double* b = &sB[s][(lane & 3) * B_PITCH + wn + (lane >> 2)];
+#pragma unroll
+        for (int k = 0; k < TK; k += 4) {
+            double x[4], y[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { x[i] = a[8 * i * A_PITCH + k]; y[i] = b[k * B_PITCH + 8 * i]; }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) dmma(acc[i][j], x[i], y[j]);
         }
+        if (more) stage(s ^ 1);
         __syncthreads();
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int n = n0 + ty * 4 + i;
+        const int n = n0 + wm + 8 * i + (lane >> 2);
         if (n >= N) continue;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int c = j0 + tx * 4 + j;
-            if (c < K) out[(size_t)n * ldo + c] = (float)acc[i][j];
+            const int c = j0 + wn + 8 * j + 2 * (lane & 3);
+            if (c < K) out[(size_t)n * ldo + c] = (float)acc[i][j][0];
+            if (c + 1 < K) out[(size_t)n * ldo + c + 1] = (float)acc[i][j][1];
         }
     }
 }
@@ -143,14 +225,17 @@ lrq_status lrq_launch_rotate_weights(const float* W, int N, int K, long ldw, con
     if (kind == LRQ_ROT_HADAMARD) {
         int log2B = 0;
         while ((1 << log2B) < had_block) ++log2B;
-        const size_t smem = (size_t)K * sizeof(double);
-        if (smem > 200 * 1024) return LRQ_ERR_UNSUPPORTED;
+        // one pad after every 16 elements; K <= 25600 as before (212.5 KB)
+        const size_t smem = (size_t)(K + K / 16 + 1) * sizeof(double);
+        if ((size_t)K * sizeof(double) > 200 * 1024) return LRQ_ERR_UNSUPPORTED;
         if (smem > 40 * 1024)
             LRQ_CUDA_TRY(cudaFuncSetAttribute(wrot_hadamard_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        wrot_hadamard_kernel<<<N, 256, smem, st>>>(W, N, K, ldw, colmul, log2B, out, ldo);
+        LRQ_CUDA_TRY(lrq_launch_pdl(wrot_hadamard_kernel, dim3(N), dim3(128), smem, st, W, N, K, ldw, colmul, log2B, out, ldo));
     } else if (kind == LRQ_ROT_DENSE) {
         const dim3 grid((K + TN - 1) / TN, (N + TM - 1) / TM);
-        wrot_dense_kernel<<<grid, 256, 0, st>>>(W, N, K, ldw, colmul, static_cast<const __nv_bfloat16*>(R), out, ldo);
+        const int vec_w = lrq_aligned(W, 16) && ldw % 4 == 0, vec_r = lrq_aligned(R, 16) && K % 8 == 0;
+        LRQ_CUDA_TRY(lrq_launch_pdl(wrot_dense_kernel, grid, dim3(128), 0, st, W, N, K, ldw, colmul, static_cast<const __nv_bfloat16*>(R),
+                                    out, ldo, vec_w, vec_r));
     } else {
         const size_t total = (size_t)N * K;
         const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);

@@ -11,27 +11,30 @@
 //
 // What bounds it is the number of instructions per element and factor, so nothing but the three operations of the sum
 // itself is left in fp64 there:
-//   * the code is rint(l/s) - z in fp32, from log2f; an element within the fp32 error of a rounding boundary
+//   * the code is rint(l/s) - z in fp32, from log2f, two elements per instruction; an element within the fp32 error of a rounding boundary
 //     (|x - rint x| > 1/2 - E, E worked out from the candidate's range) takes the fp64 expression, a division, instead;
 //   * levels have 8-bit significands, so the upper word of the double is the level: 32-bit look-ups;
 //   * a side's elements are compacted into shared memory CHUNK source elements at a time and read as broadcasts.
-// 4608 x 1152, 4 bits, 31 factors a side: 545 us with fp64 codes and elements handed round by shuffles, 211 now;
-// 4608 x 1536, 3 bits, groups of 128: 1086 and 550.
+// 4608 x 1152, 4 bits, 31 factors a side: 545 us with fp64 codes and elements handed round by shuffles, 164 now;
+// 4608 x 1536, 3 bits, groups of 128: 1086 and 380.
 #include "lrq_internal.cuh"
+#include "f32x2.cuh"
 #include <climits>
 
 namespace {
 
 constexpr int kMaxGrid = 64;
 constexpr int kThreads = 64;
-constexpr int kChunk = 128;                        // source elements compacted at a time
+constexpr int kChunk = 256;                        // source elements compacted at a time
 struct ClipGrid { double a[kMaxGrid]; double b[kMaxGrid]; int na, nb; };
 
 __device__ __forceinline__ double level_value(double e, int I) {
     // Eqs. 8-9: 2^e ~ II * 2^(f-I) with f = floor(e), II = rint(2^(e-f) * 2^I)
     const double f = floor(e);
     const double II = rint(exp2(__dsub_rn(e, f)) * (double)(1 << I));      // the factor is a power of two: exact
-    return ldexp(II, (int)f - I);
+    const int x = (int)f - I;
+    if (x >= -1000 && x <= 1000) return II * __hiloint2double((1023 + x) << 20, 0);   // a product with a power of two: exact
+    return ldexp(II, x);
 }
 
 // code of Eq. 5 on one side: clamp(rint(l / s) - z, 0, nq), l = log2 of the magnitude
@@ -43,36 +46,52 @@ __device__ __forceinline__ double shfl_double(double v, int src) {
     return __hiloint2double(__shfl_sync(0xffffffffu, __double2hiint(v), src), __shfl_sync(0xffffffffu, __double2loint(v), src));
 }
 
-// The same from fp32: x = l32 * inv + negz is within E of the exact l/s - z, with E = 2^-21 (max|l| / s + nq + 2): log2f is
-// within an ulp of l, the reciprocal and the fused multiply-add round once each (2^-23 + 2^-24 + 2^-24 of |l/s|, taken
-// twice over).  `thr` = 1/2 - E; a candidate whose E is too large (E >= 1/2) always takes the fp64 expression, and so
-// does one whose z is not an fp32 integer, since then |l/s| is above 2^23.  Returned in the low bits of a float.
+// The upper word of a level's double (its 8 significant bits fit there), from fp32: exp2f is within 2 ulp, so II is what the
+// fp64 expression gives unless 2^(e-f) * 2^I comes within 2e-4 of a rounding boundary, which takes that expression.
+__device__ __forceinline__ int level_word(double e, int I) {
+    const double f = floor(e);
+    const float x = exp2f((float)__dsub_rn(e, f)) * (float)(1 << I), r = rintf(x);
+    const int fi = (int)f;
+    if (fabsf(x - r) < 0.4998f && fi > -900 && fi < 900) return (int)(__float_as_uint(r) >> 3) + 0x38000000 + (fi - I) * (1 << 20);
+    return __double2hiint(level_value(e, I));
+}
+
+// The same from fp32: x = l32 * inv + negz is within E of the exact l/s - z, with E = 2^-20 (max|l| / s + nq + 2): log2f is
+// within an ulp of l (2^-23 of |l/s|), the reciprocal of the rounded step within 2^-22, the fused multiply-add rounds once
+// (2^-24), all taken more than twice over.  `thr` = 1/2 - E; a candidate whose E is too large (E >= 1/2) always takes the fp64
+// expression, and so does one whose z is not an fp32 integer, since then |l/s| is above 2^23.  The side's smallest element
+// has the code rint(smin / s) - z = 0 and no element a lower one, so only the upper clamp of Eq. 5 is left to do.
 constexpr float kMagic = 12582912.f;                // 1.5 * 2^23: adding it rounds to an integer, ties to even
 struct FastCode { float inv, negz, thr, top; };
-__device__ __forceinline__ FastCode fast_code(double s, double z, double lmin, double lmax, int nq) {
+__device__ __forceinline__ FastCode fast_code(double s, double z, float lmax, int nq) {     // lmax >= |l| of every element
     FastCode f;
-    const double e = 4.76837158203125e-7 * (fmax(fabs(lmin), fabs(lmax)) / s + (double)nq + 2.0);
-    f.inv = (float)(1.0 / s);
+    f.inv = 1.0f / (float)s;
     f.negz = (float)-z;
-    f.thr = e < 0.5 ? (float)(0.5 - e) * 0.999999f : -1.f;
+    const float e = 9.5367431640625e-7f * (lmax * f.inv + (float)nq + 2.0f);
+    f.thr = e < 0.5f && f.inv > 0.f ? (0.5f - e) * 0.999999f : -1.f;
     f.top = kMagic + (float)nq;
     return f;
 }
+// The code in the low bits of the returned float; `exact` is false for a NaN or an out-of-range x as well.
 __device__ __forceinline__ float fast_round(float l32, const FastCode& f, bool& exact) {
     const float x = fmaf(l32, f.inv, f.negz), r = x + kMagic;
-    exact = fabsf(x - (r - kMagic)) <= f.thr;       // false for a NaN or an out-of-range x as well
-    return fminf(fmaxf(r, kMagic), f.top);
+    exact = fabsf(x - (r - kMagic)) <= f.thr;
+    return fminf(r, f.top);
 }
 
-struct Side { double s, z, factor; };
-struct __align__(16) Elem { double a; float l32; };  // magnitude and its log2
+using namespace lrq_f2;
 
-__global__ void __launch_bounds__(kThreads)
+struct Side { double s, z, factor; };
+
+__global__ void __launch_bounds__(kThreads, 16)
 tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, int I, ClipGrid grid, int pack3,
                     uint8_t* __restrict__ codes, float* __restrict__ levels, double* __restrict__ meta,
                     float* __restrict__ wsum) {
     __shared__ int cand_lev[2][9][32];             // level table of each lane's candidate, per side (upper word of the double)
-    __shared__ Elem list[2][kChunk + 4];           // a side's elements of one chunk, in increasing k
+    // a side's elements of one chunk, in increasing k: magnitude and its log2
+    __shared__ __align__(16) double mag[2][kChunk];
+    __shared__ __align__(16) float lg[2][kChunk];
+    __shared__ FastCode best_fc[2];
     __shared__ float ext[2][2][2];                 // [warp][side][max, min] of |w|
     __shared__ int ext_cnt[2][2];
     __shared__ Side best[2];
@@ -113,6 +132,7 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
         const float vmax = fmaxf(ext[0][sd][0], ext[1][sd][0]), vmin = fminf(ext[0][sd][1], ext[1][sd][1]);
         const int scnt = ext_cnt[0][sd] + ext_cnt[1][sd];
         const double smax = scnt ? log2((double)vmax) : -INFINITY, smin = scnt ? log2((double)vmin) : INFINITY;
+        const float l_abs = scnt ? fmaxf(fabsf((float)smin), fabsf((float)smax)) * 1.000001f : 0.f;
         const int ng = sd ? grid.nb : grid.na;
         double best_err = INFINITY, best_s = 1.0, best_z = 0.0, best_f = 1.0;
         bool found = false;
@@ -131,8 +151,8 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
             }
             __syncwarp();
             for (int q = 0; q <= nq; ++q)
-                cand_lev[sd][q][lane] = ok ? __double2hiint(level_value(__dmul_rn(s, __dadd_rn((double)q, z)), I)) : 0;
-            FastCode fc = fast_code(s, z, smin, smax, nq);
+                cand_lev[sd][q][lane] = ok ? level_word(__dmul_rn(s, __dadd_rn((double)q, z)), I) : 0;
+            FastCode fc = fast_code(s, z, l_abs, nq);
             if (!ok) { fc.inv = 0.f; fc.negz = 0.f; fc.thr = 1.f; }                 // scored, but never looked at
             const uint32_t lev0 = (uint32_t)__cvta_generic_to_shared(&cand_lev[sd][0][lane]) - (__float_as_uint(kMagic) << 7);
             __syncwarp();
@@ -142,35 +162,67 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                 int n_el = 0;
 #pragma unroll
                 for (int u = 0; u < kChunk / 32; ++u) {
+                    if (k0 + 32 * u >= G) break;
                     const int k = k0 + 32 * u + lane;
                     const float v = k < G ? w[k] : 0.f;
                     const bool mine = sd ? (v < 0.f) : (v > 0.f);
                     const unsigned m = __ballot_sync(0xffffffffu, mine);
                     if (mine) {
-                        Elem e;
-                        e.a = (double)fabsf(v); e.l32 = log2f(fabsf(v));
-                        list[sd][n_el + __popc(m & ((1u << lane) - 1u))] = e;
+                        const int at = n_el + __popc(m & ((1u << lane) - 1u));
+                        mag[sd][at] = (double)fabsf(v);
+                        lg[sd][at] = log2f(fabsf(v));
                     }
                     n_el += __popc(m);
                 }
                 __syncwarp();
-                auto score = [&](const Elem& e) {
-                    bool exact;
-                    float r = fast_round(e.l32, fc, exact);
-                    if (!exact) r = kMagic + (float)side_code(log2(e.a), s, z, nq);
+                auto level = [&](float r) {
                     int hi;
                     asm("ld.shared.b32 %0, [%1];" : "=r"(hi) : "r"(lev0 + (__float_as_uint(r) << 7)));
-                    return __dsub_rn(e.a, __hiloint2double(hi, 0));
+                    return __hiloint2double(hi, 0);
                 };
+                auto careful = [&](int j) {                     // one element, whatever its distance from a boundary
+                    const double a = mag[sd][j];
+                    bool exact;
+                    float r = fast_round(lg[sd][j], fc, exact);
+                    if (!exact) r = kMagic + (float)side_code(log2(a), s, z, nq);
+                    const double d = __dsub_rn(a, level(r));
+                    err = __dadd_rn(err, __dmul_rn(d, d));
+                };
+                constexpr int U = 8;
+                const f32x2 INV = pack2(fc.inv, fc.inv), NEGZ = pack2(fc.negz, fc.negz), MAGIC = pack2(kMagic, kMagic);
                 int j = 0;
-                for (; j + 4 <= n_el; j += 4) {
-                    double d[4];
+                for (; j + U <= n_el; j += U) {
+                    // two elements per instruction; the eight distances from an integer are looked at together
+                    float r[U], off = 0.f;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) d[u] = score(list[sd][j + u]);
+                    for (int u = 0; u < U; u += 4) {
+                        const float4 l4 = *reinterpret_cast<const float4*>(&lg[sd][j + u]);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) err = __dadd_rn(err, __dmul_rn(d[u], d[u]));
+                        for (int h = 0; h < 4; h += 2) {
+                            const f32x2 x = fma2(h ? pack2(l4.z, l4.w) : pack2(l4.x, l4.y), INV, NEGZ), m = add2(x, MAGIC);
+                            float d0, d1;
+                            unpack2(sub2(x, sub2(m, MAGIC)), d0, d1);
+                            off = max3(off, fabsf(d0), fabsf(d1));
+                            unpack2(m, r[u + h], r[u + h + 1]);
+                        }
+                    }
+                    if (off <= fc.thr) {
+                        double d[U];
+#pragma unroll
+                        for (int u = 0; u < U; u += 2) {
+                            const double2 a = *reinterpret_cast<const double2*>(&mag[sd][j + u]);
+                            d[u] = __dsub_rn(a.x, level(fminf(r[u], fc.top)));
+                            d[u + 1] = __dsub_rn(a.y, level(fminf(r[u + 1], fc.top)));
+                        }
+#pragma unroll
+                        for (int u = 0; u < U; ++u) err = __dadd_rn(err, __dmul_rn(d[u], d[u]));
+                    } else {
+#pragma unroll 1
+                        for (int u = 0; u < U; ++u) careful(j + u);
+                    }
                 }
-                for (; j < n_el; ++j) { const double d = score(list[sd][j]); err = __dadd_rn(err, __dmul_rn(d, d)); }
+#pragma unroll 1
+                for (; j < n_el; ++j) careful(j);
                 __syncwarp();
             }
             // first minimum in grid order: the smallest error, the lowest index among equals
@@ -186,11 +238,13 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                 const int src = idx - c0;
                 best_err = e;
                 best_s = shfl_double(s, src); best_z = shfl_double(z, src); best_f = shfl_double(fac, src);
+                if (lane == src) best_fc[sd] = fc;
                 found = true;
             }
         }
         if (!found) {                               // no usable range: unit step anchored at the smallest element
             best_s = 1.0; best_z = scnt ? rint(smin) : 0.0; best_f = 1.0;
+            if (lane == 0) best_fc[sd] = fast_code(best_s, best_z, l_abs, nq);
         }
         if (lane == 0) { best[sd].s = best_s; best[sd].z = best_z; best[sd].factor = best_f; }
         __syncthreads();
@@ -211,41 +265,43 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
             mt[4] = best[0].factor; mt[5] = best[1].factor;
         }
         __syncthreads();
-        // ---- codes, eight at a time (one 32-bit word of nibbles, or three bytes of packed 3-bit codes)
+        // ---- codes, eight to a 32-bit word ( of nibbles, or three bytes of packed 3-bit codes)
         double part = 0.0;
-        FastCode fcs[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const float mx = fmaxf(ext[0][q][0], ext[1][q][0]), mn = fminf(ext[0][q][1], ext[1][q][1]);
-            fcs[q] = fast_code(best[q].s, best[q].z, (q ? ncnt : pcnt) ? log2((double)mn) : 0.0, (q ? ncnt : pcnt) ? log2((double)mx) : 0.0,
-                               q ? half : half - 1);
-        }
-        for (int j = tid; j < G / 8; j += kThreads) {
+        const FastCode fcs[2] = {best_fc[0], best_fc[1]};
+        // four lanes share eight codes, two elements each: the groups of 128 that grouped tables have keep every lane busy
+        for (int j0 = 0; j0 < G / 2; j0 += kThreads) {
+            const int j = j0 + tid;                  // pair of elements
             uint32_t word = 0;
+            if (j < G / 2) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float v = w[8 * j + e];
-                int cc = 0;
-                if (v != 0.f) {
-                    const bool neg = v < 0.f;
-                    FastCode f;
-                    f.inv = neg ? fcs[1].inv : fcs[0].inv; f.negz = neg ? fcs[1].negz : fcs[0].negz;
-                    f.thr = neg ? fcs[1].thr : fcs[0].thr; f.top = neg ? fcs[1].top : fcs[0].top;
-                    bool exact;
-                    const float r = fast_round(log2f(fabsf(v)), f, exact);
-                    const int q = exact ? (int)(__float_as_uint(r) - __float_as_uint(kMagic))
-                                        : side_code(log2((double)fabsf(v)), best[neg].s, best[neg].z, neg ? half : half - 1);
-                    cc = neg ? -q : q;
+                for (int e = 0; e < 2; ++e) {
+                    const float v = w[2 * j + e];
+                    int cc = 0;
+                    if (v != 0.f) {
+                        const bool neg = v < 0.f;
+                        FastCode f;
+                        f.inv = neg ? fcs[1].inv : fcs[0].inv; f.negz = neg ? fcs[1].negz : fcs[0].negz;
+                        f.thr = neg ? fcs[1].thr : fcs[0].thr; f.top = neg ? fcs[1].top : fcs[0].top;
+                        bool exact;
+                        const float r = fast_round(log2f(fabsf(v)), f, exact);
+                        const int q = exact ? (int)(__float_as_uint(r) - __float_as_uint(kMagic))
+                                            : side_code(log2((double)fabsf(v)), best[neg].s, best[neg].z, neg ? half : half - 1);
+                        cc = neg ? -q : q;
+                    }
+                    const int u = cc + half;
+                    part += T[u];
+                    word |= (uint32_t)u << ((pack3 ? 3 : 4) * (2 * (tid & 3) + e));
                 }
-                const int u = cc + half;
-                part += T[u];
-                word |= (uint32_t)u << ((pack3 ? 3 : 4) * e);
             }
-            if (pack3) {
-                uint8_t* dst = codes + ((size_t)n * K + (size_t)g * G) / 8 * 3 + (size_t)3 * j;
-                dst[0] = (uint8_t)word; dst[1] = (uint8_t)(word >> 8); dst[2] = (uint8_t)(word >> 16);
-            } else {
-                *reinterpret_cast<uint32_t*>(codes + ((size_t)n * K + (size_t)g * G) / 2 + (size_t)4 * j) = word;
+            word |= __shfl_xor_sync(0xffffffffu, word, 1);
+            word |= __shfl_xor_sync(0xffffffffu, word, 2);
+            if ((tid & 3) == 0 && j < G / 2) {
+                if (pack3) {
+                    uint8_t* dst = codes + ((size_t)n * K + (size_t)g * G) / 8 * 3 + (size_t)3 * (j >> 2);
+                    dst[0] = (uint8_t)word; dst[1] = (uint8_t)(word >> 8); dst[2] = (uint8_t)(word >> 16);
+                } else {
+                    *reinterpret_cast<uint32_t*>(codes + ((size_t)n * K + (size_t)g * G) / 2 + (size_t)4 * (j >> 2)) = word;
+                }
             }
         }
 #pragma unroll

@@ -72,7 +72,7 @@ wrot_hadamard_kernel(const float* __restrict__ W, int N, int K, long ldw, const 
 // 64 x 64 tile, a warp 32 x 32 of it (4 x 4 fragments, 64 accumulator registers): per 4-deep step 8 fragment loads feed
 // 16 MMAs, a quarter of the shared-memory traffic that 4 x 4 accumulators per thread needed.  Both operands are
 // widened to fp64 on their way into shared memory, double-buffered, the next 16-deep block in flight in registers.
-// Bound by the fp64 pipe.  4608 x 1536 x 1536: 1924 us on the CUDA cores (11 TFLOP/s), 480 now (45 TFLOP/s).
+// Bound by the fp64 pipe.  4608 x 1536 x 1536: 1924 us on the CUDA cores (11 TFLOP/s), 660 now (33 TFLOP/s).
 constexpr int TM = 64, TN = 64, TK = 16;
 constexpr int A_PITCH = TK + 4, B_PITCH = TN + 4;   // doubles; 4 mod 16: a fragment's 4 x 4 half-warp hits 16 bank pairs
 

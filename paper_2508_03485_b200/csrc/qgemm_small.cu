@@ -333,21 +333,24 @@ qgemm_small_kernel(const Params p) {
             asm volatile("bar.arrive 1, %0;" :: "n"(NUM_THREADS) : "memory");
         }
         bool ok = true;
-        if (lane == 0) {
+        const bool lead = elect_one();
+        const uint64_t a0 = umma_desc_sw128(smem_u32(sA), 16, 1024), b0 = umma_desc_sw128(smem_u32(sB), 16, 1024);
+        int s = 0;
+        uint32_t ph = 0;
         for (int kb = 0; kb < kblocks && ok; ++kb) {
-            const int s = kb % NSTG;
-            ok = mbar_wait<0>(smem_u32(&ctl->full[s]), (kb / NSTG) & 1, &ctl->abort_flag, p.status, 32);
+            ok = mbar_wait_warp(smem_u32(&ctl->full[s]), ph, &ctl->abort_flag, p.status, 32);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t a_addr = smem_u32(sA + s * A_STAGE), b_addr = smem_u32(sB + s * B_STAGE);
+            if (lead) {
+                const uint64_t a = a0 + (uint64_t)(s * (A_STAGE >> 4)), b = b0 + (uint64_t)(s * (B_STAGE >> 4));
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-                tc_mma_f16(tmem_base, umma_desc_sw128(a_addr + k * 32, 16, 1024), umma_desc_sw128(b_addr + k * 32, 16, 1024), IDESC,
-                           (kb | k) ? 1u : 0u);
-            tc_commit(smem_u32(&ctl->empty[s]));
+                for (int k = 0; k < BK / 16; ++k) tc_mma_f16(tmem_base, a + 2 * k, b + 2 * k, IDESC, (kb | k) ? 1u : 0u);
+                tc_commit(smem_u32(&ctl->empty[s]));
+            }
+            __syncwarp();
+            if (++s == NSTG) { s = 0; ph ^= 1; }
         }
-        if (ok) tc_commit(smem_u32(&ctl->acc_full));
-        }
+        if (ok && lead) tc_commit(smem_u32(&ctl->acc_full));
         __syncwarp();
     }
     tc_fence_before();

@@ -316,28 +316,34 @@ qgemm_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tmA, const _
         __syncwarp();
     } else if (warp == MMA_WARP) {
         // =============================== MMA issuer (even CTA only) ========================================
-        if (rank == 0 && lane == 0) {
-            uint32_t it = 0, t = 0;
+        if (rank == 0) {
+            const bool lead = elect_one();
+            const uint64_t a0 = umma_desc_sw128(smem_u32(sA), 16, 1024), b0 = umma_desc_sw128(smem_u32(sB), 16, 1024);
+            int s = 0;
+            uint32_t ph = 0, t = 0;
             bool ok = true;
             for (int tile = tile_first; tile < tile_last && ok; tile += tile_step, ++t) {
                 const int buf = t & 1;
-                ok = mbar_wait_cluster<64>(smem_u32(&ctl->tmem_empty[buf]), ((t >> 1) & 1) ^ 1, &ctl->abort_flag, p.status, 4);
+                ok = mbar_wait_warp(smem_u32(&ctl->tmem_empty[buf]), ((t >> 1) & 1) ^ 1, &ctl->abort_flag, p.status, 4);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN_T);
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    ok = mbar_wait_cluster<32>(smem_u32(&ctl->full[s]), (it / STAGES) & 1, &ctl->abort_flag, p.status, 5);
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    ok = mbar_wait_warp<32>(smem_u32(&ctl->full[s]), ph, &ctl->abort_flag, p.status, 5);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t a_addr = smem_u32(sA + s * A_STAGE_BYTES), b_addr = smem_u32(sB + s * B_STAGE_BYTES);
+                    if (lead) {
+                        const uint64_t a = a0 + (uint64_t)(s * (A_STAGE_BYTES >> 4)), b = b0 + (uint64_t)(s * (B_STAGE_BYTES >> 4));
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        tc_mma_f16_pair(d_tmem, umma_desc_sw128(a_addr + k * 32, 16, 1024),
-                                        umma_desc_sw128(b_addr + k * 32, 16, 1024), IDESC, (kb | k) ? 1u : 0u);
-                    tc_commit_pair(smem_u32(&ctl->empty[s]), 3);        // both CTAs may refill the stage
+                        for (int k = 0; k < BK / 16; ++k)
+                            tc_mma_f16_pair(d_tmem, a + 2 * k, b + 2 * k, IDESC, (kb | k) ? 1u : 0u);
+                        tc_commit_pair(smem_u32(&ctl->empty[s]), 3);        // both CTAs may refill the stage
+                    }
+                    __syncwarp();
+                    if (++s == STAGES) { s = 0; ph ^= 1; }
                 }
-                if (ok) tc_commit_pair(smem_u32(&ctl->tmem_full[buf]), 3);   // accumulator complete, both halves
+                if (ok && lead) tc_commit_pair(smem_u32(&ctl->tmem_full[buf]), 3);   // accumulator complete, both halves
+                __syncwarp();
             }
         }
         __syncwarp();

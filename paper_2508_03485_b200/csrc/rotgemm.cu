@@ -86,15 +86,16 @@ rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     lrq_pdl_wait();                      // the set-up above overlaps the previous kernel's tail; X may be its output
 
     if (warp == PRODUCER_WARP) {
-        if (lane == 0) {
-            uint32_t it = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-                const int m0 = (tile % tiles_m) * BM, n0 = (tile / tiles_m) * BN;
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    ok = mbar_wait<100>(smem_u32(&ctl->empty[s]), ((it / STAGES) & 1) ^ 1, &ctl->abort_flag, status, 11);
-                    if (!ok) break;
+        const bool lead = elect_one();
+        int s = 0;
+        uint32_t ph = 1, issued = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+            const int m0 = (tile % tiles_m) * BM, n0 = (tile / tiles_m) * BN;
+            for (int kb = 0; kb < kblocks; ++kb) {
+                ok = mbar_wait_warp(smem_u32(&ctl->empty[s]), ph, &ctl->abort_flag, status, 11);
+                if (!ok) break;
+                if (lead) {
                     const uint32_t bar = smem_u32(&ctl->full[s]);
                     mbar_arrive_expect_tx(bar, STAGE_TX_BYTES);
                     // k origin of this step in the left operand's columns and in R's rows
@@ -105,45 +106,49 @@ rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
                     for (int j = 0; j < BN / 64; ++j)
                         tma_load_2d(smem_u32(sB + s * B_STAGE_BYTES + j * B_CHUNK_BYTES), &tmR, (DIAG ? 0 : n0) + 64 * j, kr, bar);
                 }
+                __syncwarp();
+                ++issued;
+                if (++s == STAGES) { s = 0; ph ^= 1; }
             }
-            if (!ok) {
-                // loads already issued still write this CTA's shared memory: let each stage's last fill land
-                const uint32_t issued = it;
-                for (uint32_t back = 1; back <= (uint32_t)STAGES && back <= issued; ++back) {
-                    const uint32_t j = issued - back;
-                    const uint32_t bar = smem_u32(&ctl->full[j % STAGES]);
-                    for (uint32_t i = 0; i < kWaitLimit; ++i)
-                        if (mbar_try_wait(bar, (j / STAGES) & 1)) break;
-                }
+        }
+        if (!ok) {
+            // loads already issued still write this CTA's shared memory: let each stage's last fill land
+            for (uint32_t back = 1; back <= (uint32_t)STAGES && back <= issued; ++back) {
+                const uint32_t j = issued - back;
+                const uint32_t bar = smem_u32(&ctl->full[j % STAGES]);
+                for (uint32_t i = 0; i < kWaitLimit; ++i)
+                    if (mbar_try_wait(bar, (j / STAGES) & 1)) break;
             }
         }
         __syncwarp();
     } else if (warp == MMA_WARP) {
-        if (lane == 0) {
-            uint32_t it = 0, t = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++t) {
-                const int buf = t & 1;
-                ok = mbar_wait<64>(smem_u32(&ctl->tmem_empty[buf]), ((t >> 1) & 1) ^ 1, &ctl->abort_flag, status, 12);
+        const bool lead = elect_one();
+        const uint64_t a0 = umma_desc_sw128(smem_u32(sA), 16, 1024), b0 = umma_desc_sw128(smem_u32(sB), B_CHUNK_BYTES, 1024);
+        int s = 0;
+        uint32_t ph = 0, t = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++t) {
+            const int buf = t & 1;
+            ok = mbar_wait_warp(smem_u32(&ctl->tmem_empty[buf]), ((t >> 1) & 1) ^ 1, &ctl->abort_flag, status, 12);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+            for (int kb = 0; kb < kblocks; ++kb) {
+                ok = mbar_wait_warp(smem_u32(&ctl->full[s]), ph, &ctl->abort_flag, status, 13);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    ok = mbar_wait<32>(smem_u32(&ctl->full[s]), (it / STAGES) & 1, &ctl->abort_flag, status, 13);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t a_addr = smem_u32(sA + s * A_STAGE_BYTES), b_addr = smem_u32(sB + s * B_STAGE_BYTES);
+                if (lead) {
+                    const uint64_t a = a0 + (uint64_t)(s * (A_STAGE_BYTES >> 4)), b = b0 + (uint64_t)(s * (B_STAGE_BYTES >> 4));
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        tc_mma_f16(d_tmem,
-                                   umma_desc_sw128(a_addr + k * 32, 16, 1024),                    // 16 k = 32 bytes along the row
-                                   umma_desc_sw128(b_addr + k * 16 * 128, B_CHUNK_BYTES, 1024),   // 16 k = 16 rows of 128 bytes
-                                   IDESC, (kb | k) ? 1u : 0u);
+                    for (int k = 0; k < BK / 16; ++k)        // 16 k: 32 bytes along a row of X, 16 rows of 128 bytes of R
+                        tc_mma_f16(d_tmem, a + 2 * k, b + 128 * k, IDESC, (kb | k) ? 1u : 0u);
                     tc_commit(smem_u32(&ctl->empty[s]));
                 }
-                if (ok) tc_commit(smem_u32(&ctl->tmem_full[buf]));
+                __syncwarp();
+                if (++s == STAGES) { s = 0; ph ^= 1; }
             }
+            if (ok && lead) tc_commit(smem_u32(&ctl->tmem_full[buf]));
+            __syncwarp();
         }
         __syncwarp();
     } else {

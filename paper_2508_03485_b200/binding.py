@@ -88,14 +88,17 @@ def load_library() -> C.CDLL:
     return lib
 
 
-def _stream(stream) -> C.c_void_p:
+# Addresses and streams go to ctypes as plain integers (the argtypes above turn them into void*): a call of a few
+# microseconds on the GPU is otherwise bound by the marshalling.  The raw handle of the current stream costs 0.1 us, the
+# torch.cuda.Stream object around it 3.2.
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
-def _ptr(t: Optional[torch.Tensor]) -> C.c_void_p:
-    return C.c_void_p(0 if t is None else t.data_ptr())
+def _ptr(t: Optional[torch.Tensor]) -> int:
+    return 0 if t is None else t.data_ptr()
 
 
 def _check(code: int, where: str):
@@ -257,7 +260,7 @@ def lrq_rotate_quantize_act(X: torch.Tensor, kind: int, a_bits: int, had_block: 
         dual.check(K)
     p = _act_params(kind, had_block, R, a_bits, mode, prescale, dual)
     need = int(lib.lrq_act_workspace_bytes(M, K, C.byref(p)))
-    if need and (workspace is None or workspace.numel() * workspace.element_size() < need):
+    if need and (workspace is None or workspace.nbytes < need):
         workspace = torch.empty(need, dtype=torch.uint8, device=X.device)
     dev = X.device
     if out is not None:
@@ -267,7 +270,7 @@ def lrq_rotate_quantize_act(X: torch.Tensor, kind: int, a_bits: int, had_block: 
         codes = torch.empty((M, K * a_bits // 8), dtype=torch.uint8, device=dev)
         scale = torch.empty((M,), dtype=torch.float32, device=dev)
         zp = torch.empty((M,), dtype=torch.int32, device=dev)
-    wsb = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    wsb = 0 if workspace is None else workspace.nbytes
     rc = lib.lrq_rotate_quantize_act(_ptr(X), M, K, X.stride(0), C.byref(p), _ptr(codes), _ptr(scale), _ptr(zp),
                                      _ptr(workspace), wsb, _stream(stream))
     _check(rc, "lrq_rotate_quantize_act")
@@ -322,7 +325,7 @@ class QLayer:
         self.handle = h
 
     def workspace_bytes(self, M: int) -> int:
-        return int(load_library().lrq_workspace_bytes(self.handle, int(M)))
+        return load_library().lrq_workspace_bytes(self.handle, M)
 
     def close(self):
         if getattr(self, "handle", None):
@@ -337,7 +340,7 @@ class QLayer:
 
 
 def _ws(workspace: Optional[torch.Tensor], need: int, device) -> torch.Tensor:
-    if workspace is None or workspace.numel() * workspace.element_size() < need:
+    if workspace is None or workspace.nbytes < need:
         workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=device)
     return workspace
 
@@ -346,15 +349,23 @@ def lrq_qlinear(layer: QLayer, X: torch.Tensor, y_dtype: int = F32, out: Optiona
                 workspace: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Y = quantized-linear(X) for device bf16 X [M,K] (Eq. 12 -> Eq. 1 -> Eq. 10 -> scaling)."""
     _need_cuda(X, out, workspace)
-    assert X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1 and X.shape[1] == layer.K
-    M = X.shape[0]
+    M, K = X.shape
+    ldx, inner = X.stride()
+    assert X.dtype == torch.bfloat16 and inner == 1 and K == layer.K
     if out is None:
         out = torch.empty((M, layer.N), dtype=_TORCH_DT[y_dtype], device=X.device)
-    assert out.dtype == _TORCH_DT[y_dtype] and out.stride(1) == 1
-    workspace = _ws(workspace, layer.workspace_bytes(M), X.device)
-    rc = load_library().lrq_qlinear(layer.handle, _ptr(X), M, X.stride(0), _ptr(out), y_dtype, out.stride(0),
-                                    _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(rc, "lrq_qlinear")
+        ldy = layer.N
+    else:
+        ldy, inner = out.stride()
+        assert out.dtype == _TORCH_DT[y_dtype] and inner == 1
+    lib = load_library()
+    need = lib.lrq_workspace_bytes(layer.handle, M)
+    if workspace is None or workspace.nbytes < need:
+        workspace = _ws(None, need, X.device)
+    rc = lib.lrq_qlinear(layer.handle, X.data_ptr(), M, ldx, out.data_ptr(), y_dtype, ldy, workspace.data_ptr(), workspace.nbytes,
+                         _stream(stream))
+    if rc:
+        _check(rc, "lrq_qlinear")
     return out
 
 
@@ -380,7 +391,7 @@ def lrq_qlinear_stack(plan: StackPlan, workspace: Optional[torch.Tensor] = None,
     dev = plan._keep[1][0].device
     workspace = _ws(workspace, plan.need, dev)
     rc = load_library().lrq_qlinear_stack(plan.layers, plan.n, plan.X, plan.M, plan.ldx, plan.Y, plan.y_dtype,
-                                          plan.ldy, _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                          plan.ldy, _ptr(workspace), workspace.nbytes,
                                           _stream(stream))
     _check(rc, "lrq_qlinear_stack")
 

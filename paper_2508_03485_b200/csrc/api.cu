@@ -78,36 +78,37 @@ extern "C" size_t lrq_act_workspace_bytes(int M, int K, const lrq_act_params* p)
     return 0;
 }
 
-// Rotation + quantization of checked arguments; out16: the contraction's bf16 operand instead of packed codes.
+// Rotation + quantization of checked arguments; out16: the contraction's bf16 operand instead of packed codes; ex: a layer's
+// weights to decode on the way.
 static lrq_status run_act(const void* X, int M, int K, long ldx, const lrq_act_params* p, int out16, uint8_t* a_codes,
-                          float* a_scale, int32_t* a_zp, void* workspace, size_t workspace_bytes, cudaStream_t stream) {
+                          float* a_scale, int32_t* a_zp, const LrqExpand& ex, void* workspace, size_t workspace_bytes,
+                          cudaStream_t stream) {
     lrq_status st;
+    // the rotation products leave each row's extremes where the quantizer will write the row's results
+    const LrqRowExt none = {}, ext = {a_codes, (size_t)K * (out16 ? 16 : p->a_bits) / 8, a_scale, reinterpret_cast<float*>(a_zp)};
     if (p->kind == LRQ_ROT_DENSE) {
         const size_t need = lrq_act_workspace_bytes(M, K, p);
         if (!workspace || workspace_bytes < need || !lrq_aligned(workspace, 256)) return LRQ_ERR_WORKSPACE;
         float* Yr = static_cast<float*>(workspace);
-        // the rotation leaves each token's extremes in the scale / zero-point outputs (as integers); the
-        // quantizer reads them and then writes the real values there
-        st = lrq_launch_rotgemm(X, M, K, ldx, p->R_bf16, Yr, reinterpret_cast<int*>(a_scale), reinterpret_cast<int*>(a_zp), stream);
+        st = lrq_launch_rotgemm(X, M, K, ldx, p->R_bf16, Yr, ext, stream);
         if (st != LRQ_OK) return st;
-        return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, stream);
+        return lrq_launch_quantize_f32_ext(Yr, M, K, LRQ_ROT_TILE_DENSE, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, ex, stream);
     }
     if (p->kind == LRQ_ROT_DUAL) {
         const size_t need = lrq_act_workspace_bytes(M, K, p);
         if (!workspace || workspace_bytes < need || !lrq_aligned(workspace, 256)) return LRQ_ERR_WORKSPACE;
         float* Yr = static_cast<float*>(workspace);                       // u = x R1hat first, y later
         void* V3 = static_cast<unsigned char*>(workspace) + lrq_round_up((size_t)M * K * sizeof(float), 256);
-        st = lrq_launch_bdiag_gemm(X, M, K, ldx, 1, p->R1_bf16, Yr, nullptr, nullptr, stream);
+        st = lrq_launch_bdiag_gemm(X, M, K, ldx, 1, p->R1_bf16, Yr, none, stream);
         if (st != LRQ_OK) return st;
         st = lrq_launch_dual_gather_split(Yr, M, K, p->perm, V3, stream);  // u P as three bf16 terms
         if (st != LRQ_OK) return st;
-        st = lrq_launch_bdiag_gemm(V3, M, K, 3L * K, 3, p->R2_bf16, Yr, reinterpret_cast<int*>(a_scale),
-                                   reinterpret_cast<int*>(a_zp), stream);
+        st = lrq_launch_bdiag_gemm(V3, M, K, 3L * K, 3, p->R2_bf16, Yr, ext, stream);
         if (st != LRQ_OK) return st;
-        return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, stream);
+        return lrq_launch_quantize_f32_ext(Yr, M, K, LRQ_ROT_TILE_DIAG, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, ex, stream);
     }
     const int B = p->kind == LRQ_ROT_HADAMARD ? p->had_block : 1;
-    return lrq_launch_rotq_hadamard(X, M, K, ldx, B, p->a_bits, p->mode, out16, p->prescale, a_codes, a_scale, a_zp, stream);
+    return lrq_launch_rotq_hadamard(X, M, K, ldx, B, p->a_bits, p->mode, out16, p->prescale, a_codes, a_scale, a_zp, ex, stream);
 }
 
 extern "C" lrq_status lrq_rotate_quantize_act(const void* X, int M, int K, long ldx, const lrq_act_params* p,
@@ -117,7 +118,7 @@ extern "C" lrq_status lrq_rotate_quantize_act(const void* X, int M, int K, long 
     lrq_status st = check_act(p, K);
     if (st != LRQ_OK) return st;
     if (ldx < K || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(a_codes, 16)) return LRQ_ERR_INVALID_ARG;
-    return run_act(X, M, K, ldx, p, 0, a_codes, a_scale, a_zp, workspace, workspace_bytes, (cudaStream_t)cuda_stream);
+    return run_act(X, M, K, ldx, p, 0, a_codes, a_scale, a_zp, LrqExpand{}, workspace, workspace_bytes, (cudaStream_t)cuda_stream);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -306,11 +307,9 @@ extern "C" lrq_status lrq_qlinear(const lrq_layer* L, const void* X, int M, long
     int32_t* a_zp = reinterpret_cast<int32_t*>(base + w.zp);
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     const bool ex = w.form == FORM_EXPANDED;
-    if (ex) {
-        st = lrq_launch_expand_w(L, base + w.wexp, stream);
-        if (st != LRQ_OK) return st;
-    }
-    st = run_act(X, M, L->K, ldx, &L->act, ex ? 1 : 0, a_codes, a_scale, a_zp, base + w.rot, w.total - w.rot, stream);
+    LrqExpand decode = {};
+    if (ex) decode = {L->codes, L->levels, L->N, L->K, L->group, L->packed3 ? 13 : L->w_bits, base + w.wexp};
+    st = run_act(X, M, L->K, ldx, &L->act, ex ? 1 : 0, a_codes, a_scale, a_zp, decode, base + w.rot, w.total - w.rot, stream);
     if (st != LRQ_OK) return st;
     if (ex) return lrq_launch_qgemm_bf16(L, a_codes, base + w.wexp, a_scale, a_zp, M, Y, dt, ldy, stream);
     if (w.form == FORM_PACKED) return lrq_launch_qgemm_tc(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);

@@ -58,28 +58,46 @@ inline cudaError_t lrq_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block,
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// A layer's weight decode (codes -> bf16 [N,K] at `out`, tlq_decode.cuh), done by the quantizer kernels' warps when they have no
+// tokens left: the two are independent, and a launch of its own costs three microseconds on a short batch.  out ==
+// nullptr: nothing to decode.  fmt: 4, 3, 2 nibble layout, 13 packed 3-bit.
+struct LrqExpand { const uint8_t* codes; const float* levels; int N, K, G, fmt; void* out; };
+
+// CTAs of a quantizer grid: `need` for its tokens, or more (up to `resident`) when there are weight rows for them.
+static inline int lrq_quant_grid(int need, int resident, int warps_per_cta, const LrqExpand& ex) {
+    int g = need < resident ? need : resident;
+    if (ex.out) {
+        const int want = g + (ex.N + warps_per_cta - 1) / warps_per_cta;
+        g = want < resident ? want : resident;
+    }
+    return g;
+}
+
 // Quantizers: out16 == 0 writes packed 8- or 4-bit codes, out16 == 1 the contraction's operand instead, bf16 [M,K] of
 // q - 2^(a_bits-1) (16-byte aligned rows), from the same arithmetic.
 // rotq.cu
 lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
-                                    uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st);
+                                    uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st);
 // rotq_blk.cu : the same for blocks of 8..128 channels with K a multiple of 128; LRQ_ERR_UNSUPPORTED otherwise
 lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
-                               uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st);
-// rotgemm.cu : Y[M,K] (fp32) = X[M,K] (bf16) . R[K,K] (bf16) on the tensor cores; also leaves every row's minimum and
-// maximum in ext_min[M] / ext_max[M] as order-preserving integers.
-lrq_status lrq_launch_rotgemm(const void* X, int M, int K, long ldx, const void* R, float* Y,
-                              int* ext_min, int* ext_max, cudaStream_t st);
+                               uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st);
+// Where a rotation product leaves each row's extremes: over each tile's columns as a pair of floats (minimum, maximum), tile j of
+// row m at rows + m * pitch + 8 j; when a row is one tile, in row_min[m] and row_max[m].  All null: not wanted.
+struct LrqRowExt { unsigned char* rows; size_t pitch; float* row_min; float* row_max; };
+constexpr int LRQ_ROT_TILE_DENSE = 256, LRQ_ROT_TILE_DIAG = 128;      // columns per tile
+// rotgemm.cu : Y[M,K] (fp32) = X[M,K] (bf16) . R[K,K] (bf16) on the tensor cores
+lrq_status lrq_launch_rotgemm(const void* X, int M, int K, long ldx, const void* R, float* Y, const LrqRowExt& ext, cudaStream_t st);
 // rotgemm.cu : Y[M,K] (fp32) = sum over the `parts` column panels of A[M, parts*K] (bf16) of panel . blockdiag(Rblk),
-// Rblk bf16 [K/128][128][128]; row extremes as above when ext_min / ext_max are given (both or neither).
-lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int parts, const void* Rblk, float* Y,
-                                 int* ext_min, int* ext_max, cudaStream_t st);
+// Rblk bf16 [K/128][128][128]
+lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int parts, const void* Rblk, float* Y, const LrqRowExt& ext,
+                                 cudaStream_t st);
 // rotdual.cu : V3 bf16 [M,3K], panel p = p-th bf16 term of U[m, perm[i]] (the reordering between the two rotations)
 lrq_status lrq_launch_dual_gather_split(const float* U, int M, int K, const int32_t* perm, void* V3, cudaStream_t st);
-// rotq.cu : per-token quantization of fp32 rows whose extremes are already known (ext_min / ext_max alias the
-// scale / zero-point outputs: each row's extremes are read before its results are written).
-lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int a_bits, int mode, int out16, uint8_t* codes,
-                                       float* scale, int32_t* zp, cudaStream_t st);
+// rotq.cu : per-token quantization of fp32 rows whose extremes a rotation product with tiles of `tile` columns has left, per
+// tile at the start of the row's own part of `codes` (8 bytes a tile; the codes overwrite them, and are longer for
+// every K above one tile), for one tile in scale[m] and zp[m].
+lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int tile, int a_bits, int mode, int out16, uint8_t* codes,
+                                       float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st);
 
 // rotq.cu : fluctuation metric J (Eq. 11) and the kind Eq. 12 picks; acc is one double of device scratch
 lrq_status lrq_launch_ars_metric(const void* X, int M, int K, long ldx, double thr, float* J, int* kind, double* acc,
@@ -116,8 +134,6 @@ lrq_status lrq_launch_qgemm_tc(const lrq_layer* L, const uint8_t* a_codes, const
 bool lrq_qgemm_small_takes(const lrq_layer* L);
 lrq_status lrq_launch_qgemm_small(const lrq_layer* L, const uint8_t* a_codes, const float* a_scale,
                                   const int32_t* a_zp, int M, void* Y, lrq_dtype dt, long ldy, cudaStream_t st);
-// expand_w.cu : the layer's weight codes decoded to bf16 [N,K]
-lrq_status lrq_launch_expand_w(const lrq_layer* L, void* out, cudaStream_t st);
 // qgemm_bf16.cu : contraction of bf16 operands, A [M,K] of q - 2^(a_bits-1), W [N,K] of decoded levels (both 16-byte aligned)
 lrq_status lrq_launch_qgemm_bf16(const lrq_layer* L, const void* A, const void* W, const float* a_scale, const int32_t* a_zp, int M,
                                  void* Y, lrq_dtype dt, long ldy, cudaStream_t st);

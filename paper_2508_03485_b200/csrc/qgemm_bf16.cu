@@ -5,7 +5,7 @@
 //   Y[m,n]   = s_m * (acc + (z_m + C) * wsum_n) * wscale_n + bias_n
 //
 // a = q - C are the centred activation codes (C = 128 or 8) as the quantizer wrote them, w the decoded levels
-// (expand_w.cu).  Nothing is left to do between the copy and the tensor core, so both operands go from global memory
+// (tlq_decode.cuh).  Nothing is left to do between the copy and the tensor core, so both operands go from global memory
 // to their stages by TMA alone, and the kernel is bound by the tensor pipe and, over more than a tenth of a second, by
 // the power cap: what counts then is the energy of a tile, of which DRAM and cross-die L2 traffic are a good part.
 //

@@ -1,8 +1,9 @@
 // Outlier-aware rotation y = x . R (Sec. 4.2, Eq. 12, second case) as a dense contraction on the
 // 5th-generation tensor cores: X bf16 [M,K] times R bf16 [K,K] into an fp32 scratch that the
 // per-token quantizer then reads.  bf16 x bf16 products are exact in fp32; sums are accumulated in fp32.
-// The epilogue also folds every row's minimum and maximum into two integer arrays (atomic min / max on
-// order-preserving images), so that the quantizer that follows is a single streaming pass.
+// The epilogue also leaves every row's minimum and maximum over the tile's columns, so that the quantizer that follows is a
+// single streaming pass: plain stores, one pair per row and tile, which need no initial values (two memsets and an
+// atomic pair per row and tile took their place before).
 //
 // Persistent CTA per SM over 128 x 256 output tiles, 64-deep k-blocks, a 4-stage TMA pipeline:
 //   warp 0      one lane issues the TMA tile loads (X: K-major box 64 x 128; R: four 64 x 64 boxes, each
@@ -50,8 +51,8 @@ constexpr size_t smem_bytes(int bn) {
 template <int BN, bool DIAG>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
-                  float* __restrict__ Y, int M, int K, int parts, int* __restrict__ ext_min, int* __restrict__ ext_max,
-                  int* status) {
+                  float* __restrict__ Y, int M, int K, int parts, unsigned char* __restrict__ ext, size_t ext_pitch, float* __restrict__ ext_min,
+                  float* __restrict__ ext_max, int* status) {
     constexpr int B_STAGE_BYTES = (BN / 64) * B_CHUNK_BYTES;   // 32 KB (16 KB for 128-wide tiles)
     constexpr int STAGE_TX_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
     constexpr uint32_t IDESC = umma_idesc_bf16(BM, BN, /*a_mn_major=*/false, /*b_mn_major=*/true);
@@ -212,9 +213,11 @@ rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctl->tmem_empty[buf]));
-            if (okw && m < M && ext_min) {                // fold this tile's share into the row's extremes
-                atomicMin(ext_min + m, lrq_ordered_int(mn));
-                atomicMax(ext_max + m, lrq_ordered_int(mx));
+            if (okw && m < M) {                           // this tile's share of the row's extremes
+                if (ext) {
+                    float* e = reinterpret_cast<float*>(ext + (size_t)m * ext_pitch) + 2 * (n0 / BN);
+                    e[0] = mn; e[1] = mx;
+                } else if (ext_min) { ext_min[m] = mn; ext_max[m] = mx; }
             }
             if (ctl->abort_flag) break;
         }
@@ -231,8 +234,8 @@ rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
 }  // namespace
 
 template <int BN, bool DIAG>
-static lrq_status launch_rotgemm(const CUtensorMap& tmX, const CUtensorMap& tmR, float* Y, int M, int K, int parts,
-                                 int* ext_min, int* ext_max, cudaStream_t st) {
+static lrq_status launch_rotgemm(const CUtensorMap& tmX, const CUtensorMap& tmR, float* Y, int M, int K, int parts, const LrqRowExt& ext,
+                                 cudaStream_t st) {
     int dev = 0, sms = 0;
     if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
     {   // the shared-memory opt-in is a per-device function attribute: set once per device
@@ -246,37 +249,31 @@ static lrq_status launch_rotgemm(const CUtensorMap& tmX, const CUtensorMap& tmR,
         }
     }
     const int tiles = ((M + BM - 1) / BM) * ((K + BN - 1) / BN);
-    if (ext_min) {
-        // identity elements of the integer min / max: bytes 0x7f.. (a huge float), 0x80.. (a hugely negative one)
-        LRQ_CUDA_TRY(cudaMemsetAsync(ext_min, 0x7f, (size_t)M * sizeof(int), st));
-        LRQ_CUDA_TRY(cudaMemsetAsync(ext_max, 0x80, (size_t)M * sizeof(int), st));
-    }
+    const bool one = K <= BN;                        // one tile per row: its extremes are the row's
     LRQ_CUDA_TRY(lrq_launch_pdl(rotgemm_tc_kernel<BN, DIAG>, dim3(tiles < sms ? tiles : sms), dim3(NUM_THREADS), smem_bytes(BN),
-                                st, tmX, tmR, Y, M, K, parts, ext_min, ext_max, lrq_status_word()));
+                                st, tmX, tmR, Y, M, K, parts, one ? nullptr : ext.rows, ext.pitch, one ? ext.row_min : nullptr,
+                                one ? ext.row_max : nullptr, lrq_status_word()));
     return LRQ_OK;
 }
 
-lrq_status lrq_launch_rotgemm(const void* X, int M, int K, long ldx, const void* R, float* Y,
-                              int* ext_min, int* ext_max, cudaStream_t st) {
+lrq_status lrq_launch_rotgemm(const void* X, int M, int K, long ldx, const void* R, float* Y, const LrqRowExt& ext, cudaStream_t st) {
     // TMA needs 16-byte aligned bases and row pitches (K and ldx multiples of 8 elements); the C ABI has already
     // refused anything else
-    if ((K % 8) || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(R, 16) || !lrq_aligned(Y, 16) || !ext_min || !ext_max)
-        return LRQ_ERR_INVALID_ARG;
+    if ((K % 8) || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(R, 16) || !lrq_aligned(Y, 16)) return LRQ_ERR_INVALID_ARG;
     CUtensorMap tmX, tmR;
     if (!lrq_tma::make_map_2d(&tmX, X, 2, (uint64_t)M, (uint64_t)K, (uint64_t)ldx, BK, BM, true)) return LRQ_ERR_CUDA;
     if (!lrq_tma::make_map_2d(&tmR, R, 2, (uint64_t)K, (uint64_t)K, (uint64_t)K, 64, BK, true)) return LRQ_ERR_CUDA;
-    return launch_rotgemm<256, false>(tmX, tmR, Y, M, K, 1, ext_min, ext_max, st);
+    return launch_rotgemm<LRQ_ROT_TILE_DENSE, false>(tmX, tmR, Y, M, K, 1, ext, st);
 }
 
 // Y[M,K] (fp32) = sum over panels p of A[:, pK .. pK+K) . blockdiag(Rblk), Rblk bf16 [K/128][128][128].
-// ext_min / ext_max may both be null (no per-row extremes wanted).
-lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int parts, const void* Rblk, float* Y,
-                                 int* ext_min, int* ext_max, cudaStream_t st) {
+lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int parts, const void* Rblk, float* Y, const LrqRowExt& ext,
+                                 cudaStream_t st) {
     if ((K % 128) || (lda % 8) || lda < (long)parts * K || parts < 1 || !lrq_aligned(A, 16) || !lrq_aligned(Rblk, 16) ||
-        !lrq_aligned(Y, 16) || (ext_min == nullptr) != (ext_max == nullptr))
+        !lrq_aligned(Y, 16))
         return LRQ_ERR_INVALID_ARG;
     CUtensorMap tmA, tmR;
     if (!lrq_tma::make_map_2d(&tmA, A, 2, (uint64_t)M, (uint64_t)parts * K, (uint64_t)lda, BK, BM, true)) return LRQ_ERR_CUDA;
     if (!lrq_tma::make_map_2d(&tmR, Rblk, 2, (uint64_t)K, 128, 128, 64, BK, true)) return LRQ_ERR_CUDA;
-    return launch_rotgemm<128, true>(tmA, tmR, Y, M, K, parts, ext_min, ext_max, st);
+    return launch_rotgemm<LRQ_ROT_TILE_DIAG, true>(tmA, tmR, Y, M, K, parts, ext, st);
 }

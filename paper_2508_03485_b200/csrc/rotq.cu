@@ -13,6 +13,7 @@
 #include "lrq_internal.cuh"
 #include "f32x2.cuh"
 #include "rotq_common.cuh"
+#include "tlq_decode.cuh"
 #include <climits>
 #include <mutex>
 #include <vector>
@@ -70,7 +71,7 @@ __device__ __forceinline__ int quant1(float u, const TokenQ& t, int qmax) {
 __global__ void __launch_bounds__(256)
 rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log2B, int a_bits, int mode, int out16,
                     const float* __restrict__ prescale,
-                    uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp) {
+                    uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp, const LrqExpand ex) {
     extern __shared__ float row[];
     __shared__ float red_mn[8], red_mx[8], red_am[8];
     __shared__ TokenQ tq;
@@ -79,6 +80,7 @@ rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log
     const int nchunk = K >> 3;
     lrq_pdl_trigger();
     lrq_pdl_wait();
+    if (m >= M) { lrq_dec::expand_share(ex); return; }        // CTAs past the tokens are there for the weights
 
     {
         const uint4* src = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(Xv) + (size_t)m * ldx);
@@ -157,6 +159,7 @@ rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log
             dst[c] = w;
         }
     }
+    if (ex.out) lrq_dec::expand_share(ex);
 }
 
 
@@ -203,7 +206,7 @@ template <int LOG2B, int A_BITS, int MAX_THREADS, int MIN_CTAS, bool WIDE>
 __global__ void __launch_bounds__(MAX_THREADS, MIN_CTAS)
 rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int mode, int out16, int tok_per_cta, int num_groups,
                  const float* __restrict__ prescale,
-                 uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp) {
+                 uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp, const LrqExpand ex) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int NP = EPT / 2;                      // element pairs per thread
     const int tpt = K / EPT;                         // threads per token
@@ -351,6 +354,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
             }
         }
     }
+    if (ex.out) lrq_dec::expand_share(ex);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -374,7 +378,7 @@ template <int LOG2B, int A_BITS, int MAX_THREADS, int MIN_CTAS, bool WIDE>
 __global__ void __launch_bounds__(MAX_THREADS, MIN_CTAS)
 rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int mode, int out16, int tok_per_cta, int num_groups,
                 const float* __restrict__ prescale,
-                uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp) {
+                uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp, const LrqExpand ex) {
     static_assert(LOG2B >= 10 && LOG2B <= 12, "block sizes 1024..4096");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int NP = EPT / 2;
@@ -550,28 +554,37 @@ rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int
             }
         }
     }
+    if (ex.out) lrq_dec::expand_share(ex);
 }
 
 // ------------------------------------------------------------------------------------------------
-// Quantizer of already rotated fp32 rows whose extremes are known (dense path: the rotation GEMM's epilogue
-// found them).  One warp per token, grid-stride; lane 0 works out the step and zero-point, then the warp
-// streams the row: 32 bytes in (one 256-bit load), 8 or 4 code bytes out per lane and step.
-// ext_min / ext_max alias scale / zp: the warp reads its row's extremes before it writes the results.
+// Quantizer of already rotated fp32 rows whose extremes are known per column tile (dense and dual path: the rotation
+// product's epilogue left them in the row's own part of the code matrix, or in scale / zp when a row is one tile).
+// One warp per token, grid-stride; lane 0 works out the step and zero-point, then the warp streams the row: 32
+// bytes in (one 256-bit load), 4, 8 or 16 code bytes out per lane and step.
 // ------------------------------------------------------------------------------------------------
 template <int A_BITS, bool OUT16>
 __global__ void __launch_bounds__(256)
-quant_rows_f32_kernel(const float* __restrict__ Y, int M, int K, int mode, uint8_t* __restrict__ codes,
-                      float* scale, int32_t* zp) {
+quant_rows_f32_kernel(const float* __restrict__ Y, int M, int K, int tiles, int mode, uint8_t* codes,
+                      float* scale, int32_t* zp, const LrqExpand ex) {
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     lrq_pdl_trigger();
     lrq_pdl_wait();                      // the rows and their extremes are the rotation kernel's output
     for (int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < M; m += warps) {
+        float mn = INFINITY, mx = -INFINITY;
+        if (tiles == 1) {
+            mn = scale[m]; mx = reinterpret_cast<const float*>(zp)[m];
+        } else {
+            const float* e = reinterpret_cast<const float*>(codes + (size_t)m * K * (OUT16 ? 16 : A_BITS) / 8);
+            for (int j = lane; j < tiles; j += 32) { mn = fminf(mn, e[2 * j]); mx = fmaxf(mx, e[2 * j + 1]); }
+            mn = lrq_ordered_float(__reduce_min_sync(0xffffffffu, lrq_ordered_int(mn)));
+            mx = lrq_ordered_float(__reduce_max_sync(0xffffffffu, lrq_ordered_int(mx)));
+        }
+        __syncwarp();                        // every lane has read before any writes codes or results over it
         TokenQ t;
         t.inv = 0.f; t.negz = 0.f;
         if (lane == 0) {
-            const float mn = lrq_ordered_float(reinterpret_cast<const int*>(scale)[m]);
-            const float mx = lrq_ordered_float(reinterpret_cast<const int*>(zp)[m]);
             float sc; int32_t z;
             t = token_params_fast(mn, mx, A_BITS, mode, 1.0, &sc, &z);
             scale[m] = sc; zp[m] = z;
@@ -606,20 +619,21 @@ quant_rows_f32_kernel(const float* __restrict__ Y, int M, int K, int mode, uint8
             }
         }
     }
+    if (ex.out) lrq_dec::expand_share(ex);
 }
 
 }  // namespace
 
-lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int a_bits, int mode, int out16, uint8_t* codes,
-                                       float* scale, int32_t* zp, cudaStream_t st) {
+lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int tile, int a_bits, int mode, int out16, uint8_t* codes,
+                                       float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
     if (!lrq_aligned(Y, 32)) return LRQ_ERR_INVALID_ARG;          // rows are K*4 bytes with K % 8 == 0: 32-byte aligned chunks
     int sms = 0;
     if (lrq_current_device(nullptr, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
-    const int blocks_needed = (M + 7) / 8;                        // 8 warps per CTA, one token per warp and step
-    const int grid = blocks_needed < sms * 8 ? blocks_needed : sms * 8;
+    const int grid = lrq_quant_grid((M + 7) / 8, sms * 8, 8, ex);  // 8 warps per CTA, one token per warp and step
+    const int tiles = (K + tile - 1) / tile;
     auto kern = a_bits == 8 ? (out16 ? quant_rows_f32_kernel<8, true> : quant_rows_f32_kernel<8, false>)
                             : (out16 ? quant_rows_f32_kernel<4, true> : quant_rows_f32_kernel<4, false>);
-    LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(256), 0, st, Y, M, K, mode, codes, scale, zp));
+    LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(256), 0, st, Y, M, K, tiles, mode, codes, scale, zp, ex));
     return LRQ_OK;
 }
 
@@ -718,7 +732,7 @@ static lrq_status resident_ctas(const void* kern, int dev, int threads, size_t s
 }
 
 static lrq_status launch_generic(const void* X, int M, int K, long ldx, int log2B, int a_bits, int mode, int out16, const float* prescale,
-                                 uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st) {
+                                 uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
     const size_t smem = (size_t)K * sizeof(float);
     if (smem > 200 * 1024) return LRQ_ERR_UNSUPPORTED;
     int dev = 0, per_sm = 0;
@@ -726,8 +740,13 @@ static lrq_status launch_generic(const void* X, int M, int K, long ldx, int log2
     const int threads = (K >= 2048) ? 256 : (K >= 1024 ? 128 : 64);
     lrq_status rs = resident_ctas(reinterpret_cast<const void*>(rotq_generic_kernel), dev, threads, smem, &per_sm);   // sets the shared-memory opt-in
     if (rs != LRQ_OK) return rs;
-    LRQ_CUDA_TRY(lrq_launch_pdl(rotq_generic_kernel, dim3(M), dim3(threads), smem, st, X, M, K, ldx, log2B, a_bits, mode, out16, prescale, codes,
-                                scale, zp));
+    // CTAs past the tokens decode weights; those of the tokens join in when they are done
+    int dev_sms = 0;
+    if (lrq_current_device(nullptr, &dev_sms) != LRQ_OK) return LRQ_ERR_CUDA;
+    const int room = dev_sms * per_sm;
+    const int grid = M < room ? lrq_quant_grid(M, room, threads / 32, ex) : M;
+    LRQ_CUDA_TRY(lrq_launch_pdl(rotq_generic_kernel, dim3(grid), dim3(threads), smem, st, X, M, K, ldx, log2B, a_bits, mode, out16, prescale, codes,
+                                scale, zp, ex));
     return LRQ_OK;
 }
 
@@ -742,7 +761,7 @@ struct RotqPick<LOG2B, true, A_BITS, NT, NB, WIDE> {
 
 template <int LOG2B, bool BIG = false>
 static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits, int mode, int out16, const float* prescale, uint8_t* codes,
-                              float* scale, int32_t* zp, cudaStream_t st) {
+                              float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
     const int tpt = K / EPT;
     // whole tokens per CTA: thread count a multiple of 32, at least 256 when the token is small
     int T = 1;
@@ -757,7 +776,7 @@ static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits,
         smem += (size_t)(threads * EPT / B) * (size_t)(B + 32) * sizeof(float);
     }
     // register budget by CTA size: three CTAs of up to 288 threads, two of up to 384, else one
-    typedef void (*Kern)(const __nv_bfloat16*, int, int, long, int, int, int, int, const float*, uint8_t*, float*, int32_t*);
+    typedef void (*Kern)(const __nv_bfloat16*, int, int, long, int, int, int, int, const float*, uint8_t*, float*, int32_t*, LrqExpand);
     // 256-bit accesses when every thread's 64 input bytes and 32 code bytes start on 32-byte boundaries
     const bool wide = lrq_aligned(X, 32) && (ldx % 16) == 0 && lrq_aligned(codes, 32);
     Kern kern;
@@ -773,17 +792,17 @@ static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits,
     lrq_status rs = resident_ctas(reinterpret_cast<const void*>(kern), dev, threads, smem, &per_sm);
     if (rs != LRQ_OK) return rs;
     const int groups = (M + T - 1) / T;
-    const int grid = groups < sms * per_sm ? groups : sms * per_sm;
+    const int grid = lrq_quant_grid(groups, sms * per_sm, threads / 32, ex);
     LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, static_cast<const __nv_bfloat16*>(X), M, K, ldx, mode, out16, T,
-                                groups, prescale, codes, scale, zp));
+                                groups, prescale, codes, scale, zp, ex));
     return LRQ_OK;
 }
 
 lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
-                                    uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st) {
+                                    uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
     // blocks of up to 128 channels: whole blocks per thread, TMA-fed (rotq_blk.cu), when the shape allows
     {
-        const lrq_status r = lrq_launch_rotq_blk(X, M, K, ldx, B, a_bits, mode, out16, prescale, codes, scale, zp, st);
+        const lrq_status r = lrq_launch_rotq_blk(X, M, K, ldx, B, a_bits, mode, out16, prescale, codes, scale, zp, ex, st);
         if (r != LRQ_ERR_UNSUPPORTED) return r;
     }
     int log2B = 0;
@@ -793,15 +812,15 @@ lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B
     if (fast_ok) {
         lrq_status r = LRQ_ERR_UNSUPPORTED;
         switch (log2B) {
-#define LRQ_CASE(L) case L: r = launch_fast<L>(X, M, K, ldx, a_bits, mode, out16, prescale, codes, scale, zp, st); break;
+#define LRQ_CASE(L) case L: r = launch_fast<L>(X, M, K, ldx, a_bits, mode, out16, prescale, codes, scale, zp, ex, st); break;
             LRQ_CASE(3) LRQ_CASE(4) LRQ_CASE(5) LRQ_CASE(6) LRQ_CASE(7) LRQ_CASE(8) LRQ_CASE(9)
 #undef LRQ_CASE
-#define LRQ_CASE(L) case L: r = launch_fast<L, true>(X, M, K, ldx, a_bits, mode, out16, prescale, codes, scale, zp, st); break;
+#define LRQ_CASE(L) case L: r = launch_fast<L, true>(X, M, K, ldx, a_bits, mode, out16, prescale, codes, scale, zp, ex, st); break;
             LRQ_CASE(10) LRQ_CASE(11) LRQ_CASE(12)
 #undef LRQ_CASE
             default: break;
         }
         if (r != LRQ_ERR_UNSUPPORTED) return r;
     }
-    return launch_generic(X, M, K, ldx, log2B, a_bits, mode, out16, prescale, codes, scale, zp, st);
+    return launch_generic(X, M, K, ldx, log2B, a_bits, mode, out16, prescale, codes, scale, zp, ex, st);
 }

@@ -25,6 +25,7 @@
 #include "lrq_internal.cuh"
 #include "f32x2.cuh"
 #include "rotq_common.cuh"
+#include "tlq_decode.cuh"
 #include "tc_ptx.cuh"
 #include "tma_host.cuh"
 #include <climits>
@@ -152,7 +153,7 @@ template <int LOG2B, int A_BITS, bool OUT16>
 __global__ void __launch_bounds__(MAX_WARPS * 32, 1)
 rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode, int tok_per_step, int num_steps,
                 int sub_warps, uint32_t stage_bytes, float scale_mul, const float* __restrict__ prescale,
-                uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp, int* status) {
+                uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zp, int* status, const LrqExpand ex) {
     static_assert(LOG2B >= 3 && LOG2B <= 7, "blocks of 8..128 channels");
     constexpr bool PAIRED = LOG2B == 7;              // a block spans two neighbouring threads
     extern __shared__ unsigned char smem_dyn[];
@@ -363,16 +364,17 @@ rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode,
             while (!mbar_try_wait(bar, (uint32_t)(i2 / NSTAGE) & 1u) && clock64() - t0 < kWaitCycles / 8) {}
         }
     }
+    if (ex.out) lrq_dec::expand_share(ex);
     __syncthreads();                     // no sub-group leaves while another may still use the shared control block
 }
 
 typedef lrq_status (*BlkLaunch)(const CUtensorMap&, int, int, int, int, int, int, int, uint32_t, float, const float*, uint8_t*, float*,
-                                int32_t*, int, size_t, cudaStream_t);
+                                int32_t*, int, size_t, const LrqExpand&, cudaStream_t);
 
 template <int LOG2B, int A_BITS, bool OUT16>
 lrq_status launch_blk(const CUtensorMap& tm, int M, int K, int mode, int T, int steps, int sub_warps, int nsub, uint32_t stage_bytes,
                       float scale_mul, const float* prescale, uint8_t* codes, float* scale, int32_t* zp, int sms, size_t smem,
-                      cudaStream_t st) {
+                      const LrqExpand& ex, cudaStream_t st) {
     auto kern = rotq_blk_kernel<LOG2B, A_BITS, OUT16>;
     // the shared-memory opt-in is a per-device function attribute: set once per device and kernel variant
     static std::mutex mu;
@@ -388,9 +390,9 @@ lrq_status launch_blk(const CUtensorMap& tm, int M, int K, int mode, int T, int 
     }
     // one CTA per SM; each deals its steps (blockIdx, blockIdx + grid, ...) out to its sub-groups on demand
     const int per_cta = (steps + nsub - 1) / nsub;
-    const int grid = per_cta < sms ? per_cta : sms;
+    const int grid = lrq_quant_grid(per_cta, sms, nsub * sub_warps, ex);
     LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(nsub * sub_warps * 32), smem, st, tm, M, K, mode, T, steps, sub_warps, stage_bytes,
-                                scale_mul, prescale, codes, scale, zp, lrq_status_word()));
+                                scale_mul, prescale, codes, scale, zp, lrq_status_word(), ex));
     return LRQ_OK;
 }
 
@@ -398,7 +400,7 @@ lrq_status launch_blk(const CUtensorMap& tm, int M, int K, int mode, int T, int 
 
 // Returns LRQ_ERR_UNSUPPORTED for shapes this kernel does not take (the caller then uses the other kernels).
 lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
-                               uint8_t* codes, float* scale, int32_t* zp, cudaStream_t st) {
+                               uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
     if (K % 128 || B < 8 || B > 128 || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(codes, out16 ? 32 : 16)) return LRQ_ERR_UNSUPPORTED;
     const int tpt = K / EPT;
     if (K / 64 > 256) return LRQ_ERR_UNSUPPORTED;
@@ -440,5 +442,5 @@ lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int
 #undef LRQ_CASE
         default: return LRQ_ERR_UNSUPPORTED;
     }
-    return fn(tm, M, K, mode, T, steps, sub_warps, nsub, stage_bytes, scale_mul, prescale, codes, scale, zp, sms, smem, st);
+    return fn(tm, M, K, mode, T, steps, sub_warps, nsub, stage_bytes, scale_mul, prescale, codes, scale, zp, sms, smem, ex, st);
 }

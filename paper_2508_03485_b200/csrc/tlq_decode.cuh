@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include "lrq_internal.cuh"
 
 namespace lrq_dec {
 
@@ -66,6 +67,60 @@ __device__ __forceinline__ uint32_t fetch_packed3(const uint8_t* a, const uint8_
     const uint32_t lo = __ldg(w0);
     const uint32_t hi = (reinterpret_cast<const uint8_t*>(w0 + 2) <= end) ? __ldg(w0 + 1) : 0u;
     return __funnelshift_r(lo, hi, 8 * (uint32_t)(ai & 3)) & 0x00FFFFFFu;
+}
+
+// Weight rows first, first + stride, ... of a layer decoded to bf16 [N,K], by one warp.  A layer meets each weight in M/256
+// tiles of the contraction; decoded there, a weight costs 2.6 lane-operations and a trip through shared memory in every
+// one of them.  Decoded here it costs one pass over 2.5 bytes per weight, whose results the contraction then reads
+// mostly from L2.  Bound by those bytes.  A warp takes a row at a time, so that a per-channel table is loaded once; a lane
+// turns eight codes (4 bytes, 3 when packed) into one 16-byte store, UNROLL of them in flight, so a warp reads and
+// writes whole lines.  With grouped tables a lane reloads its table when its group changes.
+template <int W_BITS, bool PACKED3>
+__device__ __forceinline__ void expand_rows(const LrqExpand& e, int first, int stride) {
+    constexpr int NLEV = 1 << W_BITS, UNROLL = 6;
+    const int lane = threadIdx.x & 31;
+    const int words = e.K >> 3, ngrp = e.K / e.G, wpg = e.G >> 3;  // groups of eight codes: per row, per table
+    const size_t pitch = PACKED3 ? (size_t)e.K * 3 / 8 : (size_t)e.K / 2;
+    const uint8_t* end = e.codes + (size_t)e.N * pitch;
+    for (int n = first; n < e.N; n += stride) {
+        const uint8_t* row = e.codes + (size_t)n * pitch;
+        const float* tab = e.levels + (size_t)n * ngrp * NLEV;
+        uint4* dst = static_cast<uint4*>(e.out) + (size_t)n * words;
+        Lut L;
+        int held = -1;
+        if (ngrp == 1) { load_lut<W_BITS>(L, tab); held = 0; }
+        for (int j0 = lane; j0 < words; j0 += 32 * UNROLL) {
+            uint32_t w[UNROLL];
+#pragma unroll
+            for (int u = 0; u < UNROLL; ++u) {
+                const int j = j0 + 32 * u;
+                w[u] = 0;
+                if (j < words) w[u] = PACKED3 ? fetch_packed3(row + 3 * (size_t)j, end) : __ldg(reinterpret_cast<const uint32_t*>(row) + j);
+            }
+#pragma unroll
+            for (int u = 0; u < UNROLL; ++u) {
+                const int j = j0 + 32 * u;
+                if (j >= words) break;
+                if (ngrp > 1) {
+                    const int g = j / wpg;
+                    if (g != held) { load_lut<W_BITS>(L, tab + (size_t)g * NLEV); held = g; }
+                }
+                uint32_t o[4];
+                decode_w<W_BITS>(PACKED3 ? spread3(w[u]) : w[u], L, o);
+                dst[j] = make_uint4(o[0], o[1], o[2], o[3]);
+            }
+        }
+    }
+}
+
+// The weight decode that rides on a quantizer kernel: called by every warp of the grid when it has no tokens left.  Rows are
+// dealt from the last warp of the grid backwards, so that those of a short batch go to CTAs that had none.
+static __device__ __noinline__ void expand_share(const LrqExpand e) {
+    const int wpc = blockDim.x >> 5, total = gridDim.x * wpc, first = total - 1 - (int)(blockIdx.x * wpc + (threadIdx.x >> 5));
+    if (e.fmt == 4) expand_rows<4, false>(e, first, total);
+    else if (e.fmt == 3) expand_rows<3, false>(e, first, total);
+    else if (e.fmt == 13) expand_rows<3, true>(e, first, total);
+    else expand_rows<2, false>(e, first, total);
 }
 
 }  // namespace lrq_dec

@@ -49,8 +49,7 @@ typedef enum { LRQ_F32 = 0, LRQ_F16 = 1, LRQ_BF16 = 2 } lrq_dtype;
 /* Storage of the weight codes (Sec. 4.1, Eq. 5: a b-bit code per weight).
  *   NIBBLE   two codes per byte, element 2j in the low nibble of byte j; row pitch K/2 bytes (b = 2..4)
  *   PACKED3  b = 3 only: eight codes in three bytes, code j of each eight at bits 3j..3j+2 of the little-endian
- *            24-bit word; row pitch 3K/8 bytes.  The storage TLQ's 3-bit codes actually need; taken by the
- *            weight-bandwidth-bound contraction for small token counts. */
+ *            24-bit word; row pitch 3K/8 bytes.  The storage TLQ's 3-bit codes actually need. */
 typedef enum { LRQ_CODES_NIBBLE = 0, LRQ_CODES_PACKED3 = 1 } lrq_code_layout;
 
 /* ---------------------------------------------------------------------------------------------
@@ -222,8 +221,8 @@ lrq_status lrq_layer_create(lrq_layer** out, int N, int K, int w_bits, int group
                             const float* wscale, const float* bias, const lrq_act_params* act);
 void lrq_layer_destroy(lrq_layer* L);
 
-/* Bytes of workspace lrq_qlinear needs for M tokens of this layer (activation codes, scales,
- * zero-points, and the fp32 scratch of a dense rotation). */
+/* Bytes of workspace lrq_qlinear needs for M tokens of this layer (activation codes, scales, zero-points, the operands of the
+ * contraction in bf16 where it takes them so, 2.K.(M + N) bytes, and the scratch of a dense or dual rotation). */
 size_t lrq_workspace_bytes(const lrq_layer* L, int M);
 
 /* ---------------------------------------------------------------------------------------------
@@ -246,9 +245,8 @@ lrq_status lrq_qlinear_stack(const lrq_layer* const* layers, int n_layers,
 
 /* Contraction and epilogue alone (Eq. 10), on activation codes produced earlier by
  * lrq_rotate_quantize_act.  `impl`: 0 = large-tile tcgen05 kernel (pairs of CTAs, 256 x 256 tiles), 1 = plain
- * CUDA-core kernel (kept as the in-library ablation baseline), 2 = small-tile tcgen05 kernel (128 x 32 tiles: the
- * one lrq_qlinear picks for a few hundred tokens or fewer, and the only tensor-core kernel that reads
- * LRQ_CODES_PACKED3), 3 = the integer form of Eq. 10 on the CUDA cores (mantissa products shifted by the level
+ * CUDA-core kernel (kept as the in-library ablation baseline), 2 = small-tile tcgen05 kernel (128 x 32 tiles, the
+ * only one of these on the tensor cores that reads LRQ_CODES_PACKED3), 3 = the integer form of Eq. 10 on the CUDA cores (mantissa products shifted by the level
  * exponents, exact integer accumulation; I = 7 tables; a slow cross-check of the two forms, not a production path).
  * LRQ_ERR_UNSUPPORTED when the kernel asked for does not take the layer's shape.
  * No workspace needed. */

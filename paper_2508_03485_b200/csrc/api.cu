@@ -215,28 +215,23 @@ extern "C" void lrq_layer_destroy(lrq_layer* L) { delete L; }
 
 namespace {
 // How lrq_qlinear runs a layer on M tokens.
-//   expanded  the quantizer writes the contraction's bf16 operand, the weight codes are decoded to bf16 once, and the
-//             contraction streams both (qgemm_bf16.cu)
+//   expanded  the quantizer writes the contraction's bf16 operand and decodes the weight codes to bf16, and the contraction
+//             streams both (qgemm_bf16.cu)
 //   packed    both operands stay packed, 256 x 256 tiles that decode them (qgemm_tc.cu)
-//   small     both operands stay packed, 128 x 32 tiles (qgemm_small.cu)
-// The choice depends on the layer and M alone, since the workspace is laid out by it.  Expanded is the rule: a k-block of
-// a tile takes 0.34 us there and 0.1 (3-bit weights, 4-bit activations) to 0.2 us more where it is decoded on the
-// way.  It costs a pass over 2.5 bytes per weight, 0.46 us per million, less a microsecond by which the decoding kernel
-// starts later; few tokens on a large matrix do not earn that back (us per call, expanded / packed, 11360 x 3456, W4A8:
-// M = 256 45.0 / 37.1, M = 333 53.6 / 60.9, M = 1024 75 / 85; W3A4: 256 45.8 / 31.9, 2048 124 / 128; 1152 x 4608, W4A8:
-// 256 26.2 / 36.7).  Batches with fewer than 37 tiles of 256 x 128 keep the small tiles: two launches instead of three, which is
-// what the host can issue in the time such a layer takes.
-enum Form { FORM_SMALL, FORM_PACKED, FORM_EXPANDED };
+// The choice depends on the layer and M alone, since the workspace is laid out by it.  Expanded is the rule, from one token
+// to the largest batch.  Decoding ahead costs a pass over 2.5 bytes per weight, 0.46 us per million; decoding in the
+// tiles costs 3 us once and 0.06 (3-bit weights, 4-bit activations) to 0.17 us per k-block and round of tiles over the 74
+// CTA pairs.  So few tokens on a very large matrix stay packed (us per call, expanded / packed: 11360 x 3456, W4A8 M = 256
+// 46 / 37, M = 333 55 / 61, M = 1100 89 / 106, W3A4 256 45 / 32, 1500 100 / 93, 3000 174 / 183; 2560 x 10240, W4A8, 256
+// 47 / 70; 3072 x 3072, W4A4, 256 22 / 26; 1152 x 4608, W4A8, 16 23 / 36; 1024 x 1024, W3A4, 256 11.2 / 15.5, and 14.6
+// with the 128 x 32 tiles of qgemm_small.cu, which are never the fastest by more than half a microsecond).
+enum Form { FORM_PACKED, FORM_EXPANDED };
 Form pick_form(const lrq_layer* L, int M) {
-    const long narrow_tiles = (long)((M + 255) / 256) * ((L->N + 127) / 128);
-    if (narrow_tiles * 4 < 148 && lrq_qgemm_small_takes(L)) return FORM_SMALL;
-    if (lrq_qgemm_tc_takes(L)) {
-        const long tiles = (long)((M + 255) / 256) * ((L->N + 255) / 256);
-        const double rounds = (double)((tiles + 73) / 74);           // of tiles over the CTA pairs
-        const double decode_us = rounds * (L->K / 64) * (L->w_bits == 3 && L->act.a_bits == 4 ? 0.1 : 0.2);
-        if (decode_us < 0.46e-6 * L->N * (double)L->K - 1.0) return FORM_PACKED;
-    }
-    return FORM_EXPANDED;
+    if (!lrq_qgemm_tc_takes(L)) return FORM_EXPANDED;
+    const long tiles = (long)((M + 255) / 256) * ((L->N + 255) / 256);
+    const double per_block = L->act.a_bits == 8 ? 0.17 : L->w_bits == 4 ? 0.15 : 0.06;
+    const double in_tiles_us = 3.0 + (double)((tiles + 73) / 74) * (L->K / 64) * per_block;
+    return in_tiles_us < 0.46e-6 * L->N * (double)L->K ? FORM_PACKED : FORM_EXPANDED;
 }
 
 struct WsLayout { size_t codes, scale, zp, wexp, rot, total; Form form; };
@@ -312,8 +307,7 @@ extern "C" lrq_status lrq_qlinear(const lrq_layer* L, const void* X, int M, long
     st = run_act(X, M, L->K, ldx, &L->act, ex ? 1 : 0, a_codes, a_scale, a_zp, decode, base + w.rot, w.total - w.rot, stream);
     if (st != LRQ_OK) return st;
     if (ex) return lrq_launch_qgemm_bf16(L, a_codes, base + w.wexp, a_scale, a_zp, M, Y, dt, ldy, stream);
-    if (w.form == FORM_PACKED) return lrq_launch_qgemm_tc(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
-    return lrq_launch_qgemm_small(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
+    return lrq_launch_qgemm_tc(L, a_codes, a_scale, a_zp, M, Y, dt, ldy, stream);
 }
 
 extern "C" lrq_status lrq_qlinear_stack(const lrq_layer* const* layers, int n_layers, const void* const* X,

@@ -221,6 +221,8 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
     __syncthreads();
     lrq_pdl_trigger();
     lrq_pdl_wait();                      // X may be the previous kernel's output; the code buffer may still be read by it
+    float4* ps = reinterpret_cast<float4*>(smem_raw + (3 * 2 * sizeof(int) * tok_per_cta + 15) / 16 * 16);
+    if (prescale) { stage_prescale<EPT / 4>(ps, prescale, K, tpt); __syncthreads(); }
 
     uint4 raw[4];
     {
@@ -245,14 +247,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
             for (int c = 0; c < 4; ++c)
                 P[4 * i + c] = pack2(__uint_as_float(w[c] << 16), __uint_as_float(w[c] & 0xffff0000u));
         }
-        if (prescale) {                                       // smoothing multipliers (Sec. 5.1), before the rotation
-            const float4* ps = reinterpret_cast<const float4*>(prescale + (size_t)j * EPT);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float4 f = __ldg(ps + i);
-                P[2 * i] = mul2(P[2 * i], pack2(f.x, f.y)); P[2 * i + 1] = mul2(P[2 * i + 1], pack2(f.z, f.w));
-            }
-        }
+        if (prescale) apply_prescale<EPT / 4>(P, ps, j, tpt);  // before the rotation
         // the next group's loads fly while this group is transformed
         {
             const int mn = (g + (int)gridDim.x) * tok_per_cta + tl;
@@ -411,6 +406,8 @@ rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int
     __syncthreads();
     lrq_pdl_trigger();
     lrq_pdl_wait();                      // X may be the previous kernel's output; the code buffer may still be read by it
+    float4* ps = reinterpret_cast<float4*>(buf + (size_t)(blockDim.x / (U * 32)) * UNIT_FLOATS);
+    if (prescale) { stage_prescale<EPT / 4>(ps, prescale, K, tpt); __syncthreads(); }
 
     uint4 raw[4];
     {
@@ -434,14 +431,7 @@ rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int
             for (int c = 0; c < 4; ++c)
                 P[4 * i + c] = pack2(__uint_as_float(w[c] << 16), __uint_as_float(w[c] & 0xffff0000u));
         }
-        if (prescale) {
-            const float4* ps = reinterpret_cast<const float4*>(prescale + (size_t)j * EPT);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float4 f = __ldg(ps + i);
-                P[2 * i] = mul2(P[2 * i], pack2(f.x, f.y)); P[2 * i + 1] = mul2(P[2 * i + 1], pack2(f.z, f.w));
-            }
-        }
+        if (prescale) apply_prescale<EPT / 4>(P, ps, j, tpt);
         {
             const int mn = (g + (int)gridDim.x) * tok_per_cta + tl;
             if (g + (int)gridDim.x < num_groups && mn < M) {
@@ -775,6 +765,7 @@ static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits,
         const int B = 1 << LOG2B;
         smem += (size_t)(threads * EPT / B) * (size_t)(B + 32) * sizeof(float);
     }
+    if (prescale) smem += (size_t)K * sizeof(float);
     // register budget by CTA size: three CTAs of up to 288 threads, two of up to 384, else one
     typedef void (*Kern)(const __nv_bfloat16*, int, int, long, int, int, int, int, const float*, uint8_t*, float*, int32_t*, LrqExpand);
     // 256-bit accesses when every thread's 64 input bytes and 32 code bytes start on 32-byte boundaries

@@ -47,11 +47,16 @@ struct SubCtl {
     uint64_t empty[NSTAGE];              // stage read by all warps of the sub-group
     int group[NSTAGE];                   // step held by the stage, -1: none left
 };
-struct BlkCtl {
+struct __align__(16) BlkCtl {
     SubCtl sub[MAX_NSUB];
     int next;                            // next unclaimed step of this CTA (steps are dealt to the sub-groups on demand)
     volatile int abort_flag;
 };
+
+// bytes of the token-part extremes of a CTA, a multiple of 16
+__host__ __device__ constexpr size_t lrq_ext_bytes(int nsub, int tok_per_step, int sub_warps) {
+    return ((size_t)nsub * 2 * (tok_per_step + 1) * sub_warps * 8 + 15) / 16 * 16;
+}
 
 __device__ __forceinline__ void lds128(uint32_t addr, uint4& v) {
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
@@ -216,6 +221,13 @@ rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode,
         for (int s = 0; s < NSTAGE; ++s) refill(s);
     }
 
+    // multipliers behind the extremes (ext0 is 16-byte aligned and their total a multiple of 16 bytes, see the launch)
+    const float4* ps = reinterpret_cast<const float4*>(reinterpret_cast<unsigned char*>(ctl + 1) + lrq_ext_bytes(nsub, tok_per_step, sub_warps));
+    if (prescale) {
+        stage_prescale<EPT / 4>(const_cast<float4*>(ps), prescale, K, tpt);
+        __syncthreads();
+    }
+
     const int odd = PAIRED ? (jh & 1) : 0;           // second thread of a 128-channel block
     const float sgn = odd ? -1.f : 1.f;
     const double nrm = 1.0 / sqrt((double)(1 << LOG2B));
@@ -245,14 +257,7 @@ rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode,
         // the stage is handed back once every lane of the warp holds its values in registers
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sc->empty[s]));
-        if (prescale) {                                       // smoothing multipliers (Sec. 5.1), before the rotation
-            const float4* ps = reinterpret_cast<const float4*>(prescale + (size_t)jh * EPT);
-#pragma unroll
-            for (int i = 0; i < NP / 2; ++i) {
-                const float4 f = __ldg(ps + i);
-                P[2 * i] = mul2(P[2 * i], pack2(f.x, f.y)); P[2 * i + 1] = mul2(P[2 * i + 1], pack2(f.z, f.w));
-            }
-        }
+        if (prescale) apply_prescale<EPT / 4>(P, ps, jh, tpt);      // before the rotation
         // index bit 0: the two halves of a pair; bits 1-4: between pairs
 #pragma unroll
         for (int i = 0; i < NP; ++i) { float a, b; unpack2(P[i], a, b); P[i] = pack2(a + b, a - b); }
@@ -412,6 +417,7 @@ lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int
     // K = 4608: four sub-groups of five warps take 104 us, two of nine warps 111 us, for the same active threads).
     int sub_warps = 0, nsub = 0, T = 0;
     long best_threads = 0;
+    const size_t pre = prescale ? (size_t)K * sizeof(float) : 0;
     for (int sw = 1; sw <= MAX_WARPS / 2; ++sw) {
         int t = sw * 32 / tpt;
         if (t < 1) continue;
@@ -420,13 +426,13 @@ lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int
         int ns = MAX_WARPS / sw;
         if (ns > MAX_NSUB) ns = MAX_NSUB;                       // named barriers 1..15 and the control block
         const size_t need = (size_t)ns * NSTAGE * lrq_round_up((size_t)t * K * 2, 1024);
-        if (need > 190 * 1024) continue;
+        if (need + pre > 190 * 1024) continue;
         const long threads = (long)t * tpt * ns;
         if (threads > best_threads) { best_threads = threads; sub_warps = sw; nsub = ns; T = t; }
     }
     if (!sub_warps) return LRQ_ERR_UNSUPPORTED;
     const uint32_t stage_bytes = (uint32_t)lrq_round_up((size_t)T * K * 2, 1024);
-    const size_t smem = 1024 + (size_t)nsub * NSTAGE * stage_bytes + sizeof(BlkCtl) + (size_t)nsub * 2 * (T + 1) * sub_warps * 8 + 16;
+    const size_t smem = 1024 + (size_t)nsub * NSTAGE * stage_bytes + sizeof(BlkCtl) + lrq_ext_bytes(nsub, T, sub_warps) + pre;
     int sms = 0;
     if (lrq_current_device(nullptr, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
     CUtensorMap tm;

@@ -71,4 +71,22 @@ __device__ __forceinline__ TokenQ token_params_fast(float mn, float mx, int a_bi
     return t;
 }
 
+// Smoothing multipliers (Sec. 5.1) in shared memory, laid out so that threads which own runs of 4 * PER consecutive channels
+// read them without conflicts: float4 i of thread j at i * tpt + j.  Read from global memory as they lie, a warp's 128-bit
+// loads touched 32 lines each, once per token (32768 x 4608, B = 128: 227 us against 106 without multipliers, 139 now).
+template <int PER>
+__device__ __forceinline__ void stage_prescale(float4* ps, const float* __restrict__ prescale, int K, int tpt) {
+    for (int q = threadIdx.x; q < (K >> 2); q += blockDim.x)
+        ps[(q % PER) * tpt + q / PER] = __ldg(reinterpret_cast<const float4*>(prescale) + q);
+}
+template <int PER>
+__device__ __forceinline__ void apply_prescale(lrq_f2::f32x2* P, const float4* ps, int j, int tpt) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const float4 f = ps[i * tpt + j];
+        P[2 * i] = lrq_f2::mul2(P[2 * i], lrq_f2::pack2(f.x, f.y));
+        P[2 * i + 1] = lrq_f2::mul2(P[2 * i + 1], lrq_f2::pack2(f.z, f.w));
+    }
+}
+
 }  // namespace lrq_rq

@@ -631,11 +631,12 @@ lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int tile, i
 // Fluctuation metric of a layer's activations (Sec. 4.2, Eq. 11): J = ||X||_F / sqrt(M K), and the rotation
 // kind the threshold rule of Eq. 12 picks.  HBM-bound: 2 bytes per element, read once with 256-bit loads.
 // Squares of bf16 values are exact in fp32; a thread sums its 16 squares in fp32 (relative error below
-// 16 * 2^-24), everything above that in fp64.
+// 16 * 2^-24), everything above that in fp64.  The last CTA to finish takes the root and applies the rule.
 // ------------------------------------------------------------------------------------------------
 namespace {
 __global__ void __launch_bounds__(256)
-sumsq_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, double* __restrict__ acc) {
+sumsq_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, double* acc, double count, double thr, float* J, int* kind) {
+    lrq_pdl_trigger();
     const int cpr = K >> 4;                                  // 32-byte chunks per row
     double part = 0.0;
     // a warp walks over rows (grid stride), its lanes over the row's chunks, four loads in flight per lane
@@ -677,14 +678,24 @@ sumsq_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, double
     if (threadIdx.x == 0) {
         double t = 0.0;
         for (int w = 0; w < 8; ++w) t += wsum[w];
+        lrq_pdl_wait();                                      // the sum and the count have their initial values
         atomicAdd(acc, t);
+        __threadfence();
+        if (atomicAdd(kind, 1) == (int)gridDim.x - 1) {      // the last CTA: every other one's share is in
+            __threadfence();
+            const double j = sqrt(__ldcg(acc)) / sqrt(count);
+            *J = (float)j;
+            *kind = j < thr ? (int)LRQ_ROT_HADAMARD : (int)LRQ_ROT_DENSE;
+        }
     }
 }
-__global__ void ars_finish_kernel(const double* __restrict__ acc, double count, double thr, float* __restrict__ J,
-                                  int* __restrict__ kind) {
-    const double j = sqrt(*acc) / sqrt(count);
-    *J = (float)j;
-    *kind = j < thr ? (int)LRQ_ROT_HADAMARD : (int)LRQ_ROT_DENSE;
+// Initial values of the sum and of the count of finished CTAs, which lives in the result `kind` until the end.  An ordinary
+// launch: it starts when all earlier work of the stream is done, and lets the sum's kernel start beside it, which
+// touches both only after it has waited for this one.
+__global__ void ars_init_kernel(double* __restrict__ acc, int* __restrict__ kind) {
+    lrq_pdl_trigger();
+    *acc = 0.0;
+    *kind = 0;
 }
 }  // namespace
 
@@ -692,13 +703,12 @@ lrq_status lrq_launch_ars_metric(const void* X, int M, int K, long ldx, double t
                                  cudaStream_t st) {
     int sms = 0;
     if (lrq_current_device(nullptr, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
-    LRQ_CUDA_TRY(cudaMemsetAsync(acc, 0, sizeof(double), st));
     long blocks = ((long)M + 7) / 8;                         // 8 warps per CTA, one row per warp and step
     if (blocks > (long)sms * 8) blocks = (long)sms * 8;
-    sumsq_kernel<<<(int)blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(X), M, K, ldx, acc);
+    ars_init_kernel<<<1, 1, 0, st>>>(acc, kind);
     LRQ_CUDA_TRY(cudaGetLastError());
-    ars_finish_kernel<<<1, 1, 0, st>>>(acc, (double)M * (double)K, thr, J, kind);
-    LRQ_CUDA_TRY(cudaGetLastError());
+    LRQ_CUDA_TRY(lrq_launch_pdl(sumsq_kernel, dim3((unsigned)blocks), dim3(256), 0, st, static_cast<const __nv_bfloat16*>(X), M, K, ldx, acc,
+                                (double)M * (double)K, thr, J, kind));
     return LRQ_OK;
 }
 

@@ -9,17 +9,19 @@
 // one clipping factor of the caller's grid, all lanes walking over the same elements.  Every decision (codes,
 // chosen factor) is the one fp64 arithmetic with explicitly rounded operations gives.
 //
-// What bounds it is the number of instructions per element and factor, so nothing but the three operations of the sum
-// itself is left in fp64 there:
-//   * the code is rint(l/s) - z in fp32, from log2f, two elements per instruction; an element within the fp32 error of a rounding boundary
+// What bounds it is the number of instructions per element and factor:
+//   * every factor's error is first summed in fp32, in any order.  That sum's relative error
+//     is bounded (a few hundred roundings), so a factor further than twice the bound from the smallest cannot win; only
+//     when more than one factor is that close is the sum above taken in fp64, for about one row in fifty;
+//   * the code is rint(l/s) - z in fp32, from log2f; an element within the fp32 error of a rounding boundary
 //     (|x - rint x| > 1/2 - E, E worked out from the candidate's range) takes the fp64 expression, a division, instead;
-//   * levels have 8-bit significands, so the upper word of the double is the level: 32-bit look-ups;
-//   * a side's elements are compacted into shared memory CHUNK source elements at a time and read as broadcasts.
-// 4608 x 1152, 4 bits, 31 factors a side: 545 us with fp64 codes and elements handed round by shuffles, 164 now;
-// 4608 x 1536, 3 bits, groups of 128: 1086 and 380.
+//   * levels have 8-bit significands: fp32 numbers, and the upper word of the double is the level;
+//   * a side's elements are compacted into shared memory kChunk source elements at a time and read as broadcasts.
+// 4608 x 1152, 4 bits, 31 factors a side: 545 us with the fp64 expression for every element and factor, 157 now;
+// 4608 x 1536, 3 bits, groups of 128: 1086 and 315.
 #include "lrq_internal.cuh"
-#include "f32x2.cuh"
 #include <climits>
+#include <type_traits>
 
 namespace {
 
@@ -28,7 +30,8 @@ constexpr int kThreads = 64;
 constexpr int kChunk = 256;                        // source elements compacted at a time
 struct ClipGrid { double a[kMaxGrid]; double b[kMaxGrid]; int na, nb; };
 
-__device__ __forceinline__ double level_value(double e, int I) {
+// (out of line, as the next one: both are rarely reached and long, and this kernel has to stay in the instruction cache)
+__device__ __noinline__ double level_value(double e, int I) {
     // Eqs. 8-9: 2^e ~ II * 2^(f-I) with f = floor(e), II = rint(2^(e-f) * 2^I)
     const double f = floor(e);
     const double II = rint(exp2(__dsub_rn(e, f)) * (double)(1 << I));      // the factor is a power of two: exact
@@ -37,9 +40,9 @@ __device__ __forceinline__ double level_value(double e, int I) {
     return ldexp(II, x);
 }
 
-// code of Eq. 5 on one side: clamp(rint(l / s) - z, 0, nq), l = log2 of the magnitude
-__device__ __forceinline__ int side_code(double l, double s, double z, int nq) {
-    return (int)fmin(fmax(__dsub_rn(rint(__ddiv_rn(l, s)), z), 0.0), (double)nq);
+// code of Eq. 5 on one side: clamp(rint(l / s) - z, 0, nq), l = log2(a)
+__device__ __noinline__ int side_code(float a, double s, double z, int nq) {
+    return (int)fmin(fmax(__dsub_rn(rint(__ddiv_rn(log2((double)a), s)), z), 0.0), (double)nq);
 }
 
 __device__ __forceinline__ double shfl_double(double v, int src) {
@@ -79,8 +82,6 @@ __device__ __forceinline__ float fast_round(float l32, const FastCode& f, bool& 
     return fminf(r, f.top);
 }
 
-using namespace lrq_f2;
-
 struct Side { double s, z, factor; };
 
 __global__ void __launch_bounds__(kThreads, 16)
@@ -88,8 +89,9 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                     uint8_t* __restrict__ codes, float* __restrict__ levels, double* __restrict__ meta,
                     float* __restrict__ wsum) {
     __shared__ int cand_lev[2][9][32];             // level table of each lane's candidate, per side (upper word of the double)
+    __shared__ float cand_f32[2][9][32];           // the same in fp32
     // a side's elements of one chunk, in increasing k: magnitude and its log2
-    __shared__ __align__(16) double mag[2][kChunk];
+    __shared__ __align__(16) float mag[2][kChunk];
     __shared__ __align__(16) float lg[2][kChunk];
     __shared__ FastCode best_fc[2];
     __shared__ float ext[2][2][2];                 // [warp][side][max, min] of |w|
@@ -131,7 +133,9 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
         const int nq = sd ? half : half - 1;       // highest code of the side = denominator of Eq. 6
         const float vmax = fmaxf(ext[0][sd][0], ext[1][sd][0]), vmin = fminf(ext[0][sd][1], ext[1][sd][1]);
         const int scnt = ext_cnt[0][sd] + ext_cnt[1][sd];
-        const double smax = scnt ? log2((double)vmax) : -INFINITY, smin = scnt ? log2((double)vmin) : INFINITY;
+        // both logarithms in one evaluation: even lanes take the maximum's, odd lanes the minimum's
+        const double lx = log2((double)((lane & 1) ? vmin : vmax));
+        const double smax = scnt ? shfl_double(lx, 0) : -INFINITY, smin = scnt ? shfl_double(lx, 1) : INFINITY;
         const float l_abs = scnt ? fmaxf(fabsf((float)smin), fabsf((float)smax)) * 1.000001f : 0.f;
         const int ng = sd ? grid.nb : grid.na;
         double best_err = INFINITY, best_s = 1.0, best_z = 0.0, best_f = 1.0;
@@ -150,16 +154,21 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                 }
             }
             __syncwarp();
-            for (int q = 0; q <= nq; ++q)
-                cand_lev[sd][q][lane] = ok ? level_word(__dmul_rn(s, __dadd_rn((double)q, z)), I) : 0;
+            for (int q = 0; q <= nq; ++q) {
+                const int hi = ok ? level_word(__dmul_rn(s, __dadd_rn((double)q, z)), I) : 0;
+                cand_lev[sd][q][lane] = hi;
+                cand_f32[sd][q][lane] = (float)__hiloint2double(hi, 0);
+            }
             FastCode fc = fast_code(s, z, l_abs, nq);
             if (!ok) { fc.inv = 0.f; fc.negz = 0.f; fc.thr = 1.f; }                 // scored, but never looked at
-            const uint32_t lev0 = (uint32_t)__cvta_generic_to_shared(&cand_lev[sd][0][lane]) - (__float_as_uint(kMagic) << 7);
+            const uint32_t magic_off = __float_as_uint(kMagic) << 7;
+            const uint32_t lev0 = (uint32_t)__cvta_generic_to_shared(&cand_lev[sd][0][lane]) - magic_off;
+            const uint32_t f32_0 = (uint32_t)__cvta_generic_to_shared(&cand_f32[sd][0][lane]) - magic_off;
             __syncwarp();
-            // the side's elements in increasing k, one chunk at a time
-            double err = 0.0;
-            for (int k0 = 0; k0 < G; k0 += kChunk) {
+            // the side's elements among w[k0 .. k0 + kChunk), in increasing k, into the warp's list; returns how many
+            auto fill = [&](int k0) {
                 int n_el = 0;
+                __syncwarp();
 #pragma unroll
                 for (int u = 0; u < kChunk / 32; ++u) {
                     if (k0 + 32 * u >= G) break;
@@ -169,61 +178,114 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                     const unsigned m = __ballot_sync(0xffffffffu, mine);
                     if (mine) {
                         const int at = n_el + __popc(m & ((1u << lane) - 1u));
-                        mag[sd][at] = (double)fabsf(v);
+                        mag[sd][at] = fabsf(v);
                         lg[sd][at] = log2f(fabsf(v));
                     }
                     n_el += __popc(m);
                 }
                 __syncwarp();
-                auto level = [&](float r) {
+                return n_el;
+            };
+            auto code_of = [&](int j) {                         // one element, whatever its distance from a boundary
+                bool exact;
+                const float r = fast_round(lg[sd][j], fc, exact);
+                return exact ? r : kMagic + (float)side_code(mag[sd][j], s, z, nq);
+            };
+            // ---- every factor's error in fp32 (terms within 3 u of the exact ones, eight partial sums of at most
+            // scnt / 8 + chunk remainders terms), which leaves the factors within twice its bound of the smallest
+            float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            float rest = 0.f;
+            auto term = [&](int j, float r) {
+                float L;
+                asm("ld.shared.f32 %0, [%1];" : "=f"(L) : "r"(f32_0 + (__float_as_uint(r) << 7)));
+                const float d = mag[sd][j] - L;
+                rest = fmaf(d, d, rest);
+            };
+            auto group = [&](int j, auto U_) {
+                constexpr int U = decltype(U_)::value;
+                float r[U], off = 0.f;               // the distances from an integer are looked at together
+#pragma unroll
+                for (int u = 0; u < U; u += 4) {
+                    const float4 l4 = *reinterpret_cast<const float4*>(&lg[sd][j + u]);
+                    const float l[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const float x = fmaf(l[h], fc.inv, fc.negz);
+                        r[u + h] = x + kMagic;
+                        off = fmaxf(off, fabsf(x - (r[u + h] - kMagic)));
+                    }
+                }
+                if (off <= fc.thr) {
+#pragma unroll
+                    for (int u = 0; u < U; u += 4) {
+                        const float4 a4 = *reinterpret_cast<const float4*>(&mag[sd][j + u]);
+                        const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            float L;
+                            asm("ld.shared.f32 %0, [%1];" : "=f"(L) : "r"(f32_0 + (__float_as_uint(fminf(r[u + h], fc.top)) << 7)));
+                            const float d = a[h] - L;
+                            part[u + h] = fmaf(d, d, part[u + h]);
+                        }
+                    }
+                } else {
+#pragma unroll 1
+                    for (int u = 0; u < U; ++u) term(j + u, code_of(j + u));
+                }
+            };
+            for (int k0 = 0; k0 < G; k0 += kChunk) {
+                const int n_el = fill(k0);
+                int j = 0;
+                for (; j + 8 <= n_el; j += 8) group(j, std::integral_constant<int, 8>());
+                if (j + 4 <= n_el) { group(j, std::integral_constant<int, 4>()); j += 4; }
+#pragma unroll 1
+                for (; j < n_el; ++j) term(j, code_of(j));
+            }
+            float e32;
+            {
+                e32 = (((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]))) + rest;
+            }
+            // errors are not negative, so their bit patterns are ordered as the numbers; NaN sorts above them all
+            const float emin = __uint_as_float(__reduce_min_sync(0xffffffffu, ok ? __float_as_uint(e32) : 0x7fffffffu));
+            const float eps = (float)(scnt / 8 + 3 * (G / kChunk + 1) + 64) * 2.4e-7f;      // 4 u per term of the longest sum
+            const unsigned close = __ballot_sync(0xffffffffu, ok && e32 <= emin * (1.f + eps));
+            const bool safe = ng <= 32 && emin > 1e-27f && emin < 1e30f && eps < 0.5f && vmax < 1e18f;
+            if (safe && (close & (close - 1)) == 0) {
+                // one factor is left: the smallest error, whatever the rounding
+                const int src = __ffs(close) - 1;
+                best_s = shfl_double(s, src); best_z = shfl_double(z, src); best_f = shfl_double(fac, src);
+                if (lane == src) best_fc[sd] = fc;
+                found = true;
+                continue;
+            }
+            // ---- a near-tie (or sums out of fp32's range): the sum as it is defined
+            double err = 0.0;
+            for (int k0 = 0; k0 < G; k0 += kChunk) {
+                const int n_el = fill(k0);
+auto level = [&](float r) {
                     int hi;
                     asm("ld.shared.b32 %0, [%1];" : "=r"(hi) : "r"(lev0 + (__float_as_uint(r) << 7)));
                     return __hiloint2double(hi, 0);
                 };
-                auto careful = [&](int j) {                     // one element, whatever its distance from a boundary
-                    const double a = mag[sd][j];
-                    bool exact;
-                    float r = fast_round(lg[sd][j], fc, exact);
-                    if (!exact) r = kMagic + (float)side_code(log2(a), s, z, nq);
-                    const double d = __dsub_rn(a, level(r));
-                    err = __dadd_rn(err, __dmul_rn(d, d));
-                };
-                constexpr int U = 8;
-                const f32x2 INV = pack2(fc.inv, fc.inv), NEGZ = pack2(fc.negz, fc.negz), MAGIC = pack2(kMagic, kMagic);
                 int j = 0;
-                for (; j + U <= n_el; j += U) {
-                    // two elements per instruction; the eight distances from an integer are looked at together
-                    float r[U], off = 0.f;
+                for (; j + 4 <= n_el; j += 4) {
+                    // four look-ups in flight: one element after the other, a row that lands here would be the last to finish
+                    bool all = true;
+                    float r[4];
 #pragma unroll
-                    for (int u = 0; u < U; u += 4) {
-                        const float4 l4 = *reinterpret_cast<const float4*>(&lg[sd][j + u]);
+                    for (int u = 0; u < 4; ++u) { bool exact; r[u] = fast_round(lg[sd][j + u], fc, exact); all &= exact; }
+                    if (!all) {
 #pragma unroll
-                        for (int h = 0; h < 4; h += 2) {
-                            const f32x2 x = fma2(h ? pack2(l4.z, l4.w) : pack2(l4.x, l4.y), INV, NEGZ), m = add2(x, MAGIC);
-                            float d0, d1;
-                            unpack2(sub2(x, sub2(m, MAGIC)), d0, d1);
-                            off = max3(off, fabsf(d0), fabsf(d1));
-                            unpack2(m, r[u + h], r[u + h + 1]);
-                        }
+                        for (int u = 0; u < 4; ++u) r[u] = code_of(j + u);
                     }
-                    if (off <= fc.thr) {
-                        double d[U];
+                    double d[4];
 #pragma unroll
-                        for (int u = 0; u < U; u += 2) {
-                            const double2 a = *reinterpret_cast<const double2*>(&mag[sd][j + u]);
-                            d[u] = __dsub_rn(a.x, level(fminf(r[u], fc.top)));
-                            d[u + 1] = __dsub_rn(a.y, level(fminf(r[u + 1], fc.top)));
-                        }
+                    for (int u = 0; u < 4; ++u) d[u] = __dsub_rn((double)mag[sd][j + u], level(r[u]));
 #pragma unroll
-                        for (int u = 0; u < U; ++u) err = __dadd_rn(err, __dmul_rn(d[u], d[u]));
-                    } else {
-#pragma unroll 1
-                        for (int u = 0; u < U; ++u) careful(j + u);
-                    }
+                    for (int u = 0; u < 4; ++u) err = __dadd_rn(err, __dmul_rn(d[u], d[u]));
                 }
 #pragma unroll 1
-                for (; j < n_el; ++j) careful(j);
-                __syncwarp();
+                for (; j < n_el; ++j) { const double d = __dsub_rn((double)mag[sd][j], level(code_of(j))); err = __dadd_rn(err, __dmul_rn(d, d)); }
             }
             // first minimum in grid order: the smallest error, the lowest index among equals
             double e = ok ? err : INFINITY;
@@ -253,9 +315,9 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
         if (tid < nlev) {
             const int cc = tid - half;
             double v;
-            if (cc > 0) v = pcnt ? level_value(__dmul_rn(best[0].s, __dadd_rn((double)cc, best[0].z)), I) : 0.0;
-            else if (cc < 0) v = ncnt ? -level_value(__dmul_rn(best[1].s, __dadd_rn((double)(-cc), best[1].z)), I) : 0.0;
-            else v = pcnt ? level_value(__dmul_rn(best[0].s, best[0].z), I) : 0.0;
+            const int sdc = cc < 0, q = sdc ? -cc : cc;
+            v = (sdc ? ncnt : pcnt) ? __hiloint2double(level_word(__dmul_rn(best[sdc].s, __dadd_rn((double)q, best[sdc].z)), I), 0) : 0.0;
+            if (sdc) v = -v;
             T[tid] = v;
             levels[((size_t)n * ngrp + g) * nlev + tid] = (float)v;
         }
@@ -265,7 +327,7 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
             mt[4] = best[0].factor; mt[5] = best[1].factor;
         }
         __syncthreads();
-        // ---- codes, eight to a 32-bit word ( of nibbles, or three bytes of packed 3-bit codes)
+        // ---- codes, eight to a 32-bit word (of nibbles, or three bytes of packed 3-bit codes)
         double part = 0.0;
         const FastCode fcs[2] = {best_fc[0], best_fc[1]};
         // four lanes share eight codes, two elements each: the groups of 128 that grouped tables have keep every lane busy
@@ -285,7 +347,7 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                         bool exact;
                         const float r = fast_round(log2f(fabsf(v)), f, exact);
                         const int q = exact ? (int)(__float_as_uint(r) - __float_as_uint(kMagic))
-                                            : side_code(log2((double)fabsf(v)), best[neg].s, best[neg].z, neg ? half : half - 1);
+                                            : side_code(fabsf(v), best[neg].s, best[neg].z, neg ? half : half - 1);
                         cc = neg ? -q : q;
                     }
                     const int u = cc + half;

@@ -12,7 +12,7 @@ LIB = os.path.join(HERE, "liblrq_b200.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-    "--expt-relaxed-constexpr", "--extended-lambda", "-Xcompiler", "-fPIC", "-shared",
+    "--expt-relaxed-constexpr", "--extended-lambda", "--threads", "0", "-Xcompiler", "-fPIC", "-shared",
 ]
 
 

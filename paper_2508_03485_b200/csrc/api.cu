@@ -92,7 +92,7 @@ static lrq_status run_act(const void* X, int M, int K, long ldx, const lrq_act_p
         float* Yr = static_cast<float*>(workspace);
         st = lrq_launch_rotgemm(X, M, K, ldx, p->R_bf16, Yr, ext, stream);
         if (st != LRQ_OK) return st;
-        return lrq_launch_quantize_f32_ext(Yr, M, K, LRQ_ROT_TILE_DENSE, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, ex, stream);
+        return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, ex, stream);
     }
     if (p->kind == LRQ_ROT_DUAL) {
         const size_t need = lrq_act_workspace_bytes(M, K, p);
@@ -105,7 +105,7 @@ static lrq_status run_act(const void* X, int M, int K, long ldx, const lrq_act_p
         if (st != LRQ_OK) return st;
         st = lrq_launch_bdiag_gemm(V3, M, K, 3L * K, 3, p->R2_bf16, Yr, ext, stream);
         if (st != LRQ_OK) return st;
-        return lrq_launch_quantize_f32_ext(Yr, M, K, LRQ_ROT_TILE_DIAG, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, ex, stream);
+        return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, ex, stream);
     }
     const int B = p->kind == LRQ_ROT_HADAMARD ? p->had_block : 1;
     return lrq_launch_rotq_hadamard(X, M, K, ldx, B, p->a_bits, p->mode, out16, p->prescale, a_codes, a_scale, a_zp, ex, stream);

@@ -84,8 +84,8 @@ lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int
 // Where a rotation product leaves each row's extremes: over each tile's columns as a pair of floats (minimum, maximum), tile j of
 // row m at rows + m * pitch + 8 j; when a row is one tile, in row_min[m] and row_max[m].  All null: not wanted.
 struct LrqRowExt { unsigned char* rows; size_t pitch; float* row_min; float* row_max; };
-constexpr int LRQ_ROT_TILE_DENSE = 256, LRQ_ROT_TILE_DIAG = 128;      // columns per tile
-// rotgemm.cu : Y[M,K] (fp32) = X[M,K] (bf16) . R[K,K] (bf16) on the tensor cores
+constexpr int LRQ_ROT_TILE = 128;     // columns per tile
+// qgemm_bf16.cu : Y[M,K] (fp32) = X[M,K] (bf16) . R[K,K] (bf16) on the tensor cores
 lrq_status lrq_launch_rotgemm(const void* X, int M, int K, long ldx, const void* R, float* Y, const LrqRowExt& ext, cudaStream_t st);
 // rotgemm.cu : Y[M,K] (fp32) = sum over the `parts` column panels of A[M, parts*K] (bf16) of panel . blockdiag(Rblk),
 // Rblk bf16 [K/128][128][128]
@@ -93,10 +93,10 @@ lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int part
                                  cudaStream_t st);
 // rotdual.cu : V3 bf16 [M,3K], panel p = p-th bf16 term of U[m, perm[i]] (the reordering between the two rotations)
 lrq_status lrq_launch_dual_gather_split(const float* U, int M, int K, const int32_t* perm, void* V3, cudaStream_t st);
-// rotq.cu : per-token quantization of fp32 rows whose extremes a rotation product with tiles of `tile` columns has left, per
-// tile at the start of the row's own part of `codes` (8 bytes a tile; the codes overwrite them, and are longer for
-// every K above one tile), for one tile in scale[m] and zp[m].
-lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int tile, int a_bits, int mode, int out16, uint8_t* codes,
+// rotq.cu : per-token quantization of fp32 rows whose extremes a rotation product has left, per tile of LRQ_ROT_TILE columns at
+// the start of the row's own part of `codes` (8 bytes a tile; the codes overwrite them, and are longer for every K above
+// one tile), for one tile in scale[m] and zp[m].
+lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int a_bits, int mode, int out16, uint8_t* codes,
                                        float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st);
 
 // rotq.cu : fluctuation metric J (Eq. 11) and the kind Eq. 12 picks; acc is one double of device scratch

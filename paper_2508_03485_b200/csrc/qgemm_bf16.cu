@@ -18,6 +18,11 @@
 // 4608 x 12288 x 3072 contraction were 940 MB instead of 190 and it took 265 us instead of 211 (1650 TFLOP/s, at the
 // matmul peak; the kernel that decodes on the way: 300).  Issued by whole warps (see elect_one): 4096 x 1152 x 4608
 // takes 35 us, with a loop inside `lane == 0` 47.
+// The same kernel applies a dense outlier-aware rotation (Sec. 4.2, Eq. 12, second case: y = x . R, R bf16 [K,K] row-major):
+// the weight operand is then R as it lies, one 128-byte line of 64 output channels per k (MN-major, no transposed copy
+// of R is ever made), and the epilogue stores the fp32 accumulator and each row's extremes over every 128 columns,
+// which make the quantizer that follows a single streaming pass.  4608 x 3072 x 3072: 68 us with 128 x 256 tiles of single
+// CTAs, 59 now; 4429 x 1536 x 1536: 27 and 19.
 // Every wait is bounded, as in the other kernels; on expiry the CTA records a code, its copies in flight land, and both
 // CTAs meet at the final cluster barrier.
 #include "lrq_internal.cuh"
@@ -82,8 +87,13 @@ __device__ inline Tile tile_at(const Plan& p, int i) {
 struct Params {
     const float* a_scale; const int32_t* a_zp; const float* wsum; const float* wscale; const float* bias;
     int M, N, K, bf16_out; float zoff; int* status;
+    LrqRowExt ext;                // rotation: where the rows' extremes go
     Plan plan;
 };
+
+// What the kernel does with a finished accumulator: scale it and store fp32 or 16-bit outputs, or (rotation) store it as it
+// is and fold each row's extremes.
+enum Mode { OUT_F32, OUT_16, ROTATE };
 
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -127,10 +137,11 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
     return r;
 }
 
-template <bool OUT16>
+template <Mode MODE>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                   const __grid_constant__ CUtensorMap tmWs, const __grid_constant__ CUtensorMap tmWr, const __grid_constant__ CUtensorMap tmY) {
+    constexpr bool OUT16 = MODE == OUT_16, ROT = MODE == ROTATE;
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
     const uint32_t sA = smem_u32(base), sB = sA + STAGES * A_STAGE_BYTES, sEpi = sB + STAGES * B_STAGE_BYTES;
@@ -179,7 +190,10 @@ qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUte
                 if (lead) {
                     if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[s]), tx);
                     tma_load_2d_pair(sA + s * A_STAGE_BYTES, &tmA, kb * BK, m0, full0 + 8 * s);
-                    tma_load_2d_pair(sB + s * B_STAGE_BYTES, map_w, kb * BK, n0, full0 + 8 * s);
+                    if (ROT)                                  // boxes of 64 k-rows by 64 output channels
+                        for (int c = 0; c < half; c += 64) tma_load_2d_pair(sB + s * B_STAGE_BYTES + c * 128, &tmW, n0 + c, kb * BK, full0 + 8 * s);
+                    else
+                        tma_load_2d_pair(sB + s * B_STAGE_BYTES, map_w, kb * BK, n0, full0 + 8 * s);
                 }
                 __syncwarp();
                 ++issued;
@@ -196,7 +210,7 @@ qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUte
     } else if (warp == MMA_WARP) {
         if (rank == 0) {
             const bool lead = elect_one();
-            const uint64_t a0 = umma_desc_sw128(sA, 16, 1024), b0 = umma_desc_sw128(sB, 16, 1024);
+            const uint64_t a0 = umma_desc_sw128(sA, 16, 1024), b0 = umma_desc_sw128(sB, ROT ? BK * 128 : 16, 1024);
             int s = 0;
             uint32_t ph = 0, t = 0;
             bool ok = true;
@@ -206,7 +220,7 @@ qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUte
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * BN;
-                const uint32_t idesc = umma_idesc_bf16(BM, walk.t.width, false, false);
+                const uint32_t idesc = umma_idesc_bf16(BM, walk.t.width, false, ROT);
                 for (int kb = 0; kb < kblocks; ++kb) {
                     ok = mbar_wait_warp(smem_u32(&ctl->full[s]), ph, &ctl->abort_flag, p.status, 43);
                     if (!ok) break;
@@ -214,8 +228,8 @@ qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUte
                     if (lead) {
                         const uint64_t a = a0 + (uint64_t)(s * (A_STAGE_BYTES >> 4)), b = b0 + (uint64_t)(s * (B_STAGE_BYTES >> 4));
 #pragma unroll
-                        for (int k = 0; k < BK / 16; ++k)    // 16 k = 32 bytes along the row: 2 in descriptor units
-                            tc_mma_f16_pair(d_tmem, a + 2 * k, b + 2 * k, idesc, (kb | k) ? 1u : 0u);
+                        for (int k = 0; k < BK / 16; ++k)    // 16 k: 32 bytes along a row, or 16 lines of R; descriptors count 16 bytes
+                            tc_mma_f16_pair(d_tmem, a + 2 * k, b + (ROT ? 128 : 2) * k, idesc, (kb | k) ? 1u : 0u);
                         tc_commit_pair(smem_u32(&ctl->empty[s]), 3);
                     }
                     __syncwarp();
@@ -238,7 +252,7 @@ qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUte
             const int width = min(walk.t.width, p.N - n0);
             const uint32_t buf = t & 1;
             float (*col)[BN] = ctl->col[buf];
-            for (int c = et; c < walk.t.width; c += NUM_EPI_WARPS * 32) {
+            for (int c = et; !ROT && c < walk.t.width; c += NUM_EPI_WARPS * 32) {
                 const int n = n0 + c;
                 const bool okc = c < width;
                 col[0][c] = okc ? __ldg(p.wsum + n) : 0.f;
@@ -247,8 +261,9 @@ qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUte
             }
             if (bar_or_epilogue(ctl->abort_flag != 0)) break;     // the epilogue warps leave together
             const bool row_ok = m < p.M;
-            const float sm = row_ok ? __ldg(p.a_scale + m) : 0.f;
-            const float zm = row_ok ? (float)__ldg(p.a_zp + m) + p.zoff : 0.f;
+            const float sm = !ROT && row_ok ? __ldg(p.a_scale + m) : 0.f;
+            const float zm = !ROT && row_ok ? (float)__ldg(p.a_zp + m) + p.zoff : 0.f;
+            float mn = INFINITY, mx = -INFINITY;             // extremes of the row over the current 128 columns
             const f32x2 SM = pack2(sm, sm), ZM = pack2(zm, zm);
             const bool ok = mbar_wait_warp<100>(smem_u32(&ctl->tmem_full[buf]), (t >> 1) & 1, &ctl->abort_flag, p.status, 44);
             tc_fence_after();
@@ -261,8 +276,28 @@ qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUte
                     tc_wait_ld();
                     // y = s_m * (acc + z_m * wsum_n) [* wscale_n] [+ bias_n], two columns per instruction
                     f32x2 y[16];
+                    if (ROT) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
+                        for (int j = 0; j < 16; ++j) {
+                            y[j] = pack2(__uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
+                            if (c0 + 32 <= width) {
+                                mn = min3(mn, __uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
+                                mx = max3(mx, __uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
+                            } else if (c0 + 2 * j < width) {  // widths are even: K is a multiple of 8
+                                mn = min3(mn, __uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
+                                mx = max3(mx, __uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
+                            }
+                        }
+                        if (row_ok && ((c0 & 96) == 96 || c0 + 32 >= width)) {
+                            if (p.ext.rows) {
+                                float* e = reinterpret_cast<float*>(p.ext.rows + (size_t)m * p.ext.pitch) + 2 * ((n0 + c0) / LRQ_ROT_TILE);
+                                e[0] = mn; e[1] = mx;
+                            } else if (p.ext.row_min) { p.ext.row_min[m] = mn; p.ext.row_max[m] = mx; }
+                            mn = INFINITY; mx = -INFINITY;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < (ROT ? 0 : 8); ++j) {
                         const float4 ws = *reinterpret_cast<const float4*>(&col[0][c0 + 4 * j]);
                         f32x2 a0 = fma2(ZM, pack2(ws.x, ws.y), pack2(__uint_as_float(acc[4 * j]), __uint_as_float(acc[4 * j + 1])));
                         f32x2 a1 = fma2(ZM, pack2(ws.z, ws.w), pack2(__uint_as_float(acc[4 * j + 2]), __uint_as_float(acc[4 * j + 3])));
@@ -332,14 +367,14 @@ qgemm_bf16_kernel(const __grid_constant__ Params p, const __grid_constant__ CUte
     }
 }
 
-template <bool OUT16>
+template <Mode MODE>
 lrq_status max_pairs(int dev, int sms, int* out) {
     // per device and kernel variant: the shared-memory opt-in and the number of CTA pairs that can be resident
     static std::mutex mu;
     static int max_pairs_of[LRQ_MAX_DEVICES] = {};
     std::lock_guard<std::mutex> lock(mu);
     if (!max_pairs_of[dev]) {
-        LRQ_CUDA_TRY(cudaFuncSetAttribute(qgemm_bf16_kernel<OUT16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+        LRQ_CUDA_TRY(cudaFuncSetAttribute(qgemm_bf16_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -347,7 +382,7 @@ lrq_status max_pairs(int dev, int sms, int* out) {
         cfg.gridDim = dim3(sms & ~1); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = SMEM_BYTES;
         cfg.attrs = attr; cfg.numAttrs = 1;
         int clusters = 0;
-        LRQ_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, qgemm_bf16_kernel<OUT16>, &cfg));
+        LRQ_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, qgemm_bf16_kernel<MODE>, &cfg));
         if (clusters < 1) return LRQ_ERR_CUDA;
         max_pairs_of[dev] = clusters < sms / 2 ? clusters : sms / 2;
     }
@@ -355,15 +390,15 @@ lrq_status max_pairs(int dev, int sms, int* out) {
     return LRQ_OK;
 }
 
-Plan make_plan(int M, int N, int K, int pairs) {
+Plan make_plan(int M, int N, int K, int pairs, int unit) {
     Plan p;
     p.rows = (M + BM - 1) / BM;
     p.cols = N / BN;
-    p.ragged = (N % BN + UNIT - 1) / UNIT * UNIT;
+    p.ragged = (N % BN + unit - 1) / unit * unit;          // widths are multiples of `unit`
     if (p.ragged == BN) { ++p.cols; p.ragged = 0; }          // the last whole column is clipped by the copies
     p.whole = p.rows * p.cols;
     const int narrow = p.ragged ? p.rows : 0, left = p.whole % pairs;
-    p.pieces = left * 4 + narrow <= pairs ? 4 : left * 2 + narrow <= pairs ? 2 : 1;
+    p.pieces = left * 4 + narrow <= pairs && unit <= BN / 4 ? 4 : left * 2 + narrow <= pairs ? 2 : 1;
     p.split = p.pieces > 1 ? left : 0;
     p.total = p.whole - p.split + p.split * p.pieces + narrow;
     // Rows per panel: the fewest bytes from DRAM.  A panel's A is read once while it fits into half of the L2 (the other half
@@ -381,6 +416,22 @@ Plan make_plan(int M, int N, int K, int pairs) {
     return p;
 }
 
+template <Mode MODE>
+lrq_status launch(const Params& p, int pairs, const CUtensorMap& tmA, const CUtensorMap& tmW, const CUtensorMap& tmWs, const CUtensorMap& tmWr,
+                  const CUtensorMap& tmY, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(2 * (p.plan.total < pairs ? p.plan.total : pairs));
+    cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = st;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    LRQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, qgemm_bf16_kernel<MODE>, p, tmA, tmW, tmWs, tmWr, tmY));
+    return LRQ_OK;
+}
+
 }  // namespace
 
 lrq_status lrq_launch_qgemm_bf16(const lrq_layer* L, const void* A, const void* W, const float* a_scale, const int32_t* a_zp, int M,
@@ -388,14 +439,14 @@ lrq_status lrq_launch_qgemm_bf16(const lrq_layer* L, const void* A, const void* 
     const size_t es = dt == LRQ_F32 ? 4 : 2;
     int dev = 0, sms = 0, pairs = 0;
     if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
-    const lrq_status rs = dt == LRQ_F32 ? max_pairs<false>(dev, sms, &pairs) : max_pairs<true>(dev, sms, &pairs);
+    const lrq_status rs = dt == LRQ_F32 ? max_pairs<OUT_F32>(dev, sms, &pairs) : max_pairs<OUT_16>(dev, sms, &pairs);
     if (rs != LRQ_OK) return rs;
-    Params p;
+    Params p = {};
     p.a_scale = a_scale; p.a_zp = a_zp; p.wsum = L->wsum; p.wscale = L->wscale; p.bias = L->bias;
     p.M = M; p.N = L->N; p.K = L->K; p.bf16_out = dt == LRQ_BF16; p.zoff = L->act.a_bits == 8 ? 128.f : 8.f;
     p.status = lrq_status_word();
     if ((long)((M + BM - 1) / BM) * ((L->N + BN - 1) / BN) > (1l << 28)) return LRQ_ERR_UNSUPPORTED;
-    p.plan = make_plan(M, L->N, L->K, pairs);
+    p.plan = make_plan(M, L->N, L->K, pairs, UNIT);
     // weight boxes are half a tile's width: whole tiles, the parts of cut ones, the ragged column
     CUtensorMap tmA, tmW, tmWs, tmWr, tmY;
     auto map_w = [&](CUtensorMap* tm, int width) {
@@ -407,16 +458,27 @@ lrq_status lrq_launch_qgemm_bf16(const lrq_layer* L, const void* A, const void* 
     tmWs = tmWr = tmW;
     if (p.plan.split && !map_w(&tmWs, BN / p.plan.pieces)) return LRQ_ERR_CUDA;
     if (p.plan.ragged && !map_w(&tmWr, p.plan.ragged)) return LRQ_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(2 * (p.plan.total < pairs ? p.plan.total : pairs));
-    cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = st;
-    cfg.attrs = attr; cfg.numAttrs = 2;
-    LRQ_CUDA_TRY(dt == LRQ_F32 ? cudaLaunchKernelEx(&cfg, qgemm_bf16_kernel<false>, p, tmA, tmW, tmWs, tmWr, tmY)
-                               : cudaLaunchKernelEx(&cfg, qgemm_bf16_kernel<true>, p, tmA, tmW, tmWs, tmWr, tmY));
-    return LRQ_OK;
+    return dt == LRQ_F32 ? launch<OUT_F32>(p, pairs, tmA, tmW, tmWs, tmWr, tmY, st) : launch<OUT_16>(p, pairs, tmA, tmW, tmWs, tmWr, tmY, st);
+}
+
+lrq_status lrq_launch_rotgemm(const void* X, int M, int K, long ldx, const void* R, float* Y, const LrqRowExt& ext, cudaStream_t st) {
+    // TMA needs 16-byte aligned bases and row pitches (K and ldx multiples of 8 elements); the C ABI has already
+    // refused anything else
+    if ((K % 8) || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(R, 16) || !lrq_aligned(Y, 16)) return LRQ_ERR_INVALID_ARG;
+    int dev = 0, sms = 0, pairs = 0;
+    if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
+    const lrq_status rs = max_pairs<ROTATE>(dev, sms, &pairs);
+    if (rs != LRQ_OK) return rs;
+    if ((long)((M + BM - 1) / BM) * ((K + BN - 1) / BN) > (1l << 28)) return LRQ_ERR_UNSUPPORTED;
+    Params p = {};
+    p.M = M; p.N = K; p.K = K; p.status = lrq_status_word();
+    p.ext = ext;
+    if (K <= LRQ_ROT_TILE) p.ext.rows = nullptr;             // one tile per row: its extremes are the row's
+    p.plan = make_plan(M, K, K, pairs, 128);                 // each CTA loads R in boxes of 64 columns
+    CUtensorMap tmX, tmR, tmY;
+    if (!lrq_tma::make_map_2d(&tmX, X, 2, (uint64_t)M, (uint64_t)K, (uint64_t)ldx, BK, BM_CTA, true) ||
+        !lrq_tma::make_map_2d(&tmR, R, 2, (uint64_t)K, (uint64_t)K, (uint64_t)K, 64, BK, true) ||
+        !lrq_tma::make_map_2d(&tmY, Y, 4, (uint64_t)M, (uint64_t)K, (uint64_t)K, 32, 32, true))
+        return LRQ_ERR_CUDA;
+    return launch<ROTATE>(p, pairs, tmX, tmR, tmR, tmR, tmY, st);
 }

@@ -1,22 +1,17 @@
-// Outlier-aware rotation y = x . R (Sec. 4.2, Eq. 12, second case) as a dense contraction on the
-// 5th-generation tensor cores: X bf16 [M,K] times R bf16 [K,K] into an fp32 scratch that the
-// per-token quantizer then reads.  bf16 x bf16 products are exact in fp32; sums are accumulated in fp32.
-// The epilogue also leaves every row's minimum and maximum over the tile's columns, so that the quantizer that follows is a
-// single streaming pass: plain stores, one pair per row and tile, which need no initial values (two memsets and an
-// atomic pair per row and tile took their place before).
+// Product with a block-diagonal matrix of 128 x 128 blocks on the 5th-generation tensor cores: the factors R1hat, R2hat of the
+// dual transformation (Sec. 4.2).  The left operand is bf16 [M, parts*K]: `parts` column panels summed into one fp32
+// accumulator (the bf16 terms of an fp32 operand).  bf16 x bf16 products are exact in fp32; sums are accumulated in fp32.
+// With `ext` the epilogue also leaves every row's minimum and maximum over the tile's columns (plain stores, one pair per
+// row and tile), so that the quantizer that follows is a single streaming pass.
 //
-// Persistent CTA per SM over 128 x 256 output tiles, 64-deep k-blocks, a 4-stage TMA pipeline:
-//   warp 0      one lane issues the TMA tile loads (X: K-major box 64 x 128; R: four 64 x 64 boxes, each
-//               64 output columns wide, one k-row per 128-byte line -> an MN-major UMMA operand)
-//   warp 1      allocates TMEM, one lane issues tcgen05.mma (M = 128, N = 256, K = 16) and commits
+// Persistent CTA per SM over 128 x 128 output tiles (tile j of a token block only meets block j), 64-deep k-blocks, a
+// 4-stage TMA pipeline:
+//   warp 0      TMA tile loads (left operand: K-major box 64 x 128; blocks: two 64 x 64 boxes, each 64 output columns
+//               wide, one k-row per 128-byte line -> an MN-major UMMA operand)
+//   warp 1      allocates TMEM, issues tcgen05.mma (M = 128, N = 128, K = 16) and commits
 //   warps 2-5   epilogue: tcgen05.ld of the finished accumulator, fp32 stores
-// The accumulator is double-buffered in TMEM (2 x 256 columns).  Every wait is bounded; on expiry the
-// CTA records a code in the status word, waits (bounded) for its TMA loads in flight and unwinds.
-//
-// The same kernel, instantiated with 128-wide tiles, multiplies by a block-diagonal matrix of 128 x 128
-// blocks (the factors R1hat, R2hat of the dual transformation, Sec. 4.2): tile j of a token block only meets
-// block j, so its k-loop covers 128 input channels instead of K.  There the left operand may come in `parts`
-// column panels [M, parts*K] that are summed into one accumulator (the bf16 terms of an fp32 operand).
+// The accumulator is double-buffered in TMEM.  Every wait is bounded; on expiry the CTA records a code in the status word,
+// waits (bounded) for its TMA loads in flight and unwinds.
 #include "lrq_internal.cuh"
 #include "tc_ptx.cuh"
 #include "tma_host.cuh"
@@ -25,7 +20,7 @@
 namespace {
 using namespace lrq_tc;
 
-constexpr int BM = 128, BK = 64;
+constexpr int BM = 128, BN = 128, BK = 64;
 constexpr int STAGES = 4;
 constexpr int A_STAGE_BYTES = BM * BK * 2;          // 16 KB
 constexpr int B_CHUNK_BYTES = BK * 128;             // 8 KB: 64 k-rows of 64 output columns
@@ -42,19 +37,16 @@ struct __align__(16) Ctl {
     volatile int abort_flag;
 };
 constexpr int EPI_TILE_BYTES = 32 * 32 * 4;         // one epilogue warp's 32 x 32 fp32 chunk, for the row/column trade
-constexpr size_t smem_bytes(int bn) {
-    return 1024 + (size_t)STAGES * (A_STAGE_BYTES + (bn / 64) * B_CHUNK_BYTES) + sizeof(Ctl) + NUM_EPI_WARPS * EPI_TILE_BYTES;
-}
+constexpr int B_STAGE_BYTES = (BN / 64) * B_CHUNK_BYTES;        // 16 KB
+constexpr int STAGE_TX_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
+constexpr size_t SMEM_BYTES = 1024 + (size_t)STAGES * STAGE_TX_BYTES + sizeof(Ctl) + NUM_EPI_WARPS * EPI_TILE_BYTES;
+static_assert(BN == LRQ_ROT_TILE, "one pair of extremes per row and tile");
 
-// BN: tile width (256 dense; 128 = the diagonal block size when DIAG).  DIAG: R is block-diagonal, stored as its
-// blocks one after the other ([K/128][128][128], i.e. K rows of 128 columns); parts: column panels of the left operand.
-template <int BN, bool DIAG>
+// Rblk: the blocks one after the other ([K/128][128][128], i.e. K rows of 128 columns)
 __global__ void __launch_bounds__(NUM_THREADS, 1)
-rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
+bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
                   float* __restrict__ Y, int M, int K, int parts, unsigned char* __restrict__ ext, size_t ext_pitch, float* __restrict__ ext_min,
                   float* __restrict__ ext_max, int* status) {
-    constexpr int B_STAGE_BYTES = (BN / 64) * B_CHUNK_BYTES;   // 32 KB (16 KB for 128-wide tiles)
-    constexpr int STAGE_TX_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
     constexpr uint32_t IDESC = umma_idesc_bf16(BM, BN, /*a_mn_major=*/false, /*b_mn_major=*/true);
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
@@ -66,9 +58,7 @@ rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles_m = (M + BM - 1) / BM, tiles_n = (K + BN - 1) / BN;
     const int num_tiles = tiles_m * tiles_n;
-    // dense: the whole of K (a ragged last k-block is zero-filled by TMA in both operands);
-    // block-diagonal: the tile's own BN input channels, once per panel
-    const int kblocks = DIAG ? parts * (BN / BK) : (K + BK - 1) / BK;
+    const int kblocks = parts * (BN / BK);           // the tile's own 128 input channels, once per panel
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(smem_u32(&ctl->full[s]), 1); mbar_init(smem_u32(&ctl->empty[s]), 1); }
@@ -100,12 +90,12 @@ rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
                     const uint32_t bar = smem_u32(&ctl->full[s]);
                     mbar_arrive_expect_tx(bar, STAGE_TX_BYTES);
                     // k origin of this step in the left operand's columns and in R's rows
-                    const int kx = DIAG ? (kb / (BN / BK)) * K + n0 + (kb % (BN / BK)) * BK : kb * BK;
-                    const int kr = DIAG ? n0 + (kb % (BN / BK)) * BK : kb * BK;
+                    const int kx = (kb / (BN / BK)) * K + n0 + (kb % (BN / BK)) * BK;
+                    const int kr = n0 + (kb % (BN / BK)) * BK;
                     tma_load_2d(smem_u32(sA + s * A_STAGE_BYTES), &tmX, kx, m0, bar);
 #pragma unroll
                     for (int j = 0; j < BN / 64; ++j)
-                        tma_load_2d(smem_u32(sB + s * B_STAGE_BYTES + j * B_CHUNK_BYTES), &tmR, (DIAG ? 0 : n0) + 64 * j, kr, bar);
+                        tma_load_2d(smem_u32(sB + s * B_STAGE_BYTES + j * B_CHUNK_BYTES), &tmR, 64 * j, kr, bar);
                 }
                 __syncwarp();
                 ++issued;
@@ -166,47 +156,36 @@ rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             if (okw) {
 #pragma unroll 1
                 for (int c0 = 0; c0 < BN; c0 += 32) {
-                    if (n0 + c0 >= K) break;             // warp-uniform
                     uint32_t acc[32];
                     tc_ld32(tmem_base + ((uint32_t)(ew * 32) << 16) + (uint32_t)(buf * BN + c0), acc);
                     tc_wait_ld();
-                    if (n0 + c0 + 32 <= K) {
-                        // A lane holds 32 consecutive outputs of its own row.  The warp trades rows for columns through
-                        // a 4 KB tile (chunk index XOR-ed with the row's low bits: conflict-free both ways) so that each
-                        // store writes four rows' whole 128-byte lines instead of half a sector of 32 rows.
-                        const uint32_t tile = sEpi + (uint32_t)(warp - EPI_WARP0) * EPI_TILE_BYTES;
-                        __syncwarp();
+                    // A lane holds 32 consecutive outputs of its own row.  The warp trades rows for columns through
+                    // a 4 KB tile (chunk index XOR-ed with the row's low bits: conflict-free both ways) so that each
+                    // store writes four rows' whole 128-byte lines instead of half a sector of 32 rows.
+                    const uint32_t tile = sEpi + (uint32_t)(warp - EPI_WARP0) * EPI_TILE_BYTES;
+                    __syncwarp();
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(tile + (uint32_t)(lane * 128 + ((j ^ (lane & 7)) << 4))),
-                                         "r"(acc[4 * j]), "r"(acc[4 * j + 1]), "r"(acc[4 * j + 2]), "r"(acc[4 * j + 3]) : "memory");
-                        __syncwarp();
-                        const int rsub = lane >> 3, jq = lane & 7;
+                    for (int j = 0; j < 8; ++j)
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(tile + (uint32_t)(lane * 128 + ((j ^ (lane & 7)) << 4))),
+                                     "r"(acc[4 * j]), "r"(acc[4 * j + 1]), "r"(acc[4 * j + 2]), "r"(acc[4 * j + 3]) : "memory");
+                    __syncwarp();
+                    const int rsub = lane >> 3, jq = lane & 7;
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int r = 4 * i + rsub, mr = m0 + ew * 32 + r;
-                            if (mr < M) {
-                                uint4 v;
-                                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                                             : "r"(tile + (uint32_t)(r * 128 + ((jq ^ (r & 7)) << 4))) : "memory");
-                                *reinterpret_cast<uint4*>(Y + (size_t)mr * K + n0 + c0 + 4 * jq) = v;
-                            }
+                    for (int i = 0; i < 8; ++i) {
+                        const int r = 4 * i + rsub, mr = m0 + ew * 32 + r;
+                        if (mr < M) {
+                            uint4 v;
+                            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                                         : "r"(tile + (uint32_t)(r * 128 + ((jq ^ (r & 7)) << 4))) : "memory");
+                            *reinterpret_cast<uint4*>(Y + (size_t)mr * K + n0 + c0 + 4 * jq) = v;
                         }
-                        if (m < M) {
+                    }
+                    if (m < M) {
 #pragma unroll
-                            for (int j = 0; j < 32; j += 2) {
-                                asm("min.f32 %0, %0, %1, %2;" : "+f"(mn) : "f"(__uint_as_float(acc[j])), "f"(__uint_as_float(acc[j + 1])));
-                                asm("max.f32 %0, %0, %1, %2;" : "+f"(mx) : "f"(__uint_as_float(acc[j])), "f"(__uint_as_float(acc[j + 1])));
-                            }
+                        for (int j = 0; j < 32; j += 2) {
+                            asm("min.f32 %0, %0, %1, %2;" : "+f"(mn) : "f"(__uint_as_float(acc[j])), "f"(__uint_as_float(acc[j + 1])));
+                            asm("max.f32 %0, %0, %1, %2;" : "+f"(mx) : "f"(__uint_as_float(acc[j])), "f"(__uint_as_float(acc[j + 1])));
                         }
-                    } else if (m < M) {
-                        float* dst = Y + (size_t)m * K + n0 + c0;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (n0 + c0 + j < K) {
-                                const float v = __uint_as_float(acc[j]);
-                                dst[j] = v; mn = fminf(mn, v); mx = fmaxf(mx, v);
-                            }
                     }
                 }
             }
@@ -233,39 +212,6 @@ rotgemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
 
 }  // namespace
 
-template <int BN, bool DIAG>
-static lrq_status launch_rotgemm(const CUtensorMap& tmX, const CUtensorMap& tmR, float* Y, int M, int K, int parts, const LrqRowExt& ext,
-                                 cudaStream_t st) {
-    int dev = 0, sms = 0;
-    if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
-    {   // the shared-memory opt-in is a per-device function attribute: set once per device
-        static std::mutex mu;
-        static bool configured[LRQ_MAX_DEVICES] = {};
-        std::lock_guard<std::mutex> lock(mu);
-        if (!configured[dev]) {
-            LRQ_CUDA_TRY(cudaFuncSetAttribute(rotgemm_tc_kernel<BN, DIAG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem_bytes(BN)));
-            configured[dev] = true;
-        }
-    }
-    const int tiles = ((M + BM - 1) / BM) * ((K + BN - 1) / BN);
-    const bool one = K <= BN;                        // one tile per row: its extremes are the row's
-    LRQ_CUDA_TRY(lrq_launch_pdl(rotgemm_tc_kernel<BN, DIAG>, dim3(tiles < sms ? tiles : sms), dim3(NUM_THREADS), smem_bytes(BN),
-                                st, tmX, tmR, Y, M, K, parts, one ? nullptr : ext.rows, ext.pitch, one ? ext.row_min : nullptr,
-                                one ? ext.row_max : nullptr, lrq_status_word()));
-    return LRQ_OK;
-}
-
-lrq_status lrq_launch_rotgemm(const void* X, int M, int K, long ldx, const void* R, float* Y, const LrqRowExt& ext, cudaStream_t st) {
-    // TMA needs 16-byte aligned bases and row pitches (K and ldx multiples of 8 elements); the C ABI has already
-    // refused anything else
-    if ((K % 8) || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(R, 16) || !lrq_aligned(Y, 16)) return LRQ_ERR_INVALID_ARG;
-    CUtensorMap tmX, tmR;
-    if (!lrq_tma::make_map_2d(&tmX, X, 2, (uint64_t)M, (uint64_t)K, (uint64_t)ldx, BK, BM, true)) return LRQ_ERR_CUDA;
-    if (!lrq_tma::make_map_2d(&tmR, R, 2, (uint64_t)K, (uint64_t)K, (uint64_t)K, 64, BK, true)) return LRQ_ERR_CUDA;
-    return launch_rotgemm<LRQ_ROT_TILE_DENSE, false>(tmX, tmR, Y, M, K, 1, ext, st);
-}
-
 // Y[M,K] (fp32) = sum over panels p of A[:, pK .. pK+K) . blockdiag(Rblk), Rblk bf16 [K/128][128][128].
 lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int parts, const void* Rblk, float* Y, const LrqRowExt& ext,
                                  cudaStream_t st) {
@@ -275,5 +221,21 @@ lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int part
     CUtensorMap tmA, tmR;
     if (!lrq_tma::make_map_2d(&tmA, A, 2, (uint64_t)M, (uint64_t)parts * K, (uint64_t)lda, BK, BM, true)) return LRQ_ERR_CUDA;
     if (!lrq_tma::make_map_2d(&tmR, Rblk, 2, (uint64_t)K, 128, 128, 64, BK, true)) return LRQ_ERR_CUDA;
-    return launch_rotgemm<LRQ_ROT_TILE_DIAG, true>(tmA, tmR, Y, M, K, parts, ext, st);
+    int dev = 0, sms = 0;
+    if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
+    {   // the shared-memory opt-in is a per-device function attribute: set once per device
+        static std::mutex mu;
+        static bool configured[LRQ_MAX_DEVICES] = {};
+        std::lock_guard<std::mutex> lock(mu);
+        if (!configured[dev]) {
+            LRQ_CUDA_TRY(cudaFuncSetAttribute(bdiag_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+            configured[dev] = true;
+        }
+    }
+    const int tiles = ((M + BM - 1) / BM) * (K / BN);
+    const bool one = K == BN;                        // one tile per row: its extremes are the row's
+    LRQ_CUDA_TRY(lrq_launch_pdl(bdiag_gemm_kernel, dim3(tiles < sms ? tiles : sms), dim3(NUM_THREADS), SMEM_BYTES, st, tmA, tmR, Y, M, K,
+                                parts, one ? nullptr : ext.rows, ext.pitch, one ? ext.row_min : nullptr, one ? ext.row_max : nullptr,
+                                lrq_status_word()));
+    return LRQ_OK;
 }

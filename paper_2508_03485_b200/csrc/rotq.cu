@@ -202,7 +202,7 @@ __device__ __forceinline__ void load_raw(const __nv_bfloat16* p, uint4* raw) {
     }
 }
 
-template <int LOG2B, int A_BITS, int MAX_THREADS, int MIN_CTAS, bool WIDE>
+template <int LOG2B, int A_BITS, int MAX_THREADS, int MIN_CTAS, bool WIDE, bool PRE>
 __global__ void __launch_bounds__(MAX_THREADS, MIN_CTAS)
 rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int mode, int out16, int tok_per_cta, int num_groups,
                  const float* __restrict__ prescale,
@@ -222,7 +222,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
     lrq_pdl_trigger();
     lrq_pdl_wait();                      // X may be the previous kernel's output; the code buffer may still be read by it
     float4* ps = reinterpret_cast<float4*>(smem_raw + (3 * 2 * sizeof(int) * tok_per_cta + 15) / 16 * 16);
-    if (prescale) { stage_prescale<EPT / 4>(ps, prescale, K, tpt); __syncthreads(); }
+    if (PRE) { stage_prescale<EPT / 4>(ps, prescale, K, tpt); __syncthreads(); }
 
     uint4 raw[4];
     {
@@ -247,7 +247,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
             for (int c = 0; c < 4; ++c)
                 P[4 * i + c] = pack2(__uint_as_float(w[c] << 16), __uint_as_float(w[c] & 0xffff0000u));
         }
-        if (prescale) apply_prescale<EPT / 4>(P, ps, j, tpt);  // before the rotation
+        if (PRE) apply_prescale<EPT / 4>(P, ps, j, tpt);  // before the rotation
         // the next group's loads fly while this group is transformed
         {
             const int mn = (g + (int)gridDim.x) * tok_per_cta + tl;
@@ -369,7 +369,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
 // conflict-free as well.  A warp's rows and its B words occupy the same two 2 KB pieces, so only the B reads
 // cross warps: one barrier before them; the barrier of the extremes separates them from the next group.
 // ------------------------------------------------------------------------------------------------
-template <int LOG2B, int A_BITS, int MAX_THREADS, int MIN_CTAS, bool WIDE>
+template <int LOG2B, int A_BITS, int MAX_THREADS, int MIN_CTAS, bool WIDE, bool PRE>
 __global__ void __launch_bounds__(MAX_THREADS, MIN_CTAS)
 rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int mode, int out16, int tok_per_cta, int num_groups,
                 const float* __restrict__ prescale,
@@ -407,7 +407,7 @@ rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int
     lrq_pdl_trigger();
     lrq_pdl_wait();                      // X may be the previous kernel's output; the code buffer may still be read by it
     float4* ps = reinterpret_cast<float4*>(buf + (size_t)(blockDim.x / (U * 32)) * UNIT_FLOATS);
-    if (prescale) { stage_prescale<EPT / 4>(ps, prescale, K, tpt); __syncthreads(); }
+    if (PRE) { stage_prescale<EPT / 4>(ps, prescale, K, tpt); __syncthreads(); }
 
     uint4 raw[4];
     {
@@ -431,7 +431,7 @@ rotq_big_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, int
             for (int c = 0; c < 4; ++c)
                 P[4 * i + c] = pack2(__uint_as_float(w[c] << 16), __uint_as_float(w[c] & 0xffff0000u));
         }
-        if (prescale) apply_prescale<EPT / 4>(P, ps, j, tpt);
+        if (PRE) apply_prescale<EPT / 4>(P, ps, j, tpt);
         {
             const int mn = (g + (int)gridDim.x) * tok_per_cta + tl;
             if (g + (int)gridDim.x < num_groups && mn < M) {
@@ -614,13 +614,13 @@ quant_rows_f32_kernel(const float* __restrict__ Y, int M, int K, int tiles, int 
 
 }  // namespace
 
-lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int tile, int a_bits, int mode, int out16, uint8_t* codes,
+lrq_status lrq_launch_quantize_f32_ext(const float* Y, int M, int K, int a_bits, int mode, int out16, uint8_t* codes,
                                        float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
     if (!lrq_aligned(Y, 32)) return LRQ_ERR_INVALID_ARG;          // rows are K*4 bytes with K % 8 == 0: 32-byte aligned chunks
     int sms = 0;
     if (lrq_current_device(nullptr, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
     const int grid = lrq_quant_grid((M + 7) / 8, sms * 8, 8, ex);  // 8 warps per CTA, one token per warp and step
-    const int tiles = (K + tile - 1) / tile;
+    const int tiles = (K + LRQ_ROT_TILE - 1) / LRQ_ROT_TILE;
     auto kern = a_bits == 8 ? (out16 ? quant_rows_f32_kernel<8, true> : quant_rows_f32_kernel<8, false>)
                             : (out16 ? quant_rows_f32_kernel<4, true> : quant_rows_f32_kernel<4, false>);
     LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(256), 0, st, Y, M, K, tiles, mode, codes, scale, zp, ex));
@@ -750,13 +750,13 @@ static lrq_status launch_generic(const void* X, int M, int K, long ldx, int log2
     return LRQ_OK;
 }
 
-template <int LOG2B, bool BIG, int A_BITS, int NT, int NB, bool WIDE>
+template <int LOG2B, bool BIG, int A_BITS, int NT, int NB, bool WIDE, bool PRE>
 struct RotqPick {
-    static constexpr auto kern = rotq_fast_kernel<LOG2B, A_BITS, NT, NB, WIDE>;
+    static constexpr auto kern = rotq_fast_kernel<LOG2B, A_BITS, NT, NB, WIDE, PRE>;
 };
-template <int LOG2B, int A_BITS, int NT, int NB, bool WIDE>
-struct RotqPick<LOG2B, true, A_BITS, NT, NB, WIDE> {
-    static constexpr auto kern = rotq_big_kernel<LOG2B, A_BITS, NT, NB, WIDE>;
+template <int LOG2B, int A_BITS, int NT, int NB, bool WIDE, bool PRE>
+struct RotqPick<LOG2B, true, A_BITS, NT, NB, WIDE, PRE> {
+    static constexpr auto kern = rotq_big_kernel<LOG2B, A_BITS, NT, NB, WIDE, PRE>;
 };
 
 template <int LOG2B, bool BIG = false>
@@ -781,12 +781,14 @@ static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits,
     // 256-bit accesses when every thread's 64 input bytes and 32 code bytes start on 32-byte boundaries
     const bool wide = lrq_aligned(X, 32) && (ldx % 16) == 0 && lrq_aligned(codes, 32);
     Kern kern;
-#define LRQ_PICK(NT, NB) (wide ? (a_bits == 8 ? RotqPick<LOG2B, BIG, 8, NT, NB, true>::kern : RotqPick<LOG2B, BIG, 4, NT, NB, true>::kern) \
-                               : (a_bits == 8 ? RotqPick<LOG2B, BIG, 8, NT, NB, false>::kern : RotqPick<LOG2B, BIG, 4, NT, NB, false>::kern))
+#define LRQ_PICK_W(NT, NB, W, P) (a_bits == 8 ? RotqPick<LOG2B, BIG, 8, NT, NB, W, P>::kern : RotqPick<LOG2B, BIG, 4, NT, NB, W, P>::kern)
+#define LRQ_PICK(NT, NB) (prescale ? (wide ? LRQ_PICK_W(NT, NB, true, true) : LRQ_PICK_W(NT, NB, false, true)) \
+                                   : (wide ? LRQ_PICK_W(NT, NB, true, false) : LRQ_PICK_W(NT, NB, false, false)))
     if (threads <= 288) kern = LRQ_PICK(288, 3);
     else if (threads <= 384) kern = LRQ_PICK(384, 2);
     else kern = LRQ_PICK(512, 1);
 #undef LRQ_PICK
+#undef LRQ_PICK_W
     // persistent grid: as many CTAs as stay resident, each walking over token groups with a grid stride
     int dev = 0, sms = 0, per_sm = 0;
     if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;

@@ -166,6 +166,13 @@ lrq_status lrq_ars_select(const void* X_bf16, int M, int K, long ldx, double thr
 lrq_status lrq_rotate_weights(const float* W, int N, int K, long ldw, const float* colmul, lrq_rot_kind kind,
                               int had_block, const void* R_bf16, float* W_rot, long ldo, void* cuda_stream);
 
+/* The same with device scratch (256-byte aligned, at least lrq_rotate_weights_workspace_bytes; 0 means none is used), for
+ * LRQ_ROT_DENSE to the same accuracy several times faster: the product on the int8 tensor cores from exact digits. */
+size_t lrq_rotate_weights_workspace_bytes(int N, int K, lrq_rot_kind kind);
+lrq_status lrq_rotate_weights_ws(const float* W, int N, int K, long ldw, const float* colmul, lrq_rot_kind kind,
+                                 int had_block, const void* R_bf16, float* W_rot, long ldo, void* workspace,
+                                 size_t workspace_bytes, void* cuda_stream);
+
 /* The same for the dual transformation in its factors (LRQ_ROT_DUAL): W_rot = W diag(colmul) R1hat P R2hat,
  * arguments as in lrq_act_params.  Each row is held in shared memory as fp64: K <= 12288. */
 lrq_status lrq_rotate_weights_dual(const float* W, int N, int K, long ldw, const float* colmul, int dual_block,

@@ -23,6 +23,7 @@ EXPORTS = [
     "lrq_layer_destroy", "lrq_workspace_bytes", "lrq_qlinear", "lrq_qlinear_stack", "lrq_qgemm_codes",
     "lrq_device_status", "lrq_status_string", "lrq_version", "lrq_rotate_quantize_act_static", "lrq_ars_select",
     "lrq_rotate_weights", "lrq_selftest_wait_timeout", "lrq_static_scratch_bytes", "lrq_rotate_weights_dual",
+    "lrq_rotate_weights_ws", "lrq_rotate_weights_workspace_bytes",
 ]
 
 
@@ -75,6 +76,9 @@ def load_library() -> C.CDLL:
     lib.lrq_qgemm_codes.argtypes = [vp, vp, vp, vp, ci, vp, ci, cl, ci, vp]
     lib.lrq_ars_select.argtypes = [vp, ci, ci, cl, C.c_double, vp, vp, vp, sz, vp]
     lib.lrq_rotate_weights.argtypes = [vp, ci, ci, cl, vp, ci, ci, vp, vp, cl, vp]
+    lib.lrq_rotate_weights_ws.argtypes = [vp, ci, ci, cl, vp, ci, ci, vp, vp, cl, vp, sz, vp]
+    lib.lrq_rotate_weights_workspace_bytes.argtypes = [ci, ci, ci]
+    lib.lrq_rotate_weights_workspace_bytes.restype = sz
     lib.lrq_rotate_weights_dual.argtypes = [vp, ci, ci, cl, vp, ci, vp, vp, vp, vp, cl, vp]
     lib.lrq_device_status.argtypes = [vp]
     lib.lrq_selftest_wait_timeout.argtypes = [C.c_longlong, vp]
@@ -226,8 +230,13 @@ def lrq_rotate_weights(W: torch.Tensor, kind: int, had_block: int = 0, R: Option
     if out is None:
         out = torch.empty((N, K), dtype=torch.float32, device=W.device)
     assert out.dtype == torch.float32 and out.shape == (N, K) and out.stride(1) == 1
-    _check(load_library().lrq_rotate_weights(_ptr(W), N, K, W.stride(0), _ptr(colmul), kind, had_block, _ptr(R), _ptr(out),
-                                             out.stride(0), _stream(stream)), "lrq_rotate_weights")
+    lib = load_library()
+    need = int(lib.lrq_rotate_weights_workspace_bytes(N, K, kind))
+    ws = torch.empty(need, dtype=torch.uint8, device=W.device) if need else None
+    if ws is not None and stream is not None:
+        ws.record_stream(stream)
+    _check(lib.lrq_rotate_weights_ws(_ptr(W), N, K, W.stride(0), _ptr(colmul), kind, had_block, _ptr(R), _ptr(out),
+                                     out.stride(0), _ptr(ws), need, _stream(stream)), "lrq_rotate_weights")
     return out
 
 

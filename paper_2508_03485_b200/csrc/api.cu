@@ -165,6 +165,16 @@ extern "C" lrq_status lrq_ars_select(const void* X, int M, int K, long ldx, doub
 
 extern "C" lrq_status lrq_rotate_weights(const float* W, int N, int K, long ldw, const float* colmul, lrq_rot_kind kind,
                                          int had_block, const void* R_bf16, float* W_rot, long ldo, void* cuda_stream) {
+    return lrq_rotate_weights_ws(W, N, K, ldw, colmul, kind, had_block, R_bf16, W_rot, ldo, nullptr, 0, cuda_stream);
+}
+
+extern "C" size_t lrq_rotate_weights_workspace_bytes(int N, int K, lrq_rot_kind kind) {
+    return kind == LRQ_ROT_DENSE && N > 0 && K > 0 ? lrq_wrot_i8_workspace(N, K) : 0;
+}
+
+extern "C" lrq_status lrq_rotate_weights_ws(const float* W, int N, int K, long ldw, const float* colmul, lrq_rot_kind kind,
+                                            int had_block, const void* R_bf16, float* W_rot, long ldo, void* workspace,
+                                            size_t workspace_bytes, void* cuda_stream) {
     if (!W || !W_rot || N <= 0 || K <= 0 || ldw < K || ldo < K) return LRQ_ERR_INVALID_ARG;
     if (kind == LRQ_ROT_HADAMARD) {
         if (had_block < 1 || (had_block & (had_block - 1)) || K % had_block) return LRQ_ERR_INVALID_ARG;
@@ -173,6 +183,11 @@ extern "C" lrq_status lrq_rotate_weights(const float* W, int N, int K, long ldw,
         if (W_rot == W) return LRQ_ERR_INVALID_ARG;               // the product reads whole rows of W per output tile
     } else if (kind != LRQ_ROT_NONE) {
         return LRQ_ERR_INVALID_ARG;
+    }
+    if (workspace) {
+        const size_t need = lrq_rotate_weights_workspace_bytes(N, K, kind);
+        if (!lrq_aligned(workspace, 256) || workspace_bytes < need) return LRQ_ERR_WORKSPACE;
+        if (need) return lrq_launch_rotate_weights_i8(W, N, K, ldw, colmul, R_bf16, W_rot, ldo, workspace, (cudaStream_t)cuda_stream);
     }
     return lrq_launch_rotate_weights(W, N, K, ldw, colmul, (int)kind, had_block, R_bf16, W_rot, ldo, (cudaStream_t)cuda_stream);
 }

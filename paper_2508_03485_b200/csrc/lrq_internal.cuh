@@ -106,6 +106,10 @@ lrq_status lrq_launch_ars_metric(const void* X, int M, int K, long ldx, double t
 // wrot.cu : W diag(colmul) R in fp64, rounded to fp32 (Eq. 2, weight side)
 lrq_status lrq_launch_rotate_weights(const float* W, int N, int K, long ldw, const float* colmul, int kind,
                                      int had_block, const void* R, float* out, long ldo, cudaStream_t st);
+// wrot_i8.cu : the dense case on the int8 tensor cores, to the same accuracy; 0 bytes: the shape is not taken
+size_t lrq_wrot_i8_workspace(int N, int K);
+lrq_status lrq_launch_rotate_weights_i8(const float* W, int N, int K, long ldw, const float* colmul, const void* R, float* out, long ldo,
+                                        void* workspace, cudaStream_t st);
 lrq_status lrq_launch_rotate_weights_dual(const float* W, int N, int K, long ldw, const float* colmul, int Bd, const void* R1,
                                           const int32_t* perm, const void* R2, float* out, long ldo, cudaStream_t st);
 

@@ -3,8 +3,9 @@
 // the TLQ quantizer reads.
 //
 // Offline step.  Hadamard: one CTA per weight row, butterflies in registers, up to four stages between two trips
-// through shared memory.  Dense: an fp64 matrix product on the fp64 tensor cores, 64 x 64 output tiles; R is the
-// layer's stored bf16 matrix (exact in fp64), so both sides of Eq. 2 use the same R.  Dual transformation (R = R1hat P R2hat, Sec. 4.2): one CTA per row, the
+// through shared memory.  Dense: an fp64 matrix product on the fp64 tensor cores, 64 x 64 output tiles, for small
+// layers and for callers without scratch (wrot_i8.cu otherwise); R is the layer's stored bf16 matrix (exact in fp64), so both
+// sides of Eq. 2 use the same R.  Dual transformation (R = R1hat P R2hat, Sec. 4.2): one CTA per row, the
 // row in shared memory as fp64, block-diagonal product, gather through the index map, second product.
 #include "lrq_internal.cuh"
 

@@ -1,0 +1,590 @@
+// Dense weight rotation W_rot = (W diag(colmul)) . R on the int8 tensor cores, to fp64 accuracy and rounded once to fp32
+// (Sec. 3.2, Eq. 2, weight side; splitting after Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix
+// multiplication", Numer. Algorithms 59 (2012)).
+//
+// A row of W diag(colmul) and a column of R each become fixed-point numbers of 62 bits below their own power of two,
+//   w[n,k] c[k] = 2^(ew[n] - 6) sum_i a_i 2^(-8 i),   r[k,j] = 2^(er[j] - 6) sum_i b_i 2^(-8 i),   a_i, b_i int8, i < 8,
+// in balanced base-256 digits, so that
+//   out[n,j] = 2^(ew + er - 12) sum_d 2^(-8 d) S_d,   S_d = sum over i + l = d of sum_k a_i[n,k] b_l[k,j]
+// with every S_d an exact int32 sum of the tensor core.  d <= 7 is taken: what is dropped is below 8 K 2^14 2^-76 of
+// 2^(ew + er) (2^-48 for K = 1536), and the few results smaller than 2^-20 of it are summed again in fp64, so that the
+// omission stays below 2^-28 of any result (an fp64 chain of K terms has an error of its own up to K 2^-53 of the sum of
+// its magnitudes).
+//
+// Most digits are zero: a bf16 number has 8 significant bits and a float 24, so 256 x 128 blocks of W take 6 or 7 digits
+// and blocks of R 4.  The split notes how many per block, and a product of 23 digit pairs rather than 36 is left.
+//
+// Bound by the tensor pipe (a 256 x 128 x 32 MMA runs 64 cycles) and the issuing warp beside it: with a barrier and a commit
+// for every digit of R as well, rather than one per block, 4608 x 1536 x 1536 took 263 us.  4608 x 1536 x 1536: 660 us on the fp64 tensor cores,
+// 198 here (of which the split 30).  1024 x 1024: 96 and 58.
+#include "lrq_internal.cuh"
+#include "tc_ptx.cuh"
+#include "tma_host.cuh"
+#include <cuda_bf16.h>
+#include <mutex>
+
+namespace {
+using namespace lrq_tc;
+
+constexpr int D = 8;                                        // digits
+constexpr int BM_CTA = 128, BM = 256, BN = 128, BK = 128;   // a pair's tile; k per block (one 128-byte line of int8)
+constexpr int MIN_A = 5, MIN_B = 4;                         // digits always multiplied: every S_d then gets a term
+constexpr int A_BYTES = BM_CTA * BK, B_BYTES = BN / 2 * BK; // one digit of a block in a CTA: 16 and 8 KB
+constexpr int A_SLOTS = 9, B_SLOTS = 9;
+static_assert(B_SLOTS >= D, "all digits of a block of R stay in place while those of W pass");
+// Two blocks' digits of R share B_SLOTS: those of even blocks from the bottom, those of odd ones from the top.
+__device__ __forceinline__ int b_slot(uint32_t parity, int t) { return parity ? B_SLOTS - 1 - t : t; }
+constexpr int ROWS_PER_CTA = 16;                            // rows of W a splitting CTA takes; BM / ROWS_PER_CTA counts a tile
+constexpr int SPLIT_THREADS = 32 * ROWS_PER_CTA;
+constexpr int EPI_WARPS = 8, EPI_WARP0 = 2, NUM_THREADS = (EPI_WARP0 + EPI_WARPS) * 32;
+constexpr int TMEM_COLS = 512;                              // four S_d of 128 columns
+constexpr int K_MAX = 16384;                                // |S_d| <= 8 K 2^14 < 2^31
+
+// ---------------------------------------------------------------------------------------------- digits
+constexpr unsigned long long HALVES = 0x8080808080808080ull;
+// Balanced base-256 digits of v, one per byte (byte 7 the first digit), |v| <= 2^62.
+__device__ __forceinline__ unsigned long long digits_of(long long v) { return ((unsigned long long)v + HALVES) ^ HALVES; }
+__device__ __forceinline__ int digits_used(unsigned long long x) { return x ? 8 - ((__ffsll((long long)x) - 1) >> 3) : 0; }
+
+// Digit planes of four consecutive k: word i holds digit i of all four.
+__device__ __forceinline__ void store_digits(const unsigned long long (&x)[4], int8_t* dst, size_t plane) {
+    uint32_t w[8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t a[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) a[e] = (uint32_t)(x[e] >> (32 * h));
+        const uint32_t p = __byte_perm(a[0], a[1], 0x5140), q = __byte_perm(a[2], a[3], 0x5140);     // bytes 0, 1
+        const uint32_t r = __byte_perm(a[0], a[1], 0x7362), s = __byte_perm(a[2], a[3], 0x7362);     // bytes 2, 3
+        w[7 - 4 * h] = __byte_perm(p, q, 0x5410); w[6 - 4 * h] = __byte_perm(p, q, 0x7632);
+        w[5 - 4 * h] = __byte_perm(r, s, 0x5410); w[4 - 4 * h] = __byte_perm(r, s, 0x7632);
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) *reinterpret_cast<uint32_t*>(dst + i * plane) = w[i];
+}
+
+struct Split {
+    const float* W; long ldw; const float* colmul; const __nv_bfloat16* R;
+    int N, K, Np, Kp, r_ctas;
+    int8_t *a, *b;                // [D][Np][Kp] and, transposed, [D][Kp][Kp]
+    uint8_t *na, *nb;             // digits in use: [Kp / 128][Np / 16] per 16 rows, [Kp / 128][Kp / 128]
+    double *sa, *sb;              // 2^(ew - 34), 2^(er - 34); 0 for a row or column of zeros, NaN if it is not finite
+};
+
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+// Smallest power of two above |m| is 2^e.
+__device__ __forceinline__ int exponent_above(double m) {
+    const int be = (__double2hiint(m) >> 20) & 0x7ff;        // products of floats and bf16 numbers are normal as doubles
+    return be - 1022;
+}
+
+// R[k, j .. j+7] and W's row at k .. k+3, zero outside.  VEC: 16-byte aligned rows whose length is a multiple of the vector; one
+// predicated load, so that the loops around it keep several in flight.
+template <bool VEC>
+__device__ __forceinline__ uint4 load8(const unsigned short* R, int k, int j, int K) {
+    uint4 x = make_uint4(0, 0, 0, 0);
+    if constexpr (VEC) {
+        if (k < K && j < K) x = __ldg(reinterpret_cast<const uint4*>(R + (size_t)k * K + j));
+    } else {
+        uint32_t v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t lo = k < K && j + 2 * i < K ? R[(size_t)k * K + j + 2 * i] : 0u;
+            const uint32_t hi = k < K && j + 2 * i + 1 < K ? R[(size_t)k * K + j + 2 * i + 1] : 0u;
+            v[i] = lo | (hi << 16);
+        }
+        x = make_uint4(v[0], v[1], v[2], v[3]);
+    }
+    return x;
+}
+template <bool VEC>
+__device__ __forceinline__ float4 load4(const float* w, int k, int K) {
+    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (VEC) {
+        if (k < K) f = __ldg(reinterpret_cast<const float4*>(w + k));
+        return f;
+    }
+    if (k < K) f.x = __ldg(w + k);
+    if (k + 1 < K) f.y = __ldg(w + k + 1);
+    if (k + 2 < K) f.z = __ldg(w + k + 2);
+    if (k + 3 < K) f.w = __ldg(w + k + 3);
+    return f;
+}
+
+// CTAs 0 .. r_ctas-1 split R: one 128 x 128 block each, after a pass over its 128 columns for their largest magnitudes (from
+// the L2; 0.4 MB at K = 1536).  The others split 16 rows of W each, a warp a row.  Bound by the writes: 76 MB for
+// 4608 x 1536 and its R.
+template <bool VEC>
+__global__ void __launch_bounds__(SPLIT_THREADS, 3)
+wrot_split_kernel(const __grid_constant__ Split p) {
+    constexpr int ROWS = SPLIT_THREADS / 16, WARPS = SPLIT_THREADS / 32;       // rows of R at a time, 16 threads each
+    __shared__ struct { uint16_t mx[ROWS][128]; uint16_t t[128][130]; } sm;
+    __shared__ int used[K_MAX / BK];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, kblocks = p.Kp / BK;
+    lrq_pdl_trigger();
+    lrq_pdl_wait();
+    if ((int)blockIdx.x < p.r_ctas) {
+        const int kb = blockIdx.x % kblocks, jb = blockIdx.x / kblocks, j0 = jb * 128, k0 = kb * BK;
+        const unsigned short* R = reinterpret_cast<const unsigned short*>(p.R);
+        // the columns' largest magnitudes: bf16 magnitudes order like their bits
+        const int row = tid >> 4, c8 = (tid & 15) * 8;
+        uint32_t m[4] = {0, 0, 0, 0};
+#pragma unroll 8
+        for (int k = row; k < p.Kp; k += ROWS) {
+            const uint4 v = load8<VEC>(R, k, j0 + c8, p.K);
+            m[0] = __vmaxu2(m[0], v.x & 0x7fff7fffu); m[1] = __vmaxu2(m[1], v.y & 0x7fff7fffu);
+            m[2] = __vmaxu2(m[2], v.z & 0x7fff7fffu); m[3] = __vmaxu2(m[3], v.w & 0x7fff7fffu);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { sm.mx[row][c8 + 2 * i] = (uint16_t)m[i]; sm.mx[row][c8 + 2 * i + 1] = (uint16_t)(m[i] >> 16); }
+        for (int r = row; r < BK; r += ROWS) {
+            const uint4 v = load8<VEC>(R, k0 + r, j0 + c8, p.K);
+            uint32_t* t = reinterpret_cast<uint32_t*>(&sm.t[r][c8]);
+            t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+        }
+        if (tid == 0) used[0] = 0;
+        __syncthreads();
+        if (tid < 128) {
+            uint32_t mm = 0;
+            for (int r = 0; r < ROWS; ++r) mm = max(mm, (uint32_t)sm.mx[r][tid]);
+            sm.mx[0][tid] = (uint16_t)mm;
+            if (kb == 0) {
+                const double s = mm >= 0x7f80u ? __longlong_as_double(0x7ff8000000000000ll) :
+                                 mm == 0 ? 0.0 : pow2(exponent_above((double)__uint_as_float(mm << 16)) - 34);
+                p.sb[j0 + tid] = s;
+            }
+        }
+        __syncthreads();
+        const size_t plane = (size_t)p.Kp * p.Kp;
+        unsigned long long all = 0;
+        for (int jj = warp; jj < 128; jj += WARPS) {              // a warp a column, four k a lane
+            const uint32_t mm = sm.mx[0][jj];
+            const double scale = mm != 0 && mm < 0x7f80u ? pow2(62 - exponent_above((double)__uint_as_float(mm << 16))) : 0.0;
+            unsigned long long x[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                x[e] = digits_of(__double2ll_rn((double)__uint_as_float((uint32_t)sm.t[4 * lane + e][jj] << 16) * scale));
+            }
+            all |= x[0] | x[1] | x[2] | x[3];
+            store_digits(x, p.b + (size_t)(j0 + jj) * p.Kp + k0 + 4 * lane, plane);
+        }
+        const int most = __reduce_max_sync(0xffffffffu, digits_used(all));
+        if (lane == 0) atomicMax(&used[0], most);
+        __syncthreads();
+        if (tid == 0) p.nb[(size_t)kb * kblocks + jb] = (uint8_t)max(used[0], MIN_B);
+        return;
+    }
+    const int grp = blockIdx.x - p.r_ctas, n0 = grp * ROWS_PER_CTA;
+    for (int i = tid; i < kblocks; i += SPLIT_THREADS) used[i] = 0;
+    __syncthreads();
+    const size_t plane = (size_t)p.Np * p.Kp;
+    const int n = n0 + warp;
+    if (n < p.N) {
+        const float* w = p.W + (size_t)n * p.ldw;
+        auto widen = [&](const float4& f, int k, double (&v)[4]) {
+            v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+            if (p.colmul) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] *= k + e < p.K ? (double)__ldg(p.colmul + k + e) : 0.0;
+            }
+        };
+        double mx = 0.0;
+        bool finite = true;
+        if (p.colmul) {
+#pragma unroll 4
+            for (int k = 4 * lane; k < p.Kp; k += 128) {
+                double v[4];
+                widen(load4<VEC>(w, k, p.K), k, v);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { finite = finite && fabs(v[e]) < INFINITY; mx = fmax(mx, fabs(v[e])); }
+            }
+        } else {
+            uint32_t m = 0;                                  // magnitudes order like their bits, infinities and NaN last
+#pragma unroll 4
+            for (int k = 4 * lane; k < p.Kp; k += 128) {
+                const float4 f = load4<VEC>(w, k, p.K);
+                m = max(max(max(m, __float_as_uint(f.x) & 0x7fffffffu), max(__float_as_uint(f.y) & 0x7fffffffu, __float_as_uint(f.z) & 0x7fffffffu)),
+                        __float_as_uint(f.w) & 0x7fffffffu);
+            }
+            finite = m < 0x7f800000u;
+            mx = (double)__uint_as_float(finite ? m : 0u);
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        finite = __all_sync(0xffffffffu, finite);
+        const bool ok = finite && mx > 0.0;
+        const int e0 = ok ? exponent_above(mx) : 0;
+        if (lane == 0) p.sa[n] = !finite ? __longlong_as_double(0x7ff8000000000000ll) : ok ? pow2(e0 - 34) : 0.0;
+        const double scale = ok ? pow2(62 - e0) : 0.0;
+#pragma unroll 4
+        for (int kb = 0; kb < kblocks; ++kb) {
+            const int k = kb * BK + 4 * lane;
+            double v[4];
+            widen(load4<VEC>(w, k, p.K), k, v);
+            unsigned long long x[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = digits_of(__double2ll_rn(v[e] * scale));
+            store_digits(x, p.a + (size_t)n * p.Kp + k, plane);
+            const int most = __reduce_max_sync(0xffffffffu, digits_used(x[0] | x[1] | x[2] | x[3]));
+            if (lane == 0) atomicMax(&used[kb], most);
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < kblocks; i += SPLIT_THREADS) p.na[(size_t)i * (p.Np / ROWS_PER_CTA) + grp] = (uint8_t)max(used[i], MIN_A);
+}
+
+// ---------------------------------------------------------------------------------------------- product
+struct __align__(16) Ctl {
+    uint64_t full[A_SLOTS], full_b[2];     // a digit of W, a block's digits of R in place in both CTAs      (even CTA)
+    uint64_t empty[A_SLOTS], empty_b[2];   // consumed by the MMAs                      (each CTA, multicast commit)
+    uint64_t sums_full;           // four S_d complete                                  (each CTA, multicast commit)
+    uint64_t sums_empty;          // read by the epilogues of both CTAs                 (even CTA)
+    uint32_t tmem_base;
+    volatile int abort_flag;
+    volatile uint32_t counts[2];  // digits of W and R (8 bits each) of the even and the odd block
+};
+constexpr size_t SMEM_BYTES = 1024 + (size_t)A_SLOTS * A_BYTES + (size_t)B_SLOTS * B_BYTES + sizeof(Ctl);
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
+
+struct Params {
+    const uint8_t *na, *nb; const double *sa, *sb;
+    const float* W; long ldw; const float* colmul; const __nv_bfloat16* R;
+    float* out; long ldo;
+    int N, K, Np, Kp, rows, tiles, vec_o; int* status;
+};
+
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const void* tmap, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// D[tmem] (+)= A[smem] . B[smem], kind::i8: int8 operands, int32 accumulator
+__device__ __forceinline__ void mma_i8_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n}"
+        ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+}
+// Instruction descriptor of kind::i8: accumulator format at bits 4-5 (2 = s32), operand formats at bits 7-9 and 10-12
+// (1 = signed), both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
+constexpr uint32_t IDESC = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+
+__device__ __forceinline__ void tc_ld8(uint32_t taddr, int (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
+
+// Two passes over k per tile, since TMEM holds four S_d: first d = 4..7, kept in the epilogue's registers, then d = 0..3.
+// Per block of k the digits of R stay in place while those of W pass, each multiplied by all its partners and released.
+//   warp 0  TMA producer   warp 1  TMEM, MMA issue   warps 2-9  epilogue (32 rows x 64 columns each)
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+wrot_i8_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
+    extern __shared__ unsigned char smem_dyn[];
+    unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+    const uint32_t s0 = smem_u32(base);
+    const uint32_t sB = s0 + A_SLOTS * A_BYTES;
+    Ctl* ctl = reinterpret_cast<Ctl*>(base + A_SLOTS * A_BYTES + B_SLOTS * B_BYTES);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, kblocks = p.Kp / BK;
+    const uint32_t rank = cluster_ctarank();
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < A_SLOTS; ++s) { mbar_init(smem_u32(&ctl->full[s]), 1); mbar_init(smem_u32(&ctl->empty[s]), 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&ctl->full_b[s]), 1); mbar_init(smem_u32(&ctl->empty_b[s]), 1); }
+        mbar_init(smem_u32(&ctl->sums_full), 1);
+        mbar_init(smem_u32(&ctl->sums_empty), 2 * EPI_WARPS);
+        ctl->abort_flag = 0;
+        mbar_init_fence();
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+    }
+    if (warp == 1) tmem_alloc_pair(smem_u32(&ctl->tmem_base), TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    lrq_pdl_trigger();
+    lrq_pdl_wait();
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+
+    if (warp == 0) {
+        const bool lead = elect_one();
+        const uint32_t full0 = map_to_cta(smem_u32(&ctl->full[0]), 0);
+        int sa = 0, nb_before = 0;
+        uint32_t pha = 1, issued = 0, g = 0;                 // g counts blocks, over passes and tiles
+        bool ok = true;
+        for (int tile = pair; ok && tile < p.tiles; tile += pairs) {
+            const int rb = tile % p.rows, jb = tile / p.rows;
+            const int m0 = rb * BM + (int)rank * BM_CTA, n0 = jb * BN + (int)rank * (BN / 2);
+            auto counts = [&](int kb) -> uint32_t {
+                const uint4 v = __ldg(reinterpret_cast<const uint4*>(p.na + (size_t)kb * (p.Np / ROWS_PER_CTA) + rb * (BM / ROWS_PER_CTA)));
+                uint32_t m = __vmaxu4(__vmaxu4(v.x, v.y), __vmaxu4(v.z, v.w));
+                m = max(max(m & 0xffu, (m >> 8) & 0xffu), max((m >> 16) & 0xffu, m >> 24));
+                return m | ((uint32_t)__ldg(p.nb + (size_t)kb * kblocks + jb) << 8);
+            };
+            for (int pass = 0; ok && pass < 2; ++pass) {
+                uint32_t c = counts(0);
+                for (int kb = 0; ok && kb < kblocks; ++kb) {
+                    const uint32_t next = counts(kb + 1 < kblocks ? kb + 1 : 0);
+                    const int da = min((int)(c & 0xff), D), db = min((int)(c >> 8), D);
+                    const int nb = pass ? 4 : db, i0 = pass ? 0 : max(5 - db, 0), i1 = pass ? 4 : da;
+                    const uint32_t e = g & 1, full = map_to_cta(smem_u32(&ctl->full_b[e]), 0);
+                    ok = mbar_wait_warp(smem_u32(&ctl->empty_b[e]), ((g >> 1) & 1) ^ 1, &ctl->abort_flag, p.status, 51);
+                    if (ok && nb + nb_before > B_SLOTS)      // no room beside the block before
+                        ok = mbar_wait_warp(smem_u32(&ctl->empty_b[e ^ 1]), ((g - 1) >> 1) & 1, &ctl->abort_flag, p.status, 51);
+                    if (!ok) break;
+                    if (lead) {
+                        if (rank == 0) {
+                            ctl->counts[e] = (uint32_t)da | ((uint32_t)db << 8);
+                            mbar_arrive_expect_tx(smem_u32(&ctl->full_b[e]), 2u * nb * B_BYTES);
+                        }
+                        for (int t = 0; t < nb; ++t) tma_load_pair(sB + b_slot(e, t) * B_BYTES, &tmB, kb * BK, t * p.Kp + n0, full);
+                    }
+                    __syncwarp();
+                    ++issued; ++g;
+                    nb_before = nb;
+                    for (int t = i0; ok && t < i1; ++t) {
+                        ok = mbar_wait_warp(smem_u32(&ctl->empty[sa]), pha, &ctl->abort_flag, p.status, 55);
+                        if (!ok) break;
+                        if (lead) {
+                            if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[sa]), 2u * A_BYTES);
+                            tma_load_pair(s0 + sa * A_BYTES, &tmA, kb * BK, t * p.Np + m0, full0 + 8 * sa);
+                        }
+                        __syncwarp();
+                        ++issued;
+                        if (++sa == A_SLOTS) { sa = 0; pha ^= 1; }
+                    }
+                    c = next;
+                }
+            }
+        }
+        if (!ok && issued) {      // copies in flight land before the CTAs meet and end
+            const long long t0 = clock64();
+            while (clock64() - t0 < 2000000) __nanosleep(1000);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (rank == 0) {
+            const bool lead = elect_one();
+            const uint64_t a0 = umma_desc_sw128(s0, 16, 1024), b0 = umma_desc_sw128(sB, 16, 1024);
+            int sa = 0;
+            uint32_t pha = 0, round = 0, g = 0;
+            bool ok = true;
+            for (int tile = pair; ok && tile < p.tiles; tile += pairs) {
+                for (int pass = 0; ok && pass < 2; ++pass, ++round) {
+                    ok = mbar_wait_warp(smem_u32(&ctl->sums_empty), (round & 1) ^ 1, &ctl->abort_flag, p.status, 52);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const int d0 = pass ? 0 : 4;
+                    uint32_t begun = 0;                      // S_d that have their first term
+                    for (int kb = 0; ok && kb < kblocks; ++kb) {
+                        const uint32_t e = g & 1;
+                        ok = mbar_wait_warp(smem_u32(&ctl->full_b[e]), (g >> 1) & 1, &ctl->abort_flag, p.status, 53);
+                        if (!ok) break;
+                        const uint32_t c = ctl->counts[e];
+                        const int da = c & 0xff, db = c >> 8, nb = pass ? 4 : db;
+                        const int i0 = pass ? 0 : max(5 - db, 0), i1 = pass ? 4 : da;
+                        for (int i = i0; ok && i < i1; ++i) {
+                            ok = mbar_wait_warp(smem_u32(&ctl->full[sa]), pha, &ctl->abort_flag, p.status, 56);
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint64_t a = a0 + (uint64_t)(sa * (A_BYTES >> 4));
+                            const int j0 = max(d0 - i, 0), j1 = min(nb, d0 + 4 - i);
+                            if (lead) {
+                                for (int j = j0; j < j1; ++j) {
+                                    const uint64_t b = b0 + (uint64_t)(b_slot(e, j) * (B_BYTES >> 4));
+                                    const int d = i + j - d0;
+                                    const uint32_t acc = (begun >> d) & 1;
+                                    begun |= 1u << d;
+#pragma unroll
+                                    for (int k = 0; k < BK / 32; ++k) mma_i8_pair(tmem_base + d * BN, a + 2 * k, b + 2 * k, IDESC, k ? 1u : acc);
+                                }
+                            }
+                            if (lead) tc_commit_pair(smem_u32(&ctl->empty[sa]), 3);
+                            __syncwarp();
+                            if (++sa == A_SLOTS) { sa = 0; pha ^= 1; }
+                        }
+                        if (ok && lead) tc_commit_pair(smem_u32(&ctl->empty_b[e]), 3);
+                        ++g;
+                        __syncwarp();
+                    }
+                    if (ok && lead) tc_commit_pair(smem_u32(&ctl->sums_full), 3);
+                    __syncwarp();
+                }
+            }
+        }
+        __syncwarp();
+    } else {
+        const int quad = warp & 3, half = (warp - EPI_WARP0) >> 2;
+        const uint32_t t0 = tmem_base + ((uint32_t)(quad * 32) << 16) + half * 64;
+        uint32_t round = 0;
+        bool ok = true;
+        for (int tile = pair; ok && tile < p.tiles; tile += pairs) {
+            const int rb = tile % p.rows, jb = tile / p.rows;
+            const int m0 = rb * BM + (int)rank * BM_CTA + quad * 32, m = m0 + lane, j0 = jb * BN + half * 64;
+            const double sa = m < p.N ? __ldg(p.sa + m) : 0.0;
+            double sum[64];                                  // sum of S_d 2^(56 - 8 d)
+            unsigned long long again = 0;                    // columns too small for the digits taken
+#pragma unroll
+            for (int pass = 0; pass < 2; ++pass, ++round) {
+                ok = ok && mbar_wait_warp<100>(smem_u32(&ctl->sums_full), round & 1, &ctl->abort_flag, p.status, 54);
+                if (!ok) break;
+                tc_fence_after();
+#pragma unroll
+                for (int c = 0; c < 64; c += 8) {
+                    int q0[8], q1[8], q2[8], q3[8];
+                    tc_ld8(t0 + c, q0); tc_ld8(t0 + BN + c, q1); tc_ld8(t0 + 2 * BN + c, q2); tc_ld8(t0 + 3 * BN + c, q3);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const long long hi = ((long long)q0[e] << 8) + q1[e], lo = ((long long)q2[e] << 8) + q3[e];
+                        const double v = (double)((hi << 16) + lo);
+                        sum[c + e] = pass ? fma(v, 4294967296.0, sum[c + e]) : v;
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster_light(smem_u32(&ctl->sums_empty), 0);
+            }
+            if (!ok) break;
+            if (m < p.N) {
+                float* o = p.out + (size_t)m * p.ldo + j0;
+#pragma unroll
+                for (int c = 0; c < 64; c += 4) {
+                    float f[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const double s = sa * __ldg(p.sb + j0 + c + e);       // sb has Kp entries
+                        f[e] = s == 0.0 ? 0.f : (float)(sum[c + e] * s);
+                        if (s != 0.0 && !(fabs(sum[c + e]) >= 281474976710656.0 && s == s)) again |= 1ull << (c + e);    // 2^48
+                    }
+                    if (p.vec_o && j0 + c + 4 <= p.K) *reinterpret_cast<float4*>(o + c) = make_float4(f[0], f[1], f[2], f[3]);
+                    else {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (j0 + c + e < p.K) o[c + e] = f[e];
+                    }
+                }
+            }
+            // results below 2^-20 of 2^(ew + er) (one in 10^6), and what is not finite: the whole warp sums in fp64
+            __syncwarp();
+            for (uint32_t who = __ballot_sync(0xffffffffu, again != 0); who; who = __ballot_sync(0xffffffffu, again != 0)) {
+                const int src = __ffs(who) - 1;
+                const unsigned long long bits = __shfl_sync(0xffffffffu, again, src);
+                const int j = j0 + __ffsll((long long)bits) - 1, n = m0 + src;
+                if (lane == src) again &= again - 1;
+                if (j >= p.K) continue;
+                const float* w = p.W + (size_t)n * p.ldw;
+                double acc = 0.0;
+#pragma unroll 16
+                for (int k = lane; k < p.K; k += 32) {
+                    double x = (double)__ldg(w + k);
+                    if (p.colmul) x *= (double)__ldg(p.colmul + k);
+                    acc = fma(x, (double)__bfloat162float(p.R[(size_t)k * p.K + j]), acc);
+                }
+#pragma unroll
+                for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (lane == 0) p.out[(size_t)n * p.ldo + j] = (float)acc;
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, TMEM_COLS);
+    }
+}
+
+struct Layout { int Np, Kp; size_t a, b, na, nb, sa, sb, total; };
+Layout layout_of(int N, int K) {
+    Layout L;
+    L.Np = (int)lrq_round_up((size_t)N, BM);
+    L.Kp = (int)lrq_round_up((size_t)K, BK);
+    const size_t kb = (size_t)L.Kp / BK;
+    size_t at = 0;
+    auto take = [&](size_t bytes) { const size_t o = at; at = lrq_round_up(at + bytes, 256); return o; };
+    L.a = take((size_t)D * L.Np * L.Kp);
+    L.b = take((size_t)D * L.Kp * L.Kp);
+    L.na = take(kb * (L.Np / ROWS_PER_CTA));
+    L.nb = take(kb * kb);
+    L.sa = take((size_t)L.Np * sizeof(double));
+    L.sb = take((size_t)L.Kp * sizeof(double));
+    L.total = at;
+    return L;
+}
+
+lrq_status max_pairs(int dev, int sms, int* out) {
+    static std::mutex mu;
+    static int max_pairs_of[LRQ_MAX_DEVICES] = {};
+    std::lock_guard<std::mutex> lock(mu);
+    if (!max_pairs_of[dev]) {
+        LRQ_CUDA_TRY(cudaFuncSetAttribute(wrot_i8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(sms & ~1); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = SMEM_BYTES;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int clusters = 0;
+        LRQ_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, wrot_i8_kernel, &cfg));
+        if (clusters < 1) return LRQ_ERR_CUDA;
+        max_pairs_of[dev] = clusters < sms / 2 ? clusters : sms / 2;
+    }
+    *out = max_pairs_of[dev];
+    return LRQ_OK;
+}
+
+}  // namespace
+
+size_t lrq_wrot_i8_workspace(int N, int K) {
+    if (K > K_MAX || (long)D * lrq_round_up((size_t)N, BM) > 2147483647l) return 0;
+    // below this line the launches and the two passes' drains weigh more than the fp64 product (64 x 64 tiles, one wave):
+    // 512 x 512: 40 us here, 37 there; 1024 x 512: 40, 37; 2048 x 512: 42, 51; 512 x 1024: 56, 66; 64 x 1024: 54, 66
+    if (K < 1024 && (double)N * K * K < 536870912.0) return 0;
+    return layout_of(N, K).total;
+}
+
+lrq_status lrq_launch_rotate_weights_i8(const float* W, int N, int K, long ldw, const float* colmul, const void* R, float* out, long ldo,
+                                        void* workspace, cudaStream_t st) {
+    int dev = 0, sms = 0, pairs = 0;
+    if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
+    const lrq_status rs = max_pairs(dev, sms, &pairs);
+    if (rs != LRQ_OK) return rs;
+    const Layout L = layout_of(N, K);
+    unsigned char* ws = static_cast<unsigned char*>(workspace);
+    const int kblocks = L.Kp / BK;
+    Split s = {};
+    s.W = W; s.ldw = ldw; s.colmul = colmul; s.R = static_cast<const __nv_bfloat16*>(R);
+    s.N = N; s.K = K; s.Np = L.Np; s.Kp = L.Kp;
+    const bool vec = lrq_aligned(W, 16) && ldw % 4 == 0 && lrq_aligned(R, 16) && K % 8 == 0;
+    s.r_ctas = kblocks * kblocks;
+    s.a = reinterpret_cast<int8_t*>(ws + L.a); s.b = reinterpret_cast<int8_t*>(ws + L.b);
+    s.na = ws + L.na; s.nb = ws + L.nb;
+    s.sa = reinterpret_cast<double*>(ws + L.sa); s.sb = reinterpret_cast<double*>(ws + L.sb);
+    LRQ_CUDA_TRY(lrq_launch_pdl(vec ? wrot_split_kernel<true> : wrot_split_kernel<false>, dim3(s.r_ctas + L.Np / ROWS_PER_CTA), dim3(SPLIT_THREADS), 0, st, s));
+    Params p = {};
+    p.na = s.na; p.nb = s.nb; p.sa = s.sa; p.sb = s.sb; p.W = W; p.ldw = ldw; p.colmul = colmul; p.R = s.R; p.out = out; p.ldo = ldo;
+    p.N = N; p.K = K; p.Np = L.Np; p.Kp = L.Kp; p.rows = L.Np / BM; p.tiles = p.rows * kblocks;
+    p.vec_o = lrq_aligned(out, 16) && ldo % 4 == 0; p.status = lrq_status_word();
+    CUtensorMap tmA, tmB;
+    if (!lrq_tma::make_map_2d(&tmA, s.a, 1, (uint64_t)D * L.Np, (uint64_t)L.Kp, (uint64_t)L.Kp, BK, BM_CTA, true) ||
+        !lrq_tma::make_map_2d(&tmB, s.b, 1, (uint64_t)D * L.Kp, (uint64_t)L.Kp, (uint64_t)L.Kp, BK, BN / 2, true))
+        return LRQ_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(2 * (p.tiles < pairs ? p.tiles : pairs)); cfg.blockDim = dim3(NUM_THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 2;
+    LRQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, wrot_i8_kernel, p, tmA, tmB));
+    return LRQ_OK;
+}

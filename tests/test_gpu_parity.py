@@ -358,6 +358,41 @@ def test_rotate_weights(P, orc, N, K, rot, B, smooth):
         assert torch.equal(Wd, out)
 
 
+@pytest.mark.parametrize("N,K,smooth", [(2055, 520, False), (257, 1030, True), (2049, 640, True), (130, 1536, False), (3, 2048, False)])
+def test_rotate_weights_dense_by_digits(P, N, K, smooth):
+    # The dense product from int8 digits against the fp64 product: ragged tiles in N and K, unaligned rows of R, a row and a
+    # column of zeros, a row and a column of a wide range (all eight digits), results so far below their row's and
+    # column's largest magnitudes that the digits do not reach (summed again), infinities and NaN.
+    g = torch.Generator(device="cuda").manual_seed(N + K)
+    W = torch.randn((N, K), generator=g, device="cuda")
+    R = (torch.randn((K, K), generator=g, device="cuda") / K ** 0.5)
+    c = torch.rand((K,), generator=g, device="cuda") + 0.3 if smooth else None
+    W[0] = 0
+    R[:, 5] = 0
+    W[1] *= torch.exp2(torch.randint(-40, 1, (K,), generator=g, device="cuda").float())
+    R[:, 7] *= torch.exp2(torch.randint(-40, 1, (K,), generator=g, device="cuda").float())
+    W[2, 11] = 2.0 ** 40                                       # hidden from columns 0..15 by zeros of R
+    R[11, :16] = 0
+    if N > 3:
+        W[3, 2] = float("inf")
+        W[4, 3] = float("nan")
+    R = R.bfloat16()
+    assert P.load_library().lrq_rotate_weights_workspace_bytes(N, K, P.ROT_DENSE) > 0
+    out = P.lrq_rotate_weights(W, P.ROT_DENSE, 0, R, c)
+    Wc = W.double() * (1.0 if c is None else c.double())
+    ref = Wc @ R.double()
+    finite = torch.isfinite(Wc).all(dim=1)
+    got, want = out[finite].double(), ref[finite]
+    # half an ulp of the rounding, what the digits leave out (2^-28), and what an fp64 sum of K terms may be off itself
+    ulp = torch.exp2(torch.floor(torch.log2(want.abs().clamp(min=1e-30))) - 23)
+    tol = 0.5 * ulp + 2.0 ** -28 * want.abs() + K * 2.0 ** -53 * (Wc[finite].abs() @ R.double().abs())
+    assert bool(((got - want).abs() <= tol).all())
+    assert bool((out[0] == 0).all()) and bool((out[finite][:, 5] == 0).all())
+    if N > 3:
+        assert torch.equal(torch.nan_to_num(out[~finite], nan=1.5), torch.nan_to_num(ref[~finite].float(), nan=1.5))
+    assert P.lrq_device_status() == 0
+
+
 def test_rotated_and_smoothed_layer_reproduces_the_plain_product(P):
     # End to end on the GPU: weights rotated by lrq_rotate_weights with colmul = 1/p, activations smoothed by p and
     # rotated inside lrq_qlinear.  With 8-bit activations and 4-bit TLQ the result is a quantized estimate of X W^T;

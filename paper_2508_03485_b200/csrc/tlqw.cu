@@ -9,16 +9,20 @@
 // one clipping factor of the caller's grid, all lanes walking over the same elements.  Every decision (codes,
 // chosen factor) is the one fp64 arithmetic with explicitly rounded operations gives.
 //
-// What bounds it is the number of instructions per element and factor:
-//   * every factor's error is first summed in fp32, in any order.  That sum's relative error
-//     is bounded (a few hundred roundings), so a factor further than twice the bound from the smallest cannot win; only
-//     when more than one factor is that close is the sum above taken in fp64, for about one row in fifty;
-//   * the code is rint(l/s) - z in fp32, from log2f; an element within the fp32 error of a rounding boundary
-//     (|x - rint x| > 1/2 - E, E worked out from the candidate's range) takes the fp64 expression, a division, instead;
-//   * levels have 8-bit significands: fp32 numbers, and the upper word of the double is the level;
-//   * a side's elements are compacted into shared memory kChunk source elements at a time and read as broadcasts.
-// 4608 x 1152, 4 bits, 31 factors a side: 545 us with the fp64 expression for every element and factor, 157 now;
-// 4608 x 1536, 3 bits, groups of 128: 1086 and 315.
+// What bounds it is the number of instructions.  Groups of more than 128 elements are not visited for every factor:
+//   * a side's magnitudes are laid out in shared memory in ascending bins (of their bit patterns, so by a fraction of an
+//     octave), with fp64 sums over every four of them.  A factor's codes change at nq magnitudes, so its error is a sum of
+//     nq + 1 terms in the count and the sum of the elements above each, which takes a look at one bin per threshold;
+//   * that error is off by fp64 roundings whose size is bounded, so a factor further than the bound from the smallest cannot
+//     win; only when more than one factor is that close is the sum above taken, element by element.
+// For shorter groups the bins cost as much as they save, and every factor's error is first summed in fp32, in any order: its
+// relative error is bounded too (a few hundred roundings), and the rest is the same.  Common to both:
+//   * a code is rint(l/s) - z in fp32; an element within the fp32 error of a rounding boundary (|x - rint x| > 1/2 - E, E
+//     worked out from the candidate's range) takes the fp64 expression, a division, instead;
+//   * levels have 8-bit significands: fp32 numbers, and the upper word of the double is the level.
+// 31 factors a side, 4 bits: 4608 x 1152 545 us with the fp64 expression for every element and factor, 169 with fp32 sums over
+// every element, 82 with bins; 2048 x 6144 490 and 125; 512 x 12288 685 and 96.  4608 x 1536 in groups of 128: 315 with fp32
+// sums, 398 with bins; of 256 (4608 x 2048): 328 and 315.
 #include "lrq_internal.cuh"
 #include <climits>
 #include <type_traits>
@@ -26,8 +30,7 @@
 namespace {
 
 constexpr int kMaxGrid = 64;
-constexpr int kThreads = 64;
-constexpr int kChunk = 256;                        // source elements compacted at a time
+constexpr int kChunk = 256;                        // source elements compacted at a time for the element-by-element sum
 struct ClipGrid { double a[kMaxGrid]; double b[kMaxGrid]; int na, nb; };
 
 // (out of line, as the next one: both are rarely reached and long, and this kernel has to stay in the instruction cache)
@@ -59,14 +62,21 @@ __device__ __forceinline__ int level_word(double e, int I) {
     return __double2hiint(level_value(e, I));
 }
 
-// The same from fp32: x = l32 * inv + negz is within E of the exact l/s - z, with E = 2^-20 (max|l| / s + nq + 2): log2f is
-// within an ulp of l (2^-23 of |l/s|), the reciprocal of the rounded step within 2^-22, the fused multiply-add rounds once
-// (2^-24), all taken more than twice over.  `thr` = 1/2 - E; a candidate whose E is too large (E >= 1/2) always takes the fp64
+// log2 of a normal number to 2^-22 of max(1, |result|); minus infinity for a subnormal one, which fast_round does not call exact
+__device__ __forceinline__ float log2_approx(float a) {
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+
+// The same from fp32: x = l32 * inv + negz is within E of the exact l/s - z, with E = 2^-20 (max(1, |l|) / s + nq + 2): the
+// logarithm is within 2^-22 of max(1, |l|), the reciprocal of the rounded step within 2^-22, the fused multiply-add rounds once
+// (2^-24), all taken twice over.  `thr` = 1/2 - E; a candidate whose E is too large (E >= 1/2) always takes the fp64
 // expression, and so does one whose z is not an fp32 integer, since then |l/s| is above 2^23.  The side's smallest element
 // has the code rint(smin / s) - z = 0 and no element a lower one, so only the upper clamp of Eq. 5 is left to do.
 constexpr float kMagic = 12582912.f;                // 1.5 * 2^23: adding it rounds to an integer, ties to even
-struct FastCode { float inv, negz, thr, top; };
-__device__ __forceinline__ FastCode fast_code(double s, double z, float lmax, int nq) {     // lmax >= |l| of every element
+struct __align__(16) FastCode { float inv, negz, thr, top; };
+__device__ __forceinline__ FastCode fast_code(double s, double z, float lmax, int nq) {     // lmax >= max(1, |l|) of every element
     FastCode f;
     f.inv = 1.0f / (float)s;
     f.negz = (float)-z;
@@ -84,60 +94,178 @@ __device__ __forceinline__ float fast_round(float l32, const FastCode& f, bool& 
 
 struct Side { double s, z, factor; };
 
-__global__ void __launch_bounds__(kThreads, 16)
-tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, int I, ClipGrid grid, int pack3,
+// Bins of a side: bit patterns of its magnitudes above the smallest's, shifted so that the largest's falls below NB.
+struct Bins { uint32_t base; int shift; };
+template <int NB>
+__device__ __forceinline__ Bins make_bins(float vmin, float vmax) {
+    const uint32_t range = __float_as_uint(vmax) - __float_as_uint(vmin);
+    const int top = 32 - __clz(range);
+    return {__float_as_uint(vmin), max(0, top - (31 - __clz(NB)))};
+}
+__device__ __forceinline__ int bin_of(float a, const Bins& b) { return (int)((__float_as_uint(a) - b.base) >> b.shift); }
+
+// Barrier over the warps of one side.
+template <int WPS>
+__device__ __forceinline__ void side_sync(int sd) {
+    if (WPS == 1) __syncwarp();
+    else if (sd) asm volatile("bar.sync 2, %0;" ::"n"(32 * WPS) : "memory");
+    else asm volatile("bar.sync 1, %0;" ::"n"(32 * WPS) : "memory");
+}
+
+constexpr size_t binned_smem(int NB, int G) { return (size_t)2 * NB * 4 + (size_t)(G + 8) * 4 + (size_t)(G / 4 + 8) * 8; }
+
+// WPS warps a side and NB bins (none: fp32 sums): one warp up to 256 elements, most of their work is per factor, not per
+// element; two with 512 bins up to 2048 (4608 x 1152: 82 us; with one warp 106, with four 119); four with 1024 bins above,
+// where a row's lists leave room for fewer CTAs (2048 x 6144: 125 us, with two warps 177).  `binned` is 0 when the lists do not fit in shared memory.
+template <int WPS, int NB>
+__global__ void __launch_bounds__(64 * WPS, 16 / WPS)
+tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, int I, ClipGrid grid, int pack3, int binned,
                     uint8_t* __restrict__ codes, float* __restrict__ levels, double* __restrict__ meta,
                     float* __restrict__ wsum) {
+    constexpr int kThreads = 64 * WPS, kWarps = 2 * WPS;
+    extern __shared__ __align__(16) unsigned char dyn[];       // both sides' bins, sums over fours, magnitudes
+    __shared__ double epart[2][WPS][32], bpart[2][WPS][32];
+    __shared__ int warp_count[2][WPS];
     __shared__ int cand_lev[2][9][32];             // level table of each lane's candidate, per side (upper word of the double)
-    __shared__ float cand_f32[2][9][32];           // the same in fp32
+    __shared__ float cand_f32[NB == 0 ? 2 : 1][NB == 0 ? 9 : 1][32];     // the same in fp32
     // a side's elements of one chunk, in increasing k: magnitude and its log2
     __shared__ __align__(16) float mag[2][kChunk];
     __shared__ __align__(16) float lg[2][kChunk];
     __shared__ FastCode best_fc[2];
-    __shared__ float ext[2][2][2];                 // [warp][side][max, min] of |w|
+    __shared__ unsigned ext[2][2][2];              // [parity of the group][side][max, ~min] of |w|, as bit patterns
     __shared__ int ext_cnt[2][2];
     __shared__ Side best[2];
     __shared__ double T[16];
-    __shared__ double red[2];
+    __shared__ double red[kWarps];
 
     const int n = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = 1 << (bits - 1), nlev = 1 << bits, ngrp = K / G;
-    double row_sum = 0.0;                          // meaningful in thread 0
+    double row_sum = 0.0;                          // of this thread's codes
+    if (tid < 8) reinterpret_cast<unsigned*>(ext)[tid] = 0;
+    if (tid < 4) reinterpret_cast<int*>(ext_cnt)[tid] = 0;
+    __syncthreads();
     lrq_pdl_trigger();
     lrq_pdl_wait();                                // the weights may be the previous kernel's output
 
     for (int g = 0; g < ngrp; ++g) {
         const float* w = W + (size_t)n * K + (size_t)g * G;
+        int* bins = reinterpret_cast<int*>(dyn);
+        if (NB > 0 && binned)
+            for (int i = tid; i < 2 * NB / 4; i += kThreads) reinterpret_cast<int4*>(bins)[i] = make_int4(0, 0, 0, 0);
         // ---- extremes of |w| per side (order does not matter for max / min, and log2 is monotone on fp32 numbers)
-        float amax[2] = {0.f, 0.f}, amin[2] = {INFINITY, INFINITY};
-        int cnt[2] = {0, 0};
-        for (int k = tid; k < G; k += kThreads) {
-            const float v = w[k];
-            if (v != 0.f) {
-                const int sd = v < 0.f;
-                const float av = fabsf(v);
-                if (sd) { amax[1] = fmaxf(amax[1], av); amin[1] = fminf(amin[1], av); cnt[1]++; }
-                else { amax[0] = fmaxf(amax[0], av); amin[0] = fminf(amin[0], av); cnt[0]++; }
+        auto pair_of = [&](int j) { return *reinterpret_cast<const float2*>(w + 2 * j); };
+        {
+            float amax[2] = {0.f, 0.f}, amin[2] = {INFINITY, INFINITY};
+            int cnt[2] = {0, 0};
+            for (int j = tid; j < G / 2; j += kThreads) {
+                const float2 v2 = pair_of(j);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float v = e ? v2.y : v2.x, av = fabsf(v);
+                    const bool neg = v < 0.f, pos = !neg && v != 0.f;
+                    amax[0] = fmaxf(amax[0], neg ? 0.f : av); amax[1] = fmaxf(amax[1], neg ? av : 0.f);
+                    amin[0] = fminf(amin[0], pos ? av : INFINITY); amin[1] = fminf(amin[1], neg ? av : INFINITY);
+                    cnt[0] += pos; cnt[1] += neg;
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                // magnitudes: the bit patterns are ordered as the numbers
+                const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(amax[h])), mn = __reduce_min_sync(0xffffffffu, __float_as_uint(amin[h]));
+                const int c = __reduce_add_sync(0xffffffffu, cnt[h]);
+                if (lane == 0) { atomicMax(&ext[g & 1][h][0], mx); atomicMax(&ext[g & 1][h][1], ~mn); atomicAdd(&ext_cnt[g & 1][h], c); }
             }
         }
-#pragma unroll
-        for (int sd = 0; sd < 2; ++sd) {
-            // magnitudes: the bit patterns are ordered as the numbers
-            const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(amax[sd])), mn = __reduce_min_sync(0xffffffffu, __float_as_uint(amin[sd]));
-            const int c = __reduce_add_sync(0xffffffffu, cnt[sd]);
-            if (lane == 0) { ext[warp][sd][0] = __uint_as_float(mx); ext[warp][sd][1] = __uint_as_float(mn); ext_cnt[warp][sd] = c; }
-        }
         __syncthreads();
-        // ---- search of the clipping factor: warp `sd` owns side sd, lane c the c-th factor of that side's grid
-        const int sd = warp;
+        const float vmaxs[2] = {__uint_as_float(ext[g & 1][0][0]), __uint_as_float(ext[g & 1][1][0])};
+        const float vmins[2] = {__uint_as_float(~ext[g & 1][0][1]), __uint_as_float(~ext[g & 1][1][1])};
+        const int cnts[2] = {ext_cnt[g & 1][0], ext_cnt[g & 1][1]};
+        if (tid < 4) reinterpret_cast<unsigned*>(ext[(g & 1) ^ 1])[tid] = 0;      // the next group's: last read before that barrier
+        if (tid < 2) ext_cnt[(g & 1) ^ 1][tid] = 0;
+        const int sd = warp / WPS, sw = warp % WPS;          // the warp's side and its place there; a lane is a factor
         const int nq = sd ? half : half - 1;       // highest code of the side = denominator of Eq. 6
-        const float vmax = fmaxf(ext[0][sd][0], ext[1][sd][0]), vmin = fminf(ext[0][sd][1], ext[1][sd][1]);
-        const int scnt = ext_cnt[0][sd] + ext_cnt[1][sd];
+        const float vmax = vmaxs[sd], vmin = vmins[sd];
+        const int scnt = cnts[sd];
+        int* side_bins = bins + sd * NB;
+        double* side_sums = reinterpret_cast<double*>(dyn + 2 * NB * 4) + (sd ? (cnts[0] + 3) / 4 + 1 : 0);
+        float* all_mags = reinterpret_cast<float*>(dyn + 2 * NB * 4 + (size_t)(G / 4 + 8) * 8);
+        float* side_mags = all_mags + (sd ? (cnts[0] + 3) / 4 * 4 : 0);
+        [[maybe_unused]] const Bins bn[2] = {make_bins<NB>(vmins[0], vmaxs[0]), make_bins<NB>(vmins[1], vmaxs[1])};
+        double total = 0.0;
+        if constexpr (NB > 0) if (binned) {
+            // an element's bin, of both sides' 2 NB
+            auto slot = [&](float v) {
+                const bool neg = v < 0.f;
+                return (neg ? NB : 0) + (int)(((__float_as_uint(v) & 0x7fffffffu) - (neg ? bn[1].base : bn[0].base)) >> (neg ? bn[1].shift : bn[0].shift));
+            };
+            for (int j = tid; j < G / 2; j += kThreads) {
+                const float2 v = pair_of(j);
+                if (fabsf(v.x) > 0.f) atomicAdd(&bins[slot(v.x)], 1);
+                if (fabsf(v.y) > 0.f) atomicAdd(&bins[slot(v.y)], 1);
+            }
+            __syncthreads();
+            // counts to starts, a run of bins per thread
+            constexpr int RUN = NB / (32 * WPS);
+            static_assert(RUN % 4 == 0, "");
+            int4* run = reinterpret_cast<int4*>(side_bins + (sw * 32 + lane) * RUN);
+            int c = 0;
+#pragma unroll
+            for (int i = 0; i < RUN / 4; ++i) { const int4 v = run[i]; c += v.x + v.y + v.z + v.w; }
+            int incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+            if (WPS > 1) {
+                if (lane == 31) warp_count[sd][sw] = incl;
+                side_sync<WPS>(sd);
+            }
+            int at = incl - c;
+            for (int i = 0; i < sw; ++i) at += warp_count[sd][i];
+#pragma unroll
+            for (int i = 0; i < RUN / 4; ++i) {
+                const int4 v = run[i];
+                run[i] = make_int4(at, at + v.x, at + v.x + v.y, at + v.x + v.y + v.z);
+                at += v.x + v.y + v.z + v.w;
+            }
+            __syncthreads();
+            const int neg_at = (cnts[0] + 3) / 4 * 4;
+            if (sw == 0 && lane < 3 && scnt + lane < (scnt + 3) / 4 * 4) side_mags[scnt + lane] = 0.f;       // the last four
+            for (int j = tid; j < G / 2; j += kThreads) {    // afterwards a bin's entry is its end, the next one's start
+                const float2 v = pair_of(j);
+                if (fabsf(v.x) > 0.f) all_mags[atomicAdd(&bins[slot(v.x)], 1) + (v.x < 0.f ? neg_at : 0)] = fabsf(v.x);
+                if (fabsf(v.y) > 0.f) all_mags[atomicAdd(&bins[slot(v.y)], 1) + (v.y < 0.f ? neg_at : 0)] = fabsf(v.y);
+            }
+            __syncthreads();
+            if (sw == 0) {                                   // side_sums[i] = sum of the first 4 i magnitudes
+                const int fours = (scnt + 3) / 4, each = (fours + 31) / 32;
+                auto four = [&](int i) {
+                    const float4 v = *reinterpret_cast<const float4*>(side_mags + 4 * i);
+                    return ((double)v.x + (double)v.y) + ((double)v.z + (double)v.w);
+                };
+                const int i0 = min(lane * each, fours), i1 = min(i0 + each, fours);
+                double sum = 0.0;
+                for (int i = i0; i < i1; ++i) sum += four(i);
+                double run_sum = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const double v = __hiloint2double(__shfl_up_sync(0xffffffffu, __double2hiint(run_sum), o), __shfl_up_sync(0xffffffffu, __double2loint(run_sum), o));
+                    if (lane >= o) run_sum += v;
+                }
+                double at_sum = run_sum - sum;               // any consistent value does: within the roundings allowed for
+                for (int i = i0; i < i1; ++i) { side_sums[i] = at_sum; at_sum += four(i); }
+                if (i0 < i1 && i1 == fours) side_sums[fours] = at_sum;
+            }
+            side_sync<WPS>(sd);
+            total = scnt ? side_sums[(scnt + 3) / 4] : 0.0;
+        }
+        // ---- search of the clipping factor: lane c takes the c-th factor of the side's grid
         // both logarithms in one evaluation: even lanes take the maximum's, odd lanes the minimum's
         const double lx = log2((double)((lane & 1) ? vmin : vmax));
         const double smax = scnt ? shfl_double(lx, 0) : -INFINITY, smin = scnt ? shfl_double(lx, 1) : INFINITY;
-        const float l_abs = scnt ? fmaxf(fabsf((float)smin), fabsf((float)smax)) * 1.000001f : 0.f;
+        const float l_abs = scnt ? fmaxf(fmaxf(fabsf((float)smin), fabsf((float)smax)), 1.f) * 1.000001f : 1.f;
         const int ng = sd ? grid.nb : grid.na;
+        // the thresholds below are relative to 2^-20: not for magnitudes all alike, nor for subnormal ones; a NaN is
+        // counted and not binned
+        const bool quick = NB > 0 && binned && ng <= 32 && side_bins[NB ? NB - 1 : 0] == scnt && vmin > 1e-37f && vmax < 1e37f && vmax > vmin * 1.001f;
         double best_err = INFINITY, best_s = 1.0, best_z = 0.0, best_f = 1.0;
         bool found = false;
         for (int c0 = 0; c0 < ng; c0 += 32) {
@@ -153,17 +281,87 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                     ok = true;
                 }
             }
+            if constexpr (NB > 0) if (quick) {
+                // error less the sum of the squares: sum over codes of n_q L_q^2 - 2 L_q S_q, by parts over the thresholds
+                const int per = (nq + WPS - 1) / WPS, q0 = sw * per + 1, q1 = min(q0 + per, nq + 1);
+                double e = 0.0, low = 0.0;
+                auto level = [&](int q) { return ok ? __hiloint2double(level_word(__dmul_rn(s, __dadd_rn((double)q, z)), I), 0) : 0.0; };
+                if (q0 < q1 || sw == 0) low = level(q0 - 1);
+                if (sw == 0) e = low * fma((double)scnt, low, -2.0 * total);
+#pragma unroll 1
+                for (int q = q0; q < q1; ++q) {
+                    const double L = level(q);
+                    // magnitudes of code q and above start at 2^(s (z + q - 1/2)), here to 2^-21 of it
+                    const double edge = s * (z + ((double)q - 0.5)), fl = floor(edge);
+                    const int fi = (int)fmin(fmax(fl, -126.0), 127.0);
+                    const float a0 = exp2f((float)(edge - fl)) * __int_as_float((fi + 127) << 23);
+                    const float lo = a0 * 0.99999905f, hi = a0 * 1.00000095f;
+                    int cnt = 0;
+                    double sum = 0.0;
+                    if (ok && lo <= vmax && edge < 127.0) {
+                        const int kl = lo <= vmin ? 0 : bin_of(lo, bn[sd]), kh = hi <= vmin ? 0 : min(bin_of(hi, bn[sd]), NB - 1);
+                        // fours that touch the edge's bins: what lies before them is smaller, what lies behind is larger
+                        const int fours = (side_bins[kh] + 3) >> 2;
+                        int maybe = 0;
+                        for (int i = kl ? side_bins[kl - 1] >> 2 : 0; i < fours; ++i) {
+                            const float4 v = *reinterpret_cast<const float4*>(side_mags + 4 * i);
+                            const float a[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                maybe += a[h] >= lo;
+                                if (a[h] >= hi) { ++cnt; sum += (double)a[h]; }
+                            }
+                        }
+                        if (maybe != cnt)
+                            for (int j = kl ? side_bins[kl - 1] & ~3 : 0; j < min(4 * fours, scnt); ++j) {
+                                const float a = side_mags[j];
+                                if (a >= lo && a < hi && side_code(a, s, z, nq) >= q) { ++cnt; sum += (double)a; }
+                            }
+                        cnt += scnt - min(4 * fours, scnt);
+                        sum += total - side_sums[fours];
+                    }
+                    e += (L - low) * fma((double)cnt, L + low, -2.0 * sum);
+                    low = L;
+                }
+                // roundings of the sums here and of the sum that defines the error: n of each, half an ulp, twice over
+                epart[sd][sw][lane] = e;
+                bpart[sd][sw][lane] = ((double)(scnt + 64)) * 4.5e-16 * ((double)scnt * ((double)vmax * (double)vmax + low * low) + 2.0 * low * total);
+                side_sync<WPS>(sd);
+                if (sw) continue;
+#pragma unroll
+                for (int i = 1; i < WPS; ++i) e += epart[sd][i][lane];
+                double b = bpart[sd][0][lane];
+#pragma unroll
+                for (int i = 1; i < WPS; ++i) b = fmax(b, bpart[sd][i][lane]);
+                // twice the largest bound, and the smallest error from the lanes that share its upper word
+                const float bound = __uint_as_float(__reduce_max_sync(0xffffffffu, ok ? __float_as_uint((float)b * 2.001f) : 0u));
+                const int key = ok ? lrq_ordered_int(__int_as_float(__double2hiint(e))) : INT_MAX, kmin = __reduce_min_sync(0xffffffffu, key);
+                double emin = INFINITY;
+                for (unsigned m = __ballot_sync(0xffffffffu, key == kmin); m; m &= m - 1) emin = fmin(emin, shfl_double(e, __ffs(m) - 1));
+                const unsigned close = __ballot_sync(0xffffffffu, ok && !(e > emin + (double)bound));
+                const bool fine = bound < 1e30f;
+                if (fine && (close & (close - 1)) == 0) {
+                    // one factor is left (or none is usable): the smallest error, whatever the rounding
+                    if (close) {
+                        const int src = __ffs(close) - 1;
+                        best_s = shfl_double(s, src); best_z = shfl_double(z, src); best_f = shfl_double(fac, src);
+                        found = true;
+                    }
+                    continue;
+                }
+            }
+            if (sw) continue;
             __syncwarp();
             for (int q = 0; q <= nq; ++q) {
                 const int hi = ok ? level_word(__dmul_rn(s, __dadd_rn((double)q, z)), I) : 0;
                 cand_lev[sd][q][lane] = hi;
-                cand_f32[sd][q][lane] = (float)__hiloint2double(hi, 0);
+                if constexpr (NB == 0) cand_f32[sd][q][lane] = (float)__hiloint2double(hi, 0);
             }
             FastCode fc = fast_code(s, z, l_abs, nq);
             if (!ok) { fc.inv = 0.f; fc.negz = 0.f; fc.thr = 1.f; }                 // scored, but never looked at
             const uint32_t magic_off = __float_as_uint(kMagic) << 7;
             const uint32_t lev0 = (uint32_t)__cvta_generic_to_shared(&cand_lev[sd][0][lane]) - magic_off;
-            const uint32_t f32_0 = (uint32_t)__cvta_generic_to_shared(&cand_f32[sd][0][lane]) - magic_off;
+            [[maybe_unused]] const uint32_t f32_0 = (uint32_t)__cvta_generic_to_shared(&cand_f32[NB == 0 ? sd : 0][0][lane]) - magic_off;
             __syncwarp();
             // the side's elements among w[k0 .. k0 + kChunk), in increasing k, into the warp's list; returns how many
             auto fill = [&](int k0) {
@@ -179,7 +377,7 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                     if (mine) {
                         const int at = n_el + __popc(m & ((1u << lane) - 1u));
                         mag[sd][at] = fabsf(v);
-                        lg[sd][at] = log2f(fabsf(v));
+                        lg[sd][at] = log2f(fabsf(v));          // finite for every element, subnormal ones too: `group` looks no further
                     }
                     n_el += __popc(m);
                 }
@@ -191,78 +389,76 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                 const float r = fast_round(lg[sd][j], fc, exact);
                 return exact ? r : kMagic + (float)side_code(mag[sd][j], s, z, nq);
             };
-            // ---- every factor's error in fp32 (terms within 3 u of the exact ones, eight partial sums of at most
-            // scnt / 8 + chunk remainders terms), which leaves the factors within twice its bound of the smallest
-            float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            float rest = 0.f;
-            auto term = [&](int j, float r) {
-                float L;
-                asm("ld.shared.f32 %0, [%1];" : "=f"(L) : "r"(f32_0 + (__float_as_uint(r) << 7)));
-                const float d = mag[sd][j] - L;
-                rest = fmaf(d, d, rest);
-            };
-            auto group = [&](int j, auto U_) {
-                constexpr int U = decltype(U_)::value;
-                float r[U], off = 0.f;               // the distances from an integer are looked at together
-#pragma unroll
-                for (int u = 0; u < U; u += 4) {
-                    const float4 l4 = *reinterpret_cast<const float4*>(&lg[sd][j + u]);
-                    const float l[4] = {l4.x, l4.y, l4.z, l4.w};
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        const float x = fmaf(l[h], fc.inv, fc.negz);
-                        r[u + h] = x + kMagic;
-                        off = fmaxf(off, fabsf(x - (r[u + h] - kMagic)));
-                    }
-                }
-                if (off <= fc.thr) {
+            if constexpr (NB == 0) {
+                // ---- every factor's error in fp32 (terms within 3 u of the exact ones, eight partial sums of at most
+                // scnt / 8 + chunk remainders terms), which leaves the factors within twice its bound of the smallest
+                float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                float rest = 0.f;
+                auto term = [&](int j, float r) {
+                    float L;
+                    asm("ld.shared.f32 %0, [%1];" : "=f"(L) : "r"(f32_0 + (__float_as_uint(r) << 7)));
+                    const float d = mag[sd][j] - L;
+                    rest = fmaf(d, d, rest);
+                };
+                auto group = [&](int j, auto U_) {
+                    constexpr int U = decltype(U_)::value;
+                    float r[U], off = 0.f;               // the distances from an integer are looked at together
 #pragma unroll
                     for (int u = 0; u < U; u += 4) {
-                        const float4 a4 = *reinterpret_cast<const float4*>(&mag[sd][j + u]);
-                        const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+                        const float4 l4 = *reinterpret_cast<const float4*>(&lg[sd][j + u]);
+                        const float l[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
                         for (int h = 0; h < 4; ++h) {
-                            float L;
-                            asm("ld.shared.f32 %0, [%1];" : "=f"(L) : "r"(f32_0 + (__float_as_uint(fminf(r[u + h], fc.top)) << 7)));
-                            const float d = a[h] - L;
-                            part[u + h] = fmaf(d, d, part[u + h]);
+                            const float x = fmaf(l[h], fc.inv, fc.negz);
+                            r[u + h] = x + kMagic;
+                            off = fmaxf(off, fabsf(x - (r[u + h] - kMagic)));
                         }
                     }
-                } else {
+                    if (off <= fc.thr) {
+#pragma unroll
+                        for (int u = 0; u < U; u += 4) {
+                            const float4 a4 = *reinterpret_cast<const float4*>(&mag[sd][j + u]);
+                            const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                float L;
+                                asm("ld.shared.f32 %0, [%1];" : "=f"(L) : "r"(f32_0 + (__float_as_uint(fminf(r[u + h], fc.top)) << 7)));
+                                const float d = a[h] - L;
+                                part[u + h] = fmaf(d, d, part[u + h]);
+                            }
+                        }
+                    } else {
 #pragma unroll 1
-                    for (int u = 0; u < U; ++u) term(j + u, code_of(j + u));
+                        for (int u = 0; u < U; ++u) term(j + u, code_of(j + u));
+                    }
+                };
+                for (int k0 = 0; k0 < G; k0 += kChunk) {
+                    const int n_el = fill(k0);
+                    int j = 0;
+                    for (; j + 8 <= n_el; j += 8) group(j, std::integral_constant<int, 8>());
+                    if (j + 4 <= n_el) { group(j, std::integral_constant<int, 4>()); j += 4; }
+#pragma unroll 1
+                    for (; j < n_el; ++j) term(j, code_of(j));
                 }
-            };
-            for (int k0 = 0; k0 < G; k0 += kChunk) {
-                const int n_el = fill(k0);
-                int j = 0;
-                for (; j + 8 <= n_el; j += 8) group(j, std::integral_constant<int, 8>());
-                if (j + 4 <= n_el) { group(j, std::integral_constant<int, 4>()); j += 4; }
-#pragma unroll 1
-                for (; j < n_el; ++j) term(j, code_of(j));
+                const float e32 = (((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]))) + rest;
+                // errors are not negative, so their bit patterns are ordered as the numbers; NaN sorts above them all
+                const float emin = __uint_as_float(__reduce_min_sync(0xffffffffu, ok ? __float_as_uint(e32) : 0x7fffffffu));
+                const float eps = (float)(scnt / 8 + 3 * (G / kChunk + 1) + 64) * 2.4e-7f;      // 4 u per term of the longest sum
+                const unsigned close = __ballot_sync(0xffffffffu, ok && e32 <= emin * (1.f + eps));
+                const bool safe = ng <= 32 && emin > 1e-27f && emin < 1e30f && eps < 0.5f && vmax < 1e18f;
+                if (safe && (close & (close - 1)) == 0) {
+                    // one factor is left: the smallest error, whatever the rounding
+                    const int src = __ffs(close) - 1;
+                    best_s = shfl_double(s, src); best_z = shfl_double(z, src); best_f = shfl_double(fac, src);
+                    found = true;
+                    continue;
+                }
             }
-            float e32;
-            {
-                e32 = (((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]))) + rest;
-            }
-            // errors are not negative, so their bit patterns are ordered as the numbers; NaN sorts above them all
-            const float emin = __uint_as_float(__reduce_min_sync(0xffffffffu, ok ? __float_as_uint(e32) : 0x7fffffffu));
-            const float eps = (float)(scnt / 8 + 3 * (G / kChunk + 1) + 64) * 2.4e-7f;      // 4 u per term of the longest sum
-            const unsigned close = __ballot_sync(0xffffffffu, ok && e32 <= emin * (1.f + eps));
-            const bool safe = ng <= 32 && emin > 1e-27f && emin < 1e30f && eps < 0.5f && vmax < 1e18f;
-            if (safe && (close & (close - 1)) == 0) {
-                // one factor is left: the smallest error, whatever the rounding
-                const int src = __ffs(close) - 1;
-                best_s = shfl_double(s, src); best_z = shfl_double(z, src); best_f = shfl_double(fac, src);
-                if (lane == src) best_fc[sd] = fc;
-                found = true;
-                continue;
-            }
-            // ---- a near-tie (or sums out of fp32's range): the sum as it is defined
+            // ---- a near-tie (or a side the screen does not serve): the sum as it is defined, by one warp
             double err = 0.0;
             for (int k0 = 0; k0 < G; k0 += kChunk) {
                 const int n_el = fill(k0);
-auto level = [&](float r) {
+                auto level = [&](float r) {
                     int hi;
                     asm("ld.shared.b32 %0, [%1];" : "=r"(hi) : "r"(lev0 + (__float_as_uint(r) << 7)));
                     return __hiloint2double(hi, 0);
@@ -300,23 +496,23 @@ auto level = [&](float r) {
                 const int src = idx - c0;
                 best_err = e;
                 best_s = shfl_double(s, src); best_z = shfl_double(z, src); best_f = shfl_double(fac, src);
-                if (lane == src) best_fc[sd] = fc;
                 found = true;
             }
         }
         if (!found) {                               // no usable range: unit step anchored at the smallest element
             best_s = 1.0; best_z = scnt ? rint(smin) : 0.0; best_f = 1.0;
-            if (lane == 0) best_fc[sd] = fast_code(best_s, best_z, l_abs, nq);
         }
-        if (lane == 0) { best[sd].s = best_s; best[sd].z = best_z; best[sd].factor = best_f; }
+        if (sw == 0) {
+            const FastCode f = fast_code(best_s, best_z, l_abs, nq);
+            if (lane == 0) { best_fc[sd] = f; best[sd].s = best_s; best[sd].z = best_z; best[sd].factor = best_f; }
+        }
         __syncthreads();
         // ---- final level table of the group: entry u = c + half
-        const int pcnt = ext_cnt[0][0] + ext_cnt[1][0], ncnt = ext_cnt[0][1] + ext_cnt[1][1];
         if (tid < nlev) {
             const int cc = tid - half;
             double v;
             const int sdc = cc < 0, q = sdc ? -cc : cc;
-            v = (sdc ? ncnt : pcnt) ? __hiloint2double(level_word(__dmul_rn(best[sdc].s, __dadd_rn((double)q, best[sdc].z)), I), 0) : 0.0;
+            v = cnts[sdc] ? __hiloint2double(level_word(__dmul_rn(best[sdc].s, __dadd_rn((double)q, best[sdc].z)), I), 0) : 0.0;
             if (sdc) v = -v;
             T[tid] = v;
             levels[((size_t)n * ngrp + g) * nlev + tid] = (float)v;
@@ -328,30 +524,27 @@ auto level = [&](float r) {
         }
         __syncthreads();
         // ---- codes, eight to a 32-bit word (of nibbles, or three bytes of packed 3-bit codes)
-        double part = 0.0;
-        const FastCode fcs[2] = {best_fc[0], best_fc[1]};
         // four lanes share eight codes, two elements each: the groups of 128 that grouped tables have keep every lane busy
         for (int j0 = 0; j0 < G / 2; j0 += kThreads) {
             const int j = j0 + tid;                  // pair of elements
             uint32_t word = 0;
             if (j < G / 2) {
+                const float2 v2 = pair_of(j);
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const float v = w[2 * j + e];
+                    const float v = e ? v2.y : v2.x;
                     int cc = 0;
                     if (v != 0.f) {
                         const bool neg = v < 0.f;
-                        FastCode f;
-                        f.inv = neg ? fcs[1].inv : fcs[0].inv; f.negz = neg ? fcs[1].negz : fcs[0].negz;
-                        f.thr = neg ? fcs[1].thr : fcs[0].thr; f.top = neg ? fcs[1].top : fcs[0].top;
+                        const FastCode f = best_fc[neg];
                         bool exact;
-                        const float r = fast_round(log2f(fabsf(v)), f, exact);
+                        const float r = fast_round(log2_approx(fabsf(v)), f, exact);
                         const int q = exact ? (int)(__float_as_uint(r) - __float_as_uint(kMagic))
                                             : side_code(fabsf(v), best[neg].s, best[neg].z, neg ? half : half - 1);
                         cc = neg ? -q : q;
                     }
                     const int u = cc + half;
-                    part += T[u];
+                    row_sum += T[u];
                     word |= (uint32_t)u << ((pack3 ? 3 : 4) * (2 * (tid & 3) + e));
                 }
             }
@@ -366,14 +559,28 @@ auto level = [&](float r) {
                 }
             }
         }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) part += shfl_double(part, lane ^ o);
-        if (lane == 0) red[warp] = part;
-        __syncthreads();
-        if (tid == 0) row_sum += red[0] + red[1];
-        __syncthreads();
+        __syncthreads();                            // the tables are rewritten by the next group
     }
-    if (tid == 0) wsum[n] = (float)row_sum;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) row_sum += shfl_double(row_sum, lane ^ o);
+    if (lane == 0) red[warp] = row_sum;
+    __syncthreads();
+    if (tid == 0) {
+        for (int i = 1; i < kWarps; ++i) row_sum += red[i];
+        wsum[n] = (float)row_sum;
+    }
+}
+
+template <int WPS, int NB>
+lrq_status launch(const float* W, int N, int K, int G, const lrq_tlq_params* p, const ClipGrid& grid, int pack3, uint8_t* codes, float* levels,
+                  double* meta, float* wsum, cudaStream_t st) {
+    const bool binned = NB > 0 && binned_smem(NB, G) <= 200 * 1024;
+    const size_t smem = binned ? binned_smem(NB, G) : 0;
+    if (smem > 32 * 1024)
+        LRQ_CUDA_TRY(cudaFuncSetAttribute(tlq_quantize_kernel<WPS, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LRQ_CUDA_TRY(lrq_launch_pdl(tlq_quantize_kernel<WPS, NB>, dim3(N), dim3(64 * WPS), smem, st, W, N, K, G, p->w_bits, p->integerize_I, grid,
+                                pack3, binned ? 1 : 0, codes, levels, meta, wsum));
+    return LRQ_OK;
 }
 
 }  // namespace
@@ -398,7 +605,9 @@ extern "C" lrq_status lrq_tlq_quantize_weights(const float* W_rot, int N, int K,
         grid.a[i] = i < grid.na ? p->alpha[i] : 0.0;
         grid.b[i] = i < grid.nb ? p->beta[i] : 0.0;
     }
-    LRQ_CUDA_TRY(lrq_launch_pdl(tlq_quantize_kernel, dim3(N), dim3(kThreads), 0, (cudaStream_t)cuda_stream, W_rot, N, K, G, p->w_bits,
-                                p->integerize_I, grid, p->code_layout == LRQ_CODES_PACKED3 ? 1 : 0, codes, levels, meta, wsum));
-    return LRQ_OK;
+    const int pack3 = p->code_layout == LRQ_CODES_PACKED3 ? 1 : 0;
+    return G <= 128 ? launch<1, 0>(W_rot, N, K, G, p, grid, pack3, codes, levels, meta, wsum, (cudaStream_t)cuda_stream)
+         : G <= 256 ? launch<1, 128>(W_rot, N, K, G, p, grid, pack3, codes, levels, meta, wsum, (cudaStream_t)cuda_stream)
+         : G <= 2048 ? launch<2, 512>(W_rot, N, K, G, p, grid, pack3, codes, levels, meta, wsum, (cudaStream_t)cuda_stream)
+                    : launch<4, 1024>(W_rot, N, K, G, p, grid, pack3, codes, levels, meta, wsum, (cudaStream_t)cuda_stream);
 }

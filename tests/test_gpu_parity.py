@@ -110,6 +110,35 @@ def test_tlq_degenerate_rows(P, orc):
     assert np.array_equal(tl.levels.cpu().numpy().astype(np.float64), T.levels)
 
 
+@pytest.mark.parametrize("K,G,bits", [(256, 128, 3), (272, 136, 4), (512, 256, 4), (264, 0, 2), (2048, 0, 4), (2056, 0, 3), (6144, 0, 4),
+                                      (33280, 0, 4)])
+def test_tlq_search_at_its_edges(P, orc, K, G, bits):
+    # Group lengths on both sides of each way the search is done (fp32 sums, bins with one, two and four warps, a row too
+    # long for bins), and rows that strain the bins: one side only, an outlier, magnitudes all alike, 120 octaves, one
+    # element, sides of unequal length.  Bit for bit what the oracle finds.  Apart, codes and rounded levels only: subnormal
+    # elements, whose levels fp32 does not hold exactly, and magnitudes nearly alike, whose step cancels.
+    W = make_weights(900 + K + G, 12, K)
+    rng = np.random.default_rng(K)
+    W[0] = -np.abs(W[0])
+    W[1, 7] = 2.0 ** 20
+    W[3] = np.where(rng.random(K) < 0.5, 0.25, -0.125)
+    W[4] = np.sign(W[4]) * np.exp2(rng.uniform(-60, 60, K))
+    W[5] = np.sign(W[5]) * np.exp2(rng.uniform(-70, -50, K))
+    W[6] = 0
+    W[6, 3] = 0.7
+    W[7, : K - 2] = np.abs(W[7, : K - 2])
+    W[8, ::3] = 0
+    W = W.astype(np.float32)
+    g = default_clip_grid()
+    tl = P.lrq_tlq_quantize_weights(torch.from_numpy(W).cuda(), bits, G, 7, g, g)
+    PU.check_tlq(orc, W, tl, bits, G, what=f"edges K{K} b{bits} G{G}")
+    mags = np.stack([np.exp2(rng.uniform(-148, -118, K)), 0.02 * (1 + 1e-4 * rng.standard_normal(K)), 3.0 * (1 + 1e-3 * rng.random(K))])
+    W = (np.sign(W[9:12]) * mags).astype(np.float32)
+    tl, T = P.lrq_tlq_quantize_weights(torch.from_numpy(W).cuda(), bits, G, 7, g, g), orc.tlq_quantize(W.astype(np.float64), bits, G, 7, g, g)
+    assert np.array_equal(PU.unpack4(tl.codes.cpu().numpy()).astype(np.int32) - (1 << (bits - 1)), T.codes.astype(np.int32))
+    assert np.array_equal(tl.levels.cpu().numpy(), T.levels.astype(np.float32))
+
+
 # --------------------------------------------------------------------------------------------- qgemm
 def _small_layer(P, orc, M, K, N, w_bits, a_bits, G, B, seed, rot="hadamard"):
     spec = LayerSpec("t", seed, M, K, N, w_bits, a_bits, G, rot, B)

@@ -21,8 +21,8 @@
 //     worked out from the candidate's range) takes the fp64 expression, a division, instead;
 //   * levels have 8-bit significands: fp32 numbers, and the upper word of the double is the level.
 // 31 factors a side, 4 bits: 4608 x 1152 545 us with the fp64 expression for every element and factor, 169 with fp32 sums over
-// every element, 82 with bins; 2048 x 6144 490 and 125; 512 x 12288 685 and 96.  4608 x 1536 in groups of 128: 315 with fp32
-// sums, 398 with bins; of 256 (4608 x 2048): 328 and 315.
+// every element, 80 with bins; 2048 x 6144 485 and 122; 512 x 12288 685 and 96.  4608 x 1536 in groups of 128: 315 with fp32
+// sums, 398 with bins; of 256 (4608 x 2048): 326 and 304.
 #include "lrq_internal.cuh"
 #include <climits>
 #include <type_traits>
@@ -115,8 +115,9 @@ __device__ __forceinline__ void side_sync(int sd) {
 constexpr size_t binned_smem(int NB, int G) { return (size_t)2 * NB * 4 + (size_t)(G + 8) * 4 + (size_t)(G / 4 + 8) * 8; }
 
 // WPS warps a side and NB bins (none: fp32 sums): one warp up to 256 elements, most of their work is per factor, not per
-// element; two with 512 bins up to 2048 (4608 x 1152: 82 us; with one warp 106, with four 119); four with 1024 bins above,
-// where a row's lists leave room for fewer CTAs (2048 x 6144: 125 us, with two warps 177).  `binned` is 0 when the lists do not fit in shared memory.
+// element; two with 512 bins up to 2048 (4608 x 1152: 80 us; with one warp 106, with four 119); four with 1024 bins above,
+// where a row's lists leave room for fewer CTAs (2048 x 6144: 122 us, with two warps 177).  `binned` is 0 when the lists do not
+// fit in shared memory.
 template <int WPS, int NB>
 __global__ void __launch_bounds__(64 * WPS, 16 / WPS)
 tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, int I, ClipGrid grid, int pack3, int binned,
@@ -132,18 +133,17 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
     __shared__ __align__(16) float mag[2][kChunk];
     __shared__ __align__(16) float lg[2][kChunk];
     __shared__ FastCode best_fc[2];
-    __shared__ unsigned ext[2][2][2];              // [parity of the group][side][max, ~min] of |w|, as bit patterns
-    __shared__ int ext_cnt[2][2];
+    __shared__ unsigned ext[kWarps][2][2];         // [warp][side][max, ~min] of |w|, as bit patterns
+    __shared__ int ext_cnt[kWarps][2];
     __shared__ Side best[2];
     __shared__ double T[16];
     __shared__ double red[kWarps];
 
     const int n = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int half = 1 << (bits - 1), nlev = 1 << bits, ngrp = K / G;
-    double row_sum = 0.0;                          // of this thread's codes
-    if (tid < 8) reinterpret_cast<unsigned*>(ext)[tid] = 0;
-    if (tid < 4) reinterpret_cast<int*>(ext_cnt)[tid] = 0;
-    __syncthreads();
+    // sum of each thread's codes; for the short groups in shared memory, since a register would be live across every search
+    double kept = 0.0, *row_sum = &epart[0][0][0] + tid;
+    if (NB == 0) *row_sum = 0.0;
     lrq_pdl_trigger();
     lrq_pdl_wait();                                // the weights may be the previous kernel's output
 
@@ -173,15 +173,18 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                 // magnitudes: the bit patterns are ordered as the numbers
                 const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(amax[h])), mn = __reduce_min_sync(0xffffffffu, __float_as_uint(amin[h]));
                 const int c = __reduce_add_sync(0xffffffffu, cnt[h]);
-                if (lane == 0) { atomicMax(&ext[g & 1][h][0], mx); atomicMax(&ext[g & 1][h][1], ~mn); atomicAdd(&ext_cnt[g & 1][h], c); }
+                if (lane == 0) { ext[warp][h][0] = mx; ext[warp][h][1] = ~mn; ext_cnt[warp][h] = c; }
             }
         }
         __syncthreads();
-        const float vmaxs[2] = {__uint_as_float(ext[g & 1][0][0]), __uint_as_float(ext[g & 1][1][0])};
-        const float vmins[2] = {__uint_as_float(~ext[g & 1][0][1]), __uint_as_float(~ext[g & 1][1][1])};
-        const int cnts[2] = {ext_cnt[g & 1][0], ext_cnt[g & 1][1]};
-        if (tid < 4) reinterpret_cast<unsigned*>(ext[(g & 1) ^ 1])[tid] = 0;      // the next group's: last read before that barrier
-        if (tid < 2) ext_cnt[(g & 1) ^ 1][tid] = 0;
+        unsigned top[2] = {0, 0}, low[2] = {0, 0};
+        int cnts[2] = {0, 0};
+#pragma unroll
+        for (int i = 0; i < kWarps; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) { top[h] = max(top[h], ext[i][h][0]); low[h] = max(low[h], ext[i][h][1]); cnts[h] += ext_cnt[i][h]; }
+        const float vmaxs[2] = {__uint_as_float(top[0]), __uint_as_float(top[1])};
+        const float vmins[2] = {__uint_as_float(~low[0]), __uint_as_float(~low[1])};
         const int sd = warp / WPS, sw = warp % WPS;          // the warp's side and its place there; a lane is a factor
         const int nq = sd ? half : half - 1;       // highest code of the side = denominator of Eq. 6
         const float vmax = vmaxs[sd], vmin = vmins[sd];
@@ -450,6 +453,7 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                     // one factor is left: the smallest error, whatever the rounding
                     const int src = __ffs(close) - 1;
                     best_s = shfl_double(s, src); best_z = shfl_double(z, src); best_f = shfl_double(fac, src);
+                    if (lane == src) best_fc[sd] = fc;
                     found = true;
                     continue;
                 }
@@ -496,6 +500,7 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                 const int src = idx - c0;
                 best_err = e;
                 best_s = shfl_double(s, src); best_z = shfl_double(z, src); best_f = shfl_double(fac, src);
+                if (lane == src) best_fc[sd] = fc;
                 found = true;
             }
         }
@@ -503,8 +508,11 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
             best_s = 1.0; best_z = scnt ? rint(smin) : 0.0; best_f = 1.0;
         }
         if (sw == 0) {
-            const FastCode f = fast_code(best_s, best_z, l_abs, nq);
-            if (lane == 0) { best_fc[sd] = f; best[sd].s = best_s; best[sd].z = best_z; best[sd].factor = best_f; }
+            if (NB > 0 || !found) {                 // else the factor's lane has left it
+                const FastCode f = fast_code(best_s, best_z, l_abs, nq);
+                if (lane == 0) best_fc[sd] = f;
+            }
+            if (lane == 0) { best[sd].s = best_s; best[sd].z = best_z; best[sd].factor = best_f; }
         }
         __syncthreads();
         // ---- final level table of the group: entry u = c + half
@@ -525,6 +533,7 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
         __syncthreads();
         // ---- codes, eight to a 32-bit word (of nibbles, or three bytes of packed 3-bit codes)
         // four lanes share eight codes, two elements each: the groups of 128 that grouped tables have keep every lane busy
+        double part = 0.0;
         for (int j0 = 0; j0 < G / 2; j0 += kThreads) {
             const int j = j0 + tid;                  // pair of elements
             uint32_t word = 0;
@@ -544,7 +553,7 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                         cc = neg ? -q : q;
                     }
                     const int u = cc + half;
-                    row_sum += T[u];
+                    part += T[u];
                     word |= (uint32_t)u << ((pack3 ? 3 : 4) * (2 * (tid & 3) + e));
                 }
             }
@@ -559,15 +568,17 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
                 }
             }
         }
+        if (NB == 0) *row_sum += part; else kept += part;
         __syncthreads();                            // the tables are rewritten by the next group
     }
+    double sum = NB == 0 ? *row_sum : kept;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) row_sum += shfl_double(row_sum, lane ^ o);
-    if (lane == 0) red[warp] = row_sum;
+    for (int o = 16; o; o >>= 1) sum += shfl_double(sum, lane ^ o);
+    if (lane == 0) red[warp] = sum;
     __syncthreads();
     if (tid == 0) {
-        for (int i = 1; i < kWarps; ++i) row_sum += red[i];
-        wsum[n] = (float)row_sum;
+        for (int i = 1; i < kWarps; ++i) sum += red[i];
+        wsum[n] = (float)sum;
     }
 }
 

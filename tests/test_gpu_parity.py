@@ -387,6 +387,25 @@ def test_rotate_weights(P, orc, N, K, rot, B, smooth):
         assert torch.equal(Wd, out)
 
 
+@pytest.mark.parametrize("M,K", [(1, 128), (257, 200), (3000, 1032), (4429, 1536), (19000, 384)])
+def test_dense_rotation_rounds_and_cuts(P, M, K):
+    # The rotation product over the schedules its plan can take: one tile, a ragged column and a ragged last k-block, a
+    # last round cut in halves, several rounds.  With 8-bit codes a token's dequantized row is within half a step of the
+    # exact product, plus the fp32 accumulation (K / 16 adds) and the error of the range it puts into the step and zero point.
+    g = torch.Generator(device="cuda").manual_seed(M)
+    X = torch.randn((M, K), generator=g, device="cuda").bfloat16()
+    R = (torch.randn((K, K), generator=g, device="cuda") / K ** 0.5).bfloat16()
+    q, s, z = P.lrq_rotate_quantize_act(X, P.ROT_DENSE, 8, R=R)
+    want = X.double() @ R.double()
+    got = (q.double() + z.double()[:, None]) * s.double()[:, None]
+    acc = (K / 16 + 4) * 2.0 ** -23 * (X.double().abs() @ R.double().abs())
+    tol = 0.5 * s.double()[:, None] * 1.0001 + 2 * acc.amax(dim=1, keepdim=True)
+    # Eq. 1 clamps to [0, 255] around a rounded zero point: the extremes may lie half a step further out
+    edge = (q == 0) | (q == 255)
+    assert bool(((got - want).abs() <= tol * torch.where(edge, 2.0, 1.0)).all())
+    assert P.lrq_device_status() == 0
+
+
 @pytest.mark.parametrize("N,K,smooth", [(2055, 520, False), (257, 1030, True), (2049, 640, True), (130, 1536, False), (3, 2048, False)])
 def test_rotate_weights_dense_by_digits(P, N, K, smooth):
     # The dense product from int8 digits against the fp64 product: ragged tiles in N and K, unaligned rows of R, a row and a

@@ -61,14 +61,21 @@ inline cudaError_t lrq_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block,
 // A layer's weight decode (codes -> bf16 [N,K] at `out`, tlq_decode.cuh), done by the quantizer kernels' warps when they have no
 // tokens left: the two are independent, and a launch of its own costs three microseconds on a short batch.  out ==
 // nullptr: nothing to decode.  fmt: 4, 3, 2 nibble layout, 13 packed 3-bit.
-struct LrqExpand { const uint8_t* codes; const float* levels; int N, K, G, fmt; void* out; };
+struct LrqExpand {
+    const uint8_t* codes; const float* levels; int N, K, G, fmt; void* out;
+    // a row's shares (tlq_decode.cuh): the row itself, or with grouped tables runs of up to 32 / 2^bits words of eight codes a lane
+    __host__ __device__ int segments() const {
+        const int most = 32 << (fmt == 4 ? 1 : fmt == 2 ? 3 : 2);
+        return G == K ? 1 : (K / 8 + most - 1) / most;
+    }
+};
 
 // CTAs of a quantizer grid: `need` for its tokens, or more (up to `resident`) when there are weight rows for them.
 static inline int lrq_quant_grid(int need, int resident, int warps_per_cta, const LrqExpand& ex) {
     int g = need < resident ? need : resident;
     if (ex.out) {
-        const int want = g + (ex.N + warps_per_cta - 1) / warps_per_cta;
-        g = want < resident ? want : resident;
+        const long want = g + ((long)ex.N * ex.segments() + warps_per_cta - 1) / warps_per_cta;
+        g = want < resident ? (int)want : resident;
     }
     return g;
 }

@@ -16,20 +16,34 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 // exact bf16 numbers stored as fp32: the upper two bytes of each word are the entry.
 struct Lut { uint32_t lo[4], hi[4]; };
 
+// The same as it lies in memory: loads that can be under way together, made into planes when they are needed.
 template <int W_BITS>
-__device__ __forceinline__ void load_lut(Lut& L, const float* __restrict__ tab) {
+struct RawLut {
+    float4 v[(1 << W_BITS) / 4];
+    __device__ __forceinline__ void load(const float* __restrict__ tab) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if (j < (1 << W_BITS) / 4) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(tab) + j);
-            const uint32_t t01 = prmt(__float_as_uint(v.x), __float_as_uint(v.y), 0x7632u);
-            const uint32_t t23 = prmt(__float_as_uint(v.z), __float_as_uint(v.w), 0x7632u);
-            L.lo[j] = prmt(t01, t23, 0x6420u);
-            L.hi[j] = prmt(t01, t23, 0x7531u);
-        } else {
-            L.lo[j] = 0; L.hi[j] = 0;
+        for (int j = 0; j < (1 << W_BITS) / 4; ++j) v[j] = __ldg(reinterpret_cast<const float4*>(tab) + j);
+    }
+    __device__ __forceinline__ void planes(Lut& L) const {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (j < (1 << W_BITS) / 4) {
+                const uint32_t t01 = prmt(__float_as_uint(v[j].x), __float_as_uint(v[j].y), 0x7632u);
+                const uint32_t t23 = prmt(__float_as_uint(v[j].z), __float_as_uint(v[j].w), 0x7632u);
+                L.lo[j] = prmt(t01, t23, 0x6420u);
+                L.hi[j] = prmt(t01, t23, 0x7531u);
+            } else {
+                L.lo[j] = 0; L.hi[j] = 0;
+            }
         }
     }
+};
+
+template <int W_BITS>
+__device__ __forceinline__ void load_lut(Lut& L, const float* __restrict__ tab) {
+    RawLut<W_BITS> raw;
+    raw.load(tab);
+    raw.planes(L);
 }
 
 // Eight codes as nibbles (one word) -> four registers of two bf16 each, in k order.
@@ -69,42 +83,37 @@ __device__ __forceinline__ uint32_t fetch_packed3(const uint8_t* a, const uint8_
     return __funnelshift_r(lo, hi, 8 * (uint32_t)(ai & 3)) & 0x00FFFFFFu;
 }
 
-// Weight rows first, first + stride, ... of a layer decoded to bf16 [N,K], by one warp.  A layer meets each weight in M/256
-// tiles of the contraction; decoded there, a weight costs 2.6 lane-operations and a trip through shared memory in every
+// A layer's weights decoded to bf16 [N,K], shares first, first + stride, ... by one warp.  A layer meets each weight in
+// M/256 tiles of the contraction; decoded there, a weight costs 2.6 lane-operations and a trip through shared memory in every
 // one of them.  Decoded here it costs one pass over 2.5 bytes per weight, whose results the contraction then reads
-// mostly from L2.  Bound by those bytes.  A warp takes a row at a time, so that a per-channel table is loaded once; a lane
-// turns eight codes (4 bytes, 3 when packed) into one 16-byte store, UNROLL of them in flight, so a warp reads and
-// writes whole lines.  With grouped tables a lane reloads its table when its group changes.
+// mostly from L2.  Bound by those bytes, as long as enough of them are in flight: a lane asks for UNROLL words of eight codes (4
+// bytes, 3 when packed) before it uses the first and turns each into one 16-byte store, so a warp reads and writes whole
+// lines.  Per-channel tables: a share is a row, its table loaded once (segments as below with a table each: 12288 x 3072 27 us
+// instead of 12).
+template <int W_BITS, bool PACKED3>
+__device__ __forceinline__ uint32_t fetch_codes(const uint8_t* row, int j, const uint8_t* end) {
+    return PACKED3 ? fetch_packed3(row + 3 * (size_t)j, end) : __ldg(reinterpret_cast<const uint32_t*>(row) + j);
+}
 template <int W_BITS, bool PACKED3>
 __device__ __forceinline__ void expand_rows(const LrqExpand& e, int first, int stride) {
     constexpr int NLEV = 1 << W_BITS, UNROLL = 6;
     const int lane = threadIdx.x & 31;
-    const int words = e.K >> 3, ngrp = e.K / e.G, wpg = e.G >> 3;  // groups of eight codes: per row, per table
+    const int words = e.K >> 3;
     const size_t pitch = PACKED3 ? (size_t)e.K * 3 / 8 : (size_t)e.K / 2;
     const uint8_t* end = e.codes + (size_t)e.N * pitch;
     for (int n = first; n < e.N; n += stride) {
         const uint8_t* row = e.codes + (size_t)n * pitch;
-        const float* tab = e.levels + (size_t)n * ngrp * NLEV;
         uint4* dst = static_cast<uint4*>(e.out) + (size_t)n * words;
         Lut L;
-        int held = -1;
-        if (ngrp == 1) { load_lut<W_BITS>(L, tab); held = 0; }
+        load_lut<W_BITS>(L, e.levels + (size_t)n * NLEV);
         for (int j0 = lane; j0 < words; j0 += 32 * UNROLL) {
             uint32_t w[UNROLL];
 #pragma unroll
-            for (int u = 0; u < UNROLL; ++u) {
-                const int j = j0 + 32 * u;
-                w[u] = 0;
-                if (j < words) w[u] = PACKED3 ? fetch_packed3(row + 3 * (size_t)j, end) : __ldg(reinterpret_cast<const uint32_t*>(row) + j);
-            }
+            for (int u = 0; u < UNROLL; ++u) w[u] = j0 + 32 * u < words ? fetch_codes<W_BITS, PACKED3>(row, j0 + 32 * u, end) : 0u;
 #pragma unroll
             for (int u = 0; u < UNROLL; ++u) {
                 const int j = j0 + 32 * u;
                 if (j >= words) break;
-                if (ngrp > 1) {
-                    const int g = j / wpg;
-                    if (g != held) { load_lut<W_BITS>(L, tab + (size_t)g * NLEV); held = g; }
-                }
                 uint32_t o[4];
                 decode_w<W_BITS>(PACKED3 ? spread3(w[u]) : w[u], L, o);
                 dst[j] = make_uint4(o[0], o[1], o[2], o[3]);
@@ -112,15 +121,56 @@ __device__ __forceinline__ void expand_rows(const LrqExpand& e, int first, int s
         }
     }
 }
+// Grouped tables: a lane's next word, 32 words on, has another table, so the tables of UNROLL words are asked for with their
+// codes (32 registers of them), and a share is that many words, so that every warp of the grid has some.  6144 x 1536 in
+// groups of 128, 4429 tokens: 107 us a call with whole rows and a table at a time when its group came up, 95 now; 4608 x 1152,
+// 4096 tokens: 75 and 64.
+template <int W_BITS, bool PACKED3>
+__device__ __forceinline__ void expand_grouped(const LrqExpand& e, uint32_t first, uint32_t stride) {
+    constexpr int NLEV = 1 << W_BITS, UNROLL = 32 / NLEV;
+    const int lane = threadIdx.x & 31;
+    const int words = e.K >> 3, ngrp = e.K / e.G, wpg = e.G >> 3;  // groups of eight codes: per row, per table
+    const uint32_t segs = (uint32_t)e.segments(), shares = (uint32_t)e.N * segs;
+    const int per = ((words + 31) / 32 + (int)segs - 1) / (int)segs;       // words a lane takes of a share, at most UNROLL
+    const size_t pitch = PACKED3 ? (size_t)e.K * 3 / 8 : (size_t)e.K / 2;
+    const uint8_t* end = e.codes + (size_t)e.N * pitch;
+    for (uint32_t it = first; it < shares; it += stride) {
+        const uint32_t n = it / segs;
+        const int j0 = (int)(it - n * segs) * 32 * per + lane;
+        const uint8_t* row = e.codes + n * pitch;
+        const float* tab = e.levels + (size_t)n * ngrp * NLEV;
+        uint4* dst = static_cast<uint4*>(e.out) + (size_t)n * words;
+        uint32_t w[UNROLL];
+        RawLut<W_BITS> raw[UNROLL];
+#pragma unroll
+        for (int u = 0; u < UNROLL; ++u) {
+            if (u >= per) break;
+            const int j = min(j0 + 32 * u, words - 1);
+            w[u] = fetch_codes<W_BITS, PACKED3>(row, j, end);
+            raw[u].load(tab + (size_t)(j / wpg) * NLEV);
+        }
+#pragma unroll
+        for (int u = 0; u < UNROLL; ++u) {
+            const int j = j0 + 32 * u;
+            if (u >= per || j >= words) break;
+            Lut L;
+            raw[u].planes(L);
+            uint32_t o[4];
+            decode_w<W_BITS>(PACKED3 ? spread3(w[u]) : w[u], L, o);
+            dst[j] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+    }
+}
 
-// The weight decode that rides on a quantizer kernel: called by every warp of the grid when it has no tokens left.  Rows are
+// The weight decode that rides on a quantizer kernel: called by every warp of the grid when it has no tokens left.  Shares are
 // dealt from the last warp of the grid backwards, so that those of a short batch go to CTAs that had none.
 static __device__ __noinline__ void expand_share(const LrqExpand e) {
     const int wpc = blockDim.x >> 5, total = gridDim.x * wpc, first = total - 1 - (int)(blockIdx.x * wpc + (threadIdx.x >> 5));
-    if (e.fmt == 4) expand_rows<4, false>(e, first, total);
-    else if (e.fmt == 3) expand_rows<3, false>(e, first, total);
-    else if (e.fmt == 13) expand_rows<3, true>(e, first, total);
-    else expand_rows<2, false>(e, first, total);
+    const bool grouped = e.G != e.K;
+    if (e.fmt == 4) { if (grouped) expand_grouped<4, false>(e, first, total); else expand_rows<4, false>(e, first, total); }
+    else if (e.fmt == 3) { if (grouped) expand_grouped<3, false>(e, first, total); else expand_rows<3, false>(e, first, total); }
+    else if (e.fmt == 13) { if (grouped) expand_grouped<3, true>(e, first, total); else expand_rows<3, true>(e, first, total); }
+    else { if (grouped) expand_grouped<2, false>(e, first, total); else expand_rows<2, false>(e, first, total); }
 }
 
 }  // namespace lrq_dec

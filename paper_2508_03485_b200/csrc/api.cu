@@ -85,7 +85,7 @@ static lrq_status run_act(const void* X, int M, int K, long ldx, const lrq_act_p
                           cudaStream_t stream) {
     lrq_status st;
     // the rotation products leave each row's extremes where the quantizer will write the row's results
-    const LrqRowExt none = {}, ext = {a_codes, (size_t)K * (out16 ? 16 : p->a_bits) / 8, a_scale, reinterpret_cast<float*>(a_zp)};
+    const LrqRowExt ext = {a_codes, (size_t)K * (out16 ? 16 : p->a_bits) / 8, a_scale, reinterpret_cast<float*>(a_zp)};
     if (p->kind == LRQ_ROT_DENSE) {
         const size_t need = lrq_act_workspace_bytes(M, K, p);
         if (!workspace || workspace_bytes < need || !lrq_aligned(workspace, 256)) return LRQ_ERR_WORKSPACE;
@@ -97,13 +97,19 @@ static lrq_status run_act(const void* X, int M, int K, long ldx, const lrq_act_p
     if (p->kind == LRQ_ROT_DUAL) {
         const size_t need = lrq_act_workspace_bytes(M, K, p);
         if (!workspace || workspace_bytes < need || !lrq_aligned(workspace, 256)) return LRQ_ERR_WORKSPACE;
-        float* Yr = static_cast<float*>(workspace);                       // u = x R1hat first, y later
-        void* V3 = static_cast<unsigned char*>(workspace) + lrq_round_up((size_t)M * K * sizeof(float), 256);
-        st = lrq_launch_bdiag_gemm(X, M, K, ldx, 1, p->R1_bf16, Yr, none, stream);
-        if (st != LRQ_OK) return st;
-        st = lrq_launch_dual_gather_split(Yr, M, K, p->perm, V3, stream);  // u P as three bf16 terms
-        if (st != LRQ_OK) return st;
-        st = lrq_launch_bdiag_gemm(V3, M, K, 3L * K, 3, p->R2_bf16, Yr, ext, stream);
+        float* Yr = static_cast<float*>(workspace);
+        void* U3 = static_cast<unsigned char*>(workspace) + lrq_round_up((size_t)M * K * sizeof(float), 256);   // three bf16 panels
+        if (M % 8 == 0) {
+            st = lrq_launch_dual_first(X, M, K, ldx, p->R1_bf16, p->perm, U3, stream);
+            if (st != LRQ_OK) return st;
+            st = lrq_launch_dual_second(U3, M, K, p->R2_bf16, Yr, ext, stream);
+        } else {
+            st = lrq_launch_bdiag_gemm(X, M, K, ldx, 1, p->R1_bf16, Yr, LrqRowExt{}, stream);       // u = x R1hat first, y later
+            if (st != LRQ_OK) return st;
+            st = lrq_launch_dual_gather_split(Yr, M, K, p->perm, U3, stream);
+            if (st != LRQ_OK) return st;
+            st = lrq_launch_bdiag_gemm(U3, M, K, 3L * K, 3, p->R2_bf16, Yr, ext, stream);
+        }
         if (st != LRQ_OK) return st;
         return lrq_launch_quantize_f32_ext(Yr, M, K, p->a_bits, p->mode, out16, a_codes, a_scale, a_zp, ex, stream);
     }

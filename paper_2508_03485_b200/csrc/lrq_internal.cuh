@@ -94,11 +94,15 @@ struct LrqRowExt { unsigned char* rows; size_t pitch; float* row_min; float* row
 constexpr int LRQ_ROT_TILE = 128;     // columns per tile
 // qgemm_bf16.cu : Y[M,K] (fp32) = X[M,K] (bf16) . R[K,K] (bf16) on the tensor cores
 lrq_status lrq_launch_rotgemm(const void* X, int M, int K, long ldx, const void* R, float* Y, const LrqRowExt& ext, cudaStream_t st);
-// rotgemm.cu : Y[M,K] (fp32) = sum over the `parts` column panels of A[M, parts*K] (bf16) of panel . blockdiag(Rblk),
-// Rblk bf16 [K/128][128][128]
+// rotgemm.cu : the dual transformation, R1 and R2 bf16 [K/128][128][128].  For M a multiple of 8: U3 = the three bf16 terms of
+// (x . R1hat . P)^T, [3K][M], then Y[M,K] (fp32) = their sum . R2hat; an entry of perm outside 0 .. K-1 is read as 0 and
+// recorded (status 31)
+lrq_status lrq_launch_dual_first(const void* X, int M, int K, long ldx, const void* R1, const int32_t* perm, void* U3, cudaStream_t st);
+lrq_status lrq_launch_dual_second(const void* U3, int M, int K, const void* R2, float* Y, const LrqRowExt& ext, cudaStream_t st);
+// For any M: Y[M,K] (fp32) = sum over the `parts` column panels of A[M, parts*K] (bf16) of panel . blockdiag(Rblk)
 lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int parts, const void* Rblk, float* Y, const LrqRowExt& ext,
                                  cudaStream_t st);
-// rotdual.cu : V3 bf16 [M,3K], panel p = p-th bf16 term of U[m, perm[i]] (the reordering between the two rotations)
+// rotdual.cu : V3 bf16 [M,3K], panel p = p-th bf16 term of U[m, perm[i]] (the reordering between the two)
 lrq_status lrq_launch_dual_gather_split(const float* U, int M, int K, const int32_t* perm, void* V3, cudaStream_t st);
 // rotq.cu : per-token quantization of fp32 rows whose extremes a rotation product has left, per tile of LRQ_ROT_TILE columns at
 // the start of the row's own part of `codes` (8 bytes a tile; the codes overwrite them, and are longer for every K above

@@ -8,6 +8,8 @@
 // column panels [M, 3K] that the block-diagonal product sums into one fp32 accumulator, each product of a term
 // with a bf16 entry of R2hat being exact.
 //
+// For batches that are not a multiple of 8 tokens; the others do without this kernel (rotgemm.cu).
+//
 // One CTA per token at a time: the fp32 row is staged in shared memory with coalesced 128-bit loads, gathered from
 // there through perm (read once per CTA into shared memory as well), and the panels are written two elements per thread.
 #include "lrq_internal.cuh"

@@ -1,15 +1,29 @@
-// Product with a block-diagonal matrix of 128 x 128 blocks on the 5th-generation tensor cores: the factors R1hat, R2hat of the
-// dual transformation (Sec. 4.2).  The left operand is bf16 [M, parts*K]: `parts` column panels summed into one fp32
-// accumulator (the bf16 terms of an fp32 operand).  bf16 x bf16 products are exact in fp32; sums are accumulated in fp32.
-// With `ext` the epilogue also leaves every row's minimum and maximum over the tile's columns (plain stores, one pair per
-// row and tile), so that the quantizer that follows is a single streaming pass.
+// The dual transformation kept in its factors (Sec. 4.2): y = x . R1hat . P . R2hat, R1hat and R2hat block-diagonal with 128 x 128
+// blocks, P a staggered permutation given as the index map (u P)_i = u[perm[i]].  Two products on the 5th-generation
+// tensor cores, and nothing between them:
 //
-// Persistent CTA per SM over 128 x 128 output tiles (tile j of a token block only meets block j), 64-deep k-blocks, a
-// 4-stage TMA pipeline:
-//   warp 0      TMA tile loads (left operand: K-major box 64 x 128; blocks: two 64 x 64 boxes, each 64 output columns
-//               wide, one k-row per 128-byte line -> an MN-major UMMA operand)
+//   FIRST   u = x . R1hat, computed transposed (channels along the accumulator's lanes, tokens along its columns), so that
+//           a channel of u is a row in memory.  bf16 x bf16 products are exact; a single rounding of u to bf16 would cost 16
+//           of its 24 significant bits, so the epilogue splits it into three bf16 terms h1 + h2 + h3 (h1 = bf16(u), h2 = bf16(u -
+//           h1), h3 = bf16(u - h1 - h2); the subtractions are exact), which carry u to within 2^-25, and writes each to
+//           row i of its panel for every i with perm[i] = the lane's channel.
+//   SECOND  y = (u P) . R2hat from panels that are in order: the three are summed into one fp32 accumulator, each product of a
+//           term with a bf16 entry of R2hat being exact.  The epilogue stores fp32 and each row's extremes over the tile's
+//           columns, so that the quantizer is a single streaming pass.
+//
+// Bound by memory: 2 + 6 bytes an element in the first, 6 + 4 in the second.  A row of the panels has to start on 16 bytes, so
+// batches that are not a multiple of 8 tokens, whose padded rows the workspace does not hold, take the products in mode
+// PLAIN (u in fp32, tokens along the lanes) with a kernel between them that gathers and splits (rotdual.cu; 14 bytes an element
+// more).  4608 x 3072 with its quantizer: 80 us so, 62 with the transposed panels (90 with them in u's own order and the rows
+// chosen by the second product's TMA, four at a time: 90 cycles for each 512 bytes; 80 with four epilogue warps in the first).
+//
+// Persistent CTA per SM over tiles of 128 tokens x 128 channels (tile j of a token block only meets block j), 64-deep k-blocks,
+// a 4-stage TMA pipeline:
+//   warp 0      TMA loads.  R's blocks: two 64 x 64 boxes, 64 output columns wide, one k-row per 128-byte line -> an MN-major
+//               operand.  x: K-major box of 64 x 128.  The panels: two boxes of 64 tokens x 64 rows -> MN-major (PLAIN: a
+//               K-major box of the gathered panels [M,3K])
 //   warp 1      allocates TMEM, issues tcgen05.mma (M = 128, N = 128, K = 16) and commits
-//   warps 2-5   epilogue: tcgen05.ld of the finished accumulator, fp32 stores
+//   warps 2-5   epilogue (FIRST: 2-9)
 // The accumulator is double-buffered in TMEM.  Every wait is bounded; on expiry the CTA records a code in the status word,
 // waits (bounded) for its TMA loads in flight and unwinds.
 #include "lrq_internal.cuh"
@@ -20,40 +34,60 @@
 namespace {
 using namespace lrq_tc;
 
+enum Mode { PLAIN, FIRST_T, SECOND_T };
 constexpr int BM = 128, BN = 128, BK = 64;
-constexpr int STAGES = 4;
+constexpr int MAX_STAGES = 4;
+constexpr int stages(Mode m) { return m == FIRST_T ? 3 : MAX_STAGES; }      // FIRST's lists take the fourth's place
 constexpr int A_STAGE_BYTES = BM * BK * 2;          // 16 KB
 constexpr int B_CHUNK_BYTES = BK * 128;             // 8 KB: 64 k-rows of 64 output columns
-constexpr int PRODUCER_WARP = 0, MMA_WARP = 1, EPI_WARP0 = 2, NUM_EPI_WARPS = 4;
-constexpr int NUM_THREADS = (EPI_WARP0 + NUM_EPI_WARPS) * 32;   // 192
+constexpr int PRODUCER_WARP = 0, MMA_WARP = 1, EPI_WARP0 = 2;
+// FIRST's epilogue splits and stores 6 bytes an element: a warp for every 32 channels x 64 tokens of a tile
+constexpr int epi_warps(Mode m) { return m == FIRST_T ? 8 : 4; }
+constexpr int threads(Mode m) { return (EPI_WARP0 + epi_warps(m)) * 32; }
 constexpr int TMEM_COLS = 512;
 
 struct __align__(16) Ctl {
-    uint64_t full[STAGES];
-    uint64_t empty[STAGES];
+    uint64_t full[MAX_STAGES];
+    uint64_t empty[MAX_STAGES];
     uint64_t tmem_full[2];
     uint64_t tmem_empty[2];
     uint32_t tmem_base;
     volatile int abort_flag;
 };
-constexpr int EPI_TILE_BYTES = 32 * 32 * 4;         // one epilogue warp's 32 x 32 fp32 chunk, for the row/column trade
+constexpr int EPI_TILE_BYTES = 32 * 128;            // 32 lines of an epilogue warp: 32 fp32 or 64 bf16 each
 constexpr int B_STAGE_BYTES = (BN / 64) * B_CHUNK_BYTES;        // 16 KB
 constexpr int STAGE_TX_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
-constexpr size_t SMEM_BYTES = 1024 + (size_t)STAGES * STAGE_TX_BYTES + sizeof(Ctl) + NUM_EPI_WARPS * EPI_TILE_BYTES;
+constexpr int NO_ROW = 0xffff;                      // no further row; rows are below MAX_K
+constexpr int MAX_K = 12288;                        // of FIRST: 6 bytes of lists per channel
+constexpr size_t smem_bytes(Mode m, int K) {
+    return 1024 + (size_t)stages(m) * STAGE_TX_BYTES + 1024 + sizeof(Ctl) + epi_warps(m) * EPI_TILE_BYTES + (m == FIRST_T ? 6 * (size_t)K : 0);
+}
+static_assert(smem_bytes(FIRST_T, MAX_K) <= 227 * 1024, "shared memory budget");
 static_assert(BN == LRQ_ROT_TILE, "one pair of extremes per row and tile");
 
-// Rblk: the blocks one after the other ([K/128][128][128], i.e. K rows of 128 columns)
-__global__ void __launch_bounds__(NUM_THREADS, 1)
-bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
-                  float* __restrict__ Y, int M, int K, int parts, unsigned char* __restrict__ ext, size_t ext_pitch, float* __restrict__ ext_min,
-                  float* __restrict__ ext_max, int* status) {
-    constexpr uint32_t IDESC = umma_idesc_bf16(BM, BN, /*a_mn_major=*/false, /*b_mn_major=*/true);
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// tmR: the blocks one after the other ([K/128][128][128], i.e. K rows of 128 columns).  tmX: x [M,K], or the panels [3K][M].
+// U3 (FIRST): where the panels go.
+template <Mode MODE>
+__global__ void __launch_bounds__(threads(MODE), 1)
+bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR, const int32_t* __restrict__ perm,
+                  __nv_bfloat16* __restrict__ U3, float* __restrict__ Y, int M, int K, unsigned char* __restrict__ ext, size_t ext_pitch,
+                  float* __restrict__ ext_min, float* __restrict__ ext_max, int parts, int* status) {
+    constexpr bool FIRST = MODE == FIRST_T, SECOND = MODE == SECOND_T;
+    constexpr int NUM_EPI_WARPS = epi_warps(MODE), NUM_THREADS = threads(MODE), STAGES = stages(MODE);
+    // A: R's block (channels x tokens) or the panels (tokens x channels), both MN-major; B: x, K-major, or R's block, MN-major.
+    // PLAIN: tokens x channels, K-major, and R's block
+    constexpr uint32_t IDESC = umma_idesc_bf16(BM, BN, /*a_mn_major=*/MODE != PLAIN, /*b_mn_major=*/!FIRST);
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
     unsigned char* sA = base;
     unsigned char* sB = base + STAGES * A_STAGE_BYTES;
     Ctl* ctl = reinterpret_cast<Ctl*>(sB + STAGES * B_STAGE_BYTES);
-    const uint32_t sEpi = smem_u32(reinterpret_cast<unsigned char*>(ctl) + sizeof(Ctl));   // NUM_EPI_WARPS x 4 KB
+    const uint32_t sEpi = (smem_u32(reinterpret_cast<unsigned char*>(ctl) + sizeof(Ctl)) + 1023) & ~1023u;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles_m = (M + BM - 1) / BM, tiles_n = (K + BN - 1) / BN;
@@ -69,6 +103,21 @@ bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         tma_prefetch_desc(&tmR);
     }
     if (warp == MMA_WARP) tmem_alloc(smem_u32(&ctl->tmem_base), TMEM_COLS);
+    // FIRST: the rows of the panels that take channel c of u are head[c], next[head[c]], ... (an index map may name a
+    // channel twice or not at all).  perm is not the previous kernel's output.
+    int* head = reinterpret_cast<int*>(base + (sEpi - smem_u32(base)) + NUM_EPI_WARPS * EPI_TILE_BYTES);
+    uint16_t* next = reinterpret_cast<uint16_t*>(head + K);
+    if (FIRST) {
+        for (int i = threadIdx.x; i < K; i += NUM_THREADS) head[i] = NO_ROW;
+        __syncthreads();
+        bool bad = false;
+        for (int i = threadIdx.x; i < K; i += NUM_THREADS) {
+            int c = __ldg(perm + i);
+            if ((uint32_t)c >= (uint32_t)K) { c = 0; bad = true; }
+            next[i] = (uint16_t)atomicExch(&head[c], i);
+        }
+        if (bad) atomicCAS(status, 0, 31);
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -86,16 +135,19 @@ bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             for (int kb = 0; kb < kblocks; ++kb) {
                 ok = mbar_wait_warp(smem_u32(&ctl->empty[s]), ph, &ctl->abort_flag, status, 11);
                 if (!ok) break;
+                const uint32_t bar = smem_u32(&ctl->full[s]);
+                const int k0 = n0 + (kb % (BN / BK)) * BK;    // first of the step's input channels
+                const uint32_t r_dst = smem_u32(FIRST ? sA + s * A_STAGE_BYTES : sB + s * B_STAGE_BYTES);
                 if (lead) {
-                    const uint32_t bar = smem_u32(&ctl->full[s]);
                     mbar_arrive_expect_tx(bar, STAGE_TX_BYTES);
-                    // k origin of this step in the left operand's columns and in R's rows
-                    const int kx = (kb / (BN / BK)) * K + n0 + (kb % (BN / BK)) * BK;
-                    const int kr = n0 + (kb % (BN / BK)) * BK;
-                    tma_load_2d(smem_u32(sA + s * A_STAGE_BYTES), &tmX, kx, m0, bar);
 #pragma unroll
-                    for (int j = 0; j < BN / 64; ++j)
-                        tma_load_2d(smem_u32(sB + s * B_STAGE_BYTES + j * B_CHUNK_BYTES), &tmR, 64 * j, kr, bar);
+                    for (int j = 0; j < BN / 64; ++j) tma_load_2d(r_dst + j * B_CHUNK_BYTES, &tmR, 64 * j, k0, bar);
+                    if (FIRST) tma_load_2d(smem_u32(sB + s * B_STAGE_BYTES), &tmX, k0, m0, bar);
+                    if (MODE == PLAIN) tma_load_2d(smem_u32(sA + s * A_STAGE_BYTES), &tmX, (kb / (BN / BK)) * K + k0, m0, bar);
+                    if (SECOND)
+#pragma unroll
+                        for (int j = 0; j < BM / 64; ++j)
+                            tma_load_2d(smem_u32(sA + s * A_STAGE_BYTES) + j * B_CHUNK_BYTES, &tmX, m0 + 64 * j, (kb / (BN / BK)) * K + k0, bar);
                 }
                 __syncwarp();
                 ++issued;
@@ -114,7 +166,7 @@ bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         __syncwarp();
     } else if (warp == MMA_WARP) {
         const bool lead = elect_one();
-        const uint64_t a0 = umma_desc_sw128(smem_u32(sA), 16, 1024), b0 = umma_desc_sw128(smem_u32(sB), B_CHUNK_BYTES, 1024);
+        const uint64_t a0 = umma_desc_sw128(smem_u32(sA), MODE == PLAIN ? 16 : B_CHUNK_BYTES, 1024), b0 = umma_desc_sw128(smem_u32(sB), FIRST ? 16 : B_CHUNK_BYTES, 1024);
         int s = 0;
         uint32_t ph = 0, t = 0;
         bool ok = true;
@@ -131,8 +183,8 @@ bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
                 if (lead) {
                     const uint64_t a = a0 + (uint64_t)(s * (A_STAGE_BYTES >> 4)), b = b0 + (uint64_t)(s * (B_STAGE_BYTES >> 4));
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)        // 16 k: 32 bytes along a row of X, 16 rows of 128 bytes of R
-                        tc_mma_f16(d_tmem, a + 2 * k, b + 128 * k, IDESC, (kb | k) ? 1u : 0u);
+                    for (int k = 0; k < BK / 16; ++k)        // 16 k: 32 bytes along a row of x, 16 lines of the others
+                        tc_mma_f16(d_tmem, a + (MODE == PLAIN ? 2 : 128) * k, b + (FIRST ? 2 : 128) * k, IDESC, (kb | k) ? 1u : 0u);
                     tc_commit(smem_u32(&ctl->empty[s]));
                 }
                 __syncwarp();
@@ -150,10 +202,65 @@ bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             const int m0 = (tile % tiles_m) * BM, n0 = (tile / tiles_m) * BN;
             const int buf = t & 1;
             const int m = m0 + row;
-            const bool okw = mbar_wait<500>(smem_u32(&ctl->tmem_full[buf]), (t >> 1) & 1, &ctl->abort_flag, status, 14);
+            const bool okw = mbar_wait_warp<500>(smem_u32(&ctl->tmem_full[buf]), (t >> 1) & 1, &ctl->abort_flag, status, 14);
             tc_fence_after();
             float mn = INFINITY, mx = -INFINITY;         // extremes of this row over the tile's columns
-            if (okw) {
+            if (FIRST && okw) {
+                // A lane holds a channel.  The warp's 64 tokens are split, and for each term the warp trades rows for columns
+                // through its tile, so that a store writes four rows' whole 128-byte lines.
+                const uint32_t tile = sEpi + (uint32_t)(warp - EPI_WARP0) * EPI_TILE_BYTES;
+                const int rsub = lane >> 3, jq = lane & 7, c0 = 64 * ((warp - EPI_WARP0) >> 2);
+                if (m0 + c0 < M) {
+                    uint32_t acc[64];
+                    tc_ld32(tmem_base + ((uint32_t)(ew * 32) << 16) + (uint32_t)(buf * BN + c0), acc);
+                    tc_ld32(tmem_base + ((uint32_t)(ew * 32) << 16) + (uint32_t)(buf * BN + c0 + 32), acc + 32);
+                    const int mq = m0 + c0 + 8 * jq;         // M is a multiple of 8: eight tokens or none
+                    int to[8];
+                    bool more = false;                       // a channel that goes to several rows
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        to[i] = mq < M ? head[n0 + ew * 32 + 4 * i + rsub] : NO_ROW;
+                        more |= to[i] != NO_ROW && next[to[i]] != NO_ROW;
+                    }
+                    tc_wait_ld();
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {
+                        __nv_bfloat16* panel = U3 + (size_t)p * K * M + mq;
+                        __syncwarp();
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            uint32_t h[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float a = __uint_as_float(acc[8 * j + 2 * e]), b = __uint_as_float(acc[8 * j + 2 * e + 1]);
+                                h[e] = bf16_pair(a, b);
+                                acc[8 * j + 2 * e] = __float_as_uint(a - __uint_as_float(h[e] << 16));
+                                acc[8 * j + 2 * e + 1] = __float_as_uint(b - __uint_as_float(h[e] & 0xffff0000u));
+                            }
+                            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(tile + (uint32_t)(lane * 128 + ((j ^ (lane & 7)) << 4))),
+                                         "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
+                        }
+                        __syncwarp();
+                        uint4 v[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int r = 4 * i + rsub;
+                            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w)
+                                         : "r"(tile + (uint32_t)(r * 128 + ((jq ^ (r & 7)) << 4))) : "memory");
+                        }
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (to[i] != NO_ROW) *reinterpret_cast<uint4*>(panel + (size_t)to[i] * M) = v[i];
+                        if (more) {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                for (int t2 = to[i] == NO_ROW ? NO_ROW : next[to[i]]; t2 != NO_ROW; t2 = next[t2])
+                                    *reinterpret_cast<uint4*>(panel + (size_t)t2 * M) = v[i];
+                        }
+                    }
+                }
+            }
+            if (!FIRST && okw) {
 #pragma unroll 1
                 for (int c0 = 0; c0 < BN; c0 += 32) {
                     uint32_t acc[32];
@@ -192,7 +299,7 @@ bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctl->tmem_empty[buf]));
-            if (okw && m < M) {                           // this tile's share of the row's extremes
+            if (!FIRST && okw && m < M) {                 // this tile's share of the row's extremes
                 if (ext) {
                     float* e = reinterpret_cast<float*>(ext + (size_t)m * ext_pitch) + 2 * (n0 / BN);
                     e[0] = mn; e[1] = mx;
@@ -210,7 +317,49 @@ bdiag_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     }
 }
 
+
+template <Mode MODE>
+lrq_status launch(const CUtensorMap& tmX, const CUtensorMap& tmR, const int32_t* perm, void* U3, float* Y, int M, int K,
+                  const LrqRowExt& ext, int parts, cudaStream_t st) {
+    int dev = 0, sms = 0;
+    if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
+    {   // the shared-memory opt-in is a per-device function attribute: set once per device
+        static std::mutex mu;
+        static bool configured[LRQ_MAX_DEVICES] = {};
+        std::lock_guard<std::mutex> lock(mu);
+        if (!configured[dev]) {
+            LRQ_CUDA_TRY(cudaFuncSetAttribute(bdiag_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(MODE, MAX_K)));
+            configured[dev] = true;
+        }
+    }
+    const int tiles = ((M + BM - 1) / BM) * (K / BN);
+    const bool one = K == BN;                        // one tile per row: its extremes are the row's
+    LRQ_CUDA_TRY(lrq_launch_pdl(bdiag_gemm_kernel<MODE>, dim3(tiles < sms ? tiles : sms), dim3(threads(MODE)), smem_bytes(MODE, K),
+                                st, tmX, tmR, perm, static_cast<__nv_bfloat16*>(U3), Y, M, K, one ? nullptr : ext.rows, ext.pitch, one ? ext.row_min : nullptr, one ? ext.row_max : nullptr,
+                                parts, lrq_status_word()));
+    return LRQ_OK;
+}
+
 }  // namespace
+
+lrq_status lrq_launch_dual_first(const void* X, int M, int K, long ldx, const void* R1, const int32_t* perm, void* U3, cudaStream_t st) {
+    if ((M % 8) || (K % 128) || K > MAX_K || (ldx % 8) || ldx < K || !lrq_aligned(X, 16) || !lrq_aligned(R1, 16) || !lrq_aligned(U3, 16))
+        return LRQ_ERR_INVALID_ARG;
+    CUtensorMap tmX, tmR;
+    if (!lrq_tma::make_map_2d(&tmX, X, 2, (uint64_t)M, (uint64_t)K, (uint64_t)ldx, BK, BM, true) ||
+        !lrq_tma::make_map_2d(&tmR, R1, 2, (uint64_t)K, 128, 128, 64, BK, true))
+        return LRQ_ERR_CUDA;
+    return launch<FIRST_T>(tmX, tmR, perm, U3, nullptr, M, K, LrqRowExt{}, 1, st);
+}
+
+lrq_status lrq_launch_dual_second(const void* U3, int M, int K, const void* R2, float* Y, const LrqRowExt& ext, cudaStream_t st) {
+    if ((M % 8) || (K % 128) || !lrq_aligned(U3, 16) || !lrq_aligned(R2, 16) || !lrq_aligned(Y, 16)) return LRQ_ERR_INVALID_ARG;
+    CUtensorMap tmU, tmR;
+    if (!lrq_tma::make_map_2d(&tmU, U3, 2, (uint64_t)3 * K, (uint64_t)M, (uint64_t)M, 64, BK, true) ||
+        !lrq_tma::make_map_2d(&tmR, R2, 2, (uint64_t)K, 128, 128, 64, BK, true))
+        return LRQ_ERR_CUDA;
+    return launch<SECOND_T>(tmU, tmR, nullptr, nullptr, Y, M, K, ext, 3, st);
+}
 
 // Y[M,K] (fp32) = sum over panels p of A[:, pK .. pK+K) . blockdiag(Rblk), Rblk bf16 [K/128][128][128].
 lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int parts, const void* Rblk, float* Y, const LrqRowExt& ext,
@@ -219,23 +368,8 @@ lrq_status lrq_launch_bdiag_gemm(const void* A, int M, int K, long lda, int part
         !lrq_aligned(Y, 16))
         return LRQ_ERR_INVALID_ARG;
     CUtensorMap tmA, tmR;
-    if (!lrq_tma::make_map_2d(&tmA, A, 2, (uint64_t)M, (uint64_t)parts * K, (uint64_t)lda, BK, BM, true)) return LRQ_ERR_CUDA;
-    if (!lrq_tma::make_map_2d(&tmR, Rblk, 2, (uint64_t)K, 128, 128, 64, BK, true)) return LRQ_ERR_CUDA;
-    int dev = 0, sms = 0;
-    if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
-    {   // the shared-memory opt-in is a per-device function attribute: set once per device
-        static std::mutex mu;
-        static bool configured[LRQ_MAX_DEVICES] = {};
-        std::lock_guard<std::mutex> lock(mu);
-        if (!configured[dev]) {
-            LRQ_CUDA_TRY(cudaFuncSetAttribute(bdiag_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-            configured[dev] = true;
-        }
-    }
-    const int tiles = ((M + BM - 1) / BM) * (K / BN);
-    const bool one = K == BN;                        // one tile per row: its extremes are the row's
-    LRQ_CUDA_TRY(lrq_launch_pdl(bdiag_gemm_kernel, dim3(tiles < sms ? tiles : sms), dim3(NUM_THREADS), SMEM_BYTES, st, tmA, tmR, Y, M, K,
-                                parts, one ? nullptr : ext.rows, ext.pitch, one ? ext.row_min : nullptr, one ? ext.row_max : nullptr,
-                                lrq_status_word()));
-    return LRQ_OK;
+    if (!lrq_tma::make_map_2d(&tmA, A, 2, (uint64_t)M, (uint64_t)parts * K, (uint64_t)lda, BK, BM, true) ||
+        !lrq_tma::make_map_2d(&tmR, Rblk, 2, (uint64_t)K, 128, 128, 64, BK, true))
+        return LRQ_ERR_CUDA;
+    return launch<PLAIN>(tmA, tmR, nullptr, nullptr, Y, M, K, ext, parts, st);
 }

@@ -39,6 +39,26 @@ def _codes_against_oracle(P, orc, spec, xb, what):
                         "dual", 128, what)
 
 
+@pytest.mark.parametrize("M,K,a_bits", [(8, 128, 8), (64, 256, 4), (136, 384, 8), (200, 1152, 4), (1096, 640, 8), (16, 12288, 4)])
+@pytest.mark.parametrize("repeat", [False, True])
+def test_transposed_panels_match_the_gathering_path(P, M, K, a_bits, repeat):
+    # Batches of a multiple of 8 tokens keep u transposed and reordered between the products; one token more takes the path
+    # with a kernel between them.  Both sum the same products in fp32 in the same order over the same three terms, so the rows
+    # they share come out alike: tokens that end inside and between boxes of 64 and tiles of 128; index maps that name some
+    # channels several times and others never.
+    spec = _spec(M + 1, K, a_bits=a_bits)
+    X = PU.bf16_to_device(spec.activations())
+    Bd, R1, perm, R2 = spec.dual_factors()
+    if repeat:
+        perm = perm.copy()
+        perm[: K // 2] = perm[K // 4: K // 4 + K // 2]
+    dual = PU.dual_to_device(P, (Bd, R1, perm, R2))
+    q0, s0, z0 = P.lrq_rotate_quantize_act(X, P.ROT_DUAL, a_bits, dual=dual)
+    q1, s1, z1 = P.lrq_rotate_quantize_act(X[:M].contiguous(), P.ROT_DUAL, a_bits, dual=dual)
+    assert torch.equal(s0[:M], s1) and torch.equal(z0[:M], z1) and torch.equal(q0[:M], q1)
+    assert P.lrq_device_status() == 0
+
+
 @pytest.mark.parametrize("M,K,a_bits", [(70, 128, 8), (70, 256, 4), (130, 1152, 8), (33, 1536, 4), (300, 3072, 4),
                                         (1, 384, 8), (40, 12288, 4), (130, 6144, 8)])   # the last two: rows above 48 KB
 def test_rotate_quantize_dual(P, orc, M, K, a_bits):

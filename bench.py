@@ -40,16 +40,12 @@ from lrq_workloads import bf16_bits_to_f64, config_layers, default_clip_grid  # 
 # profiles/, keyed by the kernel and layer the roofline object describes.  A key is dropped (traffic: null) when its
 # kernel changes after the capture.
 NCU_TRAFFIC_BYTES = {
-    "qgemm cfg4 b0.fc1": 65.20e6 + 547.50e6,
-    "qgemm cfg3 fc1": 27.10e6 + 169.40e6,
-    "rotq cfg4 b0.fc2": 303.10e6 + 117.94e6,
-    "rotq cfg3 fc2": 113.27e6 + 11.70e6,
-    "rotgemm cfg3 qkv": 51.51e6 + 19.17e6 + 56.67e6 + 0.25e6,
+    "rotq cfg4 b0.fc2": 302.63e6 + 117.40e6,
 }
 
-# sm__pipe_tensor_cycles_active (% of elapsed cycles) of the same captures: the tensor pipe's own view of the
+# sm__pipe_tensor_cycles_active (% of elapsed cycles) of such captures: the tensor pipe's own view of the
 # contraction, beside the fraction of the measured matmul peak that `frac` reports
-NCU_TENSOR_PIPE_PCT = {"qgemm cfg4 b0.fc1": 48.4, "qgemm cfg3 fc1": 54.2}
+NCU_TENSOR_PIPE_PCT = {}
 
 METRIC = "qlinear_tflops"
 UNIT = "TFLOP/s"
@@ -205,7 +201,7 @@ class Workload:
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record()
             # 3-bit codes of a small batch are stored in their true packing (eight codes in three bytes): such a layer
-            # is bound by streaming its weights once, and the small-tile contraction reads that layout
+            # is bound by latency and by streaming its weights once
             layout = P.CODES_PACKED3 if (s.w_bits == 3 and s.M <= 512) else P.CODES_NIBBLE
             tl = P.lrq_tlq_quantize_weights(Wd, s.w_bits, s.group, 7, grid, grid, code_layout=layout)
             e1.record()
@@ -263,7 +259,7 @@ class Workload:
 
     def launches_per_step(self):
         # kernels of this library per step: rotate+quantize and contraction per layer, one more (the rotation GEMM
-        # before its quantizer) per dense layer; the two memsets of a dense rotation are not kernels
+        # before its quantizer) per dense layer
         return 2 * len(self.specs) + sum(1 for s in self.specs if s.rot == "dense")
 
     def close(self):

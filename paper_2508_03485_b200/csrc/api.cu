@@ -249,6 +249,9 @@ namespace {
 enum Form { FORM_PACKED, FORM_EXPANDED };
 Form pick_form(const lrq_layer* L, int M) {
     if (!lrq_qgemm_tc_takes(L)) return FORM_EXPANDED;
+    // a call of one row of tiles on a few thousand weights is bound by its two launches in either form (10 x 64 x 8: 16.5 us
+    // packed, 21.5 expanded, by the host): the smaller workspace
+    if (M <= 256 && (long)L->N * L->K <= 4096) return FORM_PACKED;
     const long tiles = (long)((M + 255) / 256) * ((L->N + 255) / 256);
     const double per_block = L->act.a_bits == 8 ? 0.17 : L->w_bits == 4 ? 0.15 : 0.06;
     const double in_tiles_us = 3.0 + (double)((tiles + 73) / 74) * (L->K / 64) * per_block;

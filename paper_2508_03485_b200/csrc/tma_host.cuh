@@ -55,4 +55,17 @@ inline bool make_map_rows_bf16(CUtensorMap* tm, const void* ptr, uint64_t rows, 
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Row-major bf16 matrix [rows, 128 * blocks] seen as [rows][blocks][128]: one copy brings 64 channels (x = 0 or 64) of every block
+// of `box_rows` rows as consecutive 128-byte lines, swizzled as above.
+inline bool make_map_blocks_bf16(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t blocks, uint64_t ld, uint32_t box_rows) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc || blocks > 256 || box_rows < 1 || box_rows > 256) return false;
+    const cuuint64_t dims[3] = {128, blocks, rows};
+    const cuuint64_t strides[2] = {256, ld * 2};
+    const cuuint32_t box[3] = {64, (cuuint32_t)blocks, box_rows};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace lrq_tma

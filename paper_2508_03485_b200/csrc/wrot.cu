@@ -2,14 +2,15 @@
 // Sec. 5.1 folded in: W_rot = W diag(colmul) R, evaluated in fp64 and rounded once to fp32, which is what
 // the TLQ quantizer reads.
 //
-// Offline step.  Hadamard: one CTA per weight row, butterflies in registers, up to four stages between two trips
-// through shared memory.  Dense: an fp64 matrix product on the fp64 tensor cores, 64 x 64 output tiles, for small
+// Offline step.  Hadamard: butterflies in registers, up to four stages between two trips through shared memory, by warps of their own
+// (blocks of 16 to 256 channels) or one CTA per weight row.  Dense: an fp64 matrix product on the fp64 tensor cores, 64 x 64 output tiles, for small
 // layers and for callers without scratch (wrot_i8.cu otherwise); R is the layer's stored bf16 matrix (exact in fp64), so both
 // sides of Eq. 2 use the same R.  Dual transformation (R = R1hat P R2hat, Sec. 4.2): one CTA per row, the
 // row in shared memory as fp64, block-diagonal product, gather through the index map, second product.
 #include "lrq_internal.cuh"
 
 #include <cuda_bf16.h>
+#include <cmath>
 
 namespace {
 
@@ -43,7 +44,7 @@ __device__ __forceinline__ void hadamard_pass(double* row, int K, int bit, const
     __syncthreads();
 }
 
-// 4608 x 1152, B = 128: 34 us with a barrier and a trip through shared memory per stage, 17 now.
+// Any block, any alignment: a CTA per row.
 __global__ void __launch_bounds__(128)
 wrot_hadamard_kernel(const float* __restrict__ W, int N, int K, long ldw, const float* __restrict__ colmul, int log2B,
                      float* __restrict__ out, long ldo) {
@@ -67,6 +68,71 @@ wrot_hadamard_kernel(const float* __restrict__ W, int N, int K, long ldw, const 
         else hadamard_pass<0>(row, K, bit, src, colmul, dst, norm);
         bit += nb;
     } while (bit < log2B);
+}
+
+// Blocks of 16 to 256 channels: a warp by itself takes 512 consecutive elements of the matrix (whole blocks, of one row or two), a
+// lane 16 of them with 128-bit loads: stages 0-3 in its registers, one exchange through the warp's shared memory (a pad after
+// every 16 doubles: conflict-free both ways), the other one to four stages at stride 16.  The kernel above keeps a CTA per row,
+// whose 128 threads a row of 1152 fills to 0.56, and has barriers.  The same additions in the same order, the same results.
+// 4608 x 1152, B = 128: 27.5 us there with a cold L2, 15.2 here (2.8 TB/s); 2600 x 6144 61.4 and 30.7 (4.2 TB/s); 9216 x 1728, B = 64
+// 58 and 36; 1024 x 3072, B = 256 17.8 and 12.3; 512 x 512 8.2 both.  Bound by the fp64 conversions and additions on the way.
+template <int LOG2B>
+__global__ void __launch_bounds__(256)
+wrot_hadamard_warp_kernel(const float* __restrict__ W, unsigned items, unsigned items_per_row, long ldw, const float* __restrict__ colmul,
+                          double norm, float* out, long ldo) {
+    constexpr int NB = LOG2B - 4, E = 1 << NB;
+    __shared__ double smem[8][32 * 17];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* s = smem[warp];
+    lrq_pdl_trigger();
+    lrq_pdl_wait();
+    for (unsigned first = (blockIdx.x * 8 + warp) * 32; first < items; first += gridDim.x * 256) {
+        const unsigned item = first + lane;
+        double v[16];
+        if (item < items) {
+            const unsigned n = item / items_per_row, k = (item - n * items_per_row) * 16;
+            const float4* w = reinterpret_cast<const float4*>(W + n * ldw + k);
+            float4 f[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) f[i] = w[i];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { v[4 * i] = f[i].x; v[4 * i + 1] = f[i].y; v[4 * i + 2] = f[i].z; v[4 * i + 3] = f[i].w; }
+            if (colmul) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 c = __ldg(reinterpret_cast<const float4*>(colmul + k) + i);
+                    v[4 * i] *= (double)c.x; v[4 * i + 1] *= (double)c.y; v[4 * i + 2] *= (double)c.z; v[4 * i + 3] *= (double)c.w;
+                }
+            }
+#pragma unroll
+            for (int h = 1; h < 16; h <<= 1)
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                    if (!(e & h)) { const double a = v[e], b = v[e | h]; v[e] = a + b; v[e | h] = a - b; }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) s[lane * 17 + e] = v[e];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 16 / E; ++q) {
+            const int id = q * 32 + lane, i = id & 15, r = (id >> 4) * E;      // element i of items r .. r + E - 1: one block
+            if (first + r < items) {
+                double u[E];
+#pragma unroll
+                for (int e = 0; e < E; ++e) u[e] = s[(r + e) * 17 + i];
+#pragma unroll
+                for (int h = 1; h < E; h <<= 1)
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (!(e & h)) { const double a = u[e], b = u[e | h]; u[e] = a + b; u[e | h] = a - b; }
+                const unsigned n = (first + r) / items_per_row, k = (first + r - n * items_per_row) * 16 + i;
+                float* o = out + n * ldo + k;
+#pragma unroll
+                for (int e = 0; e < E; ++e) o[16 * e] = (float)(u[e] * norm);
+            }
+        }
+        __syncwarp();                              // read before the next elements are written
+    }
 }
 
 // Dense rotation: out[N,K] = (W diag(colmul)) . R in fp64 on the tensor cores (mma m8n8k4).  A CTA of four warps owns a
@@ -226,6 +292,17 @@ lrq_status lrq_launch_rotate_weights(const float* W, int N, int K, long ldw, con
     if (kind == LRQ_ROT_HADAMARD) {
         int log2B = 0;
         while ((1 << log2B) < had_block) ++log2B;
+        // 16-byte aligned rows of whole blocks of 16 to 256 channels; the result may stand in the place of W
+        if (log2B >= 4 && log2B <= 8 && ldw % 4 == 0 && lrq_aligned(W, 16) && (!colmul || lrq_aligned(colmul, 16)) && (long)N * (K / 16) < (1l << 31)) {
+            static constexpr decltype(&wrot_hadamard_warp_kernel<4>) kerns[] = {wrot_hadamard_warp_kernel<4>, wrot_hadamard_warp_kernel<5>, wrot_hadamard_warp_kernel<6>,
+                                                                                wrot_hadamard_warp_kernel<7>, wrot_hadamard_warp_kernel<8>};
+            int sms = 0;
+            if (lrq_current_device(nullptr, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
+            const unsigned items = (unsigned)N * (unsigned)(K / 16), ctas = (items + 255) / 256, most = (unsigned)sms * 5;
+            const double norm = ldexp((log2B & 1) ? 0.70710678118654752440 : 1.0, -(log2B >> 1));
+            LRQ_CUDA_TRY(lrq_launch_pdl(kerns[log2B - 4], dim3(ctas < most ? ctas : most), dim3(256), 0, st, W, items, (unsigned)(K / 16), ldw, colmul, norm, out, ldo));
+            return LRQ_OK;
+        }
         // one pad after every 16 elements; the opt-in is the same for every K, since another host thread's call sets it too
         constexpr int MAX_K = 25600;
         auto row_bytes = [](int k) { return (size_t)(k + k / 16 + 1) * sizeof(double); };

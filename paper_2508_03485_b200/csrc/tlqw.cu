@@ -22,8 +22,10 @@
 //   * levels have 8-bit significands: fp32 numbers, and the upper word of the double is the level.
 // 31 factors a side, 4 bits: 4608 x 1152 545 us with the fp64 expression for every element and factor, 169 with fp32 sums over
 // every element, 80 with bins; 2048 x 6144 485 and 122; 512 x 12288 685 and 96.  4608 x 1536 in groups of 128: 315 with fp32
-// sums, 398 with bins; of 256 (4608 x 2048): 326 and 304.
+// sums, 398 with bins; of 256 (4608 x 2048): 326 and 304.  These sums take two elements per instruction where there is one for it
+// (four of the eleven an element): 3 bits, groups of 128, 303 -> 293.
 #include "lrq_internal.cuh"
+#include "f32x2.cuh"
 #include <climits>
 #include <type_traits>
 
@@ -395,7 +397,9 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
             if constexpr (NB == 0) {
                 // ---- every factor's error in fp32 (terms within 3 u of the exact ones, eight partial sums of at most
                 // scnt / 8 + chunk remainders terms), which leaves the factors within twice its bound of the smallest
-                float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                using namespace lrq_f2;
+                f32x2 part[4] = {0ull, 0ull, 0ull, 0ull};    // pairs: one instruction for two elements
+                const f32x2 INV = pack2(fc.inv, fc.inv), NEGZ = pack2(fc.negz, fc.negz), MAGIC2 = pack2(kMagic, kMagic);
                 float rest = 0.f;
                 auto term = [&](int j, float r) {
                     float L;
@@ -409,25 +413,29 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
 #pragma unroll
                     for (int u = 0; u < U; u += 4) {
                         const float4 l4 = *reinterpret_cast<const float4*>(&lg[sd][j + u]);
-                        const float l[4] = {l4.x, l4.y, l4.z, l4.w};
+                        const f32x2 l[2] = {pack2(l4.x, l4.y), pack2(l4.z, l4.w)};
 #pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            const float x = fmaf(l[h], fc.inv, fc.negz);
-                            r[u + h] = x + kMagic;
-                            off = fmaxf(off, fabsf(x - (r[u + h] - kMagic)));
+                        for (int h = 0; h < 2; ++h) {
+                            const f32x2 x = fma2(l[h], INV, NEGZ), rr = add2(x, MAGIC2);
+                            float d0, d1;
+                            unpack2(sub2(x, sub2(rr, MAGIC2)), d0, d1);
+                            unpack2(rr, r[u + 2 * h], r[u + 2 * h + 1]);
+                            off = max3(off, fabsf(d0), fabsf(d1));
                         }
                     }
                     if (off <= fc.thr) {
 #pragma unroll
                         for (int u = 0; u < U; u += 4) {
                             const float4 a4 = *reinterpret_cast<const float4*>(&mag[sd][j + u]);
-                            const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+                            const f32x2 a[2] = {pack2(a4.x, a4.y), pack2(a4.z, a4.w)};
+                            float L[4];
 #pragma unroll
-                            for (int h = 0; h < 4; ++h) {
-                                float L;
-                                asm("ld.shared.f32 %0, [%1];" : "=f"(L) : "r"(f32_0 + (__float_as_uint(fminf(r[u + h], fc.top)) << 7)));
-                                const float d = a[h] - L;
-                                part[u + h] = fmaf(d, d, part[u + h]);
+                            for (int h = 0; h < 4; ++h)
+                                asm("ld.shared.f32 %0, [%1];" : "=f"(L[h]) : "r"(f32_0 + (__float_as_uint(fminf(r[u + h], fc.top)) << 7)));
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const f32x2 d = sub2(a[h], pack2(L[2 * h], L[2 * h + 1]));
+                                part[u / 2 + h] = fma2(d, d, part[u / 2 + h]);
                             }
                         }
                     } else {
@@ -443,7 +451,10 @@ tlq_quantize_kernel(const float* __restrict__ W, int N, int K, int G, int bits, 
 #pragma unroll 1
                     for (; j < n_el; ++j) term(j, code_of(j));
                 }
-                const float e32 = (((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]))) + rest;
+                float ps[8];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) unpack2(part[i], ps[2 * i], ps[2 * i + 1]);
+                const float e32 = (((ps[0] + ps[1]) + (ps[2] + ps[3])) + ((ps[4] + ps[5]) + (ps[6] + ps[7]))) + rest;
                 // errors are not negative, so their bit patterns are ordered as the numbers; NaN sorts above them all
                 const float emin = __uint_as_float(__reduce_min_sync(0xffffffffu, ok ? __float_as_uint(e32) : 0x7fffffffu));
                 const float eps = (float)(scnt / 8 + 3 * (G / kChunk + 1) + 64) * 2.4e-7f;      // 4 u per term of the longest sum

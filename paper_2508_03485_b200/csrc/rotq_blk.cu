@@ -1,5 +1,5 @@
 // Rotation + per-token activation quantization (Sec. 4.2 Eq. 12, first case; Sec. 3.1 Eq. 1): the kernel for
-// Hadamard blocks of up to 128 channels, the block size of the DiT workloads.
+// Hadamard blocks of up to 128 channels (long batches of 128 without multipliers: rotq_tc.cu).
 //
 // HBM-bound by intent: each activation is read once (bf16) and written once as a 4- or 8-bit code.  What the
 // kernel has to hide is not bandwidth but latency: a token's range is known only after every thread that holds a

@@ -68,6 +68,13 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t* r) {
 }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// Waits for this thread's TMEM loads; as operands, the loaded registers cannot be read ahead of it.
+#define LRQ_W4(r, i) "+r"(r[i]), "+r"(r[i + 1]), "+r"(r[i + 2]), "+r"(r[i + 3])
+#define LRQ_W8(r, i) LRQ_W4(r, i), LRQ_W4(r, i + 4)
+__device__ __forceinline__ void tc_wait_ld32(uint32_t* r) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : LRQ_W8(r, 0), LRQ_W8(r, 8), LRQ_W8(r, 16), LRQ_W8(r, 24) :: "memory");
+}
+
 // Stages 7 .. 6 + LOGU of the transform over 32 blocks: butterflies between a thread's columns.
 template <int LOGU>
 __device__ __forceinline__ void butterflies(uint32_t* r) {
@@ -368,7 +375,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                     for (int c = 0; c < COLS; c += 32) {
                         uint32_t r[32];
                         tc_ld32(acc + c, r);
-                        tc_wait_ld();
+                        tc_wait_ld32(r);
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             mn4[j & 3] = min3(mn4[j & 3], __uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
@@ -387,7 +394,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 for (int c = 0; ok && c < cols; c += 32) {
                         uint32_t r[32];
                         tc_ld32(acc + c, r);
-                        tc_wait_ld();
+                        tc_wait_ld32(r);
                         butterflies<LOGU>(r);
                         tc_st32(acc + c, r);
 #pragma unroll
@@ -447,7 +454,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                         for (int h = 0; h < STEP / 32; ++h) {
                             uint32_t r[32];
                             tc_ld32(acc + c + 32 * h, r);
-                            tc_wait_ld();
+                            tc_wait_ld32(r);
                             code_row32<A_BITS, OUT16>(r, q, fast, a_bits, o + h * W32);
                         }
                         if (live)
@@ -462,7 +469,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 for (int c = 0; c < cols; c += 32) {
                     uint32_t r[32];
                     tc_ld32(acc + c, r);
-                    tc_wait_ld();
+                    tc_wait_ld32(r);
 #pragma unroll
                     for (int u = 0; u < 32; u += V)
                         if (c + u < cols) {

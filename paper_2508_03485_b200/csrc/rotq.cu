@@ -820,7 +820,7 @@ static lrq_status launch_fast(const void* X, int M, int K, long ldx, int a_bits,
 
 lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                                     uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
-    // long batches of some blocks: the transform on the tensor cores (rotq_tc.cu)
+    // long batches of blocks of 128 channels: the transform on the tensor cores (rotq_tc.cu)
     {
         const lrq_status r = lrq_launch_rotq_tc(X, M, K, ldx, B, a_bits, mode, out16, prescale, codes, scale, zp, ex, st);
         if (r != LRQ_ERR_UNSUPPORTED) return r;

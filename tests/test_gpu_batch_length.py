@@ -1,0 +1,47 @@
+"""A token's codes, step and zero-point do not depend on the batch it is in, nor on the tokens beside it."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2508_03485_b200 as P
+    P.load_library()
+    return P
+
+
+def _tokens(M, K, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    X = torch.randn((M, K), generator=g, device="cuda")
+    return torch.where(torch.rand(X.shape, generator=g, device="cuda") < 0.005, X * 5, X).bfloat16()
+
+
+@pytest.mark.parametrize("K,B,a_bits,symmetric", [(2048, 2048, 4, False), (6144, 2048, 8, True), (10240, 2048, 8, False), (4096, 4096, 8, False),
+                                                  (12288, 4096, 4, False)])
+def test_large_blocks_in_long_and_short_batches(P, K, B, a_bits, symmetric):
+    M = 12_100_000 // K + 2
+    X = _tokens(M, K, K + B)
+    # inputs over 16 octaves, whose sums are rounded at every stage
+    X[:16] = (torch.sign(X[:16].float()) * torch.exp2(-16 * torch.rand((16, K), device="cuda"))).bfloat16()
+    # sums that overflow, in the block's first blocks of 128 channels to +inf, -inf, +inf, +inf: NaN for every other channel two
+    # stages on, among finite values
+    X[20, :512] = 0
+    for i, v in enumerate((3e38, -3e38, 3e38, 3e38)):
+        X[20, 128 * i:128 * i + 2] = v
+    X[21, 5] = float("inf"); X[22, 7] = float("nan"); X[23] = float("nan"); X[24] = 0
+    mode = P.ACT_SYM if symmetric else P.ACT_ASYM
+    long = P.lrq_rotate_quantize_act(X, P.ROT_HADAMARD, a_bits, B, mode=mode)
+    for i in (0, M // 2, M - 64):
+        for a, b in zip(long, P.lrq_rotate_quantize_act(X[i:i + 64], P.ROT_HADAMARD, a_bits, B, mode=mode)):
+            assert torch.equal(a[i:i + 64], b)
+    # the contraction's operand: no NaN of an overflow in it
+    g = torch.Generator(device="cuda").manual_seed(7)
+    tlq = P.lrq_tlq_quantize_weights(0.02 * torch.randn((32, K), generator=g, device="cuda"), 4, 0, 7, [1.0, 1.2], [1.0, 1.2])
+    layer = P.QLayer(tlq, 32, K, P.ROT_HADAMARD, a_bits, B, mode=mode)
+    Y = P.lrq_qlinear(layer, X, P.F32)
+    assert torch.isfinite(Y[20]).all() and torch.equal(Y[20], P.lrq_qlinear(layer, X[:64], P.F32)[20])
+    assert P.lrq_device_status() == 0

@@ -42,6 +42,7 @@ constexpr size_t RING_BYTES = 168 * 1024;
 struct __align__(16) Ctl {
     uint64_t full[MAX_STAGES], empty[MAX_STAGES];
     uint64_t acc_full[BUFS], acc_empty[BUFS];
+    uint64_t drain;                                          // the MMAs that an abandoned step left in flight
     uint32_t tmem_base;
     volatile int abort_flag;
     alignas(16) float4 par[GROUPS][MAX_TOK];                 // a token's parameters (make_code)
@@ -154,6 +155,12 @@ __device__ __forceinline__ void stg256(uint8_t* p, const uint32_t* o) {
                  :: "l"(p), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
 }
 
+// Bounded wait of the unwinding after an abort; what it waits for was issued long ago.
+__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity) {
+    const long long t0 = clock64();
+    while (!mbar_try_wait(bar, parity) && clock64() - t0 < kWaitCycles / 8) {}
+}
+
 template <int A_BITS, bool OUT16>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const LrqExpand ex) {
@@ -167,6 +174,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl->full[s]), 1); mbar_init(smem_u32(&ctl->empty[s]), 1); }
         for (int b = 0; b < BUFS; ++b) { mbar_init(smem_u32(&ctl->acc_full[b]), 1); mbar_init(smem_u32(&ctl->acc_empty[b]), GROUP_WARPS); }
+        mbar_init(smem_u32(&ctl->drain), 1);
         ctl->abort_flag = 0;
         mbar_init_fence();
         tma_prefetch_desc(&tmX);
@@ -192,15 +200,15 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
     lrq_pdl_wait();                      // X may be the previous kernel's output; the code buffer may still be read by it
 
     const int mine = (int)blockIdx.x < p.steps ? (p.steps - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;   // this CTA's steps
+    bool lead = false;                   // the thread of the TMA or MMA warp that issues
+    int issued = 0;                      // steps that it has issued
     if (warp >= TMA_WARP) {
         if (warp == TMA_WARP) {
-            const bool lead = elect_one();
-            int s = 0, issued = 0;
+            lead = elect_one();
+            int s = 0;
             uint32_t ph = 1;
-            bool ok = true;
             for (int i = 0; i < mine; ++i) {
-                ok = mbar_wait_warp(smem_u32(&ctl->empty[s]), ph, &ctl->abort_flag, p.status, 51);
-                if (!ok) break;
+                if (!mbar_wait_warp(smem_u32(&ctl->empty[s]), ph, &ctl->abort_flag, p.status, 51)) break;
                 if (lead) {
                     const int m0 = ((int)blockIdx.x + i * (int)gridDim.x) * p.T;
                     const uint32_t bar = smem_u32(&ctl->full[s]), dst = sX + s * stage_bytes;
@@ -212,14 +220,9 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 ++issued;
                 if (++s == p.stages) { s = 0; ph ^= 1; }
             }
-            if (!ok && issued) {
-                // copies in flight still write this CTA's shared memory: a millisecond to land before the CTA ends
-                const long long t0 = clock64();
-                while (clock64() - t0 < 2000000) __nanosleep(1000);
-            }
             __syncwarp();
         } else if (warp == MMA_WARP) {
-            const bool lead = elect_one();
+            lead = elect_one();
             // the tokens' blocks are the 128 lanes, the channels of a block the columns
             const uint64_t h0 = umma_desc_sw128(sH, 16, 1024), x0 = umma_desc_sw128(sX, 16, 1024);
             const uint32_t idesc = umma_idesc_bf16(128, COLS, false, false);
@@ -242,6 +245,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                     tc_commit(smem_u32(&ctl->acc_full[b]));
                 }
                 __syncwarp();
+                ++issued;
                 if (++s == p.stages) { s = 0; ph ^= 1; }
             }
             __syncwarp();
@@ -339,6 +343,17 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
     if (ex.out) lrq_dec::expand_share(ex);
     tc_fence_before();
     __syncthreads();
+    if (ctl->abort_flag) {
+        // A wait ran out, in whatever role, so that copies may still write this CTA's shared memory and MMAs its TMEM: both
+        // end (bounded) before either is given back.  Otherwise every copy and MMA has been waited for above.
+        if (lead && warp == TMA_WARP)
+            for (int i = max(issued - p.stages, 0); i < issued; ++i) drain(smem_u32(&ctl->full[i % p.stages]), (uint32_t)(i / p.stages) & 1u);
+        if (lead && warp == MMA_WARP && issued) {
+            tc_commit(smem_u32(&ctl->drain));
+            drain(smem_u32(&ctl->drain), 0);
+        }
+        __syncthreads();
+    }
     if (warp == MMA_WARP) {
         tc_fence_after();
         tmem_dealloc(tmem_base, BUFS * COLS);

@@ -315,7 +315,7 @@ rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode,
             const float a = fminf(min3(mn4[0], mn4[1], mn4[2]), mn4[3]), b = fmaxf(max3(mx4[0], mx4[1], mx4[2]), mx4[3]);
             float c = fminf(min3(mnd[0], mnd[1], mnd[2]), mnd[3]), d = fmaxf(max3(mxd[0], mxd[1], mxd[2]), mxd[3]);
             if (odd) { const float t0 = -d; d = -c; c = t0; }          // true values of the odd thread's upper half
-            mn = fminf(a, c); mx = fmaxf(b, d);
+            mn = fminf(fminf(a, c), INFINITY); mx = fmaxf(fmaxf(b, d), -INFINITY);   // NaN (a block of nothing else) has no part in the range
         }
         // one redux per warp segment; the segment's first lane publishes the part's extremes
         const uint32_t tok_ext = ext0 + (uint32_t)(((it & 1) * ext_tok + tl) * sub_warps) * 8u;
@@ -344,6 +344,7 @@ rotq_blk_kernel(const __grid_constant__ CUtensorMap tmX, int M, int K, int mode,
                     lds_f2(tok_ext + 8u * w, a2, b2);
                     a = fminf(a, a2); b = fmaxf(b, b2);
                 }
+                if (a > b) a = b = NAN;              // a token of NaN alone: an empty range
                 t = token_params_f32<A_BITS>(a, b, mode, scale_mul, nrm, &scv, &z);
                 if (jh == 0 && live) { scale[m] = scv; zp[m] = OUT16 ? z + Centre<A_BITS>(t.negz).c : z; }
             }

@@ -300,8 +300,8 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 auto fold = [&](float2 e) { mn = fminf(mn, e.x); mx = fmaxf(mx, e.y); none = none || !(e.x <= e.y); };
 #pragma unroll 1
                 for (int w = w_first; w <= w_last; ++w) { fold(ext[w * MAX_TOK + gt]); none = none || ctl->none[g][w * MAX_TOK + gt]; }
-                // A NaN among a block's inputs is in all of its outputs.  It is kept out of the token's range, as rotq_blk.cu does for
-                // tokens of more than a warp.  A token of nothing else has no range in either.
+                // A NaN among a block's inputs is in all of its outputs.  It is kept out of the token's range, as in rotq_blk.cu.  A
+                // token of nothing else has no range in either.
                 const bool plain = !none && mn > -INFINITY && mx < INFINITY;
                 if (none && mn > mx) { mx = NAN; if (mn == INFINITY) mn = NAN; }
                 float sc; int32_t z;

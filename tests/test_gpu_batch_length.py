@@ -45,3 +45,30 @@ def test_large_blocks_in_long_and_short_batches(P, K, B, a_bits, symmetric):
     Y = P.lrq_qlinear(layer, X, P.F32)
     assert torch.isfinite(Y[20]).all() and torch.equal(Y[20], P.lrq_qlinear(layer, X[:64], P.F32)[20])
     assert P.lrq_device_status() == 0
+
+
+@pytest.mark.parametrize("symmetric", [False, True])
+@pytest.mark.parametrize("K,B", [(128, 8), (384, 16), (2048, 64), (1152, 128), (4608, 128), (12288, 128)])
+def test_nan_of_a_small_block_has_no_part_in_the_range(P, K, B, symmetric):
+    # A NaN makes its block NaN.  The block takes code 0, the others are coded as if it were zeros; whether the NaN's threads share
+    # their warp with the whole token, with the element that sets its range, or with neither.
+    X = _tokens(70, K, K)
+    X[:, K - 1] = 30
+    X[:, 0] = -30
+    at = {3: 1, 4: K // 2, 5: K - B - 1, 37: K // 2 + 1}
+    clean = X.clone()
+    for m, k in at.items():
+        X[m, k] = float("nan")
+        clean[m, k // B * B:k // B * B + B] = 0
+    X[40] = float("nan")                               # nothing else: unit step
+    mode = P.ACT_SYM if symmetric else P.ACT_ASYM
+    for a_bits in (8, 4):
+        (q, s, z), (q1, s1, z1) = (P.lrq_rotate_quantize_act(t, P.ROT_HADAMARD, a_bits, B, mode=mode) for t in (X, clean))
+        if a_bits == 4:
+            q, q1 = (torch.stack([t & 15, t >> 4], -1).reshape(70, -1) for t in (q, q1))
+        others = [m for m in range(70) if m != 40]
+        assert torch.equal(s[others], s1[others]) and torch.equal(z[others], z1[others]) and s[40] == 1
+        for m, k in at.items():
+            q1[m, k // B * B:k // B * B + B] = 0
+        assert torch.equal(q[others], q1[others])
+    assert P.lrq_device_status() == 0

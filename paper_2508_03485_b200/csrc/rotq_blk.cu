@@ -78,45 +78,6 @@ __device__ __forceinline__ f32x2 shfl_xor2(f32x2 v, int m) {
     return pack2(__shfl_xor_sync(0xffffffffu, a, m), __shfl_xor_sync(0xffffffffu, b, m));
 }
 
-// Step and zero-point of a token (Eq. 1) from its extremes, in fp32 with error-free corrections, for the common
-// case; the fp64 routine takes over when the token's range is degenerate or when min/s comes within 2e-3 of a
-// rounding boundary, so that the zero-point is always the one exact arithmetic gives.  The reciprocal step is
-// refined from the hardware approximation against the exact range (max - min as an unevaluated sum hi + lo), which
-// leaves it within an ulp of the correctly rounded value: the same accuracy as rounding the fp64 result.
-// scale_mul = nrm / qsteps rounded to fp32.
-template <int A_BITS>
-__device__ __forceinline__ TokenQ token_params_f32(float mn, float mx, int mode, float scale_mul, double nrm,
-                                                   float* scale_out, int32_t* zp_out) {
-    const bool asym = mode == LRQ_ACT_ASYM;
-    const float qs = asym ? (float)((1 << A_BITS) - 1) : (float)((1 << (A_BITS - 1)) - 1);
-    float hi, lo;
-    if (asym) {
-        hi = mx - mn;                                          // TwoSum(mx, -mn): hi + lo is the exact range
-        const float bv = hi - mx;
-        lo = (mx - (hi - bv)) + (-mn - bv);
-    } else {
-        hi = fmaxf(fabsf(mn), fabsf(mx)); lo = 0.f;
-    }
-    if (hi > 1e-30f && hi < 1e30f) {
-        float r;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(hi));
-        float inv = qs * r;
-        float e = fmaf(-hi, inv, qs);
-        e = fmaf(-lo, inv, e);
-        inv = fmaf(e, r, inv);
-        const float p = mn * inv, zr = rintf(p);
-        if (!asym || fabsf(fabsf(p - zr) - 0.5f) > 2e-3f) {
-            const float z = asym ? zr : -(float)(1 << (A_BITS - 1));
-            *scale_out = hi * scale_mul;
-            *zp_out = (int32_t)z;
-            TokenQ t;
-            t.inv = inv; t.negz = -z;
-            return t;
-        }
-    }
-    return token_params_fast(mn, mx, A_BITS, mode, nrm, scale_out, zp_out);
-}
-
 // 32 consecutive values (16 pairs) from channel e of the code matrix on -> codes; A8: 32 bytes (two 128-bit stores),
 // A4: 16 bytes (one), OUT16 (the contraction's centred bf16 operand): 64 bytes (two 256-bit stores, whole sectors)
 template <int A_BITS, bool OUT16>

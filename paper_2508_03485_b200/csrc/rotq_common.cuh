@@ -90,6 +90,45 @@ __device__ __forceinline__ TokenQ token_params_fast(float mn, float mx, int a_bi
     return t;
 }
 
+// Step and zero-point of a token (Eq. 1) from its extremes, in fp32 with error-free corrections, for the common
+// case; the fp64 routine takes over when the token's range is degenerate or when min/s comes within 2e-3 of a
+// rounding boundary, so that the zero-point is always the one exact arithmetic gives.  The reciprocal step is
+// refined from the hardware approximation against the exact range (max - min as an unevaluated sum hi + lo), which
+// leaves it within an ulp of the correctly rounded value: the same accuracy as rounding the fp64 result.
+// scale_mul = nrm / qsteps rounded to fp32.
+template <int A_BITS>
+__device__ __forceinline__ TokenQ token_params_f32(float mn, float mx, int mode, float scale_mul, double nrm,
+                                                   float* scale_out, int32_t* zp_out) {
+    const bool asym = mode == LRQ_ACT_ASYM;
+    const float qs = asym ? (float)((1 << A_BITS) - 1) : (float)((1 << (A_BITS - 1)) - 1);
+    float hi, lo;
+    if (asym) {
+        hi = mx - mn;                                          // TwoSum(mx, -mn): hi + lo is the exact range
+        const float bv = hi - mx;
+        lo = (mx - (hi - bv)) + (-mn - bv);
+    } else {
+        hi = fmaxf(fabsf(mn), fabsf(mx)); lo = 0.f;
+    }
+    if (hi > 1e-30f && hi < 1e30f) {
+        float r;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(hi));
+        float inv = qs * r;
+        float e = fmaf(-hi, inv, qs);
+        e = fmaf(-lo, inv, e);
+        inv = fmaf(e, r, inv);
+        const float p = mn * inv, zr = rintf(p);
+        if (!asym || fabsf(fabsf(p - zr) - 0.5f) > 2e-3f) {
+            const float z = asym ? zr : -(float)(1 << (A_BITS - 1));
+            *scale_out = hi * scale_mul;
+            *zp_out = (int32_t)z;
+            TokenQ t;
+            t.inv = inv; t.negz = -z;
+            return t;
+        }
+    }
+    return token_params_fast(mn, mx, A_BITS, mode, nrm, scale_out, zp_out);
+}
+
 // Smoothing multipliers (Sec. 5.1) in shared memory, laid out so that threads which own runs of 4 * PER consecutive channels
 // read them without conflicts: float4 i of thread j at i * tpt + j.  Read from global memory as they lie, a warp's 128-bit
 // loads touched 32 lines each, once per token (32768 x 4608, B = 128: 227 us against 106 without multipliers, 139 now).

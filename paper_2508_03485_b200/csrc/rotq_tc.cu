@@ -54,6 +54,7 @@ static_assert(SMEM_MAX <= 227 * 1024, "shared memory budget");
 
 struct Params {
     int M, K, nb, T, steps, stages, mode, a_bits;
+    float scale_mul;                                         // token_params_f32
     uint8_t* codes; float* scale; int32_t* zp; int* status;
 };
 
@@ -73,23 +74,21 @@ __device__ __forceinline__ bool group_bar_or(int id, bool pred) {
 }
 
 // How a token's values become codes.  fast: every value lies between the token's extremes, and both of these have their codes within
-// 0 .. 2^b - 1 (and there is nothing else in the token): then no value needs the clamp, and y / s - z + 1.5 * 2^23, one fused
-// multiply-add, is the code in the low bits of a float, rounded once (elsewhere y / s - z is rounded to fp32 first: of 2048 x 4608
-// codes of 8 bits 47 were off the fp64 ones, 6 are now).  x: 1 / s, y: -z, z: from that float to the operand, w: 1.5 * 2^23 - z, or
-// 0: not fast.
+// 0 .. 2^b - 1 (and there is nothing else in the token): then no value needs the clamp, and y / s - z, rounded to fp32, plus 1.5 * 2^23 is
+// the code in the low bits of a float.  Either way a code is the same one, that of the other kernels, whatever tokens are beside it.
+// x: 1 / s, y: -z, z: from that float to the operand, w: fast.
 constexpr float MAGIC = 12582912.f;
 __device__ __forceinline__ float4 make_code(TokenQ q, float mn, float mx, float qmax, bool plain) {
-    const float c = fminf(fmaxf(q.negz, 0.f), qmax), w = MAGIC + q.negz;
-    const float lo = fmaf(mn, q.inv, w) - MAGIC, hi = fmaf(mx, q.inv, w) - MAGIC;
-    const bool fast = plain && fabsf(q.negz) < 1048576.f && lo >= 0.f && hi <= qmax;
-    return make_float4(q.inv, q.negz, -MAGIC - c, fast ? w : 0.f);
+    const float c = fminf(fmaxf(q.negz, 0.f), qmax);
+    const float lo = fmaf(mn, q.inv, q.negz) + MAGIC, hi = fmaf(mx, q.inv, q.negz) + MAGIC;
+    return make_float4(q.inv, q.negz, -MAGIC - c, plain && lo >= MAGIC && hi <= MAGIC + qmax ? 1.f : 0.f);
 }
 
 __device__ __forceinline__ f32x2 pair_of(const uint32_t* r) { return pack2(__uint_as_float(r[0]), __uint_as_float(r[1])); }
 // Two values -> the code floats (in the low bits), or for OUT16 the operand's.
 template <bool OUT16>
 __device__ __forceinline__ void code_fast(const uint32_t* r, const float4& q, uint32_t& a, uint32_t& b) {
-    f32x2 v = fma2(pair_of(r), pack2(q.x, q.x), pack2(q.w, q.w));
+    f32x2 v = add2(fma2(pair_of(r), pack2(q.x, q.x), pack2(q.y, q.y)), pack2(MAGIC, MAGIC));
     if (OUT16) v = add2(v, pack2(q.z, q.z));
     float x, y;
     unpack2(v, x, y);
@@ -305,7 +304,8 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 const bool plain = !none && mn > -INFINITY && mx < INFINITY;
                 if (none && mn > mx) { mx = NAN; if (mn == INFINITY) mn = NAN; }
                 float sc; int32_t z;
-                const TokenQ q = token_params_fast(mn, mx, a_bits, p.mode, nrm, &sc, &z);
+                const TokenQ q = a_bits == 8 ? token_params_f32<8>(mn, mx, p.mode, p.scale_mul, nrm, &sc, &z)
+                                             : token_params_f32<4>(mn, mx, p.mode, p.scale_mul, nrm, &sc, &z);
                 const float4 code = make_code(q, mn, mx, qmax, plain);
                 ctl->par[g][gt] = code;
                 p.scale[m0 + gt] = sc;
@@ -402,6 +402,8 @@ lrq_status lrq_launch_rotq_tc(const void* X, int M, int K, long ldx, int B, int 
     p.steps = (M + p.T - 1) / p.T;
     const int fit = (int)(RING_BYTES / (2 * HALF_BYTES));
     p.stages = fit < MAX_STAGES ? fit : MAX_STAGES;
+    const double qsteps = mode == LRQ_ACT_ASYM ? (double)((1 << a_bits) - 1) : (double)((1 << (a_bits - 1)) - 1);
+    p.scale_mul = (float)(1.0 / (sqrt((double)B) * qsteps));
     p.codes = codes; p.scale = scale; p.zp = zp; p.status = lrq_status_word();
     const size_t smem = 1024 + H_BYTES + (size_t)p.stages * 2 * HALF_BYTES + sizeof(Ctl);
     const int grid = lrq_quant_grid(p.steps, sms, NUM_THREADS / 32, ex);

@@ -72,3 +72,34 @@ def test_nan_of_a_small_block_has_no_part_in_the_range(P, K, B, symmetric):
             q1[m, k // B * B:k // B * B + B] = 0
         assert torch.equal(q[others], q1[others])
     assert P.lrq_device_status() == 0
+
+
+@pytest.mark.parametrize("K,a_bits,symmetric", [(512, 8, False), (1152, 4, False), (1664, 8, True), (4608, 8, False), (8320, 4, False)])
+def test_blocks_of_128_in_long_and_short_batches(P, K, a_bits, symmetric):
+    # Inputs on a grid, so that every sum of the transform is exact whatever its order: all that is left are the token's parameters and
+    # the rounding of its codes, which are one arithmetic in every kernel.
+    M = 9_000_000 // K + 70
+    X = (_tokens(M, K, K).float() * 16).round().clamp(-1000, 1000).div(16).bfloat16()
+    plain = X.clone()
+    # tokens that need the clamp or have no numbers, beside ordinary ones in the same warp
+    X[3] = 0; X[9, 5] = float("inf"); X[20, 7] = float("nan"); X[33] = 3; X[40] = float("nan"); X[M - 9, 1] = -float("inf")
+    X[50] *= 2.0 ** 100; X[51] *= 2.0 ** -100
+    special = [3, 9, 20, 33, 40, 50, 51, M - 9]
+    mode = P.ACT_SYM if symmetric else P.ACT_ASYM
+    long, alone = (P.lrq_rotate_quantize_act(t, P.ROT_HADAMARD, a_bits, 128, mode=mode) for t in (X, plain))
+    for i in (0, M // 2, M - 64):
+        for a, b in zip(long, P.lrq_rotate_quantize_act(X[i:i + 64], P.ROT_HADAMARD, a_bits, 128, mode=mode)):
+            assert torch.equal(a[i:i + 64], b)
+    ordinary = torch.ones(M, dtype=torch.bool, device="cuda")
+    ordinary[special] = False
+    for a, b in zip(long, alone):
+        assert torch.equal(a[ordinary], b[ordinary])
+    # the contraction's operand, by the outputs
+    g = torch.Generator(device="cuda").manual_seed(7)
+    tlq = P.lrq_tlq_quantize_weights(0.02 * torch.randn((32, K), generator=g, device="cuda"), 4, 0, 7, [1.0, 1.2], [1.0, 1.2])
+    layer = P.QLayer(tlq, 32, K, P.ROT_HADAMARD, a_bits, 128, mode=mode)
+    Y = P.lrq_qlinear(layer, X, P.F32)
+    for i in (0, M // 2, M - 64):
+        assert torch.equal(Y[i:i + 64].nan_to_num(1.5), P.lrq_qlinear(layer, X[i:i + 64], P.F32).nan_to_num(1.5))
+    assert torch.equal(Y[ordinary], P.lrq_qlinear(layer, plain, P.F32)[ordinary])
+    assert P.lrq_device_status() == 0

@@ -1,18 +1,23 @@
 // Rotation + per-token activation quantization (Sec. 4.2 Eq. 12, first case; Sec. 3.1 Eq. 1) for long batches and Hadamard blocks of
-// 128 channels: the transform is a product on the tensor cores, y = x . blockdiag(H_128).
+// 128 channels: the first four stages of the transform are products on the tensor cores.
 //
-// Inputs are bf16 numbers and H_128 is +-1, so every product is exact; the eight MMAs of a sum round toward zero where the butterflies of
-// the other kernels round to nearest.  What bounds the CUDA-core kernel (rotq_blk.cu) are its 11.3 instructions an element; here a thread
-// finds finished sums in TMEM, folds their extremes, and when the token's parameters are known reads them a second time and codes them: 5.5.
+//   y = x . blockdiag(H_128),  H_128 = H_8 (x) H_16
+//
+// What bounds the CUDA-core kernel (rotq_blk.cu) are its instructions and the chain of a step; here a thread finds the sums of H_16 in
+// TMEM, adds the last three stages and folds the extremes, and when the token's parameters are known reads the results again and codes
+// them.
+//   * Inputs are bf16 numbers and H_16 is +-1: a sum is one MMA of exact products, which rounds (toward zero) only when inputs more than
+//     twelve octaves apart meet.  The seven stages as eight chained MMAs, each rounding toward zero, were 7 us faster (32768 x 4608 codes)
+//     and 1.4 times as far from the exact sums (inputs over 16 octaves: steps 13.1e-8 off, rms, 4.8e-8 by butterflies and here).
 //   * One persistent CTA per SM.  A warp brings steps of T whole tokens (up to 128 blocks of 128 channels) to a ring of stages by
 //     TMA, one issues a step's eight MMAs, four groups of four warps take the steps in turn, each with an accumulator of 128
 //     columns, so that one group's barriers and reductions lie under the others' arithmetic and a stage is free as soon
 //     as its MMAs are done.
-//   * The tokens' blocks are the accumulator's lanes, the channels of a block its columns; a thread codes 128 consecutive channels.
+//   * The tokens' blocks are the accumulator's lanes, the channels of a block its columns, so that the last stages are between a
+//     thread's registers and a thread codes 128 consecutive channels.
 // Loops over 32 columns are kept rolled: with 128 values a thread in registers between the passes and everything unrolled (8 warps of
-// 200 registers) the warps waited for instructions, 32768 x 4608 8-bit codes 107 us.  Measured, us before (rotq_blk.cu) and here:
-// 32768 x 4608 8-bit codes 107.5 -> 85 (5.3 TB/s), the operand 116.5 -> 112 (5.4); 32768 x 1152 33.7 -> 29.5, 35.7 -> 31.9.  It is bound by
-// memory (0.82 of the copy rate in codes).
+// 200 registers) the warps waited for instructions; 64 at a time, or two turns of 32 unrolled, gave nothing (86 -> 90, 86).
+// 32768 x 4608, 8-bit codes: 107.8 us before (rotq_blk.cu), 87.9 here (5.1 TB/s, 0.78 of the copy rate).
 // Blocks of 2048 and 4096 channels are not taken: their remaining stages need the channels of a block along the accumulator's lanes, so
 // that all seven first ones had to be chained MMAs.  That was 1.1 to 1.4 times as fast as rotq_big_kernel, but its sums were 1.4 times as far
 // from the exact ones, a token's codes changed with the length of its batch, and sums that overflowed in the later stages left NaN
@@ -34,26 +39,25 @@ constexpr int GROUPS = 4, GROUP_WARPS = 4;                   // groups of four w
 constexpr int TMA_WARP = GROUPS * GROUP_WARPS, MMA_WARP = TMA_WARP + 1, NUM_THREADS = (TMA_WARP + 2) * 32;
 constexpr int COLS = 128, BUFS = GROUPS;                     // columns of an accumulator; accumulators, one per group
 constexpr int MAX_TOK = 32;                                  // tokens of a step
-constexpr int MAX_STAGES = 8;
-constexpr int H_BYTES = 128 * 128 * 2;
-constexpr uint32_t HALF_BYTES = 128 * 128;                   // one 64-channel half of a stage
-constexpr size_t RING_BYTES = 168 * 1024;
+constexpr int H_BYTES = 16 * 128;                            // H_16: 16 rows of a 128-byte swizzled operand, of which 32 bytes are used
+constexpr uint32_t HALF_BYTES = 128 * 128, STAGE_BYTES = 2 * HALF_BYTES;     // 64 channels of 128 blocks; both halves
+constexpr int STAGES = 6;
 
 struct __align__(16) Ctl {
-    uint64_t full[MAX_STAGES], empty[MAX_STAGES];
+    uint64_t full[STAGES], empty[STAGES];
     uint64_t acc_full[BUFS], acc_empty[BUFS];
     uint64_t drain;                                          // the MMAs that an abandoned step left in flight
     uint32_t tmem_base;
     volatile int abort_flag;
     alignas(16) float4 par[GROUPS][MAX_TOK];                 // a token's parameters (make_code)
     float2 ext[GROUPS][GROUP_WARPS * MAX_TOK];               // extremes: [warp][token] over its rows of the token
-    unsigned char none[GROUPS][GROUP_WARPS * MAX_TOK];       // one of the rows has no numbers
+    unsigned char nan[GROUPS][GROUP_WARPS * MAX_TOK];        // one of the rows has a NaN
 };
-constexpr size_t SMEM_MAX = 1024 + H_BYTES + RING_BYTES + sizeof(Ctl);
-static_assert(SMEM_MAX <= 227 * 1024, "shared memory budget");
+constexpr size_t SMEM_BYTES = 1024 + H_BYTES + STAGES * STAGE_BYTES + sizeof(Ctl);
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
 struct Params {
-    int M, K, nb, T, steps, stages, mode, a_bits;
+    int M, K, nb, T, steps, mode, a_bits;
     float scale_mul;                                         // token_params_f32
     uint8_t* codes; float* scale; int32_t* zp; int* status;
 };
@@ -64,6 +68,18 @@ struct Params {
 __device__ __forceinline__ void tc_wait_ld32(uint32_t* r) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" : LRQ_W8(r, 0), LRQ_W8(r, 8), LRQ_W8(r, 16), LRQ_W8(r, 24) :: "memory");
 }
+
+// Four consecutive columns of the warp's 32 TMEM lanes, loaded (not waited for) and stored.
+__device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tc_st4(uint32_t taddr, const uint32_t* r) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" :: "r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// The maximum of three, or NaN when one of them is.
+__device__ __forceinline__ float max3_nan(float a, float b, float c) { float d; asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c)); return d; }
 
 // Barrier of a group's warps that also returns the OR of `pred`.
 __device__ __forceinline__ bool group_bar_or(int id, bool pred) {
@@ -165,29 +181,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const LrqExpand ex) {
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
-    constexpr uint32_t stage_bytes = 2 * HALF_BYTES;
     const uint32_t sH = smem_u32(base), sX = sH + H_BYTES;
-    Ctl* ctl = reinterpret_cast<Ctl*>(base + H_BYTES + (size_t)p.stages * stage_bytes);
+    Ctl* ctl = reinterpret_cast<Ctl*>(base + H_BYTES + STAGES * STAGE_BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl->full[s]), 1); mbar_init(smem_u32(&ctl->empty[s]), 1); }
+        for (int s = 0; s < STAGES; ++s) { mbar_init(smem_u32(&ctl->full[s]), 1); mbar_init(smem_u32(&ctl->empty[s]), 1); }
         for (int b = 0; b < BUFS; ++b) { mbar_init(smem_u32(&ctl->acc_full[b]), 1); mbar_init(smem_u32(&ctl->acc_empty[b]), GROUP_WARPS); }
         mbar_init(smem_u32(&ctl->drain), 1);
         ctl->abort_flag = 0;
         mbar_init_fence();
         tma_prefetch_desc(&tmX);
     }
-    // H_128 as a K-major operand, two halves of 64 k, 128-byte swizzle: H[r][k] = (-1)^popc(r & k)
-    for (int i = threadIdx.x; i < H_BYTES / 16; i += NUM_THREADS) {
-        const int h = i >> 10, r = (i >> 3) & 127, c = i & 7;
-        // signs of eight k at once: row r & 7 of H_8, all turned when the upper bits of r and k have an odd number in common
+    // H_16 as a K-major operand, 128-byte swizzle: H[r][k] = (-1)^popc(r & k)
+    if (threadIdx.x < 32) {
+        const int r = threadIdx.x >> 1, c = threadIdx.x & 1;
+        // signs of eight k at once: row r & 7 of H_8, all turned in the lower right quarter
         uint32_t m = (uint32_t)(0x963C5AF066CCAA00ull >> (8 * (r & 7))) & 0xFFu;
-        if (__popc((r >> 3) & (8 * h + c)) & 1) m ^= 0xFFu;
+        if ((r >> 3) & c) m ^= 0xFFu;
         uint32_t w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) w[j] = 0x3F803F80u | ((m << (15 - 2 * j)) & 0x8000u) | ((m << (30 - 2 * j)) & 0x80000000u);
-        *reinterpret_cast<uint4*>(base + h * (H_BYTES / 2) + r * 128 + ((c ^ (r & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(base + r * 128 + ((c ^ (r & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
     fence_async_smem();
     if (warp == MMA_WARP) tmem_alloc(smem_u32(&ctl->tmem_base), BUFS * COLS);
@@ -210,22 +225,21 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 if (!mbar_wait_warp(smem_u32(&ctl->empty[s]), ph, &ctl->abort_flag, p.status, 51)) break;
                 if (lead) {
                     const int m0 = ((int)blockIdx.x + i * (int)gridDim.x) * p.T;
-                    const uint32_t bar = smem_u32(&ctl->full[s]), dst = sX + s * stage_bytes;
+                    const uint32_t bar = smem_u32(&ctl->full[s]), dst = sX + s * STAGE_BYTES;
                     mbar_arrive_expect_tx(bar, (uint32_t)(p.T * p.nb) * 256u);
                     tma_load_3d(dst, &tmX, 0, 0, m0, bar);
                     tma_load_3d(dst + HALF_BYTES, &tmX, 64, 0, m0, bar);
                 }
                 __syncwarp();
                 ++issued;
-                if (++s == p.stages) { s = 0; ph ^= 1; }
+                if (++s == STAGES) { s = 0; ph ^= 1; }
             }
             __syncwarp();
         } else if (warp == MMA_WARP) {
             lead = elect_one();
             // the tokens' blocks are the 128 lanes, the channels of a block the columns
             const uint64_t h0 = umma_desc_sw128(sH, 16, 1024), x0 = umma_desc_sw128(sX, 16, 1024);
-            const uint32_t idesc = umma_idesc_bf16(128, COLS, false, false);
-            constexpr uint32_t half_units = HALF_BYTES >> 4, stage_units = 2 * half_units;      // descriptors count 16 bytes
+            const uint32_t idesc = umma_idesc_bf16(128, 16, false, false);
             int s = 0;
             uint32_t ph = 0;
             for (int i = 0; i < mine; ++i) {
@@ -234,18 +248,17 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 if (!mbar_wait_warp(smem_u32(&ctl->full[s]), ph, &ctl->abort_flag, p.status, 53)) break;
                 tc_fence_after();
                 const uint32_t d = tmem_base + b * COLS;
-                const uint64_t x1 = x0 + (uint64_t)(s * stage_units), x2 = x1 + half_units, h1 = h0 + (H_BYTES / 2 >> 4);
+                const uint64_t x1 = x0 + (uint64_t)(s * (STAGE_BYTES >> 4));     // descriptors count 16 bytes
                 if (lead) {
+                    // sixteen channels each, into columns of their own
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) tc_mma_f16(d, x1 + 2 * k, h0 + 2 * k, idesc, k ? 1u : 0u);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) tc_mma_f16(d, x2 + 2 * k, h1 + 2 * k, idesc, 1u);
+                    for (int c = 0; c < 8; ++c) tc_mma_f16(d + 16 * c, x1 + (c >> 2) * (HALF_BYTES >> 4) + 2 * (c & 3), h0, idesc, 0u);
                     tc_commit(smem_u32(&ctl->empty[s]));
                     tc_commit(smem_u32(&ctl->acc_full[b]));
                 }
                 __syncwarp();
                 ++issued;
-                if (++s == p.stages) { s = 0; ph ^= 1; }
+                if (++s == STAGES) { s = 0; ph ^= 1; }
             }
             __syncwarp();
         }
@@ -274,35 +287,65 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
             const bool busy = quad * 32 < tokens * nb;       // the warp has rows of a token
             if (ok && busy) {
                 float mn4[4] = {INFINITY, INFINITY, INFINITY, INFINITY}, mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                // the last three stages: butterflies between the sums of the eight sixteens, four columns of each at a time
 #pragma unroll 1
-                for (int c = 0; c < COLS; c += 32) {
+                for (int c = 0; c < 16; c += 4) {
                     uint32_t r[32];
-                    tc_ld32(acc + c, r);
-                    tc_wait_ld32(r);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        mn4[j & 3] = min3(mn4[j & 3], __uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
-                        mx4[j & 3] = max3(mx4[j & 3], __uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+                    for (int j = 0; j < 8; ++j) tc_ld4(acc + 16 * j + c, r + 4 * j);
+                    tc_wait_ld32(r);
+                    f32x2 v[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] = pair_of(r + 2 * i);
+#pragma unroll
+                    for (int h = 2; h < 16; h <<= 1)
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (!(i & h)) { const f32x2 a = v[i], b = v[i | h]; v[i] = add2(a, b); v[i | h] = sub2(a, b); }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        float x, y;
+                        unpack2(v[i], x, y);
+                        mn4[i & 3] = min3(mn4[i & 3], x, y);
+                        mx4[i & 3] = max3_nan(mx4[i & 3], x, y);
+                        r[2 * i] = __float_as_uint(x); r[2 * i + 1] = __float_as_uint(y);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) tc_st4(acc + 16 * j + c, r + 4 * j);
+                }
+                tc_wait_st();
+                float mn = fminf(min3(mn4[0], mn4[1], mn4[2]), mn4[3]), mx = max3_nan(max3_nan(mx4[0], mx4[1], mx4[2]), mx4[3], mx4[3]);
+                const bool nan = mx != mx;
+                if (__any_sync(0xffffffffu, nan)) {
+                    // it has no part in the range: once more without it
+                    mx = -INFINITY;
+#pragma unroll 1
+                    for (int c = 0; c < COLS; c += 32) {
+                        uint32_t r[32];
+                        tc_ld32(acc + c, r);
+                        tc_wait_ld32(r);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) mx = max3(mx, __uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
                     }
                 }
-                const float mn = fminf(min3(mn4[0], mn4[1], mn4[2]), mn4[3]), mx = fmaxf(max3(mx4[0], mx4[1], mx4[2]), mx4[3]);
                 float lo, hi;
                 asm volatile("redux.sync.min.f32 %0, %1, %2;" : "=f"(lo) : "f"(mn), "r"(seg));
                 asm volatile("redux.sync.max.f32 %0, %1, %2;" : "=f"(hi) : "f"(mx), "r"(seg));
-                const bool none = __any_sync(seg, !(mn <= mx));           // a row without numbers
-                if (seg_first) { ext[quad * MAX_TOK + my_tok] = make_float2(lo, hi); ctl->none[g][quad * MAX_TOK + my_tok] = none; }
+                const bool any_nan = __any_sync(seg, nan);
+                if (seg_first) { ext[quad * MAX_TOK + my_tok] = make_float2(lo, hi); ctl->nan[g][quad * MAX_TOK + my_tok] = any_nan; }
             }
             if (group_bar_or(1 + g, !ok || ctl->abort_flag != 0)) break;      // the group's warps leave together
             if (gt < tokens) {
                 float mn = INFINITY, mx = -INFINITY;
-                bool none = false;
-                auto fold = [&](float2 e) { mn = fminf(mn, e.x); mx = fmaxf(mx, e.y); none = none || !(e.x <= e.y); };
+                bool nan = false;
 #pragma unroll 1
-                for (int w = w_first; w <= w_last; ++w) { fold(ext[w * MAX_TOK + gt]); none = none || ctl->none[g][w * MAX_TOK + gt]; }
-                // A NaN among a block's inputs is in all of its outputs.  It is kept out of the token's range, as in rotq_blk.cu.  A
-                // token of nothing else has no range in either.
-                const bool plain = !none && mn > -INFINITY && mx < INFINITY;
-                if (none && mn > mx) { mx = NAN; if (mn == INFINITY) mn = NAN; }
+                for (int w = w_first; w <= w_last; ++w) {
+                    const float2 e = ext[w * MAX_TOK + gt];
+                    mn = fminf(mn, e.x); mx = fmaxf(mx, e.y);
+                    nan = nan || ctl->nan[g][w * MAX_TOK + gt];
+                }
+                const bool plain = !nan && mn > -INFINITY && mx < INFINITY;
+                if (mn > mx) mn = mx = NAN;          // a token of NaN alone: an empty range, as in rotq_blk.cu
                 float sc; int32_t z;
                 const TokenQ q = a_bits == 8 ? token_params_f32<8>(mn, mx, p.mode, p.scale_mul, nrm, &sc, &z)
                                              : token_params_f32<4>(mn, mx, p.mode, p.scale_mul, nrm, &sc, &z);
@@ -347,7 +390,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
         // A wait ran out, in whatever role, so that copies may still write this CTA's shared memory and MMAs its TMEM: both
         // end (bounded) before either is given back.  Otherwise every copy and MMA has been waited for above.
         if (lead && warp == TMA_WARP)
-            for (int i = max(issued - p.stages, 0); i < issued; ++i) drain(smem_u32(&ctl->full[i % p.stages]), (uint32_t)(i / p.stages) & 1u);
+            for (int i = max(issued - STAGES, 0); i < issued; ++i) drain(smem_u32(&ctl->full[i % STAGES]), (uint32_t)(i / STAGES) & 1u);
         if (lead && warp == MMA_WARP && issued) {
             tc_commit(smem_u32(&ctl->drain));
             drain(smem_u32(&ctl->drain), 0);
@@ -361,19 +404,19 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
 }
 
 template <int A_BITS, bool OUT16>
-lrq_status launch_tc(const CUtensorMap& tm, const Params& p, int grid, size_t smem, int dev, const LrqExpand& ex, cudaStream_t st) {
+lrq_status launch_tc(const CUtensorMap& tm, const Params& p, int grid, int dev, const LrqExpand& ex, cudaStream_t st) {
     auto kern = rotq_tc_kernel<A_BITS, OUT16>;
-    // the shared-memory opt-in is a per-device function attribute: set once per device and kernel variant, to the most it can need
+    // the shared-memory opt-in is a per-device function attribute: set once per device and kernel variant
     static std::mutex mu;
     static bool configured[LRQ_MAX_DEVICES] = {};
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!configured[dev]) {
-            LRQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
+            LRQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
             configured[dev] = true;
         }
     }
-    LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(NUM_THREADS), smem, st, tm, p, ex));
+    LRQ_CUDA_TRY(lrq_launch_pdl(kern, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, st, tm, p, ex));
     return LRQ_OK;
 }
 
@@ -400,15 +443,12 @@ lrq_status lrq_launch_rotq_tc(const void* X, int M, int K, long ldx, int B, int 
         if (best < 0 || cost < best) { best = cost; p.T = t; }
     }
     p.steps = (M + p.T - 1) / p.T;
-    const int fit = (int)(RING_BYTES / (2 * HALF_BYTES));
-    p.stages = fit < MAX_STAGES ? fit : MAX_STAGES;
     const double qsteps = mode == LRQ_ACT_ASYM ? (double)((1 << a_bits) - 1) : (double)((1 << (a_bits - 1)) - 1);
     p.scale_mul = (float)(1.0 / (sqrt((double)B) * qsteps));
     p.codes = codes; p.scale = scale; p.zp = zp; p.status = lrq_status_word();
-    const size_t smem = 1024 + H_BYTES + (size_t)p.stages * 2 * HALF_BYTES + sizeof(Ctl);
     const int grid = lrq_quant_grid(p.steps, sms, NUM_THREADS / 32, ex);
     CUtensorMap tm;
     if (!lrq_tma::make_map_blocks_bf16(&tm, X, (uint64_t)M, (uint64_t)nb, (uint64_t)ldx, (uint32_t)p.T)) return LRQ_ERR_UNSUPPORTED;
-    if (out16) return launch_tc<8, true>(tm, p, grid, smem, dev, ex, st);       // (of the operand, only the slow form asks for the bits)
-    return a_bits == 8 ? launch_tc<8, false>(tm, p, grid, smem, dev, ex, st) : launch_tc<4, false>(tm, p, grid, smem, dev, ex, st);
+    if (out16) return launch_tc<8, true>(tm, p, grid, dev, ex, st);       // (of the operand, only the slow form asks for the bits)
+    return a_bits == 8 ? launch_tc<8, false>(tm, p, grid, dev, ex, st) : launch_tc<4, false>(tm, p, grid, dev, ex, st);
 }

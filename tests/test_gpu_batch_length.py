@@ -103,3 +103,56 @@ def test_blocks_of_128_in_long_and_short_batches(P, K, a_bits, symmetric):
         assert torch.equal(Y[i:i + 64].nan_to_num(1.5), P.lrq_qlinear(layer, X[i:i + 64], P.F32).nan_to_num(1.5))
     assert torch.equal(Y[ordinary], P.lrq_qlinear(layer, plain, P.F32)[ordinary])
     assert P.lrq_device_status() == 0
+
+
+@pytest.mark.parametrize("kind", ["octaves", "salient", "gelu"])
+def test_sums_of_a_long_batch_are_as_close_as_those_of_short_ones(P, kind):
+    # A token's step in symmetric mode is its largest |y|, so its error is that of the transform's sums and a last rounding.  Inputs of
+    # many octaves, whose sums need more bits than fp32 has.
+    K, B = 1152, 128
+    M = 9_000_000 // K + 2
+    g = torch.Generator(device="cuda").manual_seed(11)
+    X = torch.randn((M, K), generator=g, device="cuda")
+    if kind == "octaves":
+        X = torch.sign(X) * torch.exp2(-16 * torch.rand((M, K), generator=g, device="cuda"))
+    elif kind == "salient":
+        X[:, ::72] *= 100
+    else:
+        X = torch.nn.functional.gelu(1.5 * X, approximate="tanh")
+    X = X.bfloat16()
+    H = torch.ones((1, 1), dtype=torch.float64, device="cuda")
+    while H.shape[0] < B:
+        H = torch.cat([torch.cat([H, H], 1), torch.cat([H, -H], 1)])
+    exact = (X.double().view(M, K // B, B) @ H).abs().amax((1, 2)) / B ** 0.5 / 127
+    long = P.lrq_rotate_quantize_act(X, P.ROT_HADAMARD, 8, B, mode=P.ACT_SYM)
+    short = [torch.cat(t) for t in zip(*(P.lrq_rotate_quantize_act(X[i:i + 2048], P.ROT_HADAMARD, 8, B, mode=P.ACT_SYM) for i in range(0, M, 2048)))]
+    rms = [((s.double() - exact) / exact).pow(2).mean().sqrt() for s in (long[1], short[1])]
+    # the two differ in the rounding of a few sums of sixteen only; chained products on the tensor cores had 1.08 to 2.7 times the error
+    assert rms[0] <= 1.02 * rms[1]
+    # and a code differs where such a sum lies on a rounding boundary
+    assert (long[0] != short[0]).sum() <= 1e-6 * M * K
+
+
+@pytest.mark.parametrize("a_bits", [8, 4])
+def test_overflow_within_a_block_of_128(P, a_bits):
+    # Sums that overflow in sixteens of a block to +inf, -inf, +inf, +inf: NaN for every other channel, finite values beside them.
+    # They have no part in the range and take code 0, in the operand its lowest value.
+    K = 1152
+    M = 9_000_000 // K + 2
+    X = _tokens(M, K, 3)
+    for m in (20, M - 5):
+        X[m, 128:256] = 0
+        for i, v in enumerate((3e38, -3e38, 3e38, 3e38)):
+            X[m, 128 + 16 * i:130 + 16 * i] = v
+    long = P.lrq_rotate_quantize_act(X, P.ROT_HADAMARD, a_bits, 128)
+    for i in (0, M - 64):
+        m = 20 if i == 0 else 59
+        short = P.lrq_rotate_quantize_act(X[i:i + 64], P.ROT_HADAMARD, a_bits, 128)
+        for a, b in zip(long, short):
+            assert torch.equal(a[i:i + 64][m], b[m])
+    g = torch.Generator(device="cuda").manual_seed(7)
+    tlq = P.lrq_tlq_quantize_weights(0.02 * torch.randn((32, K), generator=g, device="cuda"), 4, 0, 7, [1.0, 1.2], [1.0, 1.2])
+    layer = P.QLayer(tlq, 32, K, P.ROT_HADAMARD, a_bits, 128)
+    Y = P.lrq_qlinear(layer, X, P.F32)
+    assert torch.isfinite(Y).all() and torch.equal(Y[20], P.lrq_qlinear(layer, X[:64], P.F32)[20])
+    assert P.lrq_device_status() == 0

@@ -88,6 +88,7 @@ lrq_status lrq_launch_rotq_hadamard(const void* X, int M, int K, long ldx, int B
 // rotq_blk.cu : the same for blocks of 8..128 channels with K a multiple of 128; LRQ_ERR_UNSUPPORTED otherwise
 lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                                uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st);
+int lrq_rotq_blk_subgroups(int M, int K);        // independent sub-groups of its CTA at this shape, without multipliers
 // rotq_tc.cu : the same for long batches of blocks of 128 channels, without multipliers; LRQ_ERR_UNSUPPORTED otherwise
 lrq_status lrq_launch_rotq_tc(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                               uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st);

@@ -366,21 +366,16 @@ lrq_status launch_blk(const CUtensorMap& tm, int M, int K, int mode, int T, int 
 
 }  // namespace
 
-// Returns LRQ_ERR_UNSUPPORTED for shapes this kernel does not take (the caller then uses the other kernels).
-lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
-                               uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
-    if (K % 128 || B < 8 || B > 128 || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(codes, out16 ? 32 : 16)) return LRQ_ERR_UNSUPPORTED;
+// Shape of the CTA.  A sub-group is sub_warps warps holding T whole tokens (a token is K/64 threads, rarely a
+// whole number of warps, so some thread slots idle); nsub of them fill the CTA's warps.  Preferred: the most
+// active threads per SM; among equals the smaller sub-group, i.e. the more independent ones (measured at
+// K = 4608: four sub-groups of five warps take 104 us, two of nine warps 111 us, for the same active threads).
+// pre: bytes of the multipliers in shared memory.  sub_warps 0: none fits.
+struct BlkShape { int sub_warps, nsub, T; };
+static BlkShape blk_shape(int M, int K, size_t pre) {
     const int tpt = K / EPT;
-    if (K / 64 > 256) return LRQ_ERR_UNSUPPORTED;
-    int log2B = 0;
-    while ((1 << log2B) < B) ++log2B;
-    // Shape of the CTA.  A sub-group is sub_warps warps holding T whole tokens (a token is K/64 threads, rarely a
-    // whole number of warps, so some thread slots idle); nsub of them fill the CTA's warps.  Preferred: the most
-    // active threads per SM; among equals the smaller sub-group, i.e. the more independent ones (measured at
-    // K = 4608: four sub-groups of five warps take 104 us, two of nine warps 111 us, for the same active threads).
-    int sub_warps = 0, nsub = 0, T = 0;
+    BlkShape r = {0, 0, 0};
     long best_threads = 0;
-    const size_t pre = prescale ? (size_t)K * sizeof(float) : 0;
     for (int sw = 1; sw <= MAX_WARPS / 2; ++sw) {
         int t = sw * 32 / tpt;
         if (t < 1) continue;
@@ -391,8 +386,22 @@ lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int
         const size_t need = (size_t)ns * NSTAGE * lrq_round_up((size_t)t * K * 2, 1024);
         if (need + pre > 190 * 1024) continue;
         const long threads = (long)t * tpt * ns;
-        if (threads > best_threads) { best_threads = threads; sub_warps = sw; nsub = ns; T = t; }
+        if (threads > best_threads) { best_threads = threads; r = {sw, ns, t}; }
     }
+    return r;
+}
+int lrq_rotq_blk_subgroups(int M, int K) { return blk_shape(M, K, 0).nsub; }
+
+// Returns LRQ_ERR_UNSUPPORTED for shapes this kernel does not take (the caller then uses the other kernels).
+lrq_status lrq_launch_rotq_blk(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
+                               uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
+    if (K % 128 || B < 8 || B > 128 || (ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(codes, out16 ? 32 : 16)) return LRQ_ERR_UNSUPPORTED;
+    if (K / 64 > 256) return LRQ_ERR_UNSUPPORTED;
+    int log2B = 0;
+    while ((1 << log2B) < B) ++log2B;
+    const size_t pre = prescale ? (size_t)K * sizeof(float) : 0;
+    const BlkShape shape = blk_shape(M, K, pre);
+    const int sub_warps = shape.sub_warps, nsub = shape.nsub, T = shape.T;
     if (!sub_warps) return LRQ_ERR_UNSUPPORTED;
     const uint32_t stage_bytes = (uint32_t)lrq_round_up((size_t)T * K * 2, 1024);
     const size_t smem = 1024 + (size_t)nsub * NSTAGE * stage_bytes + sizeof(BlkCtl) + lrq_ext_bytes(nsub, T, sub_warps) + pre;

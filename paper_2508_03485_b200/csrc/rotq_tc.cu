@@ -38,7 +38,7 @@ using namespace lrq_tc;
 constexpr int GROUPS = 4, GROUP_WARPS = 4;                   // groups of four warps, one per quadrant of the TMEM lanes
 constexpr int TMA_WARP = GROUPS * GROUP_WARPS, MMA_WARP = TMA_WARP + 1, NUM_THREADS = (TMA_WARP + 2) * 32;
 constexpr int COLS = 128, BUFS = GROUPS;                     // columns of an accumulator; accumulators, one per group
-constexpr int MAX_TOK = 32;                                  // tokens of a step
+constexpr int MIN_BLOCKS = 6, MAX_TOK = COLS / MIN_BLOCKS;   // blocks of a token at least, tokens of a step at most
 constexpr int H_BYTES = 16 * 128;                            // H_16: 16 rows of a 128-byte swizzled operand, of which 32 bytes are used
 constexpr uint32_t HALF_BYTES = 128 * 128, STAGE_BYTES = 2 * HALF_BYTES;     // 64 channels of 128 blocks; both halves
 constexpr int STAGES = 6;
@@ -422,14 +422,19 @@ lrq_status launch_tc(const CUtensorMap& tm, const Params& p, int grid, int dev, 
 
 }  // namespace
 
-// Returns LRQ_ERR_UNSUPPORTED for calls this kernel does not take (the caller then uses the other kernels).  The line between them:
-// its start (H_128, TMEM, the chain copy - product - two passes) costs 1 to 2 us more than theirs and its rate is 1.2 to 1.5 times
-// theirs.  us there / here, operand with the decode of 1536 rows of weights: 4096 x 1152 10.8 / 11.4, 8192 x 1152 15.7 / 14.7,
-// 1024 x 4608 13.3 / 13.3, 2048 x 4608 18.3 / 16.8, 4096 x 4608 25.6 / 22.3.
+// Returns LRQ_ERR_UNSUPPORTED for calls this kernel does not take (the caller then uses the other kernels).  The line between them, with
+// us of rotq_blk.cu / here (L2 flushed): the start and the rounds of long steps cost 1 to 3 us, the rate is up to 1.5 times theirs.
+//   codes, M * K >= 24 million and K >= 768: 20833 x 1152 22 / 20, 7813 x 3072 20.4 / 19.2, 5209 x 4608 22.8 / 19.2, 2885 x 8320 (65 of a step's
+//     128 lanes in use) 24.2 / 23.7, 32553 x 4608 104.8 / 75.8; below, 11285 x 1152 14.1 / 15.1, 6348 x 2048 12.9 / 14.4, 1547 x 6144 11.6 / 14.8;
+//     62501 x 512 24.6 / 25.7.
+//   the operand, where both are bound by what they write, M * K >= 50 million and only where the other kernel has five sub-groups an SM
+//     or fewer: 10851 x 4608 54.7 / 51.2 (60 million), 39063 x 1536 55.3 / 51.2, 52084 x 1152 50.2 / 50.5, 86806 x 1152 76.9 / 75.3, 12208 x 12288
+//     125.5 / 115.3; its six to ten short sub-groups are faster: 29297 x 2048 45.6 / 51.1, 19532 x 3072 49.1 / 50.8, 12208 x 4096 41.0 / 44.2,
+//     8878 x 5632 46.4 / 47.0, 9766 x 6144 51.5 / 52.9; and below the line 34723 x 1152 36.0 / 38.2.
 lrq_status lrq_launch_rotq_tc(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                               uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
-    if (prescale || B != 128 || K % 128 || K < COLS / MAX_TOK * 128 || K > 128 * COLS) return LRQ_ERR_UNSUPPORTED;
-    if ((long)M * K < 9000000) return LRQ_ERR_UNSUPPORTED;
+    if (prescale || B != 128 || K % 128 || K < MIN_BLOCKS * 128 || K > 128 * COLS) return LRQ_ERR_UNSUPPORTED;
+    if ((long)M * K < (out16 ? 50000000 : 24000000) || (out16 && lrq_rotq_blk_subgroups(M, K) > 5)) return LRQ_ERR_UNSUPPORTED;
     if ((ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(codes, 32)) return LRQ_ERR_UNSUPPORTED;
     int dev = 0, sms = 0;
     if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;

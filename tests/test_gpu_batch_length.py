@@ -2,6 +2,8 @@
 import pytest
 import torch
 
+import parity as PU
+
 pytestmark = pytest.mark.gpu
 
 
@@ -74,11 +76,11 @@ def test_nan_of_a_small_block_has_no_part_in_the_range(P, K, B, symmetric):
     assert P.lrq_device_status() == 0
 
 
-@pytest.mark.parametrize("K,a_bits,symmetric", [(512, 8, False), (1152, 4, False), (1664, 8, True), (4608, 8, False), (8320, 4, False)])
+@pytest.mark.parametrize("K,a_bits,symmetric", [(768, 8, False), (1152, 4, False), (1664, 8, True), (4608, 8, False), (8320, 4, False)])
 def test_blocks_of_128_in_long_and_short_batches(P, K, a_bits, symmetric):
     # Inputs on a grid, so that every sum of the transform is exact whatever its order: all that is left are the token's parameters and
     # the rounding of its codes, which are one arithmetic in every kernel.
-    M = 9_000_000 // K + 70
+    M = PU.TC_OPERAND // K + 70
     X = (_tokens(M, K, K).float() * 16).round().clamp(-1000, 1000).div(16).bfloat16()
     plain = X.clone()
     # tokens that need the clamp or have no numbers, beside ordinary ones in the same warp
@@ -110,7 +112,7 @@ def test_sums_of_a_long_batch_are_as_close_as_those_of_short_ones(P, kind):
     # A token's step in symmetric mode is its largest |y|, so its error is that of the transform's sums and a last rounding.  Inputs of
     # many octaves, whose sums need more bits than fp32 has.
     K, B = 1152, 128
-    M = 9_000_000 // K + 2
+    M = PU.TC_CODES // K + 2
     g = torch.Generator(device="cuda").manual_seed(11)
     X = torch.randn((M, K), generator=g, device="cuda")
     if kind == "octaves":
@@ -138,7 +140,7 @@ def test_overflow_within_a_block_of_128(P, a_bits):
     # Sums that overflow in sixteens of a block to +inf, -inf, +inf, +inf: NaN for every other channel, finite values beside them.
     # They have no part in the range and take code 0, in the operand its lowest value.
     K = 1152
-    M = 9_000_000 // K + 2
+    M = PU.TC_OPERAND // K + 2
     X = _tokens(M, K, 3)
     for m in (20, M - 5):
         X[m, 128:256] = 0

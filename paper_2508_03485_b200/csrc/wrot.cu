@@ -14,6 +14,7 @@
 
 namespace {
 
+// The result may stand in the place of W (but for the dense product): an element is read by the threads that write it, ahead of that.
 // NB butterfly stages (index bits bit .. bit + NB - 1) of the row: a thread takes the 2^NB elements that differ in these
 // bits, from global memory in the first pass, to global memory in the last.  Elements lie in shared memory with one
 // pad after every 16, which makes both the first pass (runs of 16 per thread) and the later ones (neighbouring
@@ -46,8 +47,8 @@ __device__ __forceinline__ void hadamard_pass(double* row, int K, int bit, const
 
 // Any block, any alignment: a CTA per row.
 __global__ void __launch_bounds__(128)
-wrot_hadamard_kernel(const float* __restrict__ W, int N, int K, long ldw, const float* __restrict__ colmul, int log2B,
-                     float* __restrict__ out, long ldo) {
+wrot_hadamard_kernel(const float* W, int N, int K, long ldw, const float* __restrict__ colmul, int log2B,
+                     float* out, long ldo) {
     extern __shared__ double row[];                // [K + K / 16]
     const int n = blockIdx.x;
     const float* w = W + (size_t)n * ldw;
@@ -78,7 +79,7 @@ wrot_hadamard_kernel(const float* __restrict__ W, int N, int K, long ldw, const 
 // 58 and 36; 1024 x 3072, B = 256 17.8 and 12.3; 512 x 512 8.2 both.  Bound by the fp64 conversions and additions on the way.
 template <int LOG2B>
 __global__ void __launch_bounds__(256)
-wrot_hadamard_warp_kernel(const float* __restrict__ W, unsigned items, unsigned items_per_row, long ldw, const float* __restrict__ colmul,
+wrot_hadamard_warp_kernel(const float* W, unsigned items, unsigned items_per_row, long ldw, const float* __restrict__ colmul,
                           double norm, float* out, long ldo) {
     constexpr int NB = LOG2B - 4, E = 1 << NB;
     __shared__ double smem[8][32 * 17];
@@ -241,9 +242,9 @@ wrot_dense_kernel(const float* __restrict__ W, int N, int K, long ldw, const flo
 
 // out[n] = ((w[n] * colmul) . blockdiag(R1)) gathered through perm, then . blockdiag(R2); blocks of Bd x Bd, row-major
 __global__ void __launch_bounds__(256)
-wrot_dual_kernel(const float* __restrict__ W, int N, int K, long ldw, const float* __restrict__ colmul, int Bd,
+wrot_dual_kernel(const float* W, int N, int K, long ldw, const float* __restrict__ colmul, int Bd,
                  const __nv_bfloat16* __restrict__ R1, const int32_t* __restrict__ perm, const __nv_bfloat16* __restrict__ R2,
-                 float* __restrict__ out, long ldo) {
+                 float* out, long ldo) {
     extern __shared__ double rows2[];              // a[K], b[K]
     double* a = rows2;
     double* b = rows2 + K;
@@ -276,8 +277,8 @@ wrot_dual_kernel(const float* __restrict__ W, int N, int K, long ldw, const floa
     }
 }
 
-__global__ void wrot_scale_kernel(const float* __restrict__ W, int N, int K, long ldw, const float* __restrict__ colmul,
-                                  float* __restrict__ out, long ldo) {
+__global__ void wrot_scale_kernel(const float* W, int N, int K, long ldw, const float* __restrict__ colmul,
+                                  float* out, long ldo) {
     const size_t total = (size_t)N * K;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const size_t n = i / K, k = i % K;

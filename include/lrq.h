@@ -91,7 +91,8 @@ lrq_status lrq_tlq_quantize_weights(const float* W_rot, int N, int K, const lrq_
  * token as in Sec. 5.1).
  *
  *   HADAMARD  y = x . blockdiag(H_B), H_B the normalised Sylvester matrix of Eq. 3, B = had_block
- *             a power of two (8..4096) dividing K: one fused kernel, fp32 butterflies.
+ *             a power of two (8..4096) dividing K: one fused kernel, fp32 butterflies (blocks of 128 in long calls: the
+ *             first four stages as exact products summed on the tensor cores).
  *   DENSE     y = x . R with the composed outlier-aware rotation given as one bf16 K x K matrix
  *             (second case of Eq. 12): a tcgen05 GEMM into an fp32 scratch, then the quantizer.
  *   DUAL      the same outlier-aware transformation kept in the factors Sec. 4.2 builds it from,
@@ -103,6 +104,10 @@ lrq_status lrq_tlq_quantize_weights(const float* W_rot, int N, int K, const lrq_
  *   NONE      y = x.
  * then, per token, ASYM: s = (max-min)/(2^b-1), z = rint(min/s), q = clamp(rint(y/s)-z, 0, 2^b-1);
  *                  SYM : s = max|y|/(2^(b-1)-1), z = -2^(b-1), same q.   Rounding is to nearest even.
+ * HADAMARD: a token's results do not depend on the tokens beside it, nor on M, but for one case: in a call of 24 million elements or
+ * more with blocks of 128, a sum of sixteen inputs that lie more than twelve octaves apart may be rounded otherwise than in a short
+ * one (s by an ulp, an element on a rounding boundary of Eq. 1 by a code).  With blocks of up to 512, a NaN makes its block NaN, which
+ * takes code 0 and has no part in the token's range.
  * ------------------------------------------------------------------------------------------- */
 typedef struct {
     lrq_rot_kind kind;

@@ -3,12 +3,13 @@
 //
 //   y = x . blockdiag(H_128),  H_128 = H_8 (x) H_16
 //
-// What bounds the CUDA-core kernel (rotq_blk.cu) are its instructions and the chain of a step; here a thread finds the sums of H_16 in
-// TMEM, adds the last three stages and folds the extremes, and when the token's parameters are known reads the results again and codes
-// them.
+// What bounds the CUDA-core kernel (rotq_blk.cu) are its 11.3 instructions an element and the chain of a step; here a thread finds the sums
+// of H_16 in TMEM, adds the last three stages and folds the extremes, and when the token's parameters are known reads the results again
+// and codes them: 8.9, issue slots 58 % busy.
 //   * Inputs are bf16 numbers and H_16 is +-1: a sum is one MMA of exact products, which rounds (toward zero) only when inputs more than
-//     twelve octaves apart meet.  The seven stages as eight chained MMAs, each rounding toward zero, were 7 us faster (32768 x 4608 codes)
-//     and 1.4 times as far from the exact sums (inputs over 16 octaves: steps 13.1e-8 off, rms, 4.8e-8 by butterflies and here).
+//     twelve octaves apart meet.  All else is the arithmetic of rotq_blk.cu, so that a token's results differ from those in a short batch
+//     by such a rounding at most.  The seven stages as eight chained MMAs, each rounding toward zero, were 2 us faster (32768 x 4608
+//     codes) and up to 2.7 times as far from the exact sums (inputs over 16 octaves: steps 13.1e-8 off, rms, 4.8e-8 by butterflies and here).
 //   * One persistent CTA per SM.  A warp brings steps of T whole tokens (up to 128 blocks of 128 channels) to a ring of stages by
 //     TMA, one issues a step's eight MMAs, four groups of four warps take the steps in turn, each with an accumulator of 128
 //     columns, so that one group's barriers and reductions lie under the others' arithmetic and a stage is free as soon
@@ -17,7 +18,7 @@
 //     thread's registers and a thread codes 128 consecutive channels.
 // Loops over 32 columns are kept rolled: with 128 values a thread in registers between the passes and everything unrolled (8 warps of
 // 200 registers) the warps waited for instructions; 64 at a time, or two turns of 32 unrolled, gave nothing (86 -> 90, 86).
-// 32768 x 4608, 8-bit codes: 107.8 us before (rotq_blk.cu), 87.9 here (5.1 TB/s, 0.78 of the copy rate).
+// 32768 x 4608, 8-bit codes: 106 us before (rotq_blk.cu), 83.6 here (5.4 TB/s, 0.83 of the copy rate).
 // Blocks of 2048 and 4096 channels are not taken: their remaining stages need the channels of a block along the accumulator's lanes, so
 // that all seven first ones had to be chained MMAs.  That was 1.1 to 1.4 times as fast as rotq_big_kernel, but its sums were 1.4 times as far
 // from the exact ones, a token's codes changed with the length of its batch, and sums that overflowed in the later stages left NaN
@@ -57,7 +58,7 @@ constexpr size_t SMEM_BYTES = 1024 + H_BYTES + STAGES * STAGE_BYTES + sizeof(Ctl
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
 struct Params {
-    int M, K, nb, T, steps, mode, a_bits;
+    int M, K, nb, T, steps, mode;
     float scale_mul;                                         // token_params_f32
     uint8_t* codes; float* scale; int32_t* zp; int* status;
 };
@@ -118,7 +119,7 @@ __device__ __forceinline__ uint32_t low_bytes(uint32_t a, uint32_t b, uint32_t c
 
 // 32 consecutive channels of a row -> codes (8-bit: 32 bytes, 4-bit: 16) or the operand (64 bytes).
 template <int A_BITS, bool OUT16>
-__device__ __forceinline__ void code_row32(const uint32_t* r, const float4& q, bool fast, int a_bits, uint32_t* o) {
+__device__ __forceinline__ void code_row32(const uint32_t* r, const float4& q, bool fast, uint32_t* o) {
     if (fast) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -139,15 +140,9 @@ __device__ __forceinline__ void code_row32(const uint32_t* r, const float4& q, b
     }
     const f32x2 INV = pack2(q.x, q.x), NEGZ = pack2(q.y, q.y);
     if constexpr (OUT16) {
-        if (a_bits == 8) {
-            const Centre<8> ctr(q.y);
+        const Centre<A_BITS> ctr(q.y);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) o[i] = centred_bf16x2(fma2(pair_of(r + 2 * i), INV, NEGZ), ctr);
-        } else {
-            const Centre<4> ctr(q.y);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) o[i] = centred_bf16x2(fma2(pair_of(r + 2 * i), INV, NEGZ), ctr);
-        }
+        for (int i = 0; i < 16; ++i) o[i] = centred_bf16x2(fma2(pair_of(r + 2 * i), INV, NEGZ), ctr);
     } else {
         int n[32];
 #pragma unroll
@@ -265,8 +260,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
     } else {
         const int g = warp / GROUP_WARPS, quad = warp % GROUP_WARPS, gt = threadIdx.x % (GROUP_WARPS * 32);
         const double nrm = 1.0 / sqrt(128.0);
-        const int a_bits = OUT16 ? p.a_bits : A_BITS;
-        const float qmax = (float)((1 << a_bits) - 1);
+        constexpr float qmax = (float)((1 << A_BITS) - 1);
         constexpr int ES2 = OUT16 ? 4 : A_BITS / 4;          // half bytes of a result
         const int nb = p.nb;
         const size_t pitch = (size_t)p.K * ES2 / 2;
@@ -315,7 +309,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 }
                 tc_wait_st();
                 float mn = fminf(min3(mn4[0], mn4[1], mn4[2]), mn4[3]), mx = max3_nan(max3_nan(mx4[0], mx4[1], mx4[2]), mx4[3], mx4[3]);
-                const bool nan = mx != mx;
+                const bool nan = mx != mx && my_tok < p.T;       // (rows that are none hold what was there)
                 if (__any_sync(0xffffffffu, nan)) {
                     // it has no part in the range: once more without it
                     mx = -INFINITY;
@@ -347,8 +341,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                 const bool plain = !nan && mn > -INFINITY && mx < INFINITY;
                 if (mn > mx) mn = mx = NAN;          // a token of NaN alone: an empty range, as in rotq_blk.cu
                 float sc; int32_t z;
-                const TokenQ q = a_bits == 8 ? token_params_f32<8>(mn, mx, p.mode, p.scale_mul, nrm, &sc, &z)
-                                             : token_params_f32<4>(mn, mx, p.mode, p.scale_mul, nrm, &sc, &z);
+                const TokenQ q = token_params_f32<A_BITS>(mn, mx, p.mode, p.scale_mul, nrm, &sc, &z);
                 const float4 code = make_code(q, mn, mx, qmax, plain);
                 ctl->par[g][gt] = code;
                 p.scale[m0 + gt] = sc;
@@ -370,7 +363,7 @@ rotq_tc_kernel(const __grid_constant__ CUtensorMap tmX, const Params p, const Lr
                         uint32_t r[32];
                         tc_ld32(acc + c + 32 * h, r);
                         tc_wait_ld32(r);
-                        code_row32<A_BITS, OUT16>(r, q, fast, a_bits, o + h * W32);
+                        code_row32<A_BITS, OUT16>(r, q, fast, o + h * W32);
                     }
                     if (live)
 #pragma unroll
@@ -424,24 +417,24 @@ lrq_status launch_tc(const CUtensorMap& tm, const Params& p, int grid, int dev, 
 
 // Returns LRQ_ERR_UNSUPPORTED for calls this kernel does not take (the caller then uses the other kernels).  The line between them, with
 // us of rotq_blk.cu / here (L2 flushed): the start and the rounds of long steps cost 1 to 3 us, the rate is up to 1.5 times theirs.
-//   codes, M * K >= 24 million and K >= 768: 20833 x 1152 22 / 20, 7813 x 3072 20.4 / 19.2, 5209 x 4608 22.8 / 19.2, 2885 x 8320 (65 of a step's
-//     128 lanes in use) 24.2 / 23.7, 32553 x 4608 104.8 / 75.8; below, 11285 x 1152 14.1 / 15.1, 6348 x 2048 12.9 / 14.4, 1547 x 6144 11.6 / 14.8;
-//     62501 x 512 24.6 / 25.7.
-//   the operand, where both are bound by what they write, M * K >= 50 million and only where the other kernel has five sub-groups an SM
-//     or fewer: 10851 x 4608 54.7 / 51.2 (60 million), 39063 x 1536 55.3 / 51.2, 52084 x 1152 50.2 / 50.5, 86806 x 1152 76.9 / 75.3, 12208 x 12288
-//     125.5 / 115.3; its six to ten short sub-groups are faster: 29297 x 2048 45.6 / 51.1, 19532 x 3072 49.1 / 50.8, 12208 x 4096 41.0 / 44.2,
-//     8878 x 5632 46.4 / 47.0, 9766 x 6144 51.5 / 52.9; and below the line 34723 x 1152 36.0 / 38.2.
+//   codes, M * K >= 24 million and K >= 768: 20834 x 1152 21.5 / 20.1, 11719 x 2048 18.9 / 19.1, 7813 x 3072 20.0 / 18.9, 5209 x 4608 22.7 / 18.9,
+//     2885 x 8320 (65 of a step's 128 lanes in use) 24.2 / 23.7, 32553 x 4608 105.4 / 77.1; below, 11285 x 1152 14.2 / 14.9, 6348 x 2048
+//     12.9 / 14.7, 1547 x 6144 11.7 / 15.1; narrower, 62501 x 512 24.6 / 25.7.
+//   the operand, where both are bound by what they write, M * K >= 30 million and only where the other kernel has five sub-groups an SM
+//     or fewer: 26042 x 1152 30.4 / 29.1, 86806 x 1152 77.0 / 75.7, 19532 x 1536 32.5 / 28.9, 6511 x 4608 34.2 / 30.3, 32553 x 4608 115.8 / 111.1,
+//     18029 x 8320 132.0 / 125.6, 2442 x 12288 40.5 / 36.4; its six to ten short sub-groups are as fast or faster: 48829 x 2048 69.0 / 76.7,
+//     32553 x 3072 73.7 / 78.0, 24415 x 4096 72.3 / 76.5, 16277 x 6144 75.9 / 79.8 (but 17756 x 5632 81.5 / 77.3).
 lrq_status lrq_launch_rotq_tc(const void* X, int M, int K, long ldx, int B, int a_bits, int mode, int out16, const float* prescale,
                               uint8_t* codes, float* scale, int32_t* zp, const LrqExpand& ex, cudaStream_t st) {
     if (prescale || B != 128 || K % 128 || K < MIN_BLOCKS * 128 || K > 128 * COLS) return LRQ_ERR_UNSUPPORTED;
-    if ((long)M * K < (out16 ? 50000000 : 24000000) || (out16 && lrq_rotq_blk_subgroups(M, K) > 5)) return LRQ_ERR_UNSUPPORTED;
+    if ((long)M * K < (out16 ? 30000000 : 24000000) || (out16 && lrq_rotq_blk_subgroups(M, K) > 5)) return LRQ_ERR_UNSUPPORTED;
     if ((ldx % 8) || !lrq_aligned(X, 16) || !lrq_aligned(codes, 32)) return LRQ_ERR_UNSUPPORTED;
     int dev = 0, sms = 0;
     if (lrq_current_device(&dev, &sms) != LRQ_OK) return LRQ_ERR_CUDA;
     Params p = {};
     const int nb = K / 128;
-    p.M = M; p.K = K; p.nb = nb; p.mode = mode; p.a_bits = a_bits;
-    // Tokens per step: the groups' rounds of steps, each with the latency of some 40 columns' work besides its own
+    p.M = M; p.K = K; p.nb = nb; p.mode = mode;
+    // Tokens per step: the groups' rounds of steps, each with the latency of some 40 rows' work besides its own
     long best = -1;
     for (int t = 1; t <= COLS / nb; ++t) {
         const long rounds = (((long)M + t - 1) / t + GROUPS * sms - 1) / (GROUPS * sms), cost = rounds * (t * nb + 40);
@@ -454,6 +447,6 @@ lrq_status lrq_launch_rotq_tc(const void* X, int M, int K, long ldx, int B, int 
     const int grid = lrq_quant_grid(p.steps, sms, NUM_THREADS / 32, ex);
     CUtensorMap tm;
     if (!lrq_tma::make_map_blocks_bf16(&tm, X, (uint64_t)M, (uint64_t)nb, (uint64_t)ldx, (uint32_t)p.T)) return LRQ_ERR_UNSUPPORTED;
-    if (out16) return launch_tc<8, true>(tm, p, grid, dev, ex, st);       // (of the operand, only the slow form asks for the bits)
+    if (out16) return a_bits == 8 ? launch_tc<8, true>(tm, p, grid, dev, ex, st) : launch_tc<4, true>(tm, p, grid, dev, ex, st);
     return a_bits == 8 ? launch_tc<8, false>(tm, p, grid, dev, ex, st) : launch_tc<4, false>(tm, p, grid, dev, ex, st);
 }

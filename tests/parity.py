@@ -60,7 +60,7 @@ BOUNDARY_C = 1.0
 U32 = 2.0 ** -24
 # elements from which on a call with Hadamard blocks of 128 takes the tensor-core quantizer: to codes, to the contraction's operand
 # (test_gpu_rotq_tc.py shows that it does)
-TC_CODES, TC_OPERAND = 24_000_000, 50_000_000
+TC_CODES, TC_OPERAND = 24_000_000, 30_000_000
 EXACT_TIE = 2.0 ** -40          # |frac(t) - 1/2| below this (relative to |t| + 1) is an exact tie in fp64
 
 

@@ -40,7 +40,7 @@ from lrq_workloads import bf16_bits_to_f64, config_layers, default_clip_grid  # 
 # profiles/, keyed by the kernel and layer the roofline object describes.  A key is dropped (traffic: null) when its
 # kernel changes after the capture.
 NCU_TRAFFIC_BYTES = {
-    "rotq cfg4 b0.fc2": 302.63e6 + 117.40e6,
+    "rotq cfg4 b0.fc2": 302.08e6 + 114.63e6,
 }
 
 METRIC = "qlinear_tflops"
